@@ -51,7 +51,15 @@ long long gb_launches_so_far();
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    bool owned = true;
     int ensure(size_t nbytes);          // grow-only cudaMalloc
+    void lend(void *ptr, size_t nbytes) // use a piece of another allocation until it is outgrown
+    {
+        release();
+        p = ptr;
+        bytes = nbytes;
+        owned = false;
+    }
     void release();
     template <class T> T *as() const { return static_cast<T *>(p); }
     ~DevBuf() { release(); }
@@ -101,6 +109,20 @@ struct TileLists {
     DevBuf rec_entries;
     DevBuf rec_tptr;     // int [ntiles + 1]   receivers recorded by each tile
     DevBuf rec_list;     // int receiver ids, grouped by tile
+    // largest numbers of a tile: groups and entries of one source / of the receivers, receivers recorded
+    int src_most = 0, rec_most = 0, src_entries_most = 0, rec_entries_most = 0, recorded_most = 0;
+};
+
+// Tile of the resident time loop (sem_resident.cu) for one kind of pass and
+// number of shots; its injection groups pack the node as thread * 32 + q, q =
+// j * 5 + i the node of the thread's element that owns it.
+struct ResidentPlan {
+    int mode = 0, wanted = 0;
+    int NT = 0, TX = 0, TZ = 0, ntx = 0, ntz = 0;   // NT 0: the mesh does not fit
+    int per_launch = 0;                              // shots of which every tile is resident at once
+    int grp_cap = 0, ent_cap = 0, rec_cap = 0;       // most injected nodes, their entries and receivers of a tile
+    size_t smem = 0;
+    TileLists lists;
 };
 
 // ---------------------------------------------------------------------------
@@ -127,7 +149,7 @@ struct gbfwi_mesh {
     double dx_min = 0;                   // smallest GLL node spacing
 
     // device tables
-    DevBuf d_lm;        // float2 [nz][pitch]  (lambda, mu)
+    DevBuf d_lm;        // float2 [nz][pitch]  (lambda, mu) times the node's quadrature weight w_i w_j
     DevBuf d_minv;      // float  [nz][pitch]  1 / M
     DevBuf d_bnd;       // float4 [nz][pitch]  (Cx, Cz, 1/(M + dt/2 Cx), 1/(M + dt/2 Cz)); edges only
     DevBuf d_bw;        // float4 [nz][pitch]  (Wn_x, Wn_z, Wt_x, Wt_z) Stacey edge weights
@@ -153,6 +175,10 @@ struct gbfwi_mesh {
         ~Lane() { if (st) cudaStreamDestroy(st); }
     };
     std::vector<Lane *> lanes;
+    std::vector<ResidentPlan *> plans;  // of the resident time loop
+    DevBuf w_eacc;                      // its strain sums by element
+    DevBuf w_feat;                      // node-grid features of the learned preconditioner
+    DevBuf w_xch;                       // its exchange of node lines between tiles
     // CUDA graphs of whole forward / adjoint passes, keyed by schedule,
     // batch size and work-buffer addresses
     struct CachedGraph {
@@ -174,6 +200,8 @@ struct gbfwi_mesh {
 };
 
 int gb_build_tile_lists(gbfwi_mesh *m, int tile);
+// lists of the TX x TZ element tiling; per_thread: nodes packed for ResidentPlan
+int gb_build_lists(gbfwi_mesh *m, int TX, int TZ, bool per_thread, TileLists &L);
 // after the work on the mesh has completed: GBFWI_ETIMEOUT (and the flag
 // cleared) when a step kernel's bounded wait gave up since the last check
 int gb_take_status(gbfwi_mesh *m);
@@ -216,8 +244,50 @@ struct StepArgs {
     int *status;
 };
 
+// Arguments of a resident time loop: steps [n0, n1) of every shot of a batch.
+// Forward step n reads level n + 1 and writes n + 2; adjoint step n is
+// adjoint launch j = n of sem_driver.cu.
+struct ResidentArgs {
+    int nex, nez, nx, nz, pitch, nt;
+    float dt;
+    int TX, TZ, ntx, ntz, ntiles;
+    int n0, n1;
+    long long fstride;            // float2 elements between shots of every field
+    long long lev;                // between levels
+    const float2 *u0;             // level n0 + 1
+    float2 *vh;                   // half-step velocity, in place
+    float2 *out;                  // level k at slot k - out_k0 (out_ring: k % 3), written for k >= out_from
+    int out_from, out_ring, out_k0;
+    const float2 *hist; int hist_k0;   // adjoint: forward level k at slot k - hist_k0
+    const float2 *lm;             // (lambda, mu) times the quadrature weight
+    const float *minv;
+    const float4 *bnd;
+    const float *wxs, *wzs;       // 1-D quadrature weights
+    int free_top, edge_cap, grp_cap, ent_cap, rec_cap;
+    const int *gptr; const InjGroup *groups; const InjEntry *entries;
+    int per_shot_groups;
+    const float *sig; long long sig_shot_stride; int sig_chan_stride; float sig_scale;
+    const int *shot_map;
+    const int *rec_tptr, *rec_list; const float *recw; const int2 *rec_e;
+    float *seis; long long seis_shot_stride;
+    float *acc; long long acc_shot_stride; long long acc_comp_stride;
+    float *eacc;                  // adjoint: strain sums of every element, [shot][nez][nex][52] (25 points x 2)
+    void *xch; long long xslot, xstride;
+    int *status;
+};
+
+ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots);
+// acc components 0 and 1 of B shots from the elements' strain sums
+int gb_assemble_strain(const gbfwi_mesh *m, const float *eacc, int B, float *acc, long long acc_shot_stride, long long cs,
+                       cudaStream_t s);
+size_t gb_resident_exchange(const ResidentPlan &p, int nshots, long long NP);   // bytes of the exchange buffer
+int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf &xch, cudaStream_t s);
+
 int gb_launch_step(int mode, int tile, const StepArgs &a, int nbatch, cudaStream_t s);
 int gb_prepare_step(int mode, int tile);   // set kernel attributes outside any stream capture
+
+// node coordinates along one axis of ne elements (ne * 4 + 1 values, metres)
+std::vector<double> gb_axis(const gbfwi_mesh *m, int ne);
 
 // small kernels of the SEM driver
 int gb_material(gbfwi_mesh *m, cudaStream_t s);

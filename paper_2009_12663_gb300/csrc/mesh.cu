@@ -14,7 +14,7 @@
 
 #include "gbfwi_internal.h"
 
-int gb_upload_gll(const double *D, const double *w);
+int gb_upload_gll(const double *w);
 
 // ---------------------------------------------------------------------------
 // errors, buffers
@@ -36,6 +36,7 @@ gbfwi_mesh::~gbfwi_mesh()
     for (auto &g : graphs) cudaGraphExecDestroy(g.exec);
     if (cap_stream) cudaStreamDestroy(cap_stream);
     for (Lane *l : lanes) delete l;
+    for (ResidentPlan *p : plans) delete p;
 }
 
 extern "C" int gbfwi_enable_timing(gbfwi_mesh *m, int on)
@@ -84,9 +85,10 @@ int DevBuf::ensure(size_t nbytes)
 
 void DevBuf::release()
 {
-    if (p) cudaFree(p);
+    if (p && owned) cudaFree(p);
     p = nullptr;
     bytes = 0;
+    owned = true;
 }
 
 static_assert(cudaMemoryTypeUnregistered == GB_MEMTYPE_UNREGISTERED && cudaMemoryTypeHost == GB_MEMTYPE_HOST &&
@@ -165,7 +167,9 @@ static void lagrange_eval(const double c[5][5], double s, double l[5], double dl
         double v = 0, d = 0;
         for (int p = 4; p >= 0; --p) v = v * s + c[k][p];
         for (int p = 4; p >= 1; --p) d = d * s + p * c[k][p];
-        l[k] = v;
+        // at a node the other polynomials vanish: their 1e-16 of rounding would
+        // make an injected node of every node of the element
+        l[k] = std::fabs(v) < 1e-14 ? 0.0 : v;
         dl[k] = d;
     }
 }
@@ -288,10 +292,7 @@ extern "C" int gbfwi_mesh_create(const gbfwi_mesh_desc *desc, const gbfwi_source
         int dev = 0;
         cudaGetDevice(&dev);
         if (dev < 0 || dev >= 64 || !g_gll_done[dev]) {
-            double Df[25];
-            for (int i = 0; i < 5; ++i)
-                for (int k = 0; k < 5; ++k) Df[i * 5 + k] = m->D[i][k];
-            rc = gb_upload_gll(Df, m->w);
+            rc = gb_upload_gll(m->w);
             if (rc == GBFWI_OK && dev >= 0 && dev < 64) g_gll_done[dev] = true;
         }
     }
@@ -362,15 +363,24 @@ extern "C" int gbfwi_mesh_dims(const gbfwi_mesh *m, int *nx, int *nz)
     return GBFWI_OK;
 }
 
+std::vector<double> gb_axis(const gbfwi_mesh *m, int ne)
+{
+    std::vector<double> x(4 * (size_t)ne + 1);
+    for (size_t i = 0; i < x.size(); ++i) {
+        const int e = std::min((int)i / 4, ne - 1), k = (int)i - 4 * e;
+        x[i] = e * m->d.h + (1.0 + m->xi[k]) * m->d.h / 2.0;
+    }
+    return x;
+}
+
 extern "C" int gbfwi_node_coords(const gbfwi_mesh *m, double *x, double *z)
 {
     if (!m || !x || !z) return GBFWI_EINVAL;
+    const std::vector<double> X = gb_axis(m, m->d.nex), Z = gb_axis(m, m->d.nez);
     for (int iz = 0; iz < m->nz; ++iz)
         for (int ix = 0; ix < m->nx; ++ix) {
-            int ex = std::min(ix / 4, m->d.nex - 1), i = ix - 4 * ex;
-            int ez = std::min(iz / 4, m->d.nez - 1), j = iz - 4 * ez;
-            x[(size_t)iz * m->nx + ix] = ex * m->d.h + (1.0 + m->xi[i]) * m->d.h / 2.0;
-            z[(size_t)iz * m->nx + ix] = ez * m->d.h + (1.0 + m->xi[j]) * m->d.h / 2.0;
+            x[(size_t)iz * m->nx + ix] = X[ix];
+            z[(size_t)iz * m->nx + ix] = Z[iz];
         }
     return GBFWI_OK;
 }
@@ -441,11 +451,21 @@ int gb_build_tile_lists(gbfwi_mesh *m, int tile)
 {
     TileLists &L = m->lists[tile];
     if (L.built) return GBFWI_OK;
-    const int TX = kTiles[tile].tx, TZ = kTiles[tile].tz;
+    return gb_build_lists(m, kTiles[tile].tx, kTiles[tile].tz, false, L);
+}
+
+int gb_build_lists(gbfwi_mesh *m, int TX, int TZ, bool per_thread, TileLists &L)
+{
     L.ntx = (m->d.nex + TX - 1) / TX;
     L.ntz = (m->d.nez + TZ - 1) / TZ;
     const int ntiles = L.ntx * L.ntz;
     auto owner = [&](int ix, int iz, int &t, int &node) {
+        if (per_thread) {
+            const int ex = std::min(ix / 4, m->d.nex - 1), ez = std::min(iz / 4, m->d.nez - 1);
+            t = (ez / TZ) * L.ntx + ex / TX;
+            node = ((ez % TZ + 1) * (TX + 1) + ex % TX + 1) * 32 + (iz - 4 * ez) * 5 + ix - 4 * ex;
+            return;
+        }
         int tx = std::min(ix / (4 * TX), L.ntx - 1), tz = std::min(iz / (4 * TZ), L.ntz - 1);
         int ox = ix - 4 * TX * tx, oz = iz - 4 * TZ * tz;
         t = tz * L.ntx + tx;
@@ -503,6 +523,17 @@ int gb_build_tile_lists(gbfwi_mesh *m, int tile)
         return GBFWI_OK;
     };
     if (sgptr.empty()) sgptr.assign(ntiles + 1, 0);
+    auto most = [](const std::vector<int> &gp, const std::vector<InjGroup> &gr, size_t q, int &groups, int &entries) {
+        if (gp[q + 1] <= gp[q]) return;
+        groups = std::max(groups, gp[q + 1] - gp[q]);
+        entries = std::max(entries, gr[gp[q + 1] - 1].end - gr[gp[q]].begin);
+    };
+    for (size_t q = 0; q + 1 < sgptr.size(); ++q)
+        if ((q + 1) % (ntiles + 1)) most(sgptr, sgroups, q, L.src_most, L.src_entries_most);
+    for (int t = 0; t < ntiles; ++t) {
+        most(rgptr, rgroups, t, L.rec_most, L.rec_entries_most);
+        L.recorded_most = std::max(L.recorded_most, tcount[t + 1] - tcount[t]);
+    }
     GB_TRY(up(L.src_gptr, sgptr.data(), sgptr.size() * sizeof(int)));
     GB_TRY(up(L.src_groups, sgroups.data(), sgroups.size() * sizeof(InjGroup)));
     GB_TRY(up(L.src_entries, sentries.data(), sentries.size() * sizeof(InjEntry)));
@@ -541,7 +572,11 @@ __global__ void material_kernel(const float *__restrict__ model, const float *__
         float4 w = bw[g];
         float cx = rho * vp * w.x + rho * vs * w.z;
         float cz = rho * vp * w.y + rho * vs * w.w;
-        lm[g] = make_float2(lam, mu);
+        // (lambda, mu) times the quadrature weight w_i w_j of the node, which is
+        // the same in every element that shares it
+        const double w1[4] = {0.1, 49.0 / 90.0, 32.0 / 45.0, 49.0 / 90.0};
+        const float ww = (float)(w1[ix & 3] * w1[iz & 3]);
+        lm[g] = make_float2(ww * lam, ww * mu);
         minv[g] = 1.f / M;
         bnd[g] = make_float4(cx, cz, 1.f / (M + 0.5f * dt * cx), 1.f / (M + 0.5f * dt * cz));
     }

@@ -16,6 +16,7 @@
 // segment recomputed into C + 2 slots during the backward pass.
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <functional>
@@ -34,6 +35,16 @@ struct Ctx {
     cudaStream_t s;
     const int *d_shots;    // [B] source ids
     long long NP;          // nz * pitch
+    bool resident = false; // run each range of steps as one resident launch
+};
+
+// time levels of a field: level k at slot k - k0, or k % 3 of a ring
+struct Levels {
+    float2 *base = nullptr;
+    long long lev = 0;         // B * NP
+    int k0 = 0;
+    bool ring = false;
+    float2 *at(int k) const { return base + (long long)(ring ? k % 3 : k - k0) * lev; }
 };
 
 void base_args(StepArgs &a, const Ctx &c)
@@ -60,11 +71,49 @@ void base_args(StepArgs &a, const Ctx &c)
     a.status = m->w_status.as<int>();
 }
 
-using SlotFn = std::function<float2 *(int)>;
+// resident arguments shared by both directions
+void resident_args(ResidentArgs &r, const StepArgs &a, const Ctx &c, int n0, int n1, const Levels &f, int out_from)
+{
+    std::memset(&r, 0, sizeof(r));
+    r.nex = a.nex; r.nez = a.nez; r.nx = a.nx; r.nz = a.nz; r.pitch = a.pitch; r.nt = a.nt;
+    r.dt = a.dt;
+    r.n0 = n0; r.n1 = n1;
+    r.fstride = c.NP;
+    r.lev = f.lev;
+    r.u0 = f.at(n0 + 1);
+    r.vh = a.vh;
+    r.out = f.base;
+    r.out_from = out_from; r.out_ring = f.ring; r.out_k0 = f.k0;
+    r.lm = a.lm; r.minv = a.minv; r.bnd = a.bnd; r.wxs = a.wxs; r.wzs = a.wzs;
+    r.free_top = c.m->d.free_surface_top;
+    r.per_shot_groups = a.per_shot_groups;
+    r.sig = a.sig; r.sig_shot_stride = a.sig_shot_stride; r.sig_chan_stride = a.sig_chan_stride;
+    r.sig_scale = a.sig_scale;
+    r.shot_map = a.shot_map;
+    r.recw = a.recw; r.rec_e = a.rec_e;
+    r.seis = a.seis; r.seis_shot_stride = a.seis_shot_stride;
+    r.acc = a.acc; r.acc_shot_stride = a.acc_shot_stride; r.acc_comp_stride = a.acc_comp_stride;
+    r.status = a.status;
+}
 
-// forward launches n in [n0, n1)
-int fwd_range(const Ctx &c, int mode, int n0, int n1, const SlotFn &slot, float2 *vh, float *seis,
-              float *acc, long long acc_shot_stride, long long acc_comp_stride)
+int run_resident(const Ctx &c, int mode, ResidentArgs &r)
+{
+    ResidentPlan *p = gb_resident_plan(c.m, mode, c.B);
+    if (!p) return GBFWI_EINVAL;
+    const bool fwd = mode == MODE_FWD;
+    r.gptr = (fwd ? p->lists.src_gptr : p->lists.rec_gptr).as<int>();
+    r.groups = (fwd ? p->lists.src_groups : p->lists.rec_groups).as<InjGroup>();
+    r.entries = (fwd ? p->lists.src_entries : p->lists.rec_entries).as<InjEntry>();
+    r.rec_tptr = p->lists.rec_tptr.as<int>();
+    r.rec_list = p->lists.rec_list.as<int>();
+    return gb_launch_resident(*p, r, c.B, c.m->w_xch, c.s);
+}
+
+constexpr int kNoLevel = INT_MAX;
+
+// forward launches n in [n0, n1); `need`: first level that is read later
+int fwd_range(const Ctx &c, int mode, int n0, int n1, const Levels &f, int need, float2 *vh, float *seis, float *acc,
+              long long acc_shot_stride, long long acc_comp_stride)
 {
     StepArgs a;
     base_args(a, c);
@@ -82,10 +131,15 @@ int fwd_range(const Ctx &c, int mode, int n0, int n1, const SlotFn &slot, float2
     a.acc = acc;
     a.acc_shot_stride = acc_shot_stride;
     a.acc_comp_stride = acc_comp_stride;
+    if (c.resident && mode == MODE_FWD) {
+        ResidentArgs r;
+        resident_args(r, a, c, n0, n1, f, need);
+        return run_resident(c, mode, r);
+    }
     for (int n = n0; n < n1; ++n) {
-        a.ucur = slot(n + 1);
-        a.unext = slot(n + 2);
-        a.uold = slot(n);
+        a.ucur = f.at(n + 1);
+        a.unext = f.at(n + 2);
+        a.uold = f.at(n);
         a.tsig = n + 1;
         a.trec = n;
         GB_TRY(gb_launch_step(mode, c.tile, a, c.B, c.s));
@@ -93,8 +147,8 @@ int fwd_range(const Ctx &c, int mode, int n0, int n1, const SlotFn &slot, float2
     return GBFWI_OK;
 }
 
-// adjoint launches j in [j0, j1); the adjoint field cycles through wring[3]
-int adj_range(const Ctx &c, int mode, int j0, int j1, float2 *wring, float2 *wh, const SlotFn &hist,
+// adjoint launches j in [j0, j1); the adjoint field cycles through the ring w
+int adj_range(const Ctx &c, int mode, int j0, int j1, const Levels &w, float2 *wh, const Levels &hist,
               const float *sig, float *acc, long long acc_shot_stride, long long acc_comp_stride)
 {
     const int nt = c.m->d.nt;
@@ -113,18 +167,25 @@ int adj_range(const Ctx &c, int mode, int j0, int j1, float2 *wring, float2 *wh,
     a.acc = acc;
     a.acc_shot_stride = acc_shot_stride;
     a.acc_comp_stride = acc_comp_stride;
-    const long long lev = (long long)c.B * c.NP;
+    if (c.resident && mode == MODE_ADJ_G) {
+        ResidentArgs r;
+        resident_args(r, a, c, j0, j1, w, j1 < nt ? j1 : kNoLevel);
+        r.hist = hist.base;
+        r.hist_k0 = hist.k0;
+        r.eacc = c.m->w_eacc.as<float>();
+        return run_resident(c, mode, r);
+    }
     for (int j = j0; j < j1; ++j) {
         int k = nt - j;
-        a.ucur = wring + ((j + 1) % 3) * lev;
-        a.unext = wring + ((j + 2) % 3) * lev;
-        a.uold = wring + (j % 3) * lev;
+        a.ucur = w.at(j + 1);
+        a.unext = w.at(j + 2);
+        a.uold = w.at(j);
         if (mode == MODE_ADJ_G) {
-            a.h0 = hist(k);
+            a.h0 = hist.at(k);
         } else {
-            a.h0 = hist(k + 1);
-            a.h1 = hist(k);
-            a.h2 = hist(k - 1);
+            a.h0 = hist.at(k + 1);
+            a.h1 = hist.at(k);
+            a.h2 = hist.at(k - 1);
         }
         a.tsig = nt - 1 - j;
         GB_TRY(gb_launch_step(mode, c.tile, a, c.B, c.s));
@@ -227,7 +288,9 @@ __global__ void chain_kernel(const float *__restrict__ tot, const float *__restr
          q += (long long)gridDim.x * blockDim.x) {
         int iz = (int)(q / nx), ix = (int)(q - (long long)iz * nx);
         long long g = (long long)iz * pitch + ix;
-        float gl = tot[g], gm = tot[NP + g], gp = tot[3 * NP + g], gs = tot[4 * NP + g];
+        const double w1[4] = {0.1, 49.0 / 90.0, 32.0 / 45.0, 49.0 / 90.0};
+        const float ww = (float)(w1[ix & 3] * w1[iz & 3]);    // quadrature weight of the strain correlations
+        float gl = ww * tot[g], gm = ww * tot[NP + g], gp = tot[3 * NP + g], gs = tot[4 * NP + g];
         float gM = wx[ix] * wz[iz] * tot[2 * NP + g];
         float r = model[g], p = model[NP + g], s = model[2 * NP + g];
         float grho = gl * (p * p - 2.f * s * s) + gm * s * s + gM + gp * p + gs * s;
@@ -380,14 +443,22 @@ int check_shots(const gbfwi_mesh *m, const int *shot_ids, int nshot)
     return GBFWI_OK;
 }
 
-// history layout for one batch
-struct History {
-    float2 *base = nullptr;    // [slots][B][NP]
-    int slots = 0;
-    int kbase = 0;             // time level held by slot 0
-    long long lev = 0;         // B * NP
-    float2 *at(int k) const { return base + (long long)(k - kbase) * lev; }
-};
+// the exchange buffer of the resident loop (before any work is queued)
+int reserve_exchange(gbfwi_mesh *m, int mode, int B, long long NP)
+{
+    ResidentPlan *p = gb_resident_plan(m, mode, B);
+    return p ? m->w_xch.ensure(gb_resident_exchange(*p, B, NP)) : GBFWI_EINVAL;
+}
+
+// Shots advanced together by forward runs that keep no history, and whether
+// as resident launches: the resident loop takes as many shots as fit the SMs
+// at once (three levels and a velocity each), the step kernels the schedule's.
+int forward_batch(gbfwi_mesh *m, int nshot, bool &resident)
+{
+    ResidentPlan *p = gb_resident_plan(m, MODE_FWD, nshot);
+    resident = p != nullptr;
+    return std::min(nshot, p ? std::max(p->per_launch, m->sch.shots_per_launch) : m->sch.shots_per_launch);
+}
 
 }  // namespace
 
@@ -406,9 +477,11 @@ extern "C" int gbfwi_forward(gbfwi_mesh *m, const int *shot_ids, int nshot, floa
     GB_TRY(gb_build_tile_lists(m, tile));
     const int nt = m->d.nt;
     const long long NP = (long long)m->nz * m->pitch;
-    const int Bmax = std::min(m->sch.shots_per_launch, nshot);
+    bool resident = false;
+    const int Bmax = forward_batch(m, nshot, resident);
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
     const bool dev_out = gb_is_device_ptr(seis);
+    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, Bmax, NP));
     GB_TRY(m->w_hist.ensure((size_t)3 * Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
@@ -416,14 +489,12 @@ extern "C" int gbfwi_forward(gbfwi_mesh *m, const int *shot_ids, int nshot, floa
     GB_CUDA(cudaMemcpyAsync(m->w_shots.p, shot_ids, nshot * sizeof(int), cudaMemcpyHostToDevice, s));
     for (int i0 = 0; i0 < nshot; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
-        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP};
-        float2 *ring = m->w_hist.as<float2>();
-        long long lev = (long long)B * NP;
-        GB_CUDA(cudaMemsetAsync(ring, 0, 3 * lev * sizeof(float2), s));
-        GB_CUDA(cudaMemsetAsync(m->w_vh.p, 0, lev * sizeof(float2), s));
+        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, resident};
+        const Levels ring{m->w_hist.as<float2>(), (long long)B * NP, 0, true};
+        GB_CUDA(cudaMemsetAsync(ring.base, 0, 3 * ring.lev * sizeof(float2), s));
+        GB_CUDA(cudaMemsetAsync(m->w_vh.p, 0, ring.lev * sizeof(float2), s));
         float *out = dev_out ? seis + seis_shot * i0 : m->w_seis.as<float>();
-        SlotFn slot = [&](int k) { return ring + (long long)(k % 3) * lev; };
-        GB_TRY(fwd_range(c, MODE_FWD, 0, nt, slot, m->w_vh.as<float2>(), out, nullptr, 0, 0));
+        GB_TRY(fwd_range(c, MODE_FWD, 0, nt, ring, kNoLevel, m->w_vh.as<float2>(), out, nullptr, 0, 0));
         if (!dev_out)
             GB_CUDA(cudaMemcpyAsync(seis + seis_shot * i0, out, seis_shot * B * sizeof(float),
                                     cudaMemcpyDeviceToHost, s));
@@ -451,8 +522,10 @@ extern "C" int gbfwi_misfit(gbfwi_mesh *m, const int *shot_ids, int nshot, const
     GB_TRY(gb_build_tile_lists(m, tile));
     const int nt = m->d.nt;
     const long long NP = (long long)m->nz * m->pitch;
-    const int Bmax = std::min(m->sch.shots_per_launch, nshot);
+    bool resident = false;
+    const int Bmax = forward_batch(m, nshot, resident);
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
+    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, Bmax, NP));
     GB_TRY(m->w_hist.ensure((size_t)3 * Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
@@ -470,14 +543,12 @@ extern "C" int gbfwi_misfit(gbfwi_mesh *m, const int *shot_ids, int nshot, const
     GB_CUDA(cudaMemsetAsync(flag, 0, 16, s));
     for (int i0 = 0; i0 < nshot; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
-        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP};
-        float2 *ring = m->w_hist.as<float2>();
-        long long lev = (long long)B * NP;
-        GB_CUDA(cudaMemsetAsync(ring, 0, 3 * lev * sizeof(float2), s));
-        GB_CUDA(cudaMemsetAsync(m->w_vh.p, 0, lev * sizeof(float2), s));
-        SlotFn slot = [&](int k) { return ring + (long long)(k % 3) * lev; };
+        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, resident};
+        const Levels ring{m->w_hist.as<float2>(), (long long)B * NP, 0, true};
+        GB_CUDA(cudaMemsetAsync(ring.base, 0, 3 * ring.lev * sizeof(float2), s));
+        GB_CUDA(cudaMemsetAsync(m->w_vh.p, 0, ring.lev * sizeof(float2), s));
         float *seis_d = m->w_seis.as<float>();
-        GB_TRY(fwd_range(c, MODE_FWD, 0, nt, slot, m->w_vh.as<float2>(), seis_d, nullptr, 0, 0));
+        GB_TRY(fwd_range(c, MODE_FWD, 0, nt, ring, kNoLevel, m->w_vh.as<float2>(), seis_d, nullptr, 0, 0));
         residual_kernel<<<dim3(kMisfitBlocks, B), 256, 0, s>>>(seis_d, (const float *)obs_d + seis_shot * i0,
                                                               (long long)seis_shot, partial, flag);
         GB_LAUNCHED();
@@ -502,7 +573,7 @@ extern "C" int gbfwi_misfit(gbfwi_mesh *m, const int *shot_ids, int nshot, const
 namespace {
 
 struct BatchHist {
-    History full;              // ckpt == 0
+    Levels full;               // ckpt == 0
     float2 *ring = nullptr;    // ckpt > 0: 3-slot ring for the forward pass
     float2 *seg = nullptr;     // ckpt > 0: C + 2 slots
     float2 *snap = nullptr;    // ckpt > 0: [nseg][3][B][NP]: u_{sC}, u_{sC+1}, vh_{sC}
@@ -512,6 +583,10 @@ struct BatchHist {
     float2 *wh = nullptr;      // adjoint half-step velocity
     int C = 0, nseg = 0;
 };
+
+// Bytes of forward levels a gradient may keep beyond what its schedule asks
+// for, to run more shots at once on meshes too small to fill the GPU.
+constexpr long long kSmallHistory = 1LL << 30;
 
 // the work buffers of one concurrent lane
 struct LaneRef {
@@ -530,10 +605,7 @@ int alloc_hist(gbfwi_mesh *m, const LaneRef &L, int B, int ckpt, long long NP, B
     long long lev = (long long)B * NP;
     if (ckpt <= 0 || ckpt >= nt) {
         GB_TRY(L.hist->ensure((size_t)(nt + 2) * lev * sizeof(float2)));
-        h.full.base = L.hist->as<float2>();
-        h.full.slots = nt + 2;
-        h.full.kbase = 0;
-        h.full.lev = lev;
+        h.full = Levels{L.hist->as<float2>(), lev, 0, false};
         h.C = 0;
     } else {
         h.C = ckpt;
@@ -567,18 +639,17 @@ int forward_pass(const Ctx &c, BatchHist &h, float *seis)
     GB_CUDA(cudaMemsetAsync(vh, 0, lev * sizeof(float2), c.s));
     if (h.C == 0) {
         GB_CUDA(cudaMemsetAsync(h.full.base, 0, 2 * lev * sizeof(float2), c.s));
-        SlotFn slot = [&](int k) { return h.full.at(k); };
-        return fwd_range(c, MODE_FWD, 0, nt, slot, vh, seis, nullptr, 0, 0);
+        return fwd_range(c, MODE_FWD, 0, nt, h.full, 0, vh, seis, nullptr, 0, 0);
     }
     GB_CUDA(cudaMemsetAsync(h.ring, 0, 3 * lev * sizeof(float2), c.s));
-    SlotFn slot = [&](int k) { return h.ring + (long long)(k % 3) * lev; };
+    const Levels ring{h.ring, lev, 0, true};
     for (int sg = 0; sg < h.nseg; ++sg) {
         int n0 = sg * h.C, n1 = std::min(nt, n0 + h.C);
         float2 *sp = h.snap + (long long)sg * 3 * lev;
-        GB_CUDA(cudaMemcpyAsync(sp, slot(n0), lev * sizeof(float2), cudaMemcpyDeviceToDevice, c.s));
-        GB_CUDA(cudaMemcpyAsync(sp + lev, slot(n0 + 1), lev * sizeof(float2), cudaMemcpyDeviceToDevice, c.s));
+        GB_CUDA(cudaMemcpyAsync(sp, ring.at(n0), lev * sizeof(float2), cudaMemcpyDeviceToDevice, c.s));
+        GB_CUDA(cudaMemcpyAsync(sp + lev, ring.at(n0 + 1), lev * sizeof(float2), cudaMemcpyDeviceToDevice, c.s));
         GB_CUDA(cudaMemcpyAsync(sp + 2 * lev, vh, lev * sizeof(float2), cudaMemcpyDeviceToDevice, c.s));
-        GB_TRY(fwd_range(c, MODE_FWD, n0, n1, slot, vh, seis, nullptr, 0, 0));
+        GB_TRY(fwd_range(c, MODE_FWD, n0, n1, ring, n1 < nt ? n1 : kNoLevel, vh, seis, nullptr, 0, 0));
     }
     return GBFWI_OK;
 }
@@ -590,26 +661,24 @@ int adjoint_pass(const Ctx &c, BatchHist &h, int mode, const float *sig, float *
     gbfwi_mesh *m = c.m;
     const int nt = m->d.nt;
     const long long lev = (long long)c.B * c.NP;
-    float2 *wring = h.wring;
+    const Levels wring{h.wring, lev, 0, true};
     float2 *wh = h.wh;
-    GB_CUDA(cudaMemsetAsync(wring, 0, 3 * lev * sizeof(float2), c.s));
+    GB_CUDA(cudaMemsetAsync(h.wring, 0, 3 * lev * sizeof(float2), c.s));
     GB_CUDA(cudaMemsetAsync(wh, 0, lev * sizeof(float2), c.s));
     if (h.C == 0) {
-        SlotFn hist = [&](int k) { return h.full.at(k); };
-        return adj_range(c, mode, 0, nt, wring, wh, hist, sig, acc, acc_shot_stride, acc_comp_stride);
+        return adj_range(c, mode, 0, nt, wring, wh, h.full, sig, acc, acc_shot_stride, acc_comp_stride);
     }
     for (int sg = h.nseg - 1; sg >= 0; --sg) {
         int n0 = sg * h.C, n1 = std::min(nt, n0 + h.C);
         float2 *sp = h.snap + (long long)sg * 3 * lev;
-        History seg{h.seg, h.C + 2, n0, lev};
+        const Levels seg{h.seg, lev, n0, false};
         GB_CUDA(cudaMemcpyAsync(seg.at(n0), sp, lev * sizeof(float2), cudaMemcpyDeviceToDevice, c.s));
         GB_CUDA(cudaMemcpyAsync(seg.at(n0 + 1), sp + lev, lev * sizeof(float2), cudaMemcpyDeviceToDevice, c.s));
         GB_CUDA(cudaMemcpyAsync(h.vh_rec, sp + 2 * lev, lev * sizeof(float2), cudaMemcpyDeviceToDevice, c.s));
-        SlotFn slot = [&](int k) { return seg.at(k); };
-        GB_TRY(fwd_range(c, MODE_FWD, n0, n1, slot, h.vh_rec, nullptr, nullptr, 0, 0));
+        GB_TRY(fwd_range(c, MODE_FWD, n0, n1, seg, 0, h.vh_rec, nullptr, nullptr, 0, 0));
         // adjoint launches whose correlation level k lies in [n0 + 1, n1]
         int j0 = nt - n1, j1 = nt - n0;
-        GB_TRY(adj_range(c, mode, j0, j1, wring, wh, slot, sig, acc, acc_shot_stride, acc_comp_stride));
+        GB_TRY(adj_range(c, mode, j0, j1, wring, wh, seg, sig, acc, acc_shot_stride, acc_comp_stride));
     }
     return GBFWI_OK;
 }
@@ -617,9 +686,9 @@ int adjoint_pass(const Ctx &c, BatchHist &h, int mode, const float *sig, float *
 // Run body() on the caller's stream s, or, with graphs enabled, replay a CUDA
 // graph of it captured once on a private stream (the caller's stream may be
 // the legacy default stream, which cannot be captured).
-int run_pass(gbfwi_mesh *m, const std::string &key, cudaStream_t s, const std::function<int(cudaStream_t)> &body)
+int run_pass(gbfwi_mesh *m, bool replay, const std::string &key, cudaStream_t s, const std::function<int(cudaStream_t)> &body)
 {
-    if (!m->sch.use_graph) return body(s);
+    if (!replay || !m->sch.use_graph) return body(s);
     for (auto &g : m->graphs)
         if (g.key == key) {
             GB_CUDA(cudaGraphLaunch(g.exec, s));
@@ -695,10 +764,24 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
     const int ckpt = ckpt_every >= 0 ? ckpt_every : m->sch.ckpt_every;
     const long long NP = (long long)m->nz * m->pitch;
     const long long N = (long long)m->nz * m->nx;
-    const int Bmax = std::min(m->sch.shots_per_launch, nshot);
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
+    // Resident loops: one lane whose batch holds the shots the schedule keeps in
+    // flight (shots per launch x streams), or more while their histories stay small
+    const bool full = ckpt <= 0 || ckpt >= nt;
+    const long long levels = full ? nt + 2 : 3LL * ((nt + ckpt - 1) / ckpt) + ckpt + 6;
+    const long long small = kSmallHistory / (levels * NP * (long long)sizeof(float2));
+    int Bmax = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
+    const bool resident = gb_resident_plan(m, MODE_FWD, Bmax) && gb_resident_plan(m, MODE_ADJ_G, Bmax);
+    if (!resident) Bmax = std::min(m->sch.shots_per_launch, nshot);
     const int nbatch = (nshot + Bmax - 1) / Bmax;
-    const int L = std::max(1, std::min(m->sch.streams, nbatch));
+    const int L = resident ? 1 : std::max(1, std::min(m->sch.streams, nbatch));
+    const size_t eacc_shot = (size_t)m->d.nex * m->d.nez * 52 * sizeof(float);
+    if (resident) GB_TRY(m->w_eacc.ensure(eacc_shot * Bmax));
+    if (resident)
+        for (int B : {Bmax, nshot - (nbatch - 1) * Bmax}) {
+            GB_TRY(reserve_exchange(m, MODE_FWD, B, NP));
+            GB_TRY(reserve_exchange(m, MODE_ADJ_G, B, NP));
+        }
 
     // lanes: 0 = the mesh's own buffers on the caller's stream, 1.. = extra streams
     while ((int)m->lanes.size() < L - 1) m->lanes.push_back(new gbfwi_mesh::Lane());
@@ -773,7 +856,7 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
             // this batch's source ids at a fixed address, so captured passes replay for every batch
             GB_CUDA(cudaMemcpyAsync(lr.batch->p, m->w_shots.as<int>() + i0, B * sizeof(int),
                                     cudaMemcpyDeviceToDevice, ls));
-            Ctx c{m, &m->lists[tile], tile, B, ls, lr.batch->as<int>(), NP};
+            Ctx c{m, &m->lists[tile], tile, B, ls, lr.batch->as<int>(), NP, resident};
             float *seis_d = lr.seis->as<float>();
             float *acc = lr.acc->as<float>();
             const std::string kf = pass_key("fwd", m, B, h.C, {lr.hist->p, lr.vh->p, lr.seis->p, lr.snap->p,
@@ -781,7 +864,7 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
             const std::string ka = pass_key("adj", m, B, h.C, {lr.hist->p, lr.seis->p, lr.snap->p, lr.adj->p,
                                                                lr.wh->p, lr.acc->p});
             GB_TRY(mark(4 * bi));
-            GB_TRY(run_pass(m, kf, ls, [&](cudaStream_t cs) {
+            GB_TRY(run_pass(m, !resident, kf, ls, [&](cudaStream_t cs) {
                 Ctx cc = c;
                 cc.s = cs;
                 return forward_pass(cc, h, seis_d);
@@ -793,11 +876,13 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
                                                                    partial + (long long)kMisfitBlocks * i0, flag);
             GB_LAUNCHED();
             GB_TRY(mark(4 * bi + 2));
-            GB_TRY(run_pass(m, ka, ls, [&](cudaStream_t cs) -> int {
+            GB_TRY(run_pass(m, !resident, ka, ls, [&](cudaStream_t cs) -> int {
                 Ctx cc = c;
                 cc.s = cs;
                 GB_CUDA(cudaMemsetAsync(acc, 0, (size_t)B * 5 * NP * sizeof(float), cs));
-                return adjoint_pass(cc, h, MODE_ADJ_G, seis_d, acc, 5 * NP, NP);
+                if (resident) GB_CUDA(cudaMemsetAsync(m->w_eacc.p, 0, eacc_shot * B, cs));
+                GB_TRY(adjoint_pass(cc, h, MODE_ADJ_G, seis_d, acc, 5 * NP, NP));
+                return resident ? gb_assemble_strain(m, m->w_eacc.as<float>(), B, acc, 5 * NP, NP, cs) : GBFWI_OK;
             }));
             GB_TRY(mark(4 * bi + 3));
             GB_CUDA(cudaMemcpyAsync(acc_all + (long long)i0 * 5 * NP, acc, (size_t)B * 5 * NP * sizeof(float),
@@ -960,11 +1045,10 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
         GB_CUDA(cudaMemsetAsync(acc, 0, (size_t)B * 4 * NP * sizeof(float), s));
         long long blev = (long long)B * NP;
         if (kind == 1 || kind == 3) {
-            float2 *ring = m->w_hist.as<float2>();
-            GB_CUDA(cudaMemsetAsync(ring, 0, 3 * blev * sizeof(float2), s));
+            const Levels ring{m->w_hist.as<float2>(), blev, 0, true};
+            GB_CUDA(cudaMemsetAsync(ring.base, 0, 3 * blev * sizeof(float2), s));
             GB_CUDA(cudaMemsetAsync(m->w_vh.p, 0, blev * sizeof(float2), s));
-            SlotFn slot = [&](int k) { return ring + (long long)(k % 3) * blev; };
-            GB_TRY(fwd_range(c, MODE_FWD_PC, 0, nt, slot, m->w_vh.as<float2>(), nullptr, acc, 4 * NP, NP));
+            GB_TRY(fwd_range(c, MODE_FWD_PC, 0, nt, ring, 0, m->w_vh.as<float2>(), nullptr, acc, 4 * NP, NP));
         } else {
             // receiver wavefield: adjoint recurrence driven by the synthetic data s(m0)
             float *seis_d = m->w_seis.as<float>();

@@ -33,23 +33,22 @@
 // in four colour passes (sem_pc_step_kernel).
 
 #include "gbfwi_internal.h"
+#include "sem_element.h"
 #include "sm100.h"
 
 using sm100::bulk_g2s;
 using sm100::mbar_arrive_expect_tx;
 using sm100::mbar_init;
 using sm100::mbar_wait_bounded;
+using namespace sem;
 
-__constant__ float cD[GB_NG * GB_NG];   // D[i*5+k] = l_k'(xi_i)
 __constant__ float cW[GB_NG * GB_NG];   // w_i w_j at [j*5+i]
 
-int gb_upload_gll(const double *D, const double *w)
+int gb_upload_gll(const double *w)
 {
-    float hD[25], hW[25];
-    for (int i = 0; i < 25; ++i) hD[i] = (float)D[i];
+    float hW[25];
     for (int j = 0; j < 5; ++j)
         for (int i = 0; i < 5; ++i) hW[j * 5 + i] = (float)(w[i] * w[j]);
-    GB_CUDA(cudaMemcpyToSymbol(cD, hD, sizeof(hD)));
     GB_CUDA(cudaMemcpyToSymbol(cW, hW, sizeof(hW)));
     return GBFWI_OK;
 }
@@ -57,65 +56,35 @@ int gb_upload_gll(const double *D, const double *w)
 namespace {
 
 template <int NWXP>
-__device__ __forceinline__ void load_patch(const float2 *__restrict__ win, int base, float (&px)[25],
-                                           float (&pz)[25])
+__device__ __forceinline__ void load_patch(const float2 *__restrict__ win, int base, float2 (&p)[25])
 {
 #pragma unroll
     for (int j = 0; j < 5; ++j)
 #pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            float2 v = win[base + j * NWXP + i];
-            px[j * 5 + i] = v.x;
-            pz[j * 5 + i] = v.y;
-        }
-}
-
-// unscaled derivatives at local point (i, j): d/dxi and d/deta of both components
-__device__ __forceinline__ void grad_at(const float (&px)[25], const float (&pz)[25], int i, int j,
-                                        float &xx, float &xz, float &zx, float &zz)
-{
-    // xx = d ux/dxi, xz = d ux/deta, zx = d uz/dxi, zz = d uz/deta
-    float a = 0.f, b = 0.f, c = 0.f, d = 0.f;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        a = fmaf(cD[i * 5 + k], px[j * 5 + k], a);
-        c = fmaf(cD[i * 5 + k], pz[j * 5 + k], c);
-        b = fmaf(cD[j * 5 + k], px[k * 5 + i], b);
-        d = fmaf(cD[j * 5 + k], pz[k * 5 + i], d);
-    }
-    xx = a; xz = b; zx = c; zz = d;
+        for (int i = 0; i < 5; ++i) p[j * 5 + i] = win[base + j * NWXP + i];
 }
 
 // Per local point products of the unscaled strains of two fields A and B,
-// weighted by w_i w_j:
-//   NC == 2 (gradient):     [div A div B, 2 exx exx' + 2 ezz ezz' + gam gam']
-//   NC == 3 (preconditioner): [div A div B, exx exx' + ezz ezz', gam gam']
-template <int NWXP, int NC>
+// weighted by w_i w_j: [div A div B, exx exx' + ezz ezz', gam gam']
+template <int NWXP>
 __device__ __forceinline__ void element_products(const float2 *__restrict__ wa, const float2 *__restrict__ wb,
-                                                 int base, float (&out)[25 * NC])
+                                                 int base, float (&out)[75])
 {
-    float ax[25], az[25], bx[25], bz[25];
-    load_patch<NWXP>(wa, base, ax, az);
-    load_patch<NWXP>(wb, base, bx, bz);
+    float2 pa[25], pb[25];
+    load_patch<NWXP>(wa, base, pa);
+    load_patch<NWXP>(wb, base, pb);
 #pragma unroll
     for (int j = 0; j < 5; ++j)
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            float axx, axz, azx, azz, bxx, bxz, bzx, bzz;
-            grad_at(ax, az, i, j, axx, axz, azx, azz);
-            grad_at(bx, bz, i, j, bxx, bxz, bzx, bzz);
-            float ww = cW[j * 5 + i];
-            float da = axx + azz, db = bxx + bzz;
-            float ga = axz + azx, gb = bxz + bzx;
-            int q = (j * 5 + i) * NC;
-            if (NC == 2) {
-                out[q + 0] = ww * (da * db);
-                out[q + 1] = ww * fmaf(2.f * axx, bxx, fmaf(2.f * azz, bzz, ga * gb));
-            } else {
-                out[q + 0] = ww * (da * db);
-                out[q + 1] = ww * fmaf(axx, bxx, azz * bzz);
-                out[q + 2] = ww * (ga * gb);
-            }
+            float2 ax, ae, bx, be;
+            grad_at(pa, i, j, ax, ae);
+            grad_at(pb, i, j, bx, be);
+            const float ww = cW[j * 5 + i];
+            const int q = (j * 5 + i) * 3;
+            out[q + 0] = ww * ((ax.x + ae.y) * (bx.x + be.y));
+            out[q + 1] = ww * fmaf(ax.x, bx.x, ae.y * be.y);
+            out[q + 2] = ww * ((ae.x + ax.y) * (be.x + bx.y));
         }
 }
 
@@ -123,70 +92,35 @@ __device__ __forceinline__ void element_products(const float2 *__restrict__ wa, 
 template <int NWXP>
 __device__ __forceinline__ void element_squares(const float2 *__restrict__ wa, int base, float (&out)[75])
 {
-    float ax[25], az[25];
-    load_patch<NWXP>(wa, base, ax, az);
+    float2 pa[25];
+    load_patch<NWXP>(wa, base, pa);
 #pragma unroll
     for (int j = 0; j < 5; ++j)
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            float axx, axz, azx, azz;
-            grad_at(ax, az, i, j, axx, axz, azx, azz);
-            float ww = cW[j * 5 + i];
-            float da = axx + azz, ga = axz + azx;
-            int q = (j * 5 + i) * 3;
+            float2 ax, ae;
+            grad_at(pa, i, j, ax, ae);
+            const float ww = cW[j * 5 + i];
+            const float da = ax.x + ae.y, ga = ae.x + ax.y;
+            const int q = (j * 5 + i) * 3;
             out[q + 0] = ww * (da * da);
-            out[q + 1] = ww * fmaf(axx, axx, azz * azz);
+            out[q + 1] = ww * fmaf(ax.x, ax.x, ae.y * ae.y);
             out[q + 2] = ww * (ga * ga);
         }
 }
 
-// Element nodal forces accumulated row by row of local points: the
-// stresses of row j give the xi-part of the nodes of row j and the eta-part
-// of every node, so one row of stresses is live at a time.
+// forces of the element whose patch starts at `base` of the field window sw
+// and of the weighted-moduli window slm
 template <int NWXP>
-__device__ __forceinline__ void element_force_rows(const float2 *__restrict__ sw, const float2 *__restrict__ slm,
-                                                   int base, float2 (&f)[25])
+__device__ __forceinline__ void element_force_window(const float2 *__restrict__ sw, const float2 *__restrict__ slm,
+                                                     int base, float2 (&f)[25])
 {
-    float px[25], pz[25];
-    load_patch<NWXP>(sw, base, px, pz);
+    float2 p[25];
+    load_patch<NWXP>(sw, base, p);
+    element_force(p, [&](int j, float2(&lm)[5]) {
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        float txx[5], tzz[5], txz[5];
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            float xx, xz, zx, zz;
-            grad_at(px, pz, i, j, xx, xz, zx, zz);
-            float2 lm = slm[base + j * NWXP + i];
-            float l2m = fmaf(2.f, lm.y, lm.x);
-            float ww = cW[j * 5 + i];
-            txx[i] = ww * fmaf(l2m, xx, lm.x * zz);
-            tzz[i] = ww * fmaf(lm.x, xx, l2m * zz);
-            txz[i] = ww * (lm.y * (xz + zx));
-        }
-        // f(m, n) += D[j][n] (txz, tzz)(m, j) for every node; for n == j also
-        // the xi-part sum_i D[i][m] (txx, txz)(i, j)
-#pragma unroll
-        for (int n = 0; n < 5; ++n)
-#pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                float fx, fz;
-                if (j == 0) {
-                    fx = cD[n] * txz[m];
-                    fz = cD[n] * tzz[m];
-                } else {
-                    fx = fmaf(cD[j * 5 + n], txz[m], f[n * 5 + m].x);
-                    fz = fmaf(cD[j * 5 + n], tzz[m], f[n * 5 + m].y);
-                }
-                if (n == j) {
-#pragma unroll
-                    for (int i = 0; i < 5; ++i) {
-                        fx = fmaf(cD[i * 5 + m], txx[i], fx);
-                        fz = fmaf(cD[i * 5 + m], txz[i], fz);
-                    }
-                }
-                f[n * 5 + m] = make_float2(fx, fz);
-            }
-    }
+        for (int i = 0; i < 5; ++i) lm[i] = slm[base + j * NWXP + i];
+    }, f);
 }
 
 // window load: rows iz0.., node pairs from ix0 (even); out-of-mesh -> 0.
@@ -436,7 +370,7 @@ __global__ void __launch_bounds__(StepShape<TX, TZ, MODE>::NT, StepShape<TX, TZ,
     float mip[16], amp[16];
     float2 f[25];
     if (evalid) {
-        element_force_rows<NWXP>(sw, slm, ebase, f);
+        element_force_window<NWXP>(sw, slm, ebase, f);
     } else {
 #pragma unroll
         for (int q = 0; q < 25; ++q) f[q] = make_float2(0.f, 0.f);
@@ -500,27 +434,14 @@ __global__ void __launch_bounds__(StepShape<TX, TZ, MODE>::NT, StepShape<TX, TZ,
                 const int ix = 4 * ex + i, iz = 4 * ez + j;
                 const long long g = g00 + (long long)j * pitch + i;
                 float2 k = f[q];
-                if (ge > gb) {
-                    const float2 F = sF[(4 * (elz - 1) + j) * OXP + 4 * (elx - 1) + i];
-                    k.x += F.x;
-                    k.y += F.y;
-                }
+                if (ge > gb) k = add2(k, sF[(4 * (elz - 1) + j) * OXP + 4 * (elx - 1) + i]);
                 const float2 v = std16 ? svh[(4 * (elz - 1) + j) * S::VXP + 4 * (elx - 1) + i] : vhb[g];
                 const bool edge = (ix == 0) | (ix == a.nx - 1) | (iz == 0) | (iz == a.nz - 1);
-                float ax, az;
-                if (edge) {
-                    float4 bd = a.bnd[g];
-                    ax = -(k.x + bd.x * v.x) * bd.z;
-                    az = -(k.y + bd.y * v.y) * bd.w;
-                } else {
-                    const float mi = std16 ? mip[4 * j + i] : a.minv[g];
-                    ax = -k.x * mi;
-                    az = -k.y * mi;
-                }
-                const float2 vn = make_float2(fmaf(dt, ax, v.x), fmaf(dt, az, v.y));
+                const float2 ac = edge ? accel_edge(k, v, a.bnd[g]) : accel(k, std16 ? mip[4 * j + i] : a.minv[g]);
+                const float2 vn = axpy2(dt, ac, v);
                 const float2 uc = sw[ebase + j * NWXP + i];
                 vrow[i] = vn;
-                urow[i] = make_float2(fmaf(dt, vn.x, uc.x), fmaf(dt, vn.y, uc.y));
+                urow[i] = axpy2(dt, vn, uc);
                 if (!std16) {
                     vhb[g] = vrow[i];
                     a.unext[fo + g] = urow[i];
@@ -528,13 +449,11 @@ __global__ void __launch_bounds__(StepShape<TX, TZ, MODE>::NT, StepShape<TX, TZ,
                 if (MODE == MODE_ADJ_G) {
                     const float2 uk = su2[ebase + j * NWXP + i];
                     // u_k . a^w; the node's mass factor rho W_g enters once, in the chain rule
-                    const float am = std16 ? amp[4 * j + i] : accb[2 * cs + g];
-                    accb[2 * cs + g] = am + fmaf(uk.x, ax, uk.y * az);
+                    accb[2 * cs + g] = (std16 ? amp[4 * j + i] : accb[2 * cs + g]) + dot2(uk, ac);
                     if (edge) {
-                        float4 w4 = a.bw[g];
-                        float vx = 0.5f * (v.x + vn.x), vz = 0.5f * (v.y + vn.y);
-                        accb[3 * cs + g] += fmaf(w4.x * uk.x, vx, w4.y * uk.y * vz);
-                        accb[4 * cs + g] += fmaf(w4.z * uk.x, vx, w4.w * uk.y * vz);
+                        const float4 w4 = a.bw[g];
+                        accb[3 * cs + g] += edge_product(make_float2(w4.x, w4.y), uk, v, vn);
+                        accb[4 * cs + g] += edge_product(make_float2(w4.z, w4.w), uk, v, vn);
                     }
                 }
             }
@@ -552,16 +471,19 @@ __global__ void __launch_bounds__(StepShape<TX, TZ, MODE>::NT, StepShape<TX, TZ,
 
     // ---- phase 3: element strain products, assembled like the forces
     {
-        float pr[50];
+        float2 c[25];
         if (evalid) {
-            element_products<NWXP, 2>(sw, su2, ebase, pr);
+            float2 pw[25], pu[25];
+            load_patch<NWXP>(sw, ebase, pw);
+            load_patch<NWXP>(su2, ebase, pu);
+#pragma unroll
+            for (int j = 0; j < 5; ++j)
+#pragma unroll
+                for (int i = 0; i < 5; ++i) c[j * 5 + i] = strain_products(pw, pu, i, j);
         } else {
 #pragma unroll
-            for (int q = 0; q < 50; ++q) pr[q] = 0.f;
+            for (int q = 0; q < 25; ++q) c[q] = make_float2(0.f, 0.f);
         }
-        float2 c[25];
-#pragma unroll
-        for (int q = 0; q < 25; ++q) c[q] = make_float2(pr[2 * q], pr[2 * q + 1]);
         // strain accumulators of the 16 standard nodes, read ahead of the exchange
         float4 a0p[4], a1p[4];
         if (owns) {
@@ -708,7 +630,7 @@ __global__ void __launch_bounds__(PcShape<TX, TZ, MODE>::NT, PcShape<TX, TZ, MOD
     const int colour = ((ex0 - 1 + elx) & 1) | (((ez0 - 1 + elz) & 1) << 1);
     {
         float2 f[25];
-        if (evalid) element_force_rows<NWXP>(sw, slm, ebase, f);
+        if (evalid) element_force_window<NWXP>(sw, slm, ebase, f);
 #pragma unroll 1
         for (int pass = 0; pass < 4; ++pass) {
             if (evalid && colour == pass) {
@@ -804,7 +726,7 @@ __global__ void __launch_bounds__(PcShape<TX, TZ, MODE>::NT, PcShape<TX, TZ, MOD
             if constexpr (MODE == MODE_FWD_PC)
                 element_squares<NWXP>(sw, ebase, pr);
             else
-                element_products<NWXP, 3>(sw, slm, ebase, pr);
+                element_products<NWXP>(sw, slm, ebase, pr);
         }
 #pragma unroll 1
         for (int pass = 0; pass < 4; ++pass) {
