@@ -1019,7 +1019,16 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     const int nt = m->d.nt;
     const long long NP = (long long)m->nz * m->pitch;
     const long long N = (long long)m->nz * m->nx;
-    const int Bmax = std::min(m->sch.shots_per_launch, nshot);
+    // shots in one launch: what the schedule keeps in flight (shots per launch x
+    // streams), or more while their levels and maps stay small
+    const bool receiver = kind == 2 || kind == 4;
+    const int ck = m->sch.ckpt_every;
+    const long long levels = !receiver ? 4 : ck <= 0 || ck >= nt ? nt + 6 : 3LL * ((nt + ck - 1) / ck) + ck + 10;
+    const long long small = kSmallHistory / ((levels + 2) * NP * (long long)sizeof(float2));
+    const int Bmax = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
+    const bool resident = receiver && gb_resident_plan(m, MODE_FWD, Bmax);
+    if (resident)
+        for (int B : {Bmax, nshot - (nshot - 1) / Bmax * Bmax}) GB_TRY(reserve_exchange(m, MODE_FWD, B, NP));
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
     const long long lev = (long long)Bmax * NP;
     const double dt = m->d.dt;
@@ -1029,7 +1038,7 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     GB_TRY(m->w_grad.ensure((size_t)5 * NP * sizeof(float)));
     GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
     BatchHist h;
-    if (kind == 2 || kind == 4) {
+    if (receiver) {
         GB_TRY(alloc_hist(m, lane0(m, s), Bmax, m->sch.ckpt_every, NP, h, true));
         GB_TRY(m->w_seis.ensure(seis_shot * Bmax * sizeof(float)));
     } else {
@@ -1040,11 +1049,11 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     GB_CUDA(cudaMemsetAsync(tot, 0, 4 * NP * sizeof(float), s));
     for (int i0 = 0; i0 < nshot; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
-        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP};
+        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, resident};
         float *acc = m->w_pc.as<float>();
         GB_CUDA(cudaMemsetAsync(acc, 0, (size_t)B * 4 * NP * sizeof(float), s));
         long long blev = (long long)B * NP;
-        if (kind == 1 || kind == 3) {
+        if (!receiver) {
             const Levels ring{m->w_hist.as<float2>(), blev, 0, true};
             GB_CUDA(cudaMemsetAsync(ring.base, 0, 3 * blev * sizeof(float2), s));
             GB_CUDA(cudaMemsetAsync(m->w_vh.p, 0, blev * sizeof(float2), s));
