@@ -331,32 +331,82 @@ __global__ void precond_finish(const float *__restrict__ tot, const float *__res
 
 // Separable Gaussian smoothing along one axis of [3][nz][nx]:
 // out(i) = sum_j G(c_i - c_j) w_j f(j) / sum_j G(c_i - c_j) w_j over |c_i - c_j| <= 5 sigma
-__global__ void smooth_axis(const float *__restrict__ in, float *__restrict__ out, int nx, int nz, int axis,
-                            const float *__restrict__ coord, const float *__restrict__ wts,
-                            const int2 *__restrict__ range, float inv2s2)
+// A weight serves every node that shares it: along x a thread keeps one ix and
+// takes kSmoothRows rows of the three maps; along z a block keeps one iz, forms
+// its weights once in shared memory (chunks of kSmoothTaps) and spreads over ix.
+// Bound by the exponentials before (one per node, map and tap: 68 and 88 us along
+// x and z at 1361 x 281 nodes, 80 taps), by the loads of f from L1 now (38 and 31 us).
+constexpr int kSmoothRows = 4, kSmoothTaps = 256;
+
+__global__ void __launch_bounds__(128) smooth_x_kernel(const float *__restrict__ in, float *__restrict__ out, int nx, int nz,
+                                                       const float *__restrict__ coord, const float *__restrict__ wts,
+                                                       const int2 *__restrict__ range, float inv2s2, int row0)
 {
-    long long N = (long long)nx * nz;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < 3 * N;
-         q += (long long)gridDim.x * blockDim.x) {
-        long long c = q / N, r = q - c * N;
-        int iz = (int)(r / nx), ix = (int)(r - (long long)iz * nx);
-        int i = axis == 0 ? ix : iz;
-        int2 rg = range[i];
-        float ci = coord[i];
-        float num = 0.f, den = 0.f;
-        const float *base = in + c * N;
-        for (int jj = rg.x; jj <= rg.y; ++jj) {
-            float d = ci - coord[jj];
-            float gw = __expf(-d * d * inv2s2) * wts[jj];
-            float f = axis == 0 ? base[(long long)iz * nx + jj] : base[(long long)jj * nx + ix];
-            num = fmaf(gw, f, num);
-            den += gw;
+    const int ix = blockIdx.x * blockDim.x + threadIdx.x, iz0 = row0 + blockIdx.y * kSmoothRows;
+    if (ix >= nx) return;
+    const long long N = (long long)nx * nz;
+    const int rows = min(kSmoothRows, nz - iz0);
+    const int2 rg = range[ix];
+    const float ci = coord[ix];
+    float num[3][kSmoothRows], den = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int r = 0; r < kSmoothRows; ++r) num[c][r] = 0.f;
+    const float *base = in + (long long)iz0 * nx;
+    for (int jj = rg.x; jj <= rg.y; ++jj) {
+        const float d = ci - coord[jj];
+        const float gw = __expf(-d * d * inv2s2) * wts[jj];
+        den += gw;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int r = 0; r < kSmoothRows; ++r)
+                if (r < rows) num[c][r] = fmaf(gw, base[c * N + (long long)r * nx + jj], num[c][r]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int r = 0; r < kSmoothRows; ++r)
+            if (r < rows) out[c * N + (long long)(iz0 + r) * nx + ix] = num[c][r] / den;
+}
+
+__global__ void __launch_bounds__(128) smooth_z_kernel(const float *__restrict__ in, float *__restrict__ out, int nx, int nz,
+                                                       const float *__restrict__ coord, const float *__restrict__ wts,
+                                                       const int2 *__restrict__ range, float inv2s2)
+{
+    __shared__ float sg[kSmoothTaps];
+    const int ix = blockIdx.x * blockDim.x + threadIdx.x;
+    const long long N = (long long)nx * nz;
+    for (int iz = blockIdx.y; iz < nz; iz += gridDim.y) {
+        const int2 rg = range[iz];
+        const float ci = coord[iz];
+        float num[3] = {0.f, 0.f, 0.f}, den = 0.f;
+        for (int j0 = rg.x; j0 <= rg.y; j0 += kSmoothTaps) {
+            const int m = min(kSmoothTaps, rg.y - j0 + 1);
+            __syncthreads();
+            for (int q = threadIdx.x; q < m; q += blockDim.x) {
+                const float d = ci - coord[j0 + q];
+                sg[q] = __expf(-d * d * inv2s2) * wts[j0 + q];
+            }
+            __syncthreads();
+            if (ix < nx)
+                for (int q = 0; q < m; ++q) {
+                    const float gw = sg[q];
+                    const float *f = in + (long long)(j0 + q) * nx + ix;
+                    den += gw;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) num[c] = fmaf(gw, f[c * N], num[c]);
+                }
         }
-        out[q] = num / den;
+        if (ix < nx)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) out[c * N + (long long)iz * nx + ix] = num[c] / den;
     }
 }
 
-// radix select of rank k over n floats (one parameter map), 8 bits per pass
+// radix select of rank k over n floats, 8 bits per pass, the three maps at once
+// (map blockIdx.y / blockIdx.x); state [3][4] = {prefix, mask, rank, -}
 __device__ __forceinline__ unsigned fkey(float f)
 {
     unsigned u = __float_as_uint(f);
@@ -369,6 +419,9 @@ __global__ void radix_hist(const float *__restrict__ x, long long n, const unsig
     __shared__ unsigned h[256];
     for (int t = threadIdx.x; t < 256; t += blockDim.x) h[t] = 0;
     __syncthreads();
+    x += blockIdx.y * n;
+    state += blockIdx.y * 4;
+    hist += blockIdx.y * 256;
     unsigned prefix = state[0], mask = state[1];
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
          q += (long long)gridDim.x * blockDim.x) {
@@ -380,32 +433,40 @@ __global__ void radix_hist(const float *__restrict__ x, long long n, const unsig
         if (h[t]) atomicAdd(&hist[t], h[t]);
 }
 
-// state = {prefix, mask, rank}
-__global__ void radix_pick(unsigned *__restrict__ state, unsigned *__restrict__ hist, int shift,
-                           float *__restrict__ result)
+// the bin holding the rank, by a prefix sum over the 256 bins (one thread each:
+// a single thread's walk over them took 10 to 15 us a map and pass, the three
+// maps together 3 us here)
+__global__ void __launch_bounds__(256) radix_pick(unsigned *__restrict__ state, unsigned *__restrict__ hist, int shift,
+                                                  float *__restrict__ result)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    unsigned rank = state[2], cum = 0;
-    int bin = 0;
-    for (; bin < 256; ++bin) {
-        if (cum + hist[bin] > rank) break;
-        cum += hist[bin];
+    __shared__ unsigned wsum[8];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    state += blockIdx.x * 4;
+    hist += blockIdx.x * 256;
+    const unsigned rank = state[2], prefix = state[0], h = hist[t];
+    unsigned inc = h;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
     }
-    if (bin > 255) bin = 255;
-    state[0] |= ((unsigned)bin) << shift;
-    state[1] |= 0xFFu << shift;
-    state[2] = rank - cum;
-    for (int t = 0; t < 256; ++t) hist[t] = 0;
-    if (shift == 0) {
-        unsigned k = state[0];
-        unsigned u = (k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k;
-        *result = __uint_as_float(u);
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    for (int q = 0; q < w; ++q) inc += wsum[q];
+    hist[t] = 0;
+    if (inc > rank && inc - h <= rank) {
+        const unsigned p = prefix | (unsigned)t << shift;
+        state[0] = p;
+        state[1] |= 0xFFu << shift;
+        state[2] = rank - (inc - h);
+        if (shift == 0) result[blockIdx.x] = __uint_as_float((p & 0x80000000u) ? (p & 0x7FFFFFFFu) : ~p);
     }
 }
 
-__global__ void radix_init(unsigned *__restrict__ state, unsigned rank)
+__global__ void radix_init(unsigned *__restrict__ state, unsigned *__restrict__ hist, unsigned rank)
 {
-    if (threadIdx.x == 0) { state[0] = 0; state[1] = 0; state[2] = rank; }
+    for (int t = threadIdx.x; t < 768; t += blockDim.x) hist[t] = 0;
+    if (threadIdx.x < 12) state[threadIdx.x] = threadIdx.x % 4 == 2 ? rank : 0u;
 }
 
 __global__ void b0_kernel(const float *__restrict__ S, const float *__restrict__ med, long long N, float damp,
@@ -948,54 +1009,50 @@ static int b0_from_map(gbfwi_mesh *m, const float *Hd, float *S1, float *S2, dou
                        cudaStream_t s)
 {
     const long long N = (long long)m->nx * m->nz;
-    // smoothing tables (node coordinates along each axis, 5-sigma index ranges)
-    std::vector<float> cx(m->nx), cz(m->nz);
-    std::vector<int2> rx(m->nx), rz(m->nz);
-    {
-        std::vector<double> X((size_t)m->nx * m->nz), Z((size_t)m->nx * m->nz);
-        gbfwi_node_coords(m, X.data(), Z.data());
-        for (int i = 0; i < m->nx; ++i) cx[i] = (float)X[i];
-        for (int i = 0; i < m->nz; ++i) cz[i] = (float)Z[(size_t)i * m->nx];
-        auto ranges = [&](const std::vector<float> &c, std::vector<int2> &r) {
-            int n = (int)c.size();
-            for (int i = 0; i < n; ++i) {
-                int lo = i, hi = i;
-                while (lo > 0 && c[i] - c[lo - 1] <= 5.0 * sigma) --lo;
-                while (hi < n - 1 && c[hi + 1] - c[i] <= 5.0 * sigma) ++hi;
-                r[i] = make_int2(lo, hi);
-            }
-        };
-        ranges(cx, rx);
-        ranges(cz, rz);
+    // smoothing tables (node coordinates and weights along each axis, 5-sigma
+    // index ranges), in one upload
+    const int nx = m->nx, nz = m->nz;
+    std::vector<int2> tab(2 * (size_t)(nx + nz));       // (coordinate, weight) as bits, then the ranges
+    for (int ax = 0, o = 0; ax < 2; o += ax == 0 ? nx : 0, ++ax) {
+        const int n = ax == 0 ? nx : nz;
+        const std::vector<double> X = gb_axis(m, ax == 0 ? m->d.nex : m->d.nez);
+        const std::vector<double> &w = ax == 0 ? m->wx1 : m->wz1;
+        float *c = reinterpret_cast<float *>(tab.data()) + 2 * o;
+        for (int i = 0; i < n; ++i) {
+            c[i] = (float)X[i];
+            c[n + i] = (float)w[i];
+        }
+        for (int i = 0, lo = 0, hi = 0; i < n; ++i) {
+            while (c[i] - c[lo] > 5.0 * sigma) ++lo;
+            hi = std::max(hi, i);
+            while (hi < n - 1 && c[hi + 1] - c[i] <= 5.0 * sigma) ++hi;
+            tab[nx + nz + o + i] = make_int2(lo, hi);
+        }
     }
-    std::vector<float> wxf(m->wx1.begin(), m->wx1.end()), wzf(m->wz1.begin(), m->wz1.end());
-    GB_TRY(m->w_stage.ensure((size_t)(m->nx + m->nz) * (2 * sizeof(float) + sizeof(int2)) + 64));
-    char *tb = m->w_stage.as<char>();
-    float *dcx = (float *)tb, *dcz = dcx + m->nx, *dwx = dcz + m->nz, *dwz = dwx + m->nx;
-    int2 *drx = (int2 *)(((uintptr_t)(dwz + m->nz) + 15) & ~(uintptr_t)15), *drz = drx + m->nx;
-    GB_CUDA(cudaMemcpyAsync(dcx, cx.data(), m->nx * sizeof(float), cudaMemcpyHostToDevice, s));
-    GB_CUDA(cudaMemcpyAsync(dcz, cz.data(), m->nz * sizeof(float), cudaMemcpyHostToDevice, s));
-    GB_CUDA(cudaMemcpyAsync(dwx, wxf.data(), m->nx * sizeof(float), cudaMemcpyHostToDevice, s));
-    GB_CUDA(cudaMemcpyAsync(dwz, wzf.data(), m->nz * sizeof(float), cudaMemcpyHostToDevice, s));
-    GB_CUDA(cudaMemcpyAsync(drx, rx.data(), m->nx * sizeof(int2), cudaMemcpyHostToDevice, s));
-    GB_CUDA(cudaMemcpyAsync(drz, rz.data(), m->nz * sizeof(int2), cudaMemcpyHostToDevice, s));
+    GB_TRY(m->w_stage.ensure(tab.size() * sizeof(int2) + 64));
+    GB_CUDA(cudaMemcpyAsync(m->w_stage.p, tab.data(), tab.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+    const float *dcx = m->w_stage.as<float>(), *dcz = dcx + 2 * nx;
+    const int2 *drx = m->w_stage.as<int2>() + nx + nz, *drz = drx + nx;
     float inv2s2 = (float)(1.0 / (2.0 * sigma * sigma));
-    smooth_axis<<<grid_for(3 * N), 256, 0, s>>>(Hd, S1, m->nx, m->nz, 0, dcx, dwx, drx, inv2s2);
-    GB_LAUNCHED();
-    smooth_axis<<<grid_for(3 * N), 256, 0, s>>>(S1, S2, m->nx, m->nz, 1, dcz, dwz, drz, inv2s2);
+    const unsigned gx = (unsigned)((nx + 127) / 128);
+    for (int z0 = 0; z0 < nz; z0 += 65535 * kSmoothRows) {
+        const unsigned gy = (unsigned)std::min((nz - z0 + kSmoothRows - 1) / kSmoothRows, 65535);
+        smooth_x_kernel<<<dim3(gx, gy), 128, 0, s>>>(Hd, S1, nx, nz, dcx, dcx + nx, drx, inv2s2, z0);
+        GB_LAUNCHED();
+    }
+    smooth_z_kernel<<<dim3(gx, (unsigned)std::min(nz, 65535)), 128, 0, s>>>(S1, S2, nx, nz, dcz, dcz + nz, drz, inv2s2);
     GB_LAUNCHED();
     // medians of the smoothed maps (rank (N-1)/2)
     GB_TRY(m->w_red.ensure((1024 + 8) * sizeof(double) + 4096));
     unsigned *rstate = (unsigned *)(m->w_red.as<char>() + (1024 + 8) * sizeof(double));   // radix-select state
-    unsigned *rhist = rstate + 4;
-    float *med = (float *)(rhist + 256);
-    GB_CUDA(cudaMemsetAsync(rhist, 0, 256 * sizeof(unsigned), s));
-    for (int c = 0; c < 3; ++c) {
-        radix_init<<<1, 32, 0, s>>>(rstate, (unsigned)((N - 1) / 2));
-        for (int shift = 24; shift >= 0; shift -= 8) {
-            radix_hist<<<grid_for(N), 256, 0, s>>>(S2 + c * N, N, rstate, shift, rhist);
-            radix_pick<<<1, 32, 0, s>>>(rstate, rhist, shift, med + c);
-        }
+    unsigned *rhist = rstate + 12;
+    float *med = (float *)(rhist + 768);
+    radix_init<<<1, 256, 0, s>>>(rstate, rhist, (unsigned)((N - 1) / 2));
+    GB_LAUNCHED();
+    for (int shift = 24; shift >= 0; shift -= 8) {
+        radix_hist<<<dim3((unsigned)std::min<long long>(grid_for(N), 304), 3), 256, 0, s>>>(S2, N, rstate, shift, rhist);
+        GB_LAUNCHED();
+        radix_pick<<<3, 256, 0, s>>>(rstate, rhist, shift, med);
         GB_LAUNCHED();
     }
     const bool dev_b0 = gb_is_device_ptr(B0);
