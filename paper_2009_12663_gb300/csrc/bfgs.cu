@@ -39,19 +39,21 @@ struct gbfwi_bfgs {
     long long n = 0;
     long long ld = 0;          // row pitch of every [rows][n] block: n rounded up to 64
     int kmax = 0, k = 0;
-    DevBuf S, Y, BY, B0;       // [kmax][n] x 3, [n]
-    std::vector<double> SY;    // [kmax][kmax]: SY[i*kmax + j] = s_i^T y_j (i <= j)
-    std::vector<double> YBY;   // [kmax][kmax]: y_i^T B0 y_j
-    std::vector<double> SS, SB, BB;   // [kmax][kmax]: s_i^T s_j, s_i^T B0 y_j, (B0 y_i)^T (B0 y_j)
-    DevBuf dSY, dYBY;          // device copies
+    // one allocation for everything whose size is known at creation (an L-BFGS
+    // direction makes and frees a store each iteration)
+    DevBuf arena;
+    float *S = nullptr, *Y = nullptr, *BY = nullptr;   // [kmax][ld]
+    float *B0 = nullptr;                               // [n]
+    double *dSY = nullptr, *dYBY = nullptr;            // [kmax][kmax]: s_i^T y_j (i <= j), y_i^T B0 y_j
+    double *dSS = nullptr, *dSB = nullptr, *dBB = nullptr;   // s_i^T s_j, s_i^T B0 y_j, (B0 y_i)^T (B0 y_j)
+    int *status = nullptr;     // nonzero after a product kernel's bounded wait gave up
+    int *flag = nullptr;
     DevBuf dG;                 // [2k][2k] FP64: W^T W with W = [S, B0 Y] (rows s_i, then B0 y_i)
     DevBuf part;               // split-K partials
     DevBuf small;              // FP64 small matrices
     DevBuf coef;               // FP32 combination coefficients
     DevBuf X, E, Q, V;         // [p][n] blocks
     DevBuf stage;              // host staging
-    DevBuf flag;
-    DevBuf status;             // int: nonzero after a product kernel's bounded wait gave up
     DevBuf ex;                 // FP64 scratch of the low-rank decompositions
 };
 
@@ -75,62 +77,164 @@ __device__ __forceinline__ void dot2_term(float a, float b, float &hi, float &lo
     lo = __fadd_rn(lo, __fadd_rn(se, pe));
 }
 
-// Products with kb <= 2 columns (dot products of the pair updates, the
-// search direction): CTA (split, a) accumulates row a against the kb
-// columns with compensated (Dot2) sums, then an FP64 tree over its threads;
-// part[sx][a][b] is reduced over the splits by atb_reduce.
-template <int KB>
-__global__ void __launch_bounds__(256) atb_thin(const float *__restrict__ A, long long lda,
-                                                const float *__restrict__ Bm, long long ldb,
-                                                const float *__restrict__ w, long long n, long long chunk, int ka,
-                                                double *__restrict__ part)
+// Products of the rows [S; B0 Y] with one or two columns (the search
+// direction).  A CTA keeps its chunk of the columns in registers (4 float4 a
+// thread) and streams every row of its group past it, so a column is read once
+// instead of once per row; compensated (Dot2) sums in four lanes per thread.
+// The sums of eight rows are then reduced together over the warp in
+// compensated pairs, each exchange halving the values a lane holds: 9 merges
+// instead of 40, and FP32 ones (the FP64 pipe takes 16 cycles a warp
+// instruction); FP64 only over the warps.  Bound by the row reads (459 MB for
+// 100 rows of n = 1,147,323): 108 us, 317 us with each row reduced in FP64,
+// 160 us with a CTA per row and chunk, which reads the column again for each row.
+// part[chunk][a][b] is summed over the chunks by thin_reduce.
+constexpr int kThinChunk = 4096;           // elements of a chunk: 256 threads x 16
+
+__device__ __forceinline__ double warp_sum(double v)
 {
-    __shared__ double red[KB][256];
-    const int sx = blockIdx.x, a = blockIdx.y, t = threadIdx.x;
-    const long long ib = (long long)sx * chunk, ie = min(n, ib + chunk);
-    float hi[KB], lo[KB];
 #pragma unroll
-    for (int b = 0; b < KB; ++b) hi[b] = lo[b] = 0.f;
-    const float *ar = A + (long long)a * lda;
-    for (long long i = ib + t; i < ie; i += blockDim.x) {
-        const float av = __ldg(ar + i);
-#pragma unroll
-        for (int b = 0; b < KB; ++b) {
-            float bv = __ldg(Bm + (long long)b * ldb + i);
-            if (w) bv *= __ldg(w + i);
-            dot2_term(av, bv, hi[b], lo[b]);
-        }
-    }
-#pragma unroll
-    for (int b = 0; b < KB; ++b) red[b][t] = (double)hi[b] + (double)lo[b];
-    __syncthreads();
-    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-        if (t < h)
-#pragma unroll
-            for (int b = 0; b < KB; ++b) red[b][t] += red[b][t + h];
-        __syncthreads();
-    }
-    if (t == 0)
-#pragma unroll
-        for (int b = 0; b < KB; ++b) part[((long long)sx * ka + a) * KB + b] = red[b][0];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-__global__ void atb_reduce(const double *__restrict__ part, int nsplit, int nab, double *__restrict__ out,
-                           long long ldo, int kb)
+// (h, l) += (h2, l2)
+__device__ __forceinline__ void merge_pair(float &h, float &l, float h2, float l2)
 {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nab) return;
+    const float sm = __fadd_rn(h, h2);
+    const float z = __fsub_rn(sm, h);
+    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(sm, z)), __fsub_rn(h2, z));
+    h = sm;
+    l = __fadd_rn(__fadd_rn(l, l2), e);
+}
+
+template <int KB>
+__global__ void __launch_bounds__(256, 2) thin_rows_kernel(const float *__restrict__ A1, const float *__restrict__ A2, int k1,
+                                                           int rows, int group, long long lda, const float *__restrict__ X,
+                                                           long long ldx, long long n, double *__restrict__ part)
+{
+    extern __shared__ double tsum[];       // [group][KB][8]
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const long long i0 = blockIdx.x * (long long)kThinChunk;
+    const int r0 = blockIdx.y * group, r1 = min(rows, r0 + group);
+    float x[KB][16];
+#pragma unroll
+    for (int b = 0; b < KB; ++b)
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const long long i = i0 + (q >> 2) * 1024 + 4 * t + (q & 3);
+            x[b][q] = i < n ? __ldg(X + b * ldx + i) : 0.f;
+        }
+#pragma unroll 1
+    for (int rb = r0; rb < r1; rb += 8) {
+        float h[KB][8], l[KB][8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int r = rb + u;
+            const float *row = (r < k1 ? A1 + (long long)r * lda : A2 + (long long)(r - k1) * lda) + i0 + 4 * t;
+            float4 a[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)    // rows are readable to their pitch
+                a[q] = r < r1 && i0 + q * 1024 + 4 * t < lda ? __ldcs(reinterpret_cast<const float4 *>(row + q * 1024))
+                                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int b = 0; b < KB; ++b) {
+                float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    dot2_term(a[q].x, x[b][4 * q], hi[0], lo[0]);
+                    dot2_term(a[q].y, x[b][4 * q + 1], hi[1], lo[1]);
+                    dot2_term(a[q].z, x[b][4 * q + 2], hi[2], lo[2]);
+                    dot2_term(a[q].w, x[b][4 * q + 3], hi[3], lo[3]);
+                }
+                merge_pair(hi[0], lo[0], hi[1], lo[1]);
+                merge_pair(hi[2], lo[2], hi[3], lo[3]);
+                merge_pair(hi[0], lo[0], hi[2], lo[2]);
+                h[b][u] = hi[0];
+                l[b][u] = lo[0];
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < KB; ++b) {
+#pragma unroll
+            for (int s = 4; s >= 1; s >>= 1) {            // lanes whose bit 4 s is set keep the upper s values
+                const bool up = lane & 4 * s;
+#pragma unroll
+                for (int u = 0; u < s; ++u) {
+                    const float oh = __shfl_xor_sync(0xffffffffu, up ? h[b][u] : h[b][u + s], 4 * s);
+                    const float ol = __shfl_xor_sync(0xffffffffu, up ? l[b][u] : l[b][u + s], 4 * s);
+                    if (up) {
+                        h[b][u] = h[b][u + s];
+                        l[b][u] = l[b][u + s];
+                    }
+                    merge_pair(h[b][u], l[b][u], oh, ol);
+                }
+            }
+#pragma unroll
+            for (int o = 2; o >= 1; o >>= 1)
+                merge_pair(h[b][0], l[b][0], __shfl_xor_sync(0xffffffffu, h[b][0], o), __shfl_xor_sync(0xffffffffu, l[b][0], o));
+            const int r = rb + (lane >> 2);               // bits 4, 3, 2 of the lane: row 4, 2, 1
+            if ((lane & 3) == 0 && r < r1) tsum[((r - r0) * KB + b) * 8 + w] = (double)h[b][0] + (double)l[b][0];
+        }
+    }
+    __syncthreads();
+    for (int q = t; q < (r1 - r0) * KB; q += 256) {
+        double s = 0.0;
+#pragma unroll
+        for (int v = 0; v < 8; ++v) s += tsum[q * 8 + v];
+        part[(blockIdx.x * (long long)rows + r0) * KB + q] = s;
+    }
+}
+
+// out[q] = sum over the splits of part[sx][q]: one warp per output, the lanes
+// over the splits
+__global__ void __launch_bounds__(128) thin_reduce(const double *__restrict__ part, int nsplit, int nq, double *__restrict__ out)
+{
+    const int q = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (q >= nq) return;
     double s = 0.0;
-    for (int sx = 0; sx < nsplit; ++sx) s += part[(long long)sx * nab + q];
-    int a = q / kb, b = q - a * kb;
-    out[(long long)a * ldo + b] = s;
+    for (int sx = lane; sx < nsplit; sx += 32) s += part[(long long)sx * nq + q];
+    s = warp_sum(s);
+    if (lane == 0) out[q] = s;
+}
+
+// the same with the splits added in ascending order (the Gram matrices of the
+// update: their last bits decide pivots and the order of close eigenvalues in
+// the decompositions): the partials pass through shared memory, so only the
+// additions form a chain
+constexpr int kPairSplits = 304;
+
+__global__ void __launch_bounds__(128) pair_reduce(const double *__restrict__ part, int nsplit, int nq, double *__restrict__ out)
+{
+    __shared__ double v[4][kPairSplits];
+    const int w = threadIdx.x >> 5, q = blockIdx.x * 4 + w, lane = threadIdx.x & 31;
+    if (q >= nq) return;
+    for (int sx = lane; sx < nsplit; sx += 32) v[w][sx] = part[(long long)sx * nq + q];
+    __syncwarp();
+    if (lane) return;
+    double s = 0.0;
+#pragma unroll 8
+    for (int sx = 0; sx < nsplit; ++sx) s += v[w][sx];
+    out[q] = s;
+}
+
+// The new pair of an update: rows s, y and B0 y of the store from the caller's
+// vectors, in one pass
+__global__ void __launch_bounds__(256) append_rows_kernel(const float *__restrict__ s, const float *__restrict__ y,
+                                                          const float *__restrict__ B0, long long n, float *__restrict__ sk,
+                                                          float *__restrict__ yk, float *__restrict__ byk)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const float yv = y[i];
+        sk[i] = s[i];
+        yk[i] = yv;
+        byk[i] = B0[i] * yv;
+    }
 }
 
 // Dot products of a new pair with the store (the update of the Gram
-// matrices): CTA (split, a) takes row a of [S_0..S_{k1-1}, B0Y_0..B0Y_{k1-1}]
+// matrices): CTA (split, a) takes row a of [S_0..S_{k1-1}, B0Y_0..B0Y_{k1-1}, y]
 // against the three vectors (y, s, B0 y) with compensated (Dot2) sums, then
-// an FP64 tree over its threads; part[sx][a][b] is reduced over the splits
-// by atb_reduce.
+// an FP64 tree over its threads; part[sx][a][b] is reduced over the splits.
 __global__ void __launch_bounds__(256) pair_dots_kernel(const float *__restrict__ S, const float *__restrict__ BY,
                                                         long long ld, int k1, const float *__restrict__ y,
                                                         const float *__restrict__ sv, const float *__restrict__ by,
@@ -139,7 +243,7 @@ __global__ void __launch_bounds__(256) pair_dots_kernel(const float *__restrict_
     __shared__ double red[3][256];
     const int sx = blockIdx.x, a = blockIdx.y, t = threadIdx.x;
     const long long ib = (long long)sx * chunk, ie = min(n, ib + chunk);
-    const float *ar = a < k1 ? S + (long long)a * ld : BY + (long long)(a - k1) * ld;
+    const float *ar = a < k1 ? S + (long long)a * ld : a < 2 * k1 ? BY + (long long)(a - k1) * ld : y;
     float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f};
     for (long long i = ib + t; i < ie; i += blockDim.x) {
         const float av = __ldg(ar + i);
@@ -158,7 +262,88 @@ __global__ void __launch_bounds__(256) pair_dots_kernel(const float *__restrict_
     }
     if (t == 0)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) part[((long long)sx * 2 * k1 + a) * 3 + b] = red[b][0];
+        for (int b = 0; b < 3; ++b) part[((long long)sx * (2 * k1 + 1) + a) * 3 + b] = red[b][0];
+}
+
+// a new pair's dots d[2 k1 + 1][3] (rows s_a, B0 y_a, y against y_k, s_k,
+// B0 y_k) into the store's FP64 matrices, k1 = k + 1
+__global__ void append_dots_kernel(const double *__restrict__ d, int k, int kmax, double *__restrict__ SY,
+                                   double *__restrict__ YBY, double *__restrict__ SS, double *__restrict__ SB,
+                                   double *__restrict__ BB)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i > k) return;
+    const double *sr = d + 3 * (long long)i, *br = d + 3 * (long long)(k + 1 + i);
+    const long long km = kmax, ik = i * km + k, ki = k * km + i;
+    SY[ik] = sr[0];
+    YBY[ik] = YBY[ki] = br[0];
+    SS[ik] = SS[ki] = sr[1];
+    SB[ik] = sr[2];                          // s_i^T B0 y_k
+    if (i < k) SB[ki] = br[1];               // s_k^T B0 y_i
+    BB[ik] = BB[ki] = br[2];
+}
+
+// W^T W = [[S^T S, S^T B0 Y], [(S^T B0 Y)^T, (B0 Y)^T B0 Y]] for k pairs
+__global__ void gram_kernel(const double *__restrict__ SS, const double *__restrict__ SB, const double *__restrict__ BB, int k,
+                            int kmax, double *__restrict__ G)
+{
+    const int m = 2 * k;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m * m; q += gridDim.x * blockDim.x) {
+        const int a = q / m, c = q - a * m;
+        const long long km = kmax;
+        G[q] = a < k ? (c < k ? SS[a * km + c] : SB[a * km + c - k]) : (c < k ? SB[c * km + a - k] : BB[(a - k) * km + c - k]);
+    }
+}
+
+// out[c][i] = sum_a coef[c][a] row_a[i] + beta * dw[i] * Xc[c][i] for one or two
+// outputs: a thread takes four columns i, the rows streamed as float4, the sums
+// compensated like the products above (the reads bound it, not the arithmetic).
+// Takes the place of the tensor-core combination there, which fills 64 outputs
+// (n = 1,147,323, 100 rows, one output: 276 us there, 82 us here).
+template <int KB>
+__global__ void __launch_bounds__(256) combine_thin_kernel(const float *__restrict__ A1, const float *__restrict__ A2, int k1,
+                                                           int ktot, long long lda, const float *__restrict__ coef,
+                                                           long long n, float *__restrict__ out, long long ldo,
+                                                           const float *__restrict__ dw, const float *__restrict__ Xc,
+                                                           long long ldx, float beta)
+{
+    const long long i0 = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
+    if (i0 >= n) return;
+    float hi[KB][4], lo[KB][4];
+#pragma unroll
+    for (int b = 0; b < KB; ++b)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) hi[b][e] = lo[b][e] = 0.f;
+    auto row = [&](int a) { return (a < k1 ? A1 + (long long)a * lda : A2 + (long long)(a - k1) * lda) + i0; };
+    auto add = [&](int a, float4 v) {
+#pragma unroll
+        for (int b = 0; b < KB; ++b) {
+            const float c = __ldg(coef + (long long)b * ktot + a);
+            dot2_term(c, v.x, hi[b][0], lo[b][0]);
+            dot2_term(c, v.y, hi[b][1], lo[b][1]);
+            dot2_term(c, v.z, hi[b][2], lo[b][2]);
+            dot2_term(c, v.w, hi[b][3], lo[b][3]);
+        }
+    };
+    int a = 0;
+    for (; a + 8 <= ktot; a += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldcs(reinterpret_cast<const float4 *>(row(a + u)));
+#pragma unroll
+        for (int u = 0; u < 8; ++u) add(a + u, v[u]);
+    }
+    for (; a < ktot; ++a) add(a, __ldcs(reinterpret_cast<const float4 *>(row(a))));
+#pragma unroll
+    for (int b = 0; b < KB; ++b)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const long long i = i0 + e;
+            if (i >= n) break;
+            float r = hi[b][e] + lo[b][e];
+            if (beta != 0.f) r = fmaf(beta * dw[i], Xc[b * ldx + i], r);
+            out[b * ldo + i] = r;
+        }
 }
 
 // out[c][i] = sum_a coef[c][a] row_a[i] + beta * dw[i] * Xc[c][i]  for c in [c0, c0 + cn)
@@ -229,14 +414,6 @@ __global__ void __launch_bounds__(128) combine_kernel(const float *__restrict__ 
     }
 }
 
-__global__ void mul_kernel(const float *__restrict__ a, const float *__restrict__ b, long long n,
-                           float *__restrict__ out)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        out[i] = a[i] * b[i];
-}
-
 // Largest of the lanes' values (first index among equals; idx < 0: none),
 // broadcast to the warp.  The values are compared through their IEEE bit
 // patterns as signed 64-bit integers, which orders every non-negative double
@@ -254,13 +431,6 @@ __device__ __forceinline__ void warp_argmax_nonneg(double &v, int &idx)
     key = __shfl_sync(0xffffffffu, key, 0);
     idx = __shfl_sync(0xffffffffu, idx, 0);
     v = __longlong_as_double(key);
-}
-
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
 }
 
 // Compact-form middle product for each column c of T ([2k][p], row stride
@@ -281,20 +451,20 @@ __host__ __device__ inline size_t middle_smem_bytes(int k, bool mats)
     return ((mats ? 2 * (size_t)k * k : 0) + 3 * (size_t)k) * sizeof(double);
 }
 
-__global__ void __launch_bounds__(32) middle_kernel(const double *__restrict__ T, const double *__restrict__ SYg,
+__global__ void __launch_bounds__(256) middle_kernel(const double *__restrict__ T, const double *__restrict__ SYg,
                                                     const double *__restrict__ YBYg, int k, int kmax, int p,
                                                     double gamma, int mats, float *__restrict__ coef,
                                                     double *__restrict__ coefd)
 {
     extern __shared__ double msm[];
-    const int c = blockIdx.x, lane = threadIdx.x;
+    const int c = blockIdx.x, lane = threadIdx.x & 31;
     if (c >= p) return;
     double *cv = msm, *d = cv + k, *rdiag = d + k;
     const double *SY = SYg, *YBY = YBYg;
     long long ls = kmax;                                // row stride of SY / YBY
     if (mats) {
         double *S1 = rdiag + k, *S2 = S1 + (size_t)k * k;
-        for (int q = lane; q < k * k; q += 32) {
+        for (int q = threadIdx.x; q < k * k; q += blockDim.x) {
             const int i = q / k, j = q - i * k;
             S1[q] = __ldg(SYg + (long long)i * kmax + j);
             S2[q] = __ldg(YBYg + (long long)i * kmax + j);
@@ -303,8 +473,10 @@ __global__ void __launch_bounds__(32) middle_kernel(const double *__restrict__ T
         YBY = S2;
         ls = k;
     }
-    for (int i = lane; i < k; i += 32) rdiag[i] = 1.0 / __ldg(SYg + (long long)i * kmax + i);
-    __syncwarp();
+    for (int i = threadIdx.x; i < k; i += blockDim.x) rdiag[i] = 1.0 / __ldg(SYg + (long long)i * kmax + i);
+    // the block's warps load; the chains run in the first
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
     // R cv = T_top (back substitution), R_ij = s_i^T y_j upper
     for (int i = k - 1; i >= 0; --i) {
         double s = 0.0;
@@ -359,20 +531,20 @@ __device__ __forceinline__ double pick_nj(const double (&v)[NJ], int t)
 }
 
 template <int NJ>
-__global__ void __launch_bounds__(32) middle_col_kernel(const double *__restrict__ T, const double *__restrict__ SYg,
+__global__ void __launch_bounds__(256) middle_col_kernel(const double *__restrict__ T, const double *__restrict__ SYg,
                                                         const double *__restrict__ YBYg, int k, int kmax, int p,
                                                         double gamma, int mats, float *__restrict__ coef,
                                                         double *__restrict__ coefd)
 {
     extern __shared__ double msm[];
-    const int c = blockIdx.x, lane = threadIdx.x;
+    const int c = blockIdx.x, lane = threadIdx.x & 31;
     if (c >= p) return;
     double *rdiag = msm + 2 * k;                        // the layout of middle_kernel: cv, d, rdiag, R, YBY
     const double *SY = SYg, *YBY = YBYg;
     long long ls = kmax;
     if (mats) {
         double *S1 = rdiag + k, *S2 = S1 + (size_t)k * k;
-        for (int q = lane; q < k * k; q += 32) {
+        for (int q = threadIdx.x; q < k * k; q += blockDim.x) {
             const int i = q / k, j = q - i * k;
             S1[q] = __ldg(SYg + (long long)i * kmax + j);
             S2[q] = __ldg(YBYg + (long long)i * kmax + j);
@@ -381,8 +553,10 @@ __global__ void __launch_bounds__(32) middle_col_kernel(const double *__restrict
         YBY = S2;
         ls = k;
     }
-    for (int i = lane; i < k; i += 32) rdiag[i] = 1.0 / __ldg(SYg + (long long)i * kmax + i);
-    __syncwarp();
+    for (int i = threadIdx.x; i < k; i += blockDim.x) rdiag[i] = 1.0 / __ldg(SYg + (long long)i * kmax + i);
+    // the block's warps load; the chains run in the first
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
     double x[NJ], cv[NJ], acc[NJ];
 #pragma unroll
     for (int t = 0; t < NJ; ++t) {
@@ -1068,9 +1242,9 @@ __global__ void philox_normal_kernel(float *__restrict__ X, long long total, lon
 int take_status(gbfwi_bfgs *h)
 {
     int st = 0;
-    GB_CUDA(cudaMemcpy(&st, h->status.p, sizeof(int), cudaMemcpyDeviceToHost));
+    GB_CUDA(cudaMemcpy(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost));
     if (st) {
-        GB_CUDA(cudaMemset(h->status.p, 0, sizeof(int)));
+        GB_CUDA(cudaMemset(h->status, 0, sizeof(int)));
         return GBFWI_ETIMEOUT;
     }
     return GBFWI_OK;
@@ -1078,16 +1252,40 @@ int take_status(gbfwi_bfgs *h)
 
 int grid_n(long long n) { return (int)std::min<long long>(std::max<long long>((n + 255) / 256, 1), 152 * 8); }
 
-// splits of the one- and two-column products
-long long thin_splits(long long n) { return std::min<long long>(304, std::max<long long>(1, (n + 4095) / 4096)); }
+// splits of the pair update's dots
+long long pair_splits(long long n) { return std::min<long long>(kPairSplits, std::max<long long>(1, (n + 4095) / 4096)); }
+
+long long thin_chunks(long long n) { return (n + kThinChunk - 1) / kThinChunk; }
 
 // FP64 split-K partials an (ka x kb) product of this store takes
 size_t part_need(const gbfwi_bfgs *h, int ka, int kb)
 {
     if (ka < 1 || kb < 1) return 0;
-    if (kb <= 2) return (size_t)thin_splits(h->n) * ka * kb;
+    if (kb <= 2) return (size_t)thin_chunks(h->n) * ka * kb;
     const long long ns = gb_tc_atb_splits(ka, kb, h->n);
     return ns < 1 ? 0 : (size_t)ns * ka * kb;
+}
+
+// out[a][b] = sum_i A_a[i] X_b[i] (device FP64, [rows][p]) for p <= 2 columns of
+// pitch ldx; the rows a < k1 come from A1, the rest from A2 (store pitch)
+int thin_product(gbfwi_bfgs *h, const float *A1, const float *A2, int k1, int rows, const float *X, long long ldx, int p,
+                 double *out, cudaStream_t s)
+{
+    const long long nc = thin_chunks(h->n);
+    if ((size_t)nc * rows * p > h->part.bytes / sizeof(double)) return GBFWI_EINVAL;
+    // about four CTAs an SM: a group takes all rows when the chunks alone give that
+    const long long want = std::max<long long>(1, 4 * 152 / nc);
+    const int group = std::min(128, (int)std::max<long long>(1, (rows + want - 1) / want));
+    const dim3 grid((unsigned)nc, (unsigned)((rows + group - 1) / group));
+    const size_t smem = (size_t)group * p * 8 * sizeof(double);
+    if (p == 1)
+        thin_rows_kernel<1><<<grid, 256, smem, s>>>(A1, A2, k1, rows, group, h->ld, X, ldx, h->n, h->part.as<double>());
+    else
+        thin_rows_kernel<2><<<grid, 256, smem, s>>>(A1, A2, k1, rows, group, h->ld, X, ldx, h->n, h->part.as<double>());
+    GB_LAUNCHED();
+    thin_reduce<<<(rows * p + 3) / 4, 128, 0, s>>>(h->part.as<double>(), (int)nc, rows * p, out);
+    GB_LAUNCHED();
+    return GBFWI_OK;
 }
 
 // out[a][b] = sum_i A_a[i] B_b[i] -> out (device FP64, row stride ldo); the
@@ -1098,31 +1296,20 @@ int atb(gbfwi_bfgs *h, const float *A1, const float *A2, int ka1, int ka, const 
         int kb, double *out, long long ldo, cudaStream_t s)
 {
     if (ka == 0 || kb == 0) return GBFWI_OK;
-    const long long n = h->n, ld = h->ld;
-    if (kb <= 2 && kb1 >= kb) {
-        const long long nsplit = thin_splits(n);
-        const long long chunk = (n + nsplit - 1) / nsplit;
-        const long long ns = (n + chunk - 1) / chunk;
-        for (int blk = 0; blk < 2; ++blk) {
-            const float *A = blk == 0 ? A1 : A2;
-            const int kab = blk == 0 ? std::min(ka1, ka) : ka - ka1;
-            if (kab <= 0) continue;
-            if ((size_t)ns * kab * kb > h->part.bytes / sizeof(double)) return GBFWI_EINVAL;
-            dim3 tg((unsigned)ns, (unsigned)kab);
-            if (kb == 1)
-                atb_thin<1><<<tg, 256, 0, s>>>(A, ld, B1, ld, nullptr, n, chunk, kab, h->part.as<double>());
-            else
-                atb_thin<2><<<tg, 256, 0, s>>>(A, ld, B1, ld, nullptr, n, chunk, kab, h->part.as<double>());
-            GB_LAUNCHED();
-            const int nab = kab * kb;
-            atb_reduce<<<(nab + 255) / 256, 256, 0, s>>>(h->part.as<double>(), (int)ns, nab,
-                                                         out + (blk == 0 ? 0 : (long long)ka1 * ldo), ldo, kb);
-            GB_LAUNCHED();
-        }
-        return GBFWI_OK;
-    }
-    return gb_tc_atb(A1, A2, ka1, ka, B1, B2, kb1, kb, ld, n, h->part.as<double>(), h->part.bytes / sizeof(double),
-                     out, ldo, h->status.as<int>(), s);
+    if (kb <= 2 && kb1 >= kb && ldo == kb) return thin_product(h, A1, A2, ka1, ka, B1, h->ld, kb, out, s);
+    return gb_tc_atb(A1, A2, ka1, ka, B1, B2, kb1, kb, h->ld, h->n, h->part.as<double>(), h->part.bytes / sizeof(double),
+                     out, ldo, h->status, s);
+}
+
+// dG = W^T W for the stored pairs
+int gram_matrix(gbfwi_bfgs *h, cudaStream_t s)
+{
+    const size_t m = 2 * (size_t)h->k;
+    GB_TRY(h->dG.ensure(m * m * sizeof(double)));
+    gram_kernel<<<(unsigned)std::min<size_t>((m * m + 255) / 256, 1024), 256, 0, s>>>(h->dSS, h->dSB, h->dBB, h->k, h->kmax,
+                                                                                     h->dG.as<double>());
+    GB_LAUNCHED();
+    return GBFWI_OK;
 }
 
 // out[c] = sum_a coef[c][a] row_a + beta * dw * Xc[c], c < nc; rows a < k1
@@ -1131,8 +1318,17 @@ int combine(gbfwi_bfgs *h, const float *A1, const float *A2, int k1, int ktot, c
             float *out, long long ldo, const float *dw, const float *Xc, long long ldx, float beta, cudaStream_t s)
 {
     const long long n = h->n, ld = h->ld;
+    if (ktot >= 1 && nc <= 2) {
+        const unsigned g = (unsigned)((n + 1023) / 1024);
+        if (nc == 1)
+            combine_thin_kernel<1><<<g, 256, 0, s>>>(A1, A2, k1, ktot, ld, coef, n, out, ldo, dw, Xc, ldx, beta);
+        else
+            combine_thin_kernel<2><<<g, 256, 0, s>>>(A1, A2, k1, ktot, ld, coef, n, out, ldo, dw, Xc, ldx, beta);
+        GB_LAUNCHED();
+        return GBFWI_OK;
+    }
     if (ktot >= 1 && ktot <= 128)
-        return gb_tc_combine(A1, A2, k1, ktot, ld, coef, nc, n, out, ldo, dw, Xc, ldx, beta, h->status.as<int>(), s);
+        return gb_tc_combine(A1, A2, k1, ktot, ld, coef, nc, n, out, ldo, dw, Xc, ldx, beta, h->status, s);
     // no rows (out = beta dw Xc) or more than 128: CUDA-core combination
     for (int c0 = 0; c0 < nc; c0 += 64) {
         int cn = std::min(64, nc - c0);
@@ -1177,7 +1373,7 @@ int launch_middle(gbfwi_bfgs *h, const double *T, int q, double gamma, float *co
                                                                                        : middle_kernel;
     if (bytes > 48 * 1024)
         GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    kern<<<q, 32, bytes, s>>>(T, h->dSY.as<double>(), h->dYBY.as<double>(), k, h->kmax, q, gamma, mats, coef, coefd);
+    kern<<<q, 256, bytes, s>>>(T, h->dSY, h->dYBY, k, h->kmax, q, gamma, mats, coef, coefd);
     GB_LAUNCHED();
     return GBFWI_OK;
 }
@@ -1211,34 +1407,17 @@ int apply_dev(gbfwi_bfgs *h, const float *Xd, long long ldx, int p, float *Zd, l
             GB_CUDA(cudaMemset2DAsync(Zd, ldz * sizeof(float), 0, h->n * sizeof(float), p, s));
             return GBFWI_OK;
         }
-        return combine(h, nullptr, nullptr, 0, 0, nullptr, p, Zd, ldz, h->B0.as<float>(), Xd, ldx, beta, s);
+        return combine(h, nullptr, nullptr, 0, 0, nullptr, p, Zd, ldz, h->B0, Xd, ldx, beta, s);
     }
     double *T = h->small.as<double>();
     // T = [S; B0 Y] X^T: rows 0..k-1 S^T x_c, rows k..2k-1 (B0 Y)^T x_c, one pass over X
-    if (p <= 2 && ldx != h->ld) {
-        // a caller's one or two vectors with their own pitch: thin products
-        const long long n = h->n;
-        const long long nsplit = thin_splits(n);
-        const long long chunk = (n + nsplit - 1) / nsplit;
-        const long long ns = (n + chunk - 1) / chunk;
-        for (int blk = 0; blk < 2; ++blk) {
-            const float *A = blk == 0 ? h->S.as<float>() : h->BY.as<float>();
-            dim3 tg((unsigned)ns, (unsigned)k);
-            if (p == 1)
-                atb_thin<1><<<tg, 256, 0, s>>>(A, h->ld, Xd, ldx, nullptr, n, chunk, k, h->part.as<double>());
-            else
-                atb_thin<2><<<tg, 256, 0, s>>>(A, h->ld, Xd, ldx, nullptr, n, chunk, k, h->part.as<double>());
-            GB_LAUNCHED();
-            atb_reduce<<<(k * p + 255) / 256, 256, 0, s>>>(h->part.as<double>(), (int)ns, k * p,
-                                                           T + (long long)blk * k * p, p, p);
-            GB_LAUNCHED();
-        }
-    } else {
-        GB_TRY(atb(h, h->S.as<float>(), h->BY.as<float>(), k, 2 * k, Xd, nullptr, p, p, T, p, s));
-    }
+    if (p <= 2)
+        GB_TRY(thin_product(h, h->S, h->BY, k, 2 * k, Xd, ldx, p, T, s));
+    else
+        GB_TRY(atb(h, h->S, h->BY, k, 2 * k, Xd, nullptr, p, p, T, p, s));
     GB_TRY(launch_middle(h, T, p, gamma, h->coef.as<float>(), nullptr, s));
-    return combine(h, h->S.as<float>(), h->BY.as<float>(), k, 2 * k, h->coef.as<float>(), p, Zd, ldz,
-                   h->B0.as<float>(), Xd, ldx, beta, s);
+    return combine(h, h->S, h->BY, k, 2 * k, h->coef.as<float>(), p, Zd, ldz,
+                   h->B0, Xd, ldx, beta, s);
 }
 
 }  // namespace
@@ -1256,25 +1435,45 @@ extern "C" int gbfwi_bfgs_create(long long n, int kmax, const float *B0, gbfwi_b
     h->n = n;
     h->ld = (n + 63) / 64 * 64;
     h->kmax = kmax;
-    const size_t store = (size_t)kmax * h->ld * sizeof(float);
-    int rc = h->S.ensure(store);
-    if (!rc) rc = h->Y.ensure(store);
-    if (!rc) rc = h->BY.ensure(store);
-    if (!rc) rc = h->B0.ensure((size_t)n * sizeof(float));
-    if (!rc) rc = h->dSY.ensure((size_t)kmax * kmax * sizeof(double));
-    if (!rc) rc = h->dYBY.ensure((size_t)kmax * kmax * sizeof(double));
-    if (!rc) rc = h->flag.ensure(16);
-    if (!rc) rc = h->status.ensure(16);
+    // S, Y, B0 Y, B0, the five FP64 matrices, the flags, and scratch for updates
+    // and for applies to one vector
+    const size_t store = (size_t)kmax * h->ld, mat = (size_t)kmax * kmax;
+    const size_t dots = 6 * (size_t)kmax + 96, coefs = std::max<size_t>(2 * (size_t)kmax, 16);
+    const size_t part = std::max((size_t)pair_splits(n) * (dots + 3), (size_t)thin_chunks(n) * 2 * kmax);
+    size_t bytes = 0;
+    auto piece = [&](size_t b) { const size_t at = bytes; bytes += (b + 255) / 256 * 256; return at; };
+    const size_t oS = piece(store * 4), oY = piece(store * 4), oBY = piece(store * 4), oB0 = piece((size_t)n * 4);
+    const size_t oM = piece(5 * mat * 8), oF = piece(32);
+    // (a large kmax would reserve scratch that it may never use: grown on demand then)
+    const bool scratch = kmax <= 256;
+    const size_t oP = piece(scratch ? part * 8 : 0), oD = piece(scratch ? dots * 8 : 0), oC = piece(scratch ? coefs * 4 : 0);
+    const int rc = h->arena.ensure(bytes);
     if (rc) { delete h; return rc; }
-    h->SY.assign((size_t)kmax * kmax, 0.0);
-    h->YBY.assign((size_t)kmax * kmax, 0.0);
-    h->SS.assign((size_t)kmax * kmax, 0.0);
-    h->SB.assign((size_t)kmax * kmax, 0.0);
-    h->BB.assign((size_t)kmax * kmax, 0.0);
-    // the row padding stays zero
-    if (cudaMemset(h->S.p, 0, store) != cudaSuccess || cudaMemset(h->Y.p, 0, store) != cudaSuccess ||
-        cudaMemset(h->BY.p, 0, store) != cudaSuccess || cudaMemset(h->status.p, 0, 16) != cudaSuccess ||
-        cudaMemcpy(h->B0.p, B0, (size_t)n * sizeof(float), cudaMemcpyDefault) != cudaSuccess) {
+    char *base = h->arena.as<char>();
+    h->S = reinterpret_cast<float *>(base + oS);
+    h->Y = reinterpret_cast<float *>(base + oY);
+    h->BY = reinterpret_cast<float *>(base + oBY);
+    h->B0 = reinterpret_cast<float *>(base + oB0);
+    double *mats = reinterpret_cast<double *>(base + oM);
+    h->dSY = mats;
+    h->dYBY = mats + mat;
+    h->dSS = mats + 2 * mat;
+    h->dSB = mats + 3 * mat;
+    h->dBB = mats + 4 * mat;
+    h->flag = reinterpret_cast<int *>(base + oF);
+    h->status = h->flag + 4;
+    if (scratch) {
+        h->part.lend(base + oP, part * 8);
+        h->small.lend(base + oD, dots * 8);
+        h->coef.lend(base + oC, coefs * 4);
+    }
+    // the row padding stays zero; the matrices' unset entries read as zero
+    const size_t pad = (size_t)(h->ld - n) * 4;
+    if ((pad && cudaMemset2D(h->S + n, h->ld * 4, 0, pad, (size_t)kmax) != cudaSuccess) ||
+        (pad && cudaMemset2D(h->Y + n, h->ld * 4, 0, pad, (size_t)kmax) != cudaSuccess) ||
+        (pad && cudaMemset2D(h->BY + n, h->ld * 4, 0, pad, (size_t)kmax) != cudaSuccess) ||
+        cudaMemset(base + oM, 0, oF + 32 - oM) != cudaSuccess ||
+        cudaMemcpy(h->B0, B0, (size_t)n * sizeof(float), cudaMemcpyDefault) != cudaSuccess) {
         gb_set_last_cuda_error(cudaGetLastError(), "initialise the BFGS store", __FILE__, __LINE__);
         delete h;
         return GBFWI_ECUDA;
@@ -1299,67 +1498,48 @@ extern "C" int gbfwi_bfgs_update(gbfwi_bfgs *h, const float *s_, const float *y_
     cudaStream_t s = (cudaStream_t)stream;
     const long long n = h->n, ld = h->ld;
     const int k = h->k;
-    float *sk = h->S.as<float>() + (long long)k * ld;
-    float *yk = h->Y.as<float>() + (long long)k * ld;
-    float *byk = h->BY.as<float>() + (long long)k * ld;
-    GB_CUDA(cudaMemcpyAsync(sk, s_, n * sizeof(float), cudaMemcpyDefault, s));
-    GB_CUDA(cudaMemcpyAsync(yk, y_, n * sizeof(float), cudaMemcpyDefault, s));
-    mul_kernel<<<grid_n(n), 256, 0, s>>>(h->B0.as<float>(), yk, n, byk);
-    GB_LAUNCHED();
-    // dots of the new pair with the store: rows [S_0..S_k, B0Y_0..B0Y_k]
-    // against (y_k, s_k, B0 y_k), and y_k^T y_k; they extend S^T Y, Y^T B0 Y
-    // and the Gram matrix W^T W of W = [S, B0 Y]
-    const int k1 = k + 1;
-    const long long nsplit = thin_splits(n);
+    float *sk = h->S + (long long)k * ld;
+    float *yk = h->Y + (long long)k * ld;
+    float *byk = h->BY + (long long)k * ld;
+    // dots of the new pair with the store: rows [S_0..S_k, B0Y_0..B0Y_k, y_k]
+    // against (y_k, s_k, B0 y_k); they extend S^T Y, Y^T B0 Y and the Gram matrix
+    // W^T W of W = [S, B0 Y]
+    const int k1 = k + 1, rows = 2 * k1 + 1;
+    const long long nsplit = pair_splits(n);
     const long long chunk = (n + nsplit - 1) / nsplit;
     const long long ns = (n + chunk - 1) / chunk;
-    GB_TRY(reserve(h, 1, false, {{k1, 1}}));
-    GB_TRY(h->part.ensure(std::max(h->part.bytes, (size_t)ns * 6 * k1 * sizeof(double))));
-    GB_TRY(h->small.ensure(std::max(h->small.bytes, (size_t)(6 * k1 + 8) * sizeof(double))));
-    double *d1 = h->small.as<double>();          // [2 k1][3]
-    double *d3 = d1 + 6 * k1;                    // [1]
-    const float *S = h->S.as<float>(), *BY = h->BY.as<float>();
-    pair_dots_kernel<<<dim3((unsigned)ns, (unsigned)(2 * k1)), 256, 0, s>>>(S, BY, ld, k1, yk, sk, byk, n, chunk,
-                                                                          h->part.as<double>());
+    GB_TRY(h->part.ensure((size_t)ns * 3 * rows * sizeof(double)));
+    GB_TRY(h->small.ensure((size_t)(3 * rows + 8) * sizeof(double)));
+    const float *sd = s_, *yd = y_;
+    if (!gb_is_device_ptr(s_)) {
+        GB_CUDA(cudaMemcpyAsync(sk, s_, n * sizeof(float), cudaMemcpyHostToDevice, s));
+        sd = sk;
+    }
+    if (!gb_is_device_ptr(y_)) {
+        GB_CUDA(cudaMemcpyAsync(yk, y_, n * sizeof(float), cudaMemcpyHostToDevice, s));
+        yd = yk;
+    }
+    append_rows_kernel<<<grid_n(n), 256, 0, s>>>(sd, yd, h->B0, n, sk, yk, byk);
     GB_LAUNCHED();
-    atb_reduce<<<(6 * k1 + 255) / 256, 256, 0, s>>>(h->part.as<double>(), (int)ns, 6 * k1, d1, 3, 3);
+    double *d = h->small.as<double>();           // [2 k1 + 1][3]
+    pair_dots_kernel<<<dim3((unsigned)ns, (unsigned)rows), 256, 0, s>>>(h->S, h->BY, ld, k1, yk, sk, byk, n, chunk,
+                                                                       h->part.as<double>());
     GB_LAUNCHED();
-    GB_TRY(atb(h, yk, nullptr, 1, 1, yk, nullptr, 1, 1, d3, 1, s));
-    std::vector<double> hd(6 * k1 + 1);
-    GB_CUDA(cudaMemcpyAsync(hd.data(), d1, hd.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+    pair_reduce<<<(3 * rows + 3) / 4, 128, 0, s>>>(h->part.as<double>(), (int)ns, 3 * rows, d);
+    GB_LAUNCHED();
+    // row and column k of the store's matrices: read once the pair is accepted
+    // (h->k grows), and in place when this call returns
+    append_dots_kernel<<<(k1 + 127) / 128, 128, 0, s>>>(d, k, h->kmax, h->dSY, h->dYBY, h->dSS, h->dSB, h->dBB);
+    GB_LAUNCHED();
+    std::vector<double> hd(3 * (size_t)rows);
+    GB_CUDA(cudaMemcpyAsync(hd.data(), d, hd.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
-    // hd[3 a + b]: a < k1 row s_a, a >= k1 row B0 y_(a - k1); b: y_k, s_k, B0 y_k
+    // hd[3 a + b]: a < k1 row s_a, a < 2 k1 row B0 y_(a - k1), then y_k; b: y_k, s_k, B0 y_k
     double ys = hd[3 * k], ss = hd[3 * k + 1], yy = hd[6 * k1];
     if (!std::isfinite(ys) || !std::isfinite(ss) || !std::isfinite(yy)) return gb_nonfinite("BFGS pair dot product");
     if (!(ys > 1e-12 * std::sqrt(ss) * std::sqrt(yy))) return GBFWI_ECURV;
-    for (double v : hd)
-        if (!std::isfinite(v)) return gb_nonfinite("BFGS pair dot product");
-    const int km = h->kmax;
-    auto at = [km](std::vector<double> &A, int i, int j) -> double & { return A[(size_t)i * km + j]; };
-    for (int i = 0; i <= k; ++i) {
-        const double *sr = &hd[3 * i], *br = &hd[3 * (k1 + i)];
-        at(h->SY, i, k) = sr[0];
-        at(h->YBY, i, k) = at(h->YBY, k, i) = br[0];
-        at(h->SS, i, k) = at(h->SS, k, i) = sr[1];
-        at(h->SB, i, k) = sr[2];                     // s_i^T B0 y_k
-        if (i < k) at(h->SB, k, i) = br[1];          // s_k^T B0 y_i
-        at(h->BB, i, k) = at(h->BB, k, i) = br[2];
-    }
-    GB_CUDA(cudaMemcpyAsync(h->dSY.p, h->SY.data(), h->SY.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-    GB_CUDA(cudaMemcpyAsync(h->dYBY.p, h->YBY.data(), h->YBY.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-    // W^T W for the k1 pairs: [[S^T S, S^T B0 Y], [(S^T B0 Y)^T, (B0 Y)^T B0 Y]]
-    const int m1 = 2 * k1;
-    std::vector<double> Gm((size_t)m1 * m1);
-    for (int a = 0; a < k1; ++a)
-        for (int b = 0; b < k1; ++b) {
-            Gm[(size_t)a * m1 + b] = at(h->SS, a, b);
-            Gm[(size_t)a * m1 + k1 + b] = at(h->SB, a, b);
-            Gm[(size_t)(k1 + b) * m1 + a] = at(h->SB, a, b);
-            Gm[(size_t)(k1 + a) * m1 + k1 + b] = at(h->BB, a, b);
-        }
-    GB_TRY(h->dG.ensure(Gm.size() * sizeof(double)));
-    GB_CUDA(cudaMemcpyAsync(h->dG.p, Gm.data(), Gm.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-    GB_CUDA(cudaStreamSynchronize(s));
+    for (int q = 0; q < 6 * k1; ++q)
+        if (!std::isfinite(hd[q])) return gb_nonfinite("BFGS pair dot product");
     h->k = k + 1;
     return GBFWI_OK;
 }
@@ -1531,11 +1711,11 @@ int finish_lowrank(gbfwi_bfgs *h, const double *Tq, int r, int rank, const doubl
     const bool devV = V && gb_is_device_ptr(V);
     float *Vd = devV ? V : h->E.as<float>();
     const long long ldv = devV ? n : ld;
-    GB_TRY(combine(h, h->S.as<float>(), h->BY.as<float>(), k, m, F, rank, Vd, ldv, nullptr, nullptr, 0, 0.f, s));
+    GB_TRY(combine(h, h->S, h->BY, k, m, F, rank, Vd, ldv, nullptr, nullptr, 0, 0.f, s));
     if (std_out) {
         const bool devS = gb_is_device_ptr(std_out);
         float *Sd = devS ? std_out : h->Q.as<float>();
-        std_kernel<<<grid_n(n), 256, 0, s>>>(Vd, ldv, lam, rank, h->B0.as<float>(), n, (float)eps_prior, Sd);
+        std_kernel<<<grid_n(n), 256, 0, s>>>(Vd, ldv, lam, rank, h->B0, n, (float)eps_prior, Sd);
         GB_LAUNCHED();
         if (!devS) GB_CUDA(cudaMemcpyAsync(std_out, Sd, n * sizeof(float), cudaMemcpyDeviceToHost, s));
     }
@@ -1570,6 +1750,7 @@ int lowrank_randomized(gbfwi_bfgs *h, const float *X, int p, int rank, unsigned 
     const long long n = h->n, ld = h->ld;
     const int k = h->k, m = 2 * k;
     if (k < 1) return gb_nonfinite("probe block E = (B - B0) X is zero or not finite");
+    GB_TRY(gram_matrix(h, s));
     // the probe block in a store buffer (aligned rows for the tensor cores)
     if (X) {
         GB_TRY(stage_rows(h, h->X, X, p, s));
@@ -1586,11 +1767,11 @@ int lowrank_randomized(gbfwi_bfgs *h, const float *X, int p, int rank, unsigned 
     double *Z = ar.take(pm), *Cd = ar.take(pm), *Pm = ar.take(pm), *Ge = ar.take(pp);
     double *lam = ar.take((size_t)p + 2);
     int *rdev = reinterpret_cast<int *>(ar.take(2));
-    int *flag = h->flag.as<int>();
+    int *flag = h->flag;
     const double *G = h->dG.as<double>();
     GB_CUDA(cudaMemsetAsync(flag, 0, 16, s));
     // 1. Z = W^T X (one pass over S, B0 Y and X), C = (M Z)^T: E = C W
-    GB_TRY(atb(h, h->S.as<float>(), h->BY.as<float>(), k, m, Xd, nullptr, p, p, Z, p, s));
+    GB_TRY(atb(h, h->S, h->BY, k, m, Xd, nullptr, p, p, Z, p, s));
     GB_TRY(launch_middle(h, Z, p, 1.0, nullptr, Cd, s));
     // 2. E E^T = C G C^T, the basis coordinates Tq
     GB_TRY(gemm(p, m, m, Cd, m, 1, G, m, 1, Pm, nullptr, m, s));               // P = C G
@@ -1661,11 +1842,12 @@ extern "C" int gbfwi_lowrank_exact(gbfwi_bfgs *h, int rank, double eps_prior, fl
     Arena ar{h->ex.as<double>()};
     double *Gs = ar.take(mm), *d = ar.take(m), *lam = ar.take((size_t)m + 2);
     int *rdev = reinterpret_cast<int *>(ar.take(2));
-    int *flag = h->flag.as<int>();
+    int *flag = h->flag;
     GB_CUDA(cudaMemsetAsync(flag, 0, 16, s));
     // 1. rank-revealing basis of W = [S, B0 Y]: pivoted Cholesky of the
     //    column-scaled Gram matrix D W^T W D (d_i = 1 / |w_i|), coordinates
     //    coef1 D, then a CholeskyQR pass (no n-long work: G is kept by the update)
+    GB_TRY(gram_matrix(h, s));
     GB_CUDA(cudaMemcpyAsync(Gs, h->dG.p, mm * sizeof(double), cudaMemcpyDeviceToDevice, s));
     gram_scale_kernel<<<1, 256, 0, s>>>(Gs, m, d);
     GB_LAUNCHED();
