@@ -717,7 +717,10 @@ __device__ void block_jacobi(float *A, float *U, int p, short *pairs, int max_sw
                     }
                 }
             }
-            if (warp == 0 && any) rotated = 1;
+            // a round without a rotation changes nothing (all warps see the same; the next
+            // barrier still orders their reads before any update)
+            if (!__any_sync(0xffffffffu, any)) continue;
+            if (t == 0) rotated = 1;
             __syncthreads();                    // every rotation read its pair before any update
             for (int m1 = warp; m1 < npair; m1 += nw) {
                 const int o = m1 & 31, j1 = m1 >> 5;
@@ -901,15 +904,15 @@ __global__ void __launch_bounds__(512) gram_pivchol_kernel(const double *__restr
     __syncthreads();
     for (int i = r - 1; i >= 0; --i) {
         const double rii = rinv[i];
-        for (int a = ty; a <= i; a += 16)
-            for (int c = tx; c < r; c += 32) {
-                if (c < i) continue;
-                const double xi = A[(long long)i * r + c] * rii;
+        for (int c = tx; c < r; c += 32) {
+            if (c < i) continue;
+            const double xi = A[(long long)i * r + c] * rii;
+            for (int a = ty; a <= i; a += 16)
                 if (a == i)
                     Ri[(long long)i * r + c] = xi;
                 else
                     A[(long long)a * r + c] -= R[(long long)a * p + i] * xi;
-            }
+        }
         __syncthreads();
     }
     for (long long q = t; q < pp; q += nt) coef[q] = 0.0;
@@ -968,14 +971,14 @@ __global__ void __launch_bounds__(32) omega_system_kernel(const double *__restri
 {
     const int i = blockIdx.x, lane = threadIdx.x;
     if (i >= r) return;
-    for (int j = 0; j < r; ++j) {
-        if (r == p) {
-            if (lane == 0) {
-                N[(long long)i * r + j] = QX[(long long)j * ldq + i];
-                Bt[(long long)i * r + j] = QE[(long long)j * ldq + i];
-            }
-            continue;
+    if (r == p) {
+        for (int j = lane; j < r; j += 32) {
+            N[(long long)i * r + j] = QX[(long long)j * ldq + i];
+            Bt[(long long)i * r + j] = QE[(long long)j * ldq + i];
         }
+        return;
+    }
+    for (int j = 0; j < r; ++j) {
         double nij = 0.0, bji = 0.0;
         for (int c = lane; c < p; c += 32) {
             const double xi = QX[(long long)i * ldq + c];
@@ -998,6 +1001,7 @@ __global__ void __launch_bounds__(512) lu_kernel(double *__restrict__ M, double 
     double *A = use_smem ? lu_smem : M;
     double *Ls = use_smem ? lu_smem + (size_t)r * r : L;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    __shared__ double s_inv;
     for (int a = ty; a < r; a += 16)
         for (int c = tx; c < r; c += 32) {
             if (use_smem) A[a * r + c] = M[(long long)a * r + c];
@@ -1019,6 +1023,12 @@ __global__ void __launch_bounds__(512) lu_kernel(double *__restrict__ M, double 
                 if (!(bv > 0.0)) *flag = 3;
                 perm[j] = best;
             }
+            // the reciprocal pivot once: every warp dividing for itself kept the SM's one
+            // FP64 pipe busy (r = 60: 145 us in all, 120 us so)
+            const double d = A[best * r + j];
+            const double inv = 1.0 / (d == 0.0 ? 1.0 : d);
+            if (tx == 0) s_inv = inv;
+            __syncwarp();
             if (best != j)
                 for (int c = tx; c < r; c += 32) {
                     const double x = A[j * r + c];
@@ -1032,9 +1042,7 @@ __global__ void __launch_bounds__(512) lu_kernel(double *__restrict__ M, double 
                 }
         }
         __syncthreads();
-        double d = A[j * r + j];
-        if (d == 0.0) d = 1.0;
-        const double inv = 1.0 / d;
+        const double inv = s_inv;
         for (int a = j + 1 + ty; a < r; a += 16) {
             const double l = A[a * r + j] * inv;
             for (int c = j + 1 + tx; c < r; c += 32) A[a * r + c] -= l * A[j * r + c];

