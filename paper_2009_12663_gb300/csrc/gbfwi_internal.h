@@ -177,8 +177,8 @@ struct gbfwi_mesh {
     std::vector<Lane *> lanes;
     std::vector<ResidentPlan *> plans;  // of the resident time loop
     DevBuf w_eacc;                      // its strain sums by element
-    DevBuf w_feat;                      // node-grid features of the learned preconditioner
     DevBuf w_xch;                       // its exchange of node lines between tiles
+    DevBuf w_feat;                      // node-grid features of the learned preconditioner
     // CUDA graphs of whole forward / adjoint passes, keyed by schedule,
     // batch size and work-buffer addresses
     struct CachedGraph {
@@ -211,7 +211,9 @@ int gb_take_status(gbfwi_mesh *m);
 // shot of a batch)
 // ---------------------------------------------------------------------------
 
-enum StepMode { MODE_FWD = 0, MODE_FWD_PC = 1, MODE_ADJ_G = 2, MODE_ADJ_PC = 3 };
+// (resident loops only: MODE_FWD_PC is the forward field with its velocities stored, MODE_RCV the
+// receiver field likewise, driven by the records backwards in time)
+enum StepMode { MODE_FWD = 0, MODE_FWD_PC = 1, MODE_ADJ_G = 2, MODE_ADJ_PC = 3, MODE_RCV = 4 };
 
 struct StepArgs {
     int nex, nez, nx, nz, pitch;
@@ -258,6 +260,8 @@ struct ResidentArgs {
     float2 *vh;                   // half-step velocity, in place
     float2 *out;                  // level k at slot k - out_k0 (out_ring: k % 3), written for k >= out_from
     int out_from, out_ring, out_k0;
+    float2 *vout;                 // MODE_FWD_PC, MODE_RCV: the velocity that made level k, at the same slot
+    int reverse;                  // MODE_RCV: the signals run backwards
     const float2 *hist; int hist_k0;   // adjoint: forward level k at slot k - hist_k0
     const float2 *lm;             // (lambda, mu) times the quadrature weight
     const float *minv;
@@ -282,6 +286,14 @@ int gb_assemble_strain(const gbfwi_mesh *m, const float *eacc, int B, float *acc
                        cudaStream_t s);
 size_t gb_resident_exchange(const ResidentPlan &p, int nshots, long long NP);   // bytes of the exchange buffer
 int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf &xch, cudaStream_t s);
+
+// Time integrals of the preconditioners from stored levels, B shots (sem_integrals.cu): w, v
+// the field (levels 0 .. nt + 1) and the velocity that made each level (slots 2 .. nt + 1);
+// u null: integrals of w alone (P1, P3), else with the field u backwards in time (P2, P4).
+// acc [B][4][NP]: map 0, and maps 1..3 when strains are asked for; esum: gb_integral_bytes
+size_t gb_integral_bytes(const gbfwi_mesh *m, int B);
+int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *v, const float2 *u, bool strains, float *esum,
+                      float *acc, cudaStream_t s);
 
 int gb_launch_step(int mode, int tile, const StepArgs &a, int nbatch, cudaStream_t s);
 int gb_prepare_step(int mode, int tile);   // set kernel attributes outside any stream capture

@@ -100,7 +100,7 @@ int run_resident(const Ctx &c, int mode, ResidentArgs &r)
 {
     ResidentPlan *p = gb_resident_plan(c.m, mode, c.B);
     if (!p) return GBFWI_EINVAL;
-    const bool fwd = mode == MODE_FWD;
+    const bool fwd = mode == MODE_FWD || mode == MODE_FWD_PC;
     r.gptr = (fwd ? p->lists.src_gptr : p->lists.rec_gptr).as<int>();
     r.groups = (fwd ? p->lists.src_groups : p->lists.rec_groups).as<InjGroup>();
     r.entries = (fwd ? p->lists.src_entries : p->lists.rec_entries).as<InjEntry>();
@@ -113,7 +113,7 @@ constexpr int kNoLevel = INT_MAX;
 
 // forward launches n in [n0, n1); `need`: first level that is read later
 int fwd_range(const Ctx &c, int mode, int n0, int n1, const Levels &f, int need, float2 *vh, float *seis, float *acc,
-              long long acc_shot_stride, long long acc_comp_stride)
+              long long acc_shot_stride, long long acc_comp_stride, float2 *vout = nullptr)
 {
     StepArgs a;
     base_args(a, c);
@@ -131,9 +131,10 @@ int fwd_range(const Ctx &c, int mode, int n0, int n1, const Levels &f, int need,
     a.acc = acc;
     a.acc_shot_stride = acc_shot_stride;
     a.acc_comp_stride = acc_comp_stride;
-    if (c.resident && mode == MODE_FWD) {
+    if (c.resident) {
         ResidentArgs r;
         resident_args(r, a, c, n0, n1, f, need);
+        r.vout = vout;
         return run_resident(c, mode, r);
     }
     for (int n = n0; n < n1; ++n) {
@@ -147,9 +148,10 @@ int fwd_range(const Ctx &c, int mode, int n0, int n1, const Levels &f, int need,
     return GBFWI_OK;
 }
 
-// adjoint launches j in [j0, j1); the adjoint field cycles through the ring w
+// adjoint launches j in [j0, j1); the adjoint field cycles through the ring w.
+// MODE_RCV (resident): the field alone, all levels to w and their velocities to vout
 int adj_range(const Ctx &c, int mode, int j0, int j1, const Levels &w, float2 *wh, const Levels &hist,
-              const float *sig, float *acc, long long acc_shot_stride, long long acc_comp_stride)
+              const float *sig, float *acc, long long acc_shot_stride, long long acc_comp_stride, float2 *vout = nullptr)
 {
     const int nt = c.m->d.nt;
     StepArgs a;
@@ -167,6 +169,13 @@ int adj_range(const Ctx &c, int mode, int j0, int j1, const Levels &w, float2 *w
     a.acc = acc;
     a.acc_shot_stride = acc_shot_stride;
     a.acc_comp_stride = acc_comp_stride;
+    if (c.resident && mode == MODE_RCV) {
+        ResidentArgs r;
+        resident_args(r, a, c, j0, j1, w, 0);
+        r.reverse = 1;
+        r.vout = vout;
+        return run_resident(c, mode, r);
+    }
     if (c.resident && mode == MODE_ADJ_G) {
         ResidentArgs r;
         resident_args(r, a, c, j0, j1, w, j1 < nt ? j1 : kNoLevel);
@@ -649,6 +658,10 @@ struct BatchHist {
 // for, to run more shots at once on meshes too small to fill the GPU.
 constexpr long long kSmallHistory = 1LL << 30;
 
+// Bytes of levels the preconditioner maps may keep to form their integrals from
+// (sem_integrals.cu).
+constexpr long long kMapHistory = 6LL << 30;
+
 // the work buffers of one concurrent lane
 struct LaneRef {
     DevBuf *hist, *snap, *vh, *adj, *wh, *seis, *batch, *acc;
@@ -1063,6 +1076,78 @@ static int b0_from_map(gbfwi_mesh *m, const float *Hd, float *S1, float *S2, dou
     return GBFWI_OK;
 }
 
+// Shots a resident map run takes at once (0: the preconditioner steps run). Both
+// passes keep their levels, so the batches are smaller than the steps' of Bold
+// shots; a step costs 2 x 5.3 us resident, and 8 us forward (receiver maps) and
+// 38 us a wave of 304 CTAs otherwise (measured at 81 x 21 elements, 5 shots).
+static int map_batch(gbfwi_mesh *m, int nshot, bool receiver, int tile, int Bold, long long NP)
+{
+    const long long shot = (receiver ? 3 : 2) * (m->d.nt + 2LL) * NP * (long long)sizeof(float2);
+    int B = (int)std::min<long long>(nshot, kMapHistory / shot);
+    if (B < 1 || !gb_resident_plan(m, MODE_FWD, B)) return 0;
+    B = (nshot + (nshot + B - 1) / B - 1) / ((nshot + B - 1) / B);      // equal batches
+    const ResidentPlan *f = gb_resident_plan(m, receiver ? MODE_FWD : MODE_FWD_PC, B), *r = receiver ? gb_resident_plan(m, MODE_RCV, B) : f;
+    if (!f || !r) return 0;
+    const TileShape &t = kTiles[tile];
+    const long long ctas = (long long)((m->d.nex + t.tx - 1) / t.tx) * ((m->d.nez + t.tz - 1) / t.tz) * Bold;
+    const double launches = (B + f->per_launch - 1) / f->per_launch + (receiver ? (B + r->per_launch - 1) / r->per_launch : 0);
+    const double here = (double)((nshot + B - 1) / B) * 5.3 * launches;
+    const double steps = (double)((nshot + Bold - 1) / Bold) * ((receiver ? 8.0 : 0.0) + 38.0 * (double)((ctas + 303) / 304));
+    return here < steps ? B : 0;
+}
+
+// The integrals of every shot (summed into tot) from stored levels.  GBFWI_ENOMEM
+// before anything is queued when the levels do not fit: nothing is kept then.
+static int resident_maps(gbfwi_mesh *m, int nshot, int Bmax, int kind, int tile, float *tot, long long NP, cudaStream_t s)
+{
+    const int nt = m->d.nt;
+    const bool receiver = kind == 2 || kind == 4, strains = kind >= 3;
+    const int fwd = receiver ? MODE_FWD : MODE_FWD_PC;
+    const size_t levels = (size_t)(nt + 2) * Bmax * NP * sizeof(float2), seis_shot = (size_t)m->nrec * 2 * nt;
+    DevBuf *big[] = {&m->w_hist, &m->w_snap, &m->w_adj, &m->w_eacc};
+    int rc = m->w_hist.ensure(levels);
+    if (!rc) rc = m->w_snap.ensure(levels);
+    if (!rc && receiver) rc = m->w_adj.ensure(levels);
+    if (!rc && strains) rc = m->w_eacc.ensure(gb_integral_bytes(m, Bmax));
+    if (!rc && receiver) rc = m->w_seis.ensure(seis_shot * Bmax * sizeof(float));
+    if (!rc) rc = m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2));
+    for (int B : {Bmax, nshot - (nshot - 1) / Bmax * Bmax}) {
+        if (!rc) rc = reserve_exchange(m, fwd, B, NP);
+        if (!rc && receiver) rc = reserve_exchange(m, MODE_RCV, B, NP);
+    }
+    if (rc) {
+        for (DevBuf *b : big) b->release();
+        return rc;
+    }
+    float *acc = m->w_pc.as<float>();
+    float2 *vh = m->w_vh.as<float2>();
+    for (int i0 = 0; i0 < nshot; i0 += Bmax) {
+        const int B = std::min(Bmax, nshot - i0);
+        const long long lev = B * NP;
+        const Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, true};
+        const Levels u{m->w_hist.as<float2>(), lev, 0, false}, v{m->w_snap.as<float2>(), lev, 0, false};
+        const Levels w{m->w_adj.as<float2>(), lev, 0, false};
+        auto at_rest = [&](const Levels &f) -> int {
+            GB_CUDA(cudaMemsetAsync(f.base, 0, 2 * lev * sizeof(float2), s));
+            GB_CUDA(cudaMemsetAsync(vh, 0, lev * sizeof(float2), s));
+            return GBFWI_OK;
+        };
+        GB_TRY(at_rest(u));
+        GB_CUDA(cudaMemsetAsync(acc, 0, (size_t)B * 4 * NP * sizeof(float), s));
+        float *seis = m->w_seis.as<float>();
+        GB_TRY(fwd_range(c, fwd, 0, nt, u, 0, vh, receiver ? seis : nullptr, nullptr, 0, 0, receiver ? nullptr : v.base));
+        if (receiver) {
+            GB_TRY(at_rest(w));
+            GB_TRY(adj_range(c, MODE_RCV, 0, nt, w, vh, u, seis, nullptr, 0, 0, v.base));
+        }
+        GB_TRY(gb_time_integrals(m, B, receiver ? w.base : u.base, v.base, receiver ? u.base : nullptr, strains,
+                                 m->w_eacc.as<float>(), acc, s));
+        acc_reduce<<<grid_for(4 * NP), 256, 0, s>>>(acc, B, 4, NP, tot);
+        GB_LAUNCHED();
+    }
+    return GBFWI_OK;
+}
+
 extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot, int kind, double sigma,
                                   double damp, float *H, float *B0, void *stream)
 {
@@ -1090,21 +1175,28 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     const long long lev = (long long)Bmax * NP;
     const double dt = m->d.dt;
 
+    const int Bmap = map_batch(m, nshot, receiver, tile, Bmax, NP);
     GB_TRY(m->w_vh.ensure(lev * sizeof(float2)));
-    GB_TRY(m->w_pc.ensure((size_t)Bmax * 4 * NP * sizeof(float)));
+    GB_TRY(m->w_pc.ensure((size_t)std::max(Bmax, Bmap) * 4 * NP * sizeof(float)));
     GB_TRY(m->w_grad.ensure((size_t)5 * NP * sizeof(float)));
     GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
-    BatchHist h;
-    if (receiver) {
-        GB_TRY(alloc_hist(m, lane0(m, s), Bmax, m->sch.ckpt_every, NP, h, true));
-        GB_TRY(m->w_seis.ensure(seis_shot * Bmax * sizeof(float)));
-    } else {
-        GB_TRY(m->w_hist.ensure((size_t)3 * lev * sizeof(float2)));
-    }
     GB_CUDA(cudaMemcpyAsync(m->w_shots.p, shot_ids, nshot * sizeof(int), cudaMemcpyHostToDevice, s));
     float *tot = m->w_grad.as<float>();
     GB_CUDA(cudaMemsetAsync(tot, 0, 4 * NP * sizeof(float), s));
-    for (int i0 = 0; i0 < nshot; i0 += Bmax) {
+    bool done = false;
+    if (Bmap) {
+        const int rc = resident_maps(m, nshot, Bmap, kind, tile, tot, NP, s);
+        if (rc && rc != GBFWI_ENOMEM) return rc;
+        done = rc == GBFWI_OK;
+    }
+    BatchHist h;
+    if (!done && receiver) {
+        GB_TRY(alloc_hist(m, lane0(m, s), Bmax, m->sch.ckpt_every, NP, h, true));
+        GB_TRY(m->w_seis.ensure(seis_shot * Bmax * sizeof(float)));
+    } else if (!done) {
+        GB_TRY(m->w_hist.ensure((size_t)3 * lev * sizeof(float2)));
+    }
+    for (int i0 = 0; i0 < nshot && !done; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
         Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, resident};
         float *acc = m->w_pc.as<float>();

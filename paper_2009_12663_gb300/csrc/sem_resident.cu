@@ -1,6 +1,6 @@
 // Whole time loops of the spectral-element scheme in one cooperative launch
-// (sm_103a): forward passes and adjoint-gradient passes of meshes whose
-// fields fit the SMs' shared memory.
+// (sm_103a): forward passes, receiver-field passes and adjoint-gradient passes
+// of meshes whose fields fit the SMs' shared memory.
 //
 // The step kernels of sem_step.cu read and write every field once per launch
 // (44 B a node forward, 76 B adjoint, from L2) and start cold each step; a
@@ -8,7 +8,10 @@
 // adjoint a step measured on 12 x 6 elements).  Here a CTA keeps its tile for
 // all steps: the displacement window, the weighted moduli, the velocity and
 // the accumulators stay in shared memory or registers, and between steps a
-// CTA only trades the node lines its neighbours need.
+// CTA only trades the node lines its neighbours need.  Measured a step: 3.9 us
+// forward (40 x 20 elements, one CTA an SM), 5.3 us with two shots an SM,
+// 5.3 to 5.7 us adjoint; the chain of a step is the exchange (1.5 us), the
+// forces (1.6 us), the update (0.8 us) and the sends (0.4 us).
 //
 // Tile and threads.  A CTA owns TX x TZ elements (chosen at run time) of one
 // shot and recomputes the element column to its left and the row above, one
@@ -22,6 +25,12 @@
 // cell, so a warp's patch reads are contiguous 16-byte accesses: the loop is
 // bound by shared-memory wavefronts and the FMA pipe together (72% and 61%
 // of peak measured on the force loop alone).
+//
+// Correlations.  In the adjoint pass one more thread per owned element adds
+// the step's strain and mass correlations from the forward level, beside the
+// exchange and the next forces: on the element threads they took 138 ms of the
+// gradient on 340 x 70 elements and 500 steps that takes 96 ms so (130 ms with
+// the step kernels).
 //
 // Exchange.  Every node another tile's window holds is sent as two 64-bit
 // words (component, step tag) with relaxed gpu-scope stores; the reader polls
@@ -190,7 +199,7 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
 {
     using S = Shape<NT_, MODE>;
     constexpr int NT = S::NT, PS = S::PS, NO = S::NO, NA = S::THREADS, kMaxHalo = S::L.halo;
-    constexpr bool ADJ = S::ADJ;
+    constexpr bool ADJ = S::ADJ, VEL = MODE == MODE_RCV;
     extern __shared__ float4 rsm[];
     float4 *win0 = rsm;                                          // field window [8][PS], two in the adjoint
     float4 *lmw = win0 + (ADJ ? 2 : 1) * S::WIN;                 // weighted moduli window [8][PS]
@@ -492,7 +501,7 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
 
     // signals of step n into their half of ssig (asynchronous)
     auto fetch_signals = [&](int n) {
-        const int ts = ADJ ? a.nt - 1 - n : n + 1;
+        const int ts = ADJ || (VEL && a.reverse) ? a.nt - 1 - n : n + 1;
 #pragma unroll 1
         for (int e = t; e < ne; e += NT) {
             const int4 I = sent[e];
@@ -513,6 +522,15 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
         for (int q = t; q < nextra; q += NT) {
             const int rx = q < ncol ? 4 * nex : q - ncol, rz = q < ncol ? q : 4 * nez;
             ob[(4 * ez0 + rz) * pitch + 4 * ex0 + rx] = reinterpret_cast<const float2 *>(w)[sxi[q].z];
+        }
+        if (VEL) {                                                // the velocity that made this level
+            float2 *vb = a.vout + (long long)(k - a.out_k0) * a.lev + fo;
+            if (owns)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) store_row(vb + g00 + j * pitch, vr[2 * j], vr[2 * j + 1]);
+#pragma unroll 1
+            for (int q = t; q < nextra; q += NT)
+                vb[q < ncol ? (4 * ez0 + q) * pitch + a.nx - 1 : (a.nz - 1) * pitch + 4 * ex0 + q - ncol] = svx[q];
         }
         // the next level lies in new pages: have their translation ready
         if (!a.out_ring && t < 2 && k <= a.n1) prefetch_l2(ob + a.lev + (t ? ize - 1 : 4 * ez0) * pitch + 4 * ex0);
@@ -749,6 +767,7 @@ constexpr Variant variant() {
  }
 
 const Variant kVariants[] = {variant<64, MODE_FWD>(),   variant<128, MODE_FWD>(),   variant<192, MODE_FWD>(),
+                             variant<64, MODE_RCV>(),   variant<128, MODE_RCV>(),   variant<192, MODE_RCV>(),
                              variant<64, MODE_ADJ_G>(), variant<128, MODE_ADJ_G>(), variant<192, MODE_ADJ_G>()};
 
 const Variant *find_variant(int NT, int mode)
@@ -757,6 +776,9 @@ const Variant *find_variant(int NT, int mode)
         if (v.NT == NT && v.MODE == mode) return &v;
     return nullptr;
 }
+
+// the kernel that runs a mode (MODE_RCV's also stores the velocities)
+int kernel_mode(int mode) { return mode == MODE_FWD_PC ? MODE_RCV : mode; }
 
 bool fits(int NT, int TX, int TZ)
 {
@@ -801,7 +823,7 @@ size_t smem_of(const Variant &v, int TX, int TZ, int ntx, int ntz, bool free_top
 // sem_step.cu run).
 ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
 {
-    if (mode != MODE_FWD && mode != MODE_ADJ_G) return nullptr;
+    if (mode == MODE_ADJ_PC) return nullptr;
     for (ResidentPlan *p : m->plans)
         if (p->mode == mode && p->wanted == shots) return p->NT ? p : nullptr;
     ResidentPlan best;
@@ -810,7 +832,7 @@ ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
     double best_cost = 1e300;
     const int nex = m->d.nex, nez = m->d.nez;
     for (const Variant &v : kVariants) {
-        if (v.MODE != mode) continue;
+        if (v.MODE != kernel_mode(mode)) continue;
         int nsm = 0, slots = 0;
         size_t known = 0;                        // shared bytes `slots` was looked up for
         for (int tx = 1; tx < v.NT; ++tx) {
@@ -831,8 +853,8 @@ ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
                 const double warps = ((TX + 1) * (TZ + 1) + 31) / 32 * (double)((c * T + nsm - 1) / nsm);
                 // (us; measured: 4.2 us forward and 5.7 us adjoint a step with one CTA an SM,
                 // 5.3 us forward with two)
-                const double issue = (mode == MODE_FWD ? 0.43 : 0.90) * warps;
-                const double lat = (mode == MODE_FWD ? 2.6 : 3.6) + (T > 1 ? 1.2 : 0.0) + 0.05 * warps;
+                const double issue = (v.MODE != MODE_ADJ_G ? 0.43 : 0.90) * warps;
+                const double lat = (v.MODE != MODE_ADJ_G ? 2.6 : 3.6) + (T > 1 ? 1.2 : 0.0) + 0.05 * warps;
                 const double cost = ((shots + c - 1) / c) * std::max(issue, lat);
                 if (cost < best_cost * (1 - 1e-9)) {
                     best_cost = cost;
@@ -854,10 +876,11 @@ ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
     p->TX = best.TX; p->TZ = best.TZ; p->ntx = best.ntx; p->ntz = best.ntz;
     if (gb_build_lists(m, p->TX, p->TZ, true, p->lists) != GBFWI_OK) return nullptr;
     // with the real injection lists: how many shots fit one launch
-    const Variant *v = find_variant(best.NT, mode);
-    p->grp_cap = mode == MODE_FWD ? p->lists.src_most : p->lists.rec_most;
-    p->ent_cap = mode == MODE_FWD ? p->lists.src_entries_most : p->lists.rec_entries_most;
-    p->rec_cap = mode == MODE_FWD ? p->lists.recorded_most : 0;
+    const Variant *v = find_variant(best.NT, kernel_mode(mode));
+    const bool fwd = mode == MODE_FWD || mode == MODE_FWD_PC;
+    p->grp_cap = fwd ? p->lists.src_most : p->lists.rec_most;
+    p->ent_cap = fwd ? p->lists.src_entries_most : p->lists.rec_entries_most;
+    p->rec_cap = fwd ? p->lists.recorded_most : 0;
     int nsm = 0;
     p->smem = smem_of(*v, p->TX, p->TZ, p->ntx, p->ntz, m->d.free_surface_top, p->grp_cap, p->ent_cap, p->rec_cap);
     const int slots = slots_of(*v, p->smem, &nsm);
@@ -870,9 +893,9 @@ ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
 
 int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf &xch, cudaStream_t s)
 {
-    const Variant *v = find_variant(p.NT, p.mode);
+    const Variant *v = find_variant(p.NT, kernel_mode(p.mode));
     if (!v || a.pitch % 4 != 0 || a.fstride % 4 != 0 || a.lev % 4 != 0 || a.acc_comp_stride % 4 != 0 ||
-        a.acc_shot_stride % 4 != 0 || ((uintptr_t)a.u0 & 15) || ((uintptr_t)a.out & 31) || ((uintptr_t)a.vh & 15) ||
+        a.acc_shot_stride % 4 != 0 || ((uintptr_t)a.vout & 31) || ((uintptr_t)a.u0 & 15) || ((uintptr_t)a.out & 31) || ((uintptr_t)a.vh & 15) ||
         ((uintptr_t)a.minv & 15) || ((uintptr_t)a.acc & 15) || ((uintptr_t)a.hist & 31) || ((uintptr_t)a.eacc & 15) || !a.status)
         return GBFWI_EINVAL;
     a.TX = p.TX; a.TZ = p.TZ; a.ntx = p.ntx; a.ntz = p.ntz;
@@ -888,6 +911,7 @@ int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf
         a.u0 += s0 * a.fstride;
         a.vh += s0 * a.fstride;
         a.out += s0 * a.fstride;
+        if (a.vout) a.vout += s0 * a.fstride;
         if (a.hist) a.hist += s0 * a.fstride;
         if (a.acc) a.acc += s0 * a.acc_shot_stride;
         if (a.eacc) a.eacc += (long long)s0 * a.nex * a.nez * 52;
