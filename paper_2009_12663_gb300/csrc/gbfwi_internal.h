@@ -178,6 +178,7 @@ struct gbfwi_mesh {
     std::vector<ResidentPlan *> plans;  // of the resident time loop
     DevBuf w_eacc;                      // its strain sums by element
     DevBuf w_xch;                       // its exchange of node lines between tiles
+    DevBuf w_chk;                       // model checks (and a model given on the host)
     DevBuf w_feat;                      // node-grid features of the learned preconditioner
     // CUDA graphs of whole forward / adjoint passes, keyed by schedule,
     // batch size and work-buffer addresses
