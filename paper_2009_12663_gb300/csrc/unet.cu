@@ -8,17 +8,22 @@
 // after the upsampled features, a 1x1 output convolution.
 //
 // Every convolution is a dense contraction and runs on the tensor cores as
-// one BF16 GEMM with FP32 accumulation (mma.sync m16n8k16, operands staged
-// by cp.async and fed by ldmatrix):
-//   forward        Y[co][p]     = W[co][kk] Xcol[kk][p]          (+ bias, ReLU, -> bf16)
-//   input grad     dXcol[kk][p] = W^T[kk][co] G[co][p]           (then a gathering col2im)
-//   weight grad    dW[co][kk]  += G[co][p] Xcol^T[p][kk]         (split over p, splits summed in order)
-// with kk = c*9 + ky*3 + kx and Xcol[kk][y*W + x] = X[c][y+ky-1][x+kx-1]
-// (zero outside).  The four operand layouts of these products are the
-// template arguments of one kernel.  Everything around the GEMMs (im2col
-// with fused upsampling and concatenation, col2im, pooling, the ReLU masks
-// of the gradients, bias sums, loss, Adam, resampling) is memory-bound and
-// written as plain coalesced kernels.
+// one BF16 GEMM with FP32 accumulation (mma.sync m16n8k16, fed by ldmatrix):
+//   forward        Y[co][p]   = W[co][kk] X[kk][p]          (+ bias, ReLU, -> bf16)
+//   weight grad    dW[co][kk] += G[co][p] X^T[p][kk]        (split over p, splits summed in order)
+//   input grad     dX[c][p]   = sum_tap (sum_co W[co][c, tap] G[co][p - tap])
+// with kk = c*9 + ky*3 + kx and X[kk][y*W + x] = x[c][y+ky-1][x+kx-1] (zero
+// outside).  The column matrix X is never written: the kernels gather its
+// 8-pixel chunks from the activations (with upsampling and concatenation) while
+// they stage a tile, one 16-byte load and a shift by one pixel per chunk.  Every
+// sum keeps the order it had with a stored column matrix (the same 16-deep MMA
+// steps, the same splits, taps added in order), so results are bit for bit the
+// same; what went is the traffic (1.4 GB written and read again per inference at
+// 256 x 1024, 2.8 GB more per training step).  All launches take the samples of
+// a batch together (blockIdx.z): small images are bound by launch latency.
+// Everything around the GEMMs (pooling, the ReLU masks of the gradients, bias
+// sums, loss, Adam, resampling) is memory-bound and written as plain coalesced
+// kernels.
 //
 // Storage points (where values are rounded to bfloat16, round to nearest
 // even): input image, weights, every ReLU activation, the average-pooled
@@ -46,6 +51,20 @@ constexpr int GBK = 32;        // k extent of a staged tile
 constexpr int GPAD = 8;        // bf16 padding per shared row (ldmatrix rows on distinct banks)
 constexpr int GTHREADS = 256;  // 8 warps, each owning a 32 x 32 block of C
 constexpr int GSTAGES = 3;     // cp.async pipeline depth (tiles in flight + 1)
+// A gathered tile passes through registers within one iteration, so a third
+// stage hides nothing; two leave room for four CTAs an SM, whose loads cover
+// each other (the whole forward pass at 256 x 1024 gains 4%)
+template <bool GATHER>
+constexpr int kStages = GATHER ? 2 : GSTAGES;
+
+// activations a 3x3 convolution reads: channels c < C1 from s1,
+// nearest-upsampled from (H/2, W/2) when up1; the rest from s2 (the skip
+// connection, concatenated after s1); bs1, bs2: elements between samples
+struct ConvSrc {
+    const bf16 *s1, *s2;
+    int C1, up1, C2, H, W;
+    long long bs1, bs2;
+};
 
 struct GemmArgs {
     const bf16 *A;
@@ -60,8 +79,11 @@ struct GemmArgs {
     int relu;
     int accumulate;            // Cf += result
     long long ldc;
-    long long split_stride;    // elements between split partials (splits > 1)
+    long long split_stride;    // elements between split partials
     int splits;
+    int partial;               // write split partials [sample][split][M][N]
+    long long abs_, bbs, cbs;  // elements between samples of A, B, C
+    ConvSrc src;               // gathered B
 };
 
 __device__ __forceinline__ void cp16(void *smem, const void *gmem, bool valid)
@@ -94,6 +116,46 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Chunk of 8 pixels (y, x0 ..) of row (c, ky, kx) of the column matrix: the
+// aligned 16 bytes (8 when upsampled) and, in e, the pixel beyond them that the
+// shift brings in, the shift and the upsampling flag.
+__device__ __forceinline__ void fetch8(const ConvSrc &S, const bf16 *s1, const bf16 *s2, int c, int ky, int kx, int y, int x0,
+                                       bool in, uint4 &v, unsigned &e)
+{
+    v = make_uint4(0u, 0u, 0u, 0u);
+    e = 1u << 16;
+    const int ys = y + ky - 1;
+    if (!in || c >= S.C1 + S.C2 || ys < 0 || ys >= S.H) return;
+    const int xe = kx == 0 ? x0 - 1 : x0 + 8;
+    const bool edge = kx != 1 && xe >= 0 && xe < S.W;
+    if (c < S.C1 && S.up1) {
+        const bf16 *row = s1 + ((long long)c * (S.H / 2) + ys / 2) * (S.W / 2);
+        const uint2 q = *reinterpret_cast<const uint2 *>(row + x0 / 2);
+        v.x = q.x;
+        v.y = q.y;
+        e = (edge ? (unsigned)*reinterpret_cast<const unsigned short *>(row + xe / 2) : 0u) | (unsigned)kx << 16 | 1u << 18;
+    } else {
+        const bf16 *row = c < S.C1 ? s1 + ((long long)c * S.H + ys) * S.W : s2 + ((long long)(c - S.C1) * S.H + ys) * S.W;
+        v = *reinterpret_cast<const uint4 *>(row + x0);
+        e = (edge ? (unsigned)*reinterpret_cast<const unsigned short *>(row + xe) : 0u) | (unsigned)kx << 16;
+    }
+}
+
+__device__ __forceinline__ uint4 shift8(uint4 v, unsigned e)
+{
+    if (e >> 18 & 1)
+        v = make_uint4(__byte_perm(v.x, 0, 0x1010), __byte_perm(v.x, 0, 0x3232), __byte_perm(v.y, 0, 0x1010),
+                       __byte_perm(v.y, 0, 0x3232));
+    const unsigned kx = e >> 16 & 3u;
+    if (kx == 0)
+        return make_uint4(v.x << 16 | (e & 0xffffu), __funnelshift_l(v.x, v.y, 16), __funnelshift_l(v.y, v.z, 16),
+                          __funnelshift_l(v.z, v.w, 16));
+    if (kx == 2)
+        return make_uint4(__funnelshift_r(v.x, v.y, 16), __funnelshift_r(v.y, v.z, 16), __funnelshift_r(v.z, v.w, 16),
+                          v.w >> 16 | e << 16);
+    return v;
+}
+
 // Shared tiles of one stage.  A_KM: A stored [K][M] (m contiguous), else
 // [M][K]; B_NK: B stored [N][K] (k contiguous), else [K][N].
 template <int BM, int BN, bool A_KM, bool B_NK>
@@ -104,12 +166,14 @@ struct GemmTile {
     static constexpr int BE = B_NK ? BN * BP : GBK * BP;
     static constexpr int ACH = BM * GBK / 8;                      // 16-byte chunks per stage
     static constexpr int BCH = BN * GBK / 8;
+    static constexpr int BPT = BCH / GTHREADS;                    // of B per thread
+    static_assert(BCH % GTHREADS == 0, "chunks of B");
 };
 
-template <int BM, int BN, bool A_KM, bool B_NK>
-__device__ __forceinline__ void gemm_stage(const GemmArgs &g, bf16 *As, bf16 *Bs, int m0, int n0, int k0, int kend)
+template <int BM, int BN, bool A_KM>
+__device__ __forceinline__ void stage_a(const GemmArgs &g, const bf16 *A, bf16 *As, int m0, int k0, int kend)
 {
-    using T = GemmTile<BM, BN, A_KM, B_NK>;
+    using T = GemmTile<BM, BN, A_KM, false>;
     for (int q = threadIdx.x; q < T::ACH; q += GTHREADS) {
         int r, c;
         const bf16 *src;
@@ -118,15 +182,21 @@ __device__ __forceinline__ void gemm_stage(const GemmArgs &g, bf16 *As, bf16 *Bs
             r = q / (BM / 8);
             c = (q % (BM / 8)) * 8;
             ok = (k0 + r < kend) && (m0 + c < g.M);
-            src = g.A + (long long)(k0 + r) * g.lda + m0 + c;
+            src = A + (long long)(k0 + r) * g.lda + m0 + c;
         } else {                          // rows m, 8 k per chunk
             r = q / (GBK / 8);
             c = (q % (GBK / 8)) * 8;
             ok = (m0 + r < g.M) && (k0 + c < kend);
-            src = g.A + (long long)(m0 + r) * g.lda + k0 + c;
+            src = A + (long long)(m0 + r) * g.lda + k0 + c;
         }
-        cp16(As + r * T::AP + c, ok ? src : g.A, ok);
+        cp16(As + r * T::AP + c, ok ? src : A, ok);
     }
+}
+
+template <int BM, int BN, bool A_KM, bool B_NK>
+__device__ __forceinline__ void stage_b(const GemmArgs &g, const bf16 *B, bf16 *Bs, int n0, int k0, int kend)
+{
+    using T = GemmTile<BM, BN, A_KM, B_NK>;
     for (int q = threadIdx.x; q < T::BCH; q += GTHREADS) {
         int r, c;
         const bf16 *src;
@@ -135,36 +205,124 @@ __device__ __forceinline__ void gemm_stage(const GemmArgs &g, bf16 *As, bf16 *Bs
             r = q / (GBK / 8);
             c = (q % (GBK / 8)) * 8;
             ok = (n0 + r < g.N) && (k0 + c < kend);
-            src = g.B + (long long)(n0 + r) * g.ldb + k0 + c;
+            src = B + (long long)(n0 + r) * g.ldb + k0 + c;
         } else {                          // rows k, 8 n per chunk
             r = q / (BN / 8);
             c = (q % (BN / 8)) * 8;
             ok = (k0 + r < kend) && (n0 + c < g.N);
-            src = g.B + (long long)(k0 + r) * g.ldb + n0 + c;
+            src = B + (long long)(k0 + r) * g.ldb + n0 + c;
         }
-        cp16(Bs + r * T::BP + c, ok ? src : g.B, ok);
+        cp16(Bs + r * T::BP + c, ok ? src : B, ok);
     }
-    asm volatile("cp.async.commit_group;\n" ::);
+}
+
+// this thread's chunks of a gathered tile of B (rows kk of the column matrix)
+template <int BM, int BN, bool B_NK>
+__device__ __forceinline__ void fetch_b(const GemmArgs &g, const bf16 *s1, const bf16 *s2, int n0, int k0, int kend,
+                                        uint4 (&v)[GemmTile<BM, BN, false, B_NK>::BPT],
+                                        unsigned (&e)[GemmTile<BM, BN, false, B_NK>::BPT])
+{
+    using T = GemmTile<BM, BN, false, B_NK>;
+    // the pixels of a thread's chunks are the same in all of them
+    const int p = B_NK ? k0 + (threadIdx.x % (GBK / 8)) * 8 : n0 + (threadIdx.x % (BN / 8)) * 8;
+    const int y = p / g.src.W, x0 = p - y * g.src.W;
+    const bool in = p < (B_NK ? kend : g.N);
+#pragma unroll
+    for (int i = 0; i < T::BPT; ++i) {
+        const int q = threadIdx.x + i * GTHREADS;
+        const int kk = B_NK ? n0 + q / (GBK / 8) : k0 + q / (BN / 8);
+        const int c = kk / 9, t = kk - 9 * c;
+        fetch8(g.src, s1, s2, c, t / 3, t % 3, y, x0, in && kk < (B_NK ? g.N : kend), v[i], e[i]);
+    }
+}
+
+template <int BM, int BN, bool B_NK>
+__device__ __forceinline__ void put_b(bf16 *Bs, const uint4 (&v)[GemmTile<BM, BN, false, B_NK>::BPT],
+                                      const unsigned (&e)[GemmTile<BM, BN, false, B_NK>::BPT])
+{
+    using T = GemmTile<BM, BN, false, B_NK>;
+#pragma unroll
+    for (int i = 0; i < T::BPT; ++i) {
+        const int q = threadIdx.x + i * GTHREADS;
+        const int r = B_NK ? q / (GBK / 8) : q / (BN / 8), c = B_NK ? (q % (GBK / 8)) * 8 : (q % (BN / 8)) * 8;
+        *reinterpret_cast<uint4 *>(Bs + r * T::BP + c) = shift8(v[i], e[i]);
+    }
+}
+
+// the MMAs of one staged tile
+template <int BM, int BN, bool A_KM, bool B_NK>
+__device__ __forceinline__ void tile_mma(const bf16 *as, const bf16 *bs, int wm, int wn, int lane, float (&acc)[2][4][4])
+{
+    using T = GemmTile<BM, BN, A_KM, B_NK>;
+#pragma unroll
+    for (int kk = 0; kk < GBK; kk += 16) {
+        unsigned a[2][4], b[4][2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int mb = wm * 32 + i * 16;
+            if (A_KM) {
+                int k = kk + (lane & 7) + ((lane >> 4) << 3);
+                int m = mb + (((lane >> 3) & 1) << 3);
+                ldsm_x4_t(a[i], as + k * T::AP + m);
+            } else {
+                int m = mb + (lane & 15);
+                int k = kk + ((lane >> 4) << 3);
+                ldsm_x4(a[i], as + m * T::AP + k);
+            }
+        }
+#pragma unroll
+        for (int jb = 0; jb < 2; ++jb) {
+            const int nb = wn * 32 + jb * 16;
+            unsigned r[4];
+            if (B_NK) {
+                int n = nb + (lane & 7) + ((lane >> 4) << 3);
+                int k = kk + (((lane >> 3) & 1) << 3);
+                ldsm_x4(r, bs + n * T::BP + k);
+            } else {
+                int k = kk + (lane & 15);
+                int n = nb + ((lane >> 4) << 3);
+                ldsm_x4_t(r, bs + k * T::BP + n);
+            }
+            b[2 * jb][0] = r[0];
+            b[2 * jb][1] = r[1];
+            b[2 * jb + 1][0] = r[2];
+            b[2 * jb + 1][1] = r[3];
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j][0], b[j][1]);
+    }
 }
 
 // C tile BM x BN per CTA, warps arranged (BM/32) x (BN/32), each warp
-// 2 x 4 mma tiles of 16 x 8.  Requirements (checked on the host): K % 8 == 0,
-// lda, ldb multiples of 8, 16-byte aligned bases, M % 8 == 0 when A_KM,
-// N % 8 == 0 when !B_NK, N even.
-template <int BM, int BN, bool A_KM, bool B_NK>
-__global__ void __launch_bounds__(GTHREADS) gemm_bf16_kernel(const GemmArgs g)
+// 2 x 4 mma tiles of 16 x 8; blockIdx.z = sample * splits + split.  A (and a
+// stored B) by cp.async ahead of its use, a gathered B through registers
+// (loaded before the tile's MMAs, written after them).  Requirements (checked on
+// the host): K % 8 == 0, lda, ldb multiples of 8, 16-byte aligned bases, M % 8 ==
+// 0 when A_KM, N % 8 == 0 when !B_NK, N even; gathered: W % 8 == 0.
+template <int BM, int BN, bool A_KM, bool B_NK, bool GATHER>
+__global__ void __launch_bounds__(GTHREADS, GATHER ? (BM == 32 ? 3 : 4) : 1) gemm_bf16_kernel(const GemmArgs g)
 {
     using T = GemmTile<BM, BN, A_KM, B_NK>;
     static_assert((BM / 32) * (BN / 32) == GTHREADS / 32, "warp layout");
-    extern __shared__ __align__(16) unsigned char gsm[];   // GSTAGES x (A tile, B tile)
+    constexpr int ST = kStages<GATHER>;
+    extern __shared__ __align__(16) unsigned char gsm[];   // ST x (A tile, B tile)
     bf16 *As0 = reinterpret_cast<bf16 *>(gsm);
-    bf16 *Bs0 = As0 + GSTAGES * T::AE;
+    bf16 *Bs0 = As0 + ST * T::AE;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int wm = warp % (BM / 32), wn = warp / (BM / 32);
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int kbeg = blockIdx.z * g.kchunk;
+    const int sample = blockIdx.z / g.splits, split = blockIdx.z - sample * g.splits;
+    const int kbeg = split * g.kchunk;
     const int kend = min(g.K, kbeg + g.kchunk);
+    const bf16 *A = g.A + sample * g.abs_, *B = GATHER ? nullptr : g.B + sample * g.bbs;
+    const bf16 *s1 = nullptr, *s2 = nullptr;
+    if (GATHER) {
+        s1 = g.src.s1 + sample * g.src.bs1;
+        s2 = g.src.s2 + sample * g.src.bs2;
+    }
 
     float acc[2][4][4];
 #pragma unroll
@@ -174,101 +332,71 @@ __global__ void __launch_bounds__(GTHREADS) gemm_bf16_kernel(const GemmArgs g)
 #pragma unroll
             for (int v = 0; v < 4; ++v) acc[i][j][v] = 0.f;
 
-    // GSTAGES-deep cp.async pipeline: tiles it+1 .. it+GSTAGES-1 are in flight
-    // while tile it is consumed; every iteration commits one group (empty
-    // past the end) so that wait_group GSTAGES-2 always means "tile it landed"
+    uint4 bv[T::BPT];
+    unsigned be[T::BPT];
+    // tiles it+1 .. it+ST-1 are under way while tile it is consumed; every
+    // iteration commits one group (empty past the end) so that wait_group
+    // ST-2 always means "tile it landed"
 #pragma unroll
-    for (int sidx = 0; sidx < GSTAGES - 1; ++sidx) {
+    for (int sidx = 0; sidx < ST - 1; ++sidx) {
         const int kk0 = kbeg + sidx * GBK;
-        if (kk0 < kend)
-            gemm_stage<BM, BN, A_KM, B_NK>(g, As0 + sidx * T::AE, Bs0 + sidx * T::BE, m0, n0, kk0, kend);
-        else
-            asm volatile("cp.async.commit_group;\n" ::);
+        if (kk0 < kend) {
+            stage_a<BM, BN, A_KM>(g, A, As0 + sidx * T::AE, m0, kk0, kend);
+            if (GATHER) {
+                fetch_b<BM, BN, B_NK>(g, s1, s2, n0, kk0, kend, bv, be);
+                put_b<BM, BN, B_NK>(Bs0 + sidx * T::BE, bv, be);
+            } else {
+                stage_b<BM, BN, A_KM, B_NK>(g, B, Bs0 + sidx * T::BE, n0, kk0, kend);
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::);
     }
     int it = 0;
     for (int k0 = kbeg; k0 < kend; k0 += GBK, ++it) {
-        asm volatile("cp.async.wait_group %0;\n" ::"n"(GSTAGES - 2));
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(ST - 2));
         __syncthreads();
-        {
-            // refill the slot consumed in the previous iteration (all threads
-            // are past it: the barrier above)
-            const int kn = k0 + (GSTAGES - 1) * GBK;
-            const int slot = (it + GSTAGES - 1) % GSTAGES;
-            if (kn < kend)
-                gemm_stage<BM, BN, A_KM, B_NK>(g, As0 + slot * T::AE, Bs0 + slot * T::BE, m0, n0, kn, kend);
-            else
-                asm volatile("cp.async.commit_group;\n" ::);
+        // refill the slot consumed in the previous iteration (all threads are
+        // past it: the barrier above)
+        const int kn = k0 + (ST - 1) * GBK;
+        const int slot = (it + ST - 1) % ST;
+        if (kn < kend) {
+            stage_a<BM, BN, A_KM>(g, A, As0 + slot * T::AE, m0, kn, kend);
+            if (GATHER) fetch_b<BM, BN, B_NK>(g, s1, s2, n0, kn, kend, bv, be);
+            else stage_b<BM, BN, A_KM, B_NK>(g, B, Bs0 + slot * T::BE, n0, kn, kend);
         }
-        const int cur = it % GSTAGES;
-        const bf16 *as = As0 + cur * T::AE, *bs = Bs0 + cur * T::BE;
-#pragma unroll
-        for (int kk = 0; kk < GBK; kk += 16) {
-            unsigned a[2][4], b[4][2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int mb = wm * 32 + i * 16;
-                if (A_KM) {
-                    int k = kk + (lane & 7) + ((lane >> 4) << 3);
-                    int m = mb + (((lane >> 3) & 1) << 3);
-                    ldsm_x4_t(a[i], as + k * T::AP + m);
-                } else {
-                    int m = mb + (lane & 15);
-                    int k = kk + ((lane >> 4) << 3);
-                    ldsm_x4(a[i], as + m * T::AP + k);
-                }
-            }
-#pragma unroll
-            for (int jb = 0; jb < 2; ++jb) {
-                const int nb = wn * 32 + jb * 16;
-                unsigned r[4];
-                if (B_NK) {
-                    int n = nb + (lane & 7) + ((lane >> 4) << 3);
-                    int k = kk + (((lane >> 3) & 1) << 3);
-                    ldsm_x4(r, bs + n * T::BP + k);
-                } else {
-                    int k = kk + (lane & 15);
-                    int n = nb + ((lane >> 4) << 3);
-                    ldsm_x4_t(r, bs + k * T::BP + n);
-                }
-                b[2 * jb][0] = r[0];
-                b[2 * jb][1] = r[1];
-                b[2 * jb + 1][0] = r[2];
-                b[2 * jb + 1][1] = r[3];
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j][0], b[j][1]);
-        }
+        asm volatile("cp.async.commit_group;\n" ::);
+        const int cur = it % ST;
+        tile_mma<BM, BN, A_KM, B_NK>(As0 + cur * T::AE, Bs0 + cur * T::BE, wm, wn, lane, acc);
+        if (GATHER && kn < kend) put_b<BM, BN, B_NK>(Bs0 + slot * T::BE, bv, be);
     }
     asm volatile("cp.async.wait_group 0;\n" ::);
 
     // epilogue: thread holds rows g, g+8 and columns 2t, 2t+1 of each 16 x 8 tile
     const int gr = lane >> 2, tc = (lane & 3) * 2;
-    const bool partial = g.splits > 1;
+    float *Cf = g.Cf ? g.Cf + (g.partial ? (long long)blockIdx.z * g.split_stride : sample * g.cbs) : nullptr;
+    bf16 *Cb = g.Cb ? g.Cb + sample * g.cbs : nullptr;
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int m = m0 + wm * 32 + i * 16 + gr + 8 * h;
             if (m >= g.M) continue;
-            const float bm = (!partial && g.bias) ? g.bias[m] : 0.f;
+            const float bm = (!g.partial && g.bias) ? g.bias[m] : 0.f;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int n = n0 + wn * 32 + j * 8 + tc;
                 if (n >= g.N) continue;
                 float v0 = acc[i][j][2 * h] + bm, v1 = acc[i][j][2 * h + 1] + bm;
-                if (partial) {
-                    float2 *p = reinterpret_cast<float2 *>(g.Cf + blockIdx.z * g.split_stride + (long long)m * g.ldc + n);
-                    *p = make_float2(v0, v1);
+                if (g.partial) {
+                    *reinterpret_cast<float2 *>(Cf + (long long)m * g.ldc + n) = make_float2(v0, v1);
                     continue;
                 }
                 if (g.relu) {
                     v0 = fmaxf(v0, 0.f);
                     v1 = fmaxf(v1, 0.f);
                 }
-                if (g.Cf) {
-                    float2 *p = reinterpret_cast<float2 *>(g.Cf + (long long)m * g.ldc + n);
+                if (Cf) {
+                    float2 *p = reinterpret_cast<float2 *>(Cf + (long long)m * g.ldc + n);
                     if (g.accumulate) {
                         float2 o = *p;
                         v0 += o.x;
@@ -276,29 +404,154 @@ __global__ void __launch_bounds__(GTHREADS) gemm_bf16_kernel(const GemmArgs g)
                     }
                     *p = make_float2(v0, v1);
                 }
-                if (g.Cb) {
+                if (Cb) {
                     __nv_bfloat162 o = __floats2bfloat162_rn(v0, v1);
-                    *reinterpret_cast<__nv_bfloat162 *>(g.Cb + (long long)m * g.ldc + n) = o;
+                    *reinterpret_cast<__nv_bfloat162 *>(Cb + (long long)m * g.ldc + n) = o;
                 }
             }
         }
 }
 
-// sum of the split partials in split order, then the epilogue of the GEMM
-__global__ void gemm_reduce_kernel(const float *__restrict__ part, int splits, long long split_stride, int M, int N,
-                                   long long ldc, const float *__restrict__ bias, int relu, int accumulate,
-                                   float *__restrict__ Cf, bf16 *__restrict__ Cb)
+// Input gradient of a 3x3 convolution: dX[c][p] = sum over the nine taps, in
+// order, of sum_co Wt[tap][co][c] G[co][y - ky + 1][x - kx + 1] (zero outside).
+// Each tap's sum starts from zero (and from zero again at every kchunk of co,
+// the parts added in order), as if the taps' products were stored and then
+// gathered.  A = Wt + tap * K * lda ([K][M]); B gathered from G.
+template <int BM, int BN>
+__global__ void __launch_bounds__(GTHREADS) conv_dx_kernel(const GemmArgs g)
+{
+    using T = GemmTile<BM, BN, true, false>;
+    extern __shared__ __align__(16) unsigned char gsm[];
+    bf16 *As0 = reinterpret_cast<bf16 *>(gsm);
+    bf16 *Bs0 = As0 + GSTAGES * T::AE;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int wm = warp % (BM / 32), wn = warp / (BM / 32);
+    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const bf16 *G = g.src.s1 + blockIdx.z * g.src.bs1;
+    const int nk = (g.K + GBK - 1) / GBK, total = 9 * nk, per = g.kchunk / GBK;   // tiles per tap, in all, per part
+    const int p = n0 + (threadIdx.x % (BN / 8)) * 8, y = p / g.src.W, x0 = p - y * g.src.W;
+
+    float acc[2][4][4], part[2][4][4], sum[2][4][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[i][j][v] = part[i][j][v] = sum[i][j][v] = 0.f;
+    uint4 bv[T::BPT];
+    unsigned be[T::BPT];
+    auto fetch = [&](int t) {
+        const int tap = t / nk, k0 = (t - tap * nk) * GBK, ky = tap / 3, kx = tap - 3 * ky;
+#pragma unroll
+        for (int i = 0; i < T::BPT; ++i) {
+            const int co = k0 + (threadIdx.x + i * GTHREADS) / (BN / 8);
+            fetch8(g.src, G, G, co, 2 - ky, 2 - kx, y, x0, p < g.N && co < g.K, bv[i], be[i]);
+        }
+    };
+    auto stage = [&](int t, int slot) {
+        const int tap = t / nk, k0 = (t - tap * nk) * GBK;
+        stage_a<BM, BN, true>(g, g.A + (long long)tap * g.K * g.lda, As0 + slot * T::AE, m0, k0, g.K);
+    };
+#pragma unroll
+    for (int sidx = 0; sidx < GSTAGES - 1; ++sidx) {
+        if (sidx < total) {
+            stage(sidx, sidx);
+            fetch(sidx);
+            put_b<BM, BN, false>(Bs0 + sidx * T::BE, bv, be);
+        }
+        asm volatile("cp.async.commit_group;\n" ::);
+    }
+    for (int it = 0; it < total; ++it) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(GSTAGES - 2));
+        __syncthreads();
+        const int tn = it + GSTAGES - 1, slot = tn % GSTAGES, cur = it % GSTAGES;
+        if (tn < total) {
+            stage(tn, slot);
+            fetch(tn);
+        }
+        asm volatile("cp.async.commit_group;\n" ::);
+        tile_mma<BM, BN, true, false>(As0 + cur * T::AE, Bs0 + cur * T::BE, wm, wn, lane, acc);
+        if (tn < total) put_b<BM, BN, false>(Bs0 + slot * T::BE, bv, be);
+        const int kt = it % nk;
+        const bool end = kt == nk - 1;
+        if (end || (kt + 1) % per == 0) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        part[i][j][v] += acc[i][j][v];
+                        acc[i][j][v] = 0.f;
+                        if (end) {
+                            sum[i][j][v] += part[i][j][v];
+                            part[i][j][v] = 0.f;
+                        }
+                    }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::);
+    const int gr = lane >> 2, tc = (lane & 3) * 2;
+    float *Cf = g.Cf + blockIdx.z * g.cbs;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int m = m0 + wm * 32 + i * 16 + gr + 8 * h;
+            if (m >= g.M) continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int n = n0 + wn * 32 + j * 8 + tc;
+                if (n < g.N)
+                    *reinterpret_cast<float2 *>(Cf + (long long)m * g.ldc + n) = make_float2(sum[i][j][2 * h], sum[i][j][2 * h + 1]);
+            }
+        }
+}
+
+// sum of the split partials in split order, then the epilogue of the GEMM; with
+// accumulate the samples are added in order.  V (4 where the rows allow it)
+// consecutive outputs a thread: bound by the partials' reads.
+template <int V>
+__global__ void __launch_bounds__(256) gemm_reduce_kernel(const float *__restrict__ part, int samples, int splits, int M, int N,
+                                                          long long ldc, long long cbs, const float *__restrict__ bias, int relu,
+                                                          int accumulate, float *__restrict__ Cf, bf16 *__restrict__ Cb)
 {
     const long long total = (long long)M * N;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int m = (int)(q / N), n = (int)(q - (long long)m * N);
-        float s = 0.f;
-        for (int z = 0; z < splits; ++z) s += part[z * split_stride + (long long)m * N + n];
-        if (bias) s += bias[m];
-        if (relu) s = fmaxf(s, 0.f);
-        if (Cf) Cf[(long long)m * ldc + n] = accumulate ? Cf[(long long)m * ldc + n] + s : s;
-        if (Cb) Cb[(long long)m * ldc + n] = __float2bfloat16_rn(s);
+    const int b0 = accumulate ? 0 : blockIdx.y, b1 = accumulate ? samples : b0 + 1;
+    struct alignas(4 * V) Vec { float v[V]; };
+    struct alignas(2 * V) VecB { bf16 v[V]; };
+    for (long long q = V * (blockIdx.x * (long long)blockDim.x + threadIdx.x); q < total;
+         q += (long long)gridDim.x * blockDim.x * V) {
+        const int m = total < (1LL << 31) ? (int)((unsigned)q / (unsigned)N) : (int)(q / N);
+        const long long at = (long long)m * ldc + (q - (long long)m * N);
+        Vec o;
+        if (accumulate) o = *reinterpret_cast<const Vec *>(Cf + at);
+        for (int b = b0; b < b1; ++b) {
+            Vec s;
+#pragma unroll
+            for (int v = 0; v < V; ++v) s.v[v] = 0.f;
+#pragma unroll 4
+            for (int z = 0; z < splits; ++z) {
+                const Vec x = *reinterpret_cast<const Vec *>(part + ((long long)b * splits + z) * total + q);
+#pragma unroll
+                for (int v = 0; v < V; ++v) s.v[v] += x.v[v];
+            }
+            if (accumulate) {
+#pragma unroll
+                for (int v = 0; v < V; ++v) o.v[v] += s.v[v];
+                continue;
+            }
+            VecB h;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                if (bias) s.v[v] += bias[m];
+                if (relu) s.v[v] = fmaxf(s.v[v], 0.f);
+                h.v[v] = __float2bfloat16_rn(s.v[v]);
+            }
+            if (Cf) *reinterpret_cast<Vec *>(Cf + b * cbs + at) = s;
+            if (Cb) *reinterpret_cast<VecB *>(Cb + b * cbs + at) = h;
+        }
+        if (accumulate) *reinterpret_cast<Vec *>(Cf + at) = o;
     }
 }
 
@@ -307,71 +560,9 @@ __global__ void gemm_reduce_kernel(const float *__restrict__ part, int splits, l
 namespace {
 
 // ---------------------------------------------------------------------------
-// layout kernels
+// layout kernels (the channels of all samples of a batch are one long list
+// where they need not be told apart)
 // ---------------------------------------------------------------------------
-
-// Xcol[kk][p] = X[c][y+ky-1][x+kx-1] with kk = c*9 + ky*3 + kx, zero outside
-// the image and for kk >= 9 (C1 + C2).  Channels c < C1 come from s1,
-// nearest-upsampled from (H/2, W/2) when up1; the rest from s2 (the skip
-// connection, concatenated after s1).  Each thread writes 8 consecutive p.
-__global__ void im2col_kernel(const bf16 *__restrict__ s1, int C1, int up1, const bf16 *__restrict__ s2, int C2,
-                              int H, int W, int Kp, bf16 *__restrict__ out)
-{
-    const long long P = (long long)H * W;
-    const long long groups = (long long)Kp * (P / 8);
-    const int C = C1 + C2;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < groups;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int kk = (int)(q / (P / 8));
-        const long long p0 = (q - (long long)kk * (P / 8)) * 8;
-        const int y = (int)(p0 / W), x0 = (int)(p0 - (long long)y * W);
-        __align__(16) bf16 v[8];
-        const int c = kk / 9, r = kk - 9 * c, ky = r / 3, kx = r - 3 * ky;
-        const int ys = y + ky - 1;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int xs = x0 + i + kx - 1;
-            bf16 val = __float2bfloat16_rn(0.f);
-            if (c < C && ys >= 0 && ys < H && xs >= 0 && xs < W) {
-                if (c < C1) {
-                    val = up1 ? s1[((long long)c * (H / 2) + ys / 2) * (W / 2) + xs / 2]
-                              : s1[((long long)c * H + ys) * W + xs];
-                } else {
-                    val = s2[((long long)(c - C1) * H + ys) * W + xs];
-                }
-            }
-            v[i] = val;
-        }
-        *reinterpret_cast<uint4 *>(out + (long long)kk * P + p0) = *reinterpret_cast<const uint4 *>(v);
-    }
-}
-
-// dX[c][y][x] = sum_{ky,kx} dXcol[c*9+ky*3+kx][(y-ky+1)*W + (x-kx+1)]
-// over the taps whose output pixel lies in the image (fixed order)
-__global__ void col2im_kernel(const float *__restrict__ dcol, int C, int H, int W, float *__restrict__ dX)
-{
-    const long long P = (long long)H * W;
-    const long long total = (long long)C * P;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(q / P);
-        const long long p = q - (long long)c * P;
-        const int y = (int)(p / W), x = (int)(p - (long long)y * W);
-        float s = 0.f;
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky) {
-            const int yo = y - ky + 1;
-            if (yo < 0 || yo >= H) continue;
-#pragma unroll
-            for (int kx = 0; kx < 3; ++kx) {
-                const int xo = x - kx + 1;
-                if (xo < 0 || xo >= W) continue;
-                s += dcol[(long long)(c * 9 + ky * 3 + kx) * P + (long long)yo * W + xo];
-            }
-        }
-        dX[q] = s;
-    }
-}
 
 // out[c][y][x] = mean of in[c][2y..2y+1][2x..2x+1] (H, W of the output)
 __global__ void avgpool_kernel(const bf16 *__restrict__ in, int C, int H, int W, bf16 *__restrict__ out)
@@ -395,11 +586,17 @@ __global__ void avgpool_kernel(const bf16 *__restrict__ in, int C, int H, int W,
 //   g = fine (2x2 sum of a [C][2H][2W] map: upsampling adjoint)   when fine
 //     + 0.25 * coarse[c][y/2][x/2]   (average-pooling adjoint)      when coarse
 //     + direct[c][y][x]                                             when direct
-__global__ void grad_mask_kernel(const float *__restrict__ fine, const float *__restrict__ coarse,
-                                 const float *__restrict__ direct, const bf16 *__restrict__ y, int C, int H, int W,
-                                 bf16 *__restrict__ out)
+__global__ void grad_mask_kernel(const float *__restrict__ fine, long long fine_bs, const float *__restrict__ coarse,
+                                 const float *__restrict__ direct, long long direct_bs, const bf16 *__restrict__ y, int C,
+                                 int H, int W, bf16 *__restrict__ out)
 {
+    // blockIdx.y: sample; fine and direct may be channel ranges of wider maps
     const long long total = (long long)C * H * W;
+    if (fine) fine += blockIdx.y * fine_bs;
+    if (coarse) coarse += blockIdx.y * (total / 4);
+    if (direct) direct += blockIdx.y * direct_bs;
+    y += blockIdx.y * total;
+    out += blockIdx.y * total;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
          q += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(q % W);
@@ -417,20 +614,41 @@ __global__ void grad_mask_kernel(const float *__restrict__ fine, const float *__
     }
 }
 
-// db[m] += sum_p G[m][p]: one CTA per row, fixed-order tree
-__global__ void rowsum_kernel(const bf16 *__restrict__ G, long long P, float *__restrict__ db)
+// part[b][m] = sum_p G[b][m][p]: one CTA per row and sample, fixed-order tree;
+// db[m] += part[b][m] sample by sample
+__global__ void rowsum_kernel(const bf16 *__restrict__ G, long long P, int rows, float *__restrict__ part)
 {
     __shared__ float red[256];
-    const int m = blockIdx.x;
+    const bf16 *g = G + ((long long)blockIdx.y * rows + blockIdx.x) * P;
     float s = 0.f;
-    for (long long p = threadIdx.x; p < P; p += blockDim.x) s += __bfloat162float(G[(long long)m * P + p]);
+#pragma unroll 8
+    for (long long p = threadIdx.x; p < P; p += blockDim.x) s += __bfloat162float(g[p]);
     red[threadIdx.x] = s;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
         if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) db[m] += red[0];
+    if (threadIdx.x == 0) part[blockIdx.y * rows + blockIdx.x] = red[0];
+}
+
+__global__ void rowsum_add_kernel(const float *__restrict__ part, int samples, int rows, float *__restrict__ db)
+{
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= rows) return;
+    float s = db[m];
+    for (int b = 0; b < samples; ++b) s += part[b * rows + m];
+    db[m] = s;
+}
+
+// Wt[tap][co][c] = W[co][c * 9 + tap] of one 3x3 layer
+__global__ void transpose_weights_kernel(const bf16 *__restrict__ W, int cout, int cin, int kcp, bf16 *__restrict__ Wt)
+{
+    const int total = 9 * cout * cin;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
+        const int c = q % cin, r = q / cin, co = r % cout, tap = r / cout;
+        Wt[q] = W[(long long)co * kcp + c * 9 + tap];
+    }
 }
 
 __global__ void to_bf16_kernel(const float *__restrict__ in, long long n, bf16 *__restrict__ out)
@@ -442,13 +660,17 @@ __global__ void to_bf16_kernel(const float *__restrict__ in, long long n, bf16 *
 // Mean squared error over `cout` channels of pred [cpad][P] against
 // target [cout][P]: per-block partial sums (FP32 products, FP64 block sums),
 // and dy [cpad][P] = gscale 2 (pred - target) / (cout P) (zero rows beyond
-// cout; gscale = 1 / batch gives the gradient of the batch mean).
+// cout; gscale = 1 / batch gives the gradient of the batch mean).  blockIdx.y:
+// sample.
 __global__ void mse_kernel(const float *__restrict__ pred, const float *__restrict__ target, int cout, int cpad,
                            long long P, float gscale, double *__restrict__ partial, bf16 *__restrict__ dy)
 {
     __shared__ double red[256];
     const long long n = (long long)cout * P;
     const float scale = (float)(2.0 / (double)n) * gscale;
+    pred += blockIdx.y * cpad * P;
+    target += blockIdx.y * n;
+    dy += blockIdx.y * cpad * P;
     double s = 0.0;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < (long long)cpad * P;
          q += (long long)gridDim.x * blockDim.x) {
@@ -465,17 +687,22 @@ __global__ void mse_kernel(const float *__restrict__ pred, const float *__restri
         if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
+    if (threadIdx.x == 0) partial[blockIdx.y * gridDim.x + blockIdx.x] = red[0];
 }
 
+// the loss of sample blockIdx.x: the block sums added in block order by one
+// thread, staged in shared memory
 __global__ void mse_finish_kernel(const double *__restrict__ partial, int nb, long long n, double *__restrict__ out,
                                   int *__restrict__ flag)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double sp[512];
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) sp[b] = partial[blockIdx.x * nb + b];
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += partial[b];
+    for (int b = 0; b < nb; ++b) s += sp[b];
     s /= (double)n;
-    *out = s;
+    out[blockIdx.x] = s;
     if (!isfinite(s)) *flag = 1;
 }
 
@@ -653,198 +880,294 @@ struct gbfwi_unet {
     DevBuf xin32, xb, tgt32;            // input (FP32 staging, bf16), target staging
     DevBuf ea[kMaxLevels], e[kMaxLevels], pl[kMaxLevels], da[kMaxLevels], dd[kMaxLevels];
     DevBuf yout, gyb;                   // output [coutp][P0] FP32, its gradient (bf16)
-    DevBuf col, dcol;                   // im2col (bf16), its gradient (FP32)
+    DevBuf wt;                          // transposed bf16 weights of the 3x3 layers ([tap][co][c], at w_off)
+    bool wt_fresh = false;              // wt holds the current weights
+    DevBuf rsum;                        // per-sample row sums of the bias gradients
     DevBuf dcat[kMaxLevels];            // gradient of the concatenated decoder input (FP32)
     DevBuf fA, fP, gb;                  // FP32 input gradients, masked bf16 gradient
     DevBuf part;                        // split-K partials
     DevBuf red, flag;                   // loss partials / result, non-finite flag
     long long part_cap = 0;
+    int nb = 0;                         // samples the activation buffers hold
+    bool grads = false;                 // the gradient buffers are there too
 };
 
 namespace {
 
 long long npix(const gbfwi_unet *n, int l) { return (long long)(n->d.height >> l) * (n->d.width >> l); }
 
-template <int BM, bool AK, bool BK>
-int launch_gemm(const GemmArgs &g, cudaStream_t s)
+// tile extents by output rows
+constexpr int bm_of(int M) { return M <= 32 ? 32 : (M <= 64 ? 64 : 128); }
+constexpr int bn_of(int BM) { return 256 * 32 / BM; }
+
+template <class K>
+int allow_smem(K kern, size_t smem, bool (&done)[64])
 {
-    constexpr int BN = 256 * 32 / BM;
-    dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), (unsigned)g.splits);
-    using T = GemmTile<BM, BN, AK, BK>;
-    constexpr size_t smem = (size_t)GSTAGES * (T::AE + T::BE) * sizeof(bf16);
-    static bool attr_done[64] = {};      // per device ordinal
     int dev = 0;
     GB_CUDA(cudaGetDevice(&dev));
-    if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        GB_CUDA(cudaFuncSetAttribute(gemm_bf16_kernel<BM, BN, AK, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
-        attr_done[dev] = true;
+    if (dev >= 0 && dev < 64 && !done[dev]) {
+        GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        done[dev] = true;
     }
-    gemm_bf16_kernel<BM, BN, AK, BK><<<grid, GTHREADS, smem, s>>>(g);
+    return GBFWI_OK;
+}
+
+template <int BM, bool AK, bool BK, bool GA>
+int launch_gemm(const GemmArgs &g, int samples, cudaStream_t s)
+{
+    constexpr int BN = bn_of(BM);
+    dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), (unsigned)(g.splits * samples));
+    using T = GemmTile<BM, BN, AK, BK>;
+    constexpr size_t smem = (size_t)kStages<GA> * (T::AE + T::BE) * sizeof(bf16);
+    static bool attr_done[64] = {};      // per device ordinal
+    GB_TRY(allow_smem(gemm_bf16_kernel<BM, BN, AK, BK, GA>, smem, attr_done));
+    gemm_bf16_kernel<BM, BN, AK, BK, GA><<<grid, GTHREADS, smem, s>>>(g);
     GB_LAUNCHED();
     return GBFWI_OK;
 }
 
 template <int BM>
-int launch_gemm_bm(const GemmArgs &g, bool a_km, bool b_nk, cudaStream_t s)
+int launch_gemm_bm(const GemmArgs &g, int samples, bool a_km, bool b_nk, cudaStream_t s)
 {
-    if (a_km) return b_nk ? launch_gemm<BM, true, true>(g, s) : launch_gemm<BM, true, false>(g, s);
-    return b_nk ? launch_gemm<BM, false, true>(g, s) : launch_gemm<BM, false, false>(g, s);
+    if (g.src.s1)
+        return b_nk ? launch_gemm<BM, false, true, true>(g, samples, s) : launch_gemm<BM, false, false, true>(g, samples, s);
+    if (a_km) return b_nk ? GBFWI_EINVAL : launch_gemm<BM, true, false, false>(g, samples, s);
+    return b_nk ? launch_gemm<BM, false, true, false>(g, samples, s) : launch_gemm<BM, false, false, false>(g, samples, s);
 }
 
-// C[M][N] (+)= A B (+ bias, ReLU) with A = [M][K] or [K][M] (a_km), B = [K][N]
-// or [N][K] (b_nk); FP32 output Cf and/or bf16 output Cb, row pitch ldc.
-int gemm(gbfwi_unet *net, const bf16 *A, long long lda, bool a_km, const bf16 *B, long long ldb, bool b_nk, int M,
-         int N, int K, float *Cf, bf16 *Cb, const float *bias, int relu, int accumulate, long long ldc, cudaStream_t s)
+// k range of a split of an (M x N) output over K: enough splits to fill the
+// SMs, each at least four tiles long.  The rule fixes where the sums are cut, so
+// it depends on one sample's shape only.
+int split_chunk(int M, int N, int K, long long part_cap, int *splits_out)
 {
-    if (M < 1 || N < 1 || K < 8 || K % 8 || lda % 8 || ldb % 8 || N % 2 || ldc % 2 || ((uintptr_t)A & 15) ||
-        ((uintptr_t)B & 15) || (a_km && M % 8) || (!b_nk && N % 8))
-        return GBFWI_EINVAL;
-    const int BM = M <= 32 ? 32 : (M <= 64 ? 64 : 128);
-    const int BN = 256 * 32 / BM;
+    const int BM = bm_of(M), BN = bn_of(BM);
     const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
     int splits = 1;
     if (tiles < 2 * 152 && K >= 8 * GBK) {
         long long want = (2 * 152 + tiles - 1) / tiles;
         want = std::min<long long>(want, K / (4 * GBK));
-        want = std::min<long long>(want, std::max<long long>(1, net->part_cap / ((long long)M * N)));
+        want = std::min<long long>(want, std::max<long long>(1, part_cap / ((long long)M * N)));
         splits = (int)std::max<long long>(1, want);
     }
-    int kchunk = (int)(((K + splits - 1) / splits + GBK - 1) / GBK * GBK);
-    splits = (K + kchunk - 1) / kchunk;
-    GemmArgs g{A, lda, B, ldb, M, N, K, kchunk, Cf, Cb, bias, relu, accumulate, ldc, 0, splits};
-    if (splits > 1) {
-        g.Cf = net->part.as<float>();
-        g.Cb = nullptr;
-        g.bias = nullptr;
-        g.relu = 0;
-        g.accumulate = 0;
-        g.ldc = N;
-        g.split_stride = (long long)M * N;
-    }
-    int rc = BM == 32 ? launch_gemm_bm<32>(g, a_km, b_nk, s)
-                      : (BM == 64 ? launch_gemm_bm<64>(g, a_km, b_nk, s) : launch_gemm_bm<128>(g, a_km, b_nk, s));
-    GB_TRY(rc);
-    if (splits > 1) {
-        gemm_reduce_kernel<<<grid_for((long long)M * N), 256, 0, s>>>(net->part.as<float>(), splits, (long long)M * N,
-                                                                      M, N, ldc, bias, relu, accumulate, Cf, Cb);
-        GB_LAUNCHED();
+    const int kchunk = (int)(((K + splits - 1) / splits + GBK - 1) / GBK * GBK);
+    *splits_out = (K + kchunk - 1) / kchunk;
+    return kchunk;
+}
+
+// C[M][N] (+)= A B (+ bias, ReLU) for `samples` samples with A = [M][K] or [K][M]
+// (a_km), B = [K][N] or [N][K] (b_nk), or gathered from src (B null); FP32 output
+// Cf and/or bf16 output Cb, row pitch ldc.  With accumulate one C takes the
+// samples in order.
+struct Operand { const bf16 *p; long long ld, bs; };
+
+int gemm(gbfwi_unet *net, int samples, Operand A, bool a_km, Operand B, const ConvSrc *src, bool b_nk, int M, int N, int K,
+         float *Cf, bf16 *Cb, const float *bias, int relu, int accumulate, long long ldc, long long cbs, cudaStream_t s)
+{
+    if (M < 1 || N < 1 || K < 8 || K % 8 || A.ld % 8 || N % 2 || ldc % 2 || ((uintptr_t)A.p & 15) || (a_km && M % 8) ||
+        (!b_nk && N % 8))
+        return GBFWI_EINVAL;
+    if (!src && (B.ld % 8 || ((uintptr_t)B.p & 15))) return GBFWI_EINVAL;
+    if (src && (src->W % 8 || ((uintptr_t)src->s1 & 15) || ((uintptr_t)src->s2 & 15))) return GBFWI_EINVAL;
+    const int BM = bm_of(M);
+    int splits = 1;
+    const int kchunk = split_chunk(M, N, K, net->part_cap, &splits);
+    const bool partial = splits > 1 || (accumulate && samples > 1);
+    // samples whose partials fit the scratch together
+    const int fit = partial ? (int)std::max<long long>(1, net->part_cap / ((long long)M * N * splits)) : samples;
+    for (int b0 = 0; b0 < samples; b0 += fit) {
+        const int nb = std::min(fit, samples - b0);
+        GemmArgs g{};
+        g.A = A.p + b0 * A.bs; g.lda = A.ld; g.abs_ = A.bs;
+        if (src) {
+            g.src = *src;
+            g.src.s1 += b0 * src->bs1;
+            if (g.src.s2) g.src.s2 += b0 * src->bs2;
+        } else {
+            g.B = B.p + b0 * B.bs; g.ldb = B.ld; g.bbs = B.bs;
+        }
+        g.M = M; g.N = N; g.K = K; g.kchunk = kchunk; g.splits = splits;
+        float *cf = Cf ? Cf + (accumulate ? 0 : b0 * cbs) : nullptr;
+        bf16 *cb = Cb ? Cb + b0 * cbs : nullptr;
+        if (partial) {
+            g.Cf = net->part.as<float>();
+            g.ldc = N;
+            g.split_stride = (long long)M * N;
+            g.partial = 1;
+        } else {
+            g.Cf = cf; g.Cb = cb; g.bias = bias; g.relu = relu; g.accumulate = accumulate; g.ldc = ldc; g.cbs = cbs;
+        }
+        GB_TRY(BM == 32 ? launch_gemm_bm<32>(g, nb, a_km, b_nk, s)
+                        : (BM == 64 ? launch_gemm_bm<64>(g, nb, a_km, b_nk, s) : launch_gemm_bm<128>(g, nb, a_km, b_nk, s)));
+        if (partial) {
+            // (four outputs a thread once that leaves enough threads: 16.8 us to 6.7 us for
+            // 32 x 262144 outputs; slower for the few outputs of a weight gradient)
+            const bool wide = (long long)M * N >= 4LL * 152 * 1024 && N % 4 == 0 && ldc % 4 == 0 && cbs % 4 == 0 && !((uintptr_t)cf & 15) && !((uintptr_t)cb & 7) &&
+                              !((uintptr_t)net->part.p & 15);
+            auto reduce = wide ? gemm_reduce_kernel<4> : gemm_reduce_kernel<1>;
+            reduce<<<dim3((unsigned)grid_for((long long)M * N, wide ? 4 : 1), accumulate ? 1u : (unsigned)nb), 256, 0, s>>>(
+                net->part.as<float>(), nb, splits, M, N, ldc, cbs, bias, relu, accumulate, cf, cb);
+            GB_LAUNCHED();
+        }
     }
     return GBFWI_OK;
 }
 
-int im2col(const bf16 *s1, int C1, int up1, const bf16 *s2, int C2, int H, int W, int Kp, bf16 *out, cudaStream_t s)
+template <int BM>
+int launch_dx(const GemmArgs &g, int samples, cudaStream_t s)
 {
-    im2col_kernel<<<grid_for((long long)Kp * H * W, 8), 256, 0, s>>>(s1, C1, up1, s2, C2, H, W, Kp, out);
+    constexpr int BN = bn_of(BM);
+    using T = GemmTile<BM, BN, true, false>;
+    constexpr size_t smem = (size_t)GSTAGES * (T::AE + T::BE) * sizeof(bf16);
+    static bool attr_done[64] = {};
+    GB_TRY(allow_smem(conv_dx_kernel<BM, BN>, smem, attr_done));
+    conv_dx_kernel<BM, BN><<<dim3((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), (unsigned)samples),
+                             GTHREADS, smem, s>>>(g);
     GB_LAUNCHED();
     return GBFWI_OK;
 }
 
-// 3x3 convolution + bias + ReLU -> bf16 output [cout][H][W]
-int conv_fwd(gbfwi_unet *n, const UnetLayer &L, const bf16 *s1, int C1, int up1, const bf16 *s2, int C2, int H, int W,
-             bf16 *out, cudaStream_t s)
+// 3x3 convolution + bias + ReLU -> bf16 output [sample][cout][H][W]
+int conv_fwd(gbfwi_unet *n, int nb, const UnetLayer &L, const ConvSrc &src, bf16 *out, cudaStream_t s)
 {
-    const long long P = (long long)H * W;
-    GB_TRY(im2col(s1, C1, up1, s2, C2, H, W, L.kcp, n->col.as<bf16>(), s));
-    return gemm(n, n->pb.as<bf16>() + L.w_off, L.kcp, false, n->col.as<bf16>(), P, false, L.cout, (int)P, L.kcp,
-                nullptr, out, n->p32.as<float>() + L.b_off, 1, 0, P, s);
+    const long long P = (long long)src.H * src.W;
+    return gemm(n, nb, {n->pb.as<bf16>() + L.w_off, L.kcp, 0}, false, {}, &src, false, L.cout, (int)P, L.kcp, nullptr, out,
+                n->p32.as<float>() + L.b_off, 1, 0, P, L.cout * P, s);
+}
+
+int bias_grad(gbfwi_unet *n, int nb, const bf16 *G, long long P, int rows, float *db, cudaStream_t s)
+{
+    rowsum_kernel<<<dim3((unsigned)rows, (unsigned)nb), 256, 0, s>>>(G, P, rows, n->rsum.as<float>());
+    GB_LAUNCHED();
+    rowsum_add_kernel<<<(rows + 127) / 128, 128, 0, s>>>(n->rsum.as<float>(), nb, rows, db);
+    GB_LAUNCHED();
+    return GBFWI_OK;
 }
 
 // Backward of a 3x3 convolution given its masked output gradient G
-// (bf16 [cout][P]): dW, db accumulate into the gradient buffer; when dX is
-// not null, the input gradient (FP32 [cin][P]) is written there.
-int conv_bwd(gbfwi_unet *n, const UnetLayer &L, const bf16 *s1, int C1, int up1, const bf16 *s2, int C2, int H, int W,
-             const bf16 *G, float *dX, cudaStream_t s)
+// (bf16 [sample][cout][P]): dW, db accumulate into the gradient buffer; when dX is
+// not null, the input gradient (FP32 [sample][cin][P]) is written there.
+int conv_bwd(gbfwi_unet *n, int nb, const UnetLayer &L, const ConvSrc &src, const bf16 *G, float *dX, cudaStream_t s)
 {
-    const long long P = (long long)H * W;
-    GB_TRY(im2col(s1, C1, up1, s2, C2, H, W, L.kcp, n->col.as<bf16>(), s));
-    GB_TRY(gemm(n, G, P, false, n->col.as<bf16>(), P, true, L.cout, L.kcp, (int)P, n->g32.as<float>() + L.w_off,
-                nullptr, nullptr, 0, 1, L.kcp, s));
-    rowsum_kernel<<<L.cout, 256, 0, s>>>(G, P, n->g32.as<float>() + L.b_off);
-    GB_LAUNCHED();
+    const long long P = (long long)src.H * src.W;
+    GB_TRY(gemm(n, nb, {G, P, L.cout * P}, false, {}, &src, true, L.cout, L.kcp, (int)P, n->g32.as<float>() + L.w_off, nullptr,
+                nullptr, 0, 1, L.kcp, 0, s));
+    GB_TRY(bias_grad(n, nb, G, P, L.cout, n->g32.as<float>() + L.b_off, s));
     if (!dX) return GBFWI_OK;
-    GB_TRY(gemm(n, n->pb.as<bf16>() + L.w_off, L.kcp, true, G, P, false, L.kcp, (int)P, L.coutp,
-                n->dcol.as<float>(), nullptr, nullptr, 0, 0, P, s));
-    col2im_kernel<<<grid_for((long long)L.cin * P), 256, 0, s>>>(n->dcol.as<float>(), L.cin, H, W, dX);
-    GB_LAUNCHED();
-    return GBFWI_OK;
+    GemmArgs g{};
+    g.A = n->wt.as<bf16>() + L.w_off;
+    g.lda = L.cin;
+    g.M = L.cin; g.N = (int)P; g.K = L.coutp;
+    int splits = 1;
+    // the parts the taps' sums are cut into: the split rule of a (9 cin x P) product
+    g.kchunk = split_chunk(L.kcp, (int)P, L.coutp, n->part_cap, &splits);
+    g.Cf = dX; g.ldc = P; g.cbs = L.cin * P;
+    g.src = ConvSrc{G, G, L.cout, 0, 0, src.H, src.W, L.cout * P, 0};
+    const int BM = bm_of(L.cin);
+    return BM == 32 ? launch_dx<32>(g, nb, s) : (BM == 64 ? launch_dx<64>(g, nb, s) : launch_dx<128>(g, nb, s));
 }
 
-int grad_mask(const float *fine, const float *coarse, const float *direct, const bf16 *y, int C, int H, int W,
-              bf16 *out, cudaStream_t s)
+int grad_mask(int nb, const float *fine, long long fine_bs, const float *coarse, const float *direct, long long direct_bs,
+              const bf16 *y, int C, int H, int W, bf16 *out, cudaStream_t s)
 {
-    grad_mask_kernel<<<grid_for((long long)C * H * W), 256, 0, s>>>(fine, coarse, direct, y, C, H, W, out);
+    grad_mask_kernel<<<dim3((unsigned)grid_for((long long)C * H * W), (unsigned)nb), 256, 0, s>>>(
+        fine, fine_bs, coarse, direct, direct_bs, y, C, H, W, out);
     GB_LAUNCHED();
     return GBFWI_OK;
 }
 
-// forward pass on n->xb (bf16 input already staged) -> n->yout
-int net_forward(gbfwi_unet *n, cudaStream_t s)
+// transposed weights for the input gradients, after the weights changed
+int refresh_wt(gbfwi_unet *n, cudaStream_t s)
+{
+    if (n->wt_fresh) return GBFWI_OK;
+    for (const UnetLayer &L : n->layers) {
+        if (L.k != 3) continue;
+        transpose_weights_kernel<<<grid_for(9LL * L.cout * L.cin), 256, 0, s>>>(n->pb.as<bf16>() + L.w_off, L.cout, L.cin,
+                                                                               L.kcp, n->wt.as<bf16>() + L.w_off);
+        GB_LAUNCHED();
+    }
+    n->wt_fresh = true;
+    return GBFWI_OK;
+}
+
+// plain source: one map, nothing upsampled or concatenated
+ConvSrc plain(const bf16 *x, int C, int H, int W)
+{
+    return ConvSrc{x, x, C, 0, 0, H, W, (long long)C * H * W, 0};
+}
+
+// decoder input of level l: the level below upsampled, then the skip connection
+ConvSrc decoder_src(const gbfwi_unet *n, int l, const bf16 *below)
+{
+    const int H = n->d.height >> l, W = n->d.width >> l;
+    return ConvSrc{below, n->e[l].as<bf16>(), n->ch[l + 1], 1, n->ch[l], H, W, (long long)n->ch[l + 1] * (H / 2) * (W / 2),
+                   (long long)n->ch[l] * H * W};
+}
+
+// forward pass of nb samples on n->xb (bf16 input already staged) -> n->yout
+int net_forward(gbfwi_unet *n, int nb, cudaStream_t s)
 {
     const int Lv = n->d.levels;
     int li = 0;
     for (int l = 0; l < Lv; ++l) {
         const int H = n->d.height >> l, W = n->d.width >> l;
-        const bf16 *in;
-        int cin;
-        if (l == 0) {
-            in = n->xb.as<bf16>();
-            cin = n->d.cin;
-        } else {
+        const bf16 *in = n->xb.as<bf16>();
+        int cin = n->d.cin;
+        if (l > 0) {
             cin = n->ch[l - 1];
-            avgpool_kernel<<<grid_for((long long)cin * H * W), 256, 0, s>>>(n->e[l - 1].as<bf16>(), cin, H, W,
-                                                                           n->pl[l].as<bf16>());
+            avgpool_kernel<<<grid_for((long long)nb * cin * H * W), 256, 0, s>>>(n->e[l - 1].as<bf16>(), nb * cin, H, W,
+                                                                                n->pl[l].as<bf16>());
             GB_LAUNCHED();
             in = n->pl[l].as<bf16>();
         }
-        GB_TRY(conv_fwd(n, n->layers[li++], in, cin, 0, nullptr, 0, H, W, n->ea[l].as<bf16>(), s));
-        GB_TRY(conv_fwd(n, n->layers[li++], n->ea[l].as<bf16>(), n->ch[l], 0, nullptr, 0, H, W, n->e[l].as<bf16>(), s));
+        GB_TRY(conv_fwd(n, nb, n->layers[li++], plain(in, cin, H, W), n->ea[l].as<bf16>(), s));
+        GB_TRY(conv_fwd(n, nb, n->layers[li++], plain(n->ea[l].as<bf16>(), n->ch[l], H, W), n->e[l].as<bf16>(), s));
     }
     const bf16 *h = n->e[Lv - 1].as<bf16>();
     for (int l = Lv - 2; l >= 0; --l) {
         const int H = n->d.height >> l, W = n->d.width >> l;
-        GB_TRY(conv_fwd(n, n->layers[li++], h, n->ch[l + 1], 1, n->e[l].as<bf16>(), n->ch[l], H, W,
-                        n->da[l].as<bf16>(), s));
-        GB_TRY(conv_fwd(n, n->layers[li++], n->da[l].as<bf16>(), n->ch[l], 0, nullptr, 0, H, W, n->dd[l].as<bf16>(), s));
+        GB_TRY(conv_fwd(n, nb, n->layers[li++], decoder_src(n, l, h), n->da[l].as<bf16>(), s));
+        GB_TRY(conv_fwd(n, nb, n->layers[li++], plain(n->da[l].as<bf16>(), n->ch[l], H, W), n->dd[l].as<bf16>(), s));
         h = n->dd[l].as<bf16>();
     }
     const UnetLayer &O = n->layers[li];
     const long long P0 = npix(n, 0);
-    return gemm(n, n->pb.as<bf16>() + O.w_off, O.kcp, false, h, P0, false, O.coutp, (int)P0, O.kcp,
-                n->yout.as<float>(), nullptr, n->p32.as<float>() + O.b_off, 0, 0, P0, s);
+    return gemm(n, nb, {n->pb.as<bf16>() + O.w_off, O.kcp, 0}, false, {h, P0, n->ch[0] * P0}, nullptr, false, O.coutp, (int)P0,
+                O.kcp, n->yout.as<float>(), nullptr, n->p32.as<float>() + O.b_off, 0, 0, P0, O.coutp * P0, s);
 }
 
-// backward pass from the output gradient n->gyb (bf16 [coutp][P0]);
-// parameter gradients accumulate into n->g32
-int net_backward(gbfwi_unet *n, cudaStream_t s)
+// backward pass of nb samples from the output gradient n->gyb (bf16
+// [sample][coutp][P0]); parameter gradients accumulate into n->g32
+int net_backward(gbfwi_unet *n, int nb, cudaStream_t s)
 {
     const int Lv = n->d.levels;
     const long long P0 = npix(n, 0);
     int li = (int)n->layers.size() - 1;
     const UnetLayer &O = n->layers[li];
     const bf16 *top = Lv > 1 ? n->dd[0].as<bf16>() : n->e[0].as<bf16>();
+    GB_TRY(refresh_wt(n, s));
     // output 1x1 convolution
-    GB_TRY(gemm(n, n->gyb.as<bf16>(), P0, false, top, P0, true, O.coutp, O.kcp, (int)P0, n->g32.as<float>() + O.w_off,
-                nullptr, nullptr, 0, 1, O.kcp, s));
-    rowsum_kernel<<<O.coutp, 256, 0, s>>>(n->gyb.as<bf16>(), P0, n->g32.as<float>() + O.b_off);
-    GB_LAUNCHED();
-    GB_TRY(gemm(n, n->pb.as<bf16>() + O.w_off, O.kcp, true, n->gyb.as<bf16>(), P0, false, O.kcp, (int)P0, O.coutp,
-                n->fA.as<float>(), nullptr, nullptr, 0, 0, P0, s));
+    GB_TRY(gemm(n, nb, {n->gyb.as<bf16>(), P0, O.coutp * P0}, false, {top, P0, n->ch[0] * P0}, nullptr, true, O.coutp, O.kcp,
+                (int)P0, n->g32.as<float>() + O.w_off, nullptr, nullptr, 0, 1, O.kcp, 0, s));
+    GB_TRY(bias_grad(n, nb, n->gyb.as<bf16>(), P0, O.coutp, n->g32.as<float>() + O.b_off, s));
+    GB_TRY(gemm(n, nb, {n->pb.as<bf16>() + O.w_off, O.kcp, 0}, true, {n->gyb.as<bf16>(), P0, O.coutp * P0}, nullptr, false, O.kcp,
+                (int)P0, O.coutp, n->fA.as<float>(), nullptr, nullptr, 0, 0, P0, O.kcp * P0, s));
     --li;
+    float *fA = n->fA.as<float>();
+    bf16 *gb = n->gb.as<bf16>();
+    auto wide = [&](int l) { return (long long)(n->ch[l + 1] + n->ch[l]) * npix(n, l); };   // dcat elements per sample
     // decoder, fine to coarse; the gradient of level l's output arrives as
     // fA (level 0) or as the upsampling adjoint of dcat[l-1]
     for (int l = 0; l <= Lv - 2; ++l) {
         const int H = n->d.height >> l, W = n->d.width >> l;
+        const long long own = n->ch[l] * npix(n, l);
         const float *fine = l > 0 ? n->dcat[l - 1].as<float>() : nullptr;
-        const float *direct = l == 0 ? n->fA.as<float>() : nullptr;
-        GB_TRY(grad_mask(fine, nullptr, direct, n->dd[l].as<bf16>(), n->ch[l], H, W, n->gb.as<bf16>(), s));
-        GB_TRY(conv_bwd(n, n->layers[li], n->da[l].as<bf16>(), n->ch[l], 0, nullptr, 0, H, W, n->gb.as<bf16>(),
-                        n->fA.as<float>(), s));
+        const float *direct = l == 0 ? fA : nullptr;
+        GB_TRY(grad_mask(nb, fine, l > 0 ? wide(l - 1) : 0, nullptr, direct, own, n->dd[l].as<bf16>(), n->ch[l], H, W, gb, s));
+        GB_TRY(conv_bwd(n, nb, n->layers[li], plain(n->da[l].as<bf16>(), n->ch[l], H, W), gb, fA, s));
         --li;
-        GB_TRY(grad_mask(nullptr, nullptr, n->fA.as<float>(), n->da[l].as<bf16>(), n->ch[l], H, W, n->gb.as<bf16>(), s));
+        GB_TRY(grad_mask(nb, nullptr, 0, nullptr, fA, own, n->da[l].as<bf16>(), n->ch[l], H, W, gb, s));
         const bf16 *coarse = (l + 1 <= Lv - 2) ? n->dd[l + 1].as<bf16>() : n->e[Lv - 1].as<bf16>();
-        GB_TRY(conv_bwd(n, n->layers[li], coarse, n->ch[l + 1], 1, n->e[l].as<bf16>(), n->ch[l], H, W,
-                        n->gb.as<bf16>(), n->dcat[l].as<float>(), s));
+        GB_TRY(conv_bwd(n, nb, n->layers[li], decoder_src(n, l, coarse), gb, n->dcat[l].as<float>(), s));
         --li;
     }
     // encoder, bottleneck first; the gradient of e[l] sums the decoder's
@@ -852,34 +1175,36 @@ int net_backward(gbfwi_unet *n, cudaStream_t s)
     // below and the skip connection
     for (int l = Lv - 1; l >= 0; --l) {
         const int H = n->d.height >> l, W = n->d.width >> l;
-        const long long P = (long long)H * W;
+        const long long P = (long long)H * W, own = n->ch[l] * P;
         const float *fine = nullptr, *coarse = nullptr, *direct = nullptr;
+        long long fine_bs = 0, direct_bs = own;
         if (l == Lv - 1) {
-            if (Lv > 1)
+            if (Lv > 1) {
                 fine = n->dcat[Lv - 2].as<float>();
-            else
-                direct = n->fA.as<float>();
+                fine_bs = wide(Lv - 2);
+            } else {
+                direct = fA;
+            }
         } else {
             coarse = n->fP.as<float>();
             direct = n->dcat[l].as<float>() + (long long)n->ch[l + 1] * P;
+            direct_bs = wide(l);
         }
-        GB_TRY(grad_mask(fine, coarse, direct, n->e[l].as<bf16>(), n->ch[l], H, W, n->gb.as<bf16>(), s));
-        GB_TRY(conv_bwd(n, n->layers[li], n->ea[l].as<bf16>(), n->ch[l], 0, nullptr, 0, H, W, n->gb.as<bf16>(),
-                        n->fA.as<float>(), s));
+        GB_TRY(grad_mask(nb, fine, fine_bs, coarse, direct, direct_bs, n->e[l].as<bf16>(), n->ch[l], H, W, gb, s));
+        GB_TRY(conv_bwd(n, nb, n->layers[li], plain(n->ea[l].as<bf16>(), n->ch[l], H, W), gb, fA, s));
         --li;
-        GB_TRY(grad_mask(nullptr, nullptr, n->fA.as<float>(), n->ea[l].as<bf16>(), n->ch[l], H, W, n->gb.as<bf16>(), s));
+        GB_TRY(grad_mask(nb, nullptr, 0, nullptr, fA, own, n->ea[l].as<bf16>(), n->ch[l], H, W, gb, s));
         const bf16 *in = l == 0 ? n->xb.as<bf16>() : n->pl[l].as<bf16>();
         const int cin = l == 0 ? n->d.cin : n->ch[l - 1];
-        GB_TRY(conv_bwd(n, n->layers[li], in, cin, 0, nullptr, 0, H, W, n->gb.as<bf16>(),
-                        l > 0 ? n->fP.as<float>() : nullptr, s));
+        GB_TRY(conv_bwd(n, nb, n->layers[li], plain(in, cin, H, W), gb, l > 0 ? n->fP.as<float>() : nullptr, s));
         --li;
     }
     return GBFWI_OK;
 }
 
-int stage_input(gbfwi_unet *n, const float *x, cudaStream_t s)
+int stage_input(gbfwi_unet *n, int nb, const float *x, cudaStream_t s)
 {
-    const long long cnt = (long long)n->d.cin * npix(n, 0);
+    const long long cnt = (long long)nb * n->d.cin * npix(n, 0);
     const float *src = x;
     if (!gb_is_device_ptr(x)) {
         GB_CUDA(cudaMemcpyAsync(n->xin32.p, x, cnt * sizeof(float), cudaMemcpyHostToDevice, s));
@@ -888,6 +1213,61 @@ int stage_input(gbfwi_unet *n, const float *x, cudaStream_t s)
     to_bf16_kernel<<<grid_for(cnt), 256, 0, s>>>(src, cnt, n->xb.as<bf16>());
     GB_LAUNCHED();
     return GBFWI_OK;
+}
+
+// Activation buffers for nb samples, and the gradients' when grads.  Grown on
+// demand: inference needs neither the gradients nor more than one sample.
+int reserve(gbfwi_unet *n, int nb, bool grads)
+{
+    if (nb <= n->nb && (n->grads || !grads)) return GBFWI_OK;
+    nb = std::max(nb, n->nb);
+    const int Lv = n->d.levels;
+    const long long P0 = npix(n, 0);
+    const UnetLayer &O = n->layers.back();
+    int rc = GBFWI_OK;
+    auto need = [&](DevBuf &b, long long bytes) {
+        if (!rc) rc = b.ensure((size_t)std::max<long long>(bytes * nb, 16));
+    };
+    const size_t F = sizeof(float), B2 = sizeof(bf16);
+    n->nb = 0;                          // until all of it is there
+    need(n->xin32, (long long)n->d.cin * P0 * F);
+    need(n->xb, (long long)n->d.cin * P0 * B2);
+    need(n->tgt32, (long long)n->d.cout * P0 * F);
+    need(n->yout, (long long)O.coutp * P0 * F);
+    long long cmax = (long long)O.coutp * P0;
+    for (int l = 0; l < Lv; ++l) {
+        const long long P = npix(n, l);
+        cmax = std::max(cmax, n->ch[l] * P);
+        need(n->ea[l], n->ch[l] * P * B2);
+        need(n->e[l], n->ch[l] * P * B2);
+        if (l > 0) need(n->pl[l], n->ch[l - 1] * P * B2);
+        if (l <= Lv - 2) {
+            need(n->da[l], n->ch[l] * P * B2);
+            need(n->dd[l], n->ch[l] * P * B2);
+        }
+    }
+    if (grads || n->grads) {
+        need(n->gyb, (long long)O.coutp * P0 * B2);
+        for (int l = 0; l <= Lv - 2; ++l) need(n->dcat[l], (long long)(n->ch[l + 1] + n->ch[l]) * npix(n, l) * F);
+        need(n->fA, cmax * F);
+        need(n->fP, cmax * F);
+        need(n->gb, cmax * B2);
+        need(n->rsum, (long long)std::max(n->ch[Lv - 1], O.coutp) * F);
+        if (!rc) rc = n->wt.ensure((size_t)n->nparam * B2);
+    }
+    if (rc) return rc;
+    n->nb = nb;
+    n->grads = n->grads || grads;
+    return GBFWI_OK;
+}
+
+// samples a training step takes at once: their buffers stay near 2 GiB
+int batch_group(const gbfwi_unet *n, int batch)
+{
+    long long per = 0;                  // bytes of one sample, the gradients included
+    for (int l = 0; l < n->d.levels; ++l) per += npix(n, l) * n->ch[l] * (5 * 2 + 4 + 3 * 4);
+    per += npix(n, 0) * (n->ch[0] * 10 + 64);
+    return (int)std::max<long long>(1, std::min<long long>(batch, (2LL << 30) / std::max<long long>(per, 1)));
 }
 
 int read_flag(gbfwi_unet *n, cudaStream_t s, int *out)
@@ -931,22 +1311,6 @@ extern "C" int gbfwi_unet_create(const gbfwi_unet_desc *d, gbfwi_unet **out)
         add(n->ch[l], n->ch[l], 3);
     }
     add(n->ch[0], d->cout, 1);
-    const long long P0 = npix(n, 0);
-    long long colmax = 0, cmax = 0;
-    for (int l = 0; l < Lv; ++l) cmax = std::max(cmax, (long long)n->ch[l] * npix(n, l));
-    {
-        int li = 0;
-        for (int l = 0; l < Lv; ++l) {
-            colmax = std::max(colmax, (long long)n->layers[li++].kcp * npix(n, l));
-            colmax = std::max(colmax, (long long)n->layers[li++].kcp * npix(n, l));
-        }
-        for (int l = Lv - 2; l >= 0; --l) {
-            colmax = std::max(colmax, (long long)n->layers[li++].kcp * npix(n, l));
-            colmax = std::max(colmax, (long long)n->layers[li++].kcp * npix(n, l));
-        }
-    }
-    const UnetLayer &O = n->layers.back();
-    cmax = std::max(cmax, (long long)O.coutp * P0);
     n->part_cap = 32LL << 20;   // floats of split-K partials
     int rc = GBFWI_OK;
     auto need = [&](DevBuf &b, long long bytes) {
@@ -958,30 +1322,10 @@ extern "C" int gbfwi_unet_create(const gbfwi_unet_desc *d, gbfwi_unet **out)
     need(n->m32, n->nparam * F);
     need(n->v32, n->nparam * F);
     need(n->pb, n->nparam * B2);
-    need(n->xin32, (long long)d->cin * P0 * F);
-    need(n->xb, (long long)d->cin * P0 * B2);
-    need(n->tgt32, (long long)d->cout * P0 * F);
-    for (int l = 0; l < Lv; ++l) {
-        const long long P = npix(n, l);
-        need(n->ea[l], n->ch[l] * P * B2);
-        need(n->e[l], n->ch[l] * P * B2);
-        if (l > 0) need(n->pl[l], n->ch[l - 1] * P * B2);
-        if (l <= Lv - 2) {
-            need(n->da[l], n->ch[l] * P * B2);
-            need(n->dd[l], n->ch[l] * P * B2);
-            need(n->dcat[l], (long long)(n->ch[l + 1] + n->ch[l]) * P * F);
-        }
-    }
-    need(n->yout, (long long)O.coutp * P0 * F);
-    need(n->gyb, (long long)O.coutp * P0 * B2);
-    need(n->col, colmax * B2);
-    need(n->dcol, colmax * F);
-    need(n->fA, cmax * F);
-    need(n->fP, cmax * F);
-    need(n->gb, cmax * B2);
     need(n->part, n->part_cap * F);
-    need(n->red, 4096 * sizeof(double));
+    need(n->red, (1024 + 512 * 64) * sizeof(double));
     need(n->flag, 16);
+    if (!rc) rc = reserve(n, 1, true);
     if (rc) {
         delete n;
         return rc;
@@ -1035,6 +1379,7 @@ extern "C" int gbfwi_unet_set_params(gbfwi_unet *n, const float *params, void *s
     GB_CUDA(cudaMemsetAsync(n->m32.p, 0, n->nparam * sizeof(float), s));
     GB_CUDA(cudaMemsetAsync(n->v32.p, 0, n->nparam * sizeof(float), s));
     n->step = 0;
+    n->wt_fresh = false;
     GB_CUDA(cudaStreamSynchronize(s));
     return GBFWI_OK;
 }
@@ -1056,8 +1401,9 @@ extern "C" int gbfwi_unet_forward(gbfwi_unet *n, const float *x, float *y, void 
     GB_TRY(gb_check_local(x, y));
     cudaStream_t s = (cudaStream_t)stream;
     const long long P0 = npix(n, 0);
-    GB_TRY(stage_input(n, x, s));
-    GB_TRY(net_forward(n, s));
+    GB_TRY(reserve(n, 1, true));
+    GB_TRY(stage_input(n, 1, x, s));
+    GB_TRY(net_forward(n, 1, s));
     const long long cnt = (long long)n->d.cout * P0;
     GB_CUDA(cudaMemsetAsync(n->flag.p, 0, sizeof(int), s));
     finite_flag_kernel<<<grid_for(cnt), 256, 0, s>>>(n->yout.as<float>(), cnt, n->flag.as<int>());
@@ -1076,8 +1422,9 @@ extern "C" int gbfwi_unet_gradient(gbfwi_unet *n, const float *x, const float *d
     cudaStream_t s = (cudaStream_t)stream;
     const long long P0 = npix(n, 0);
     const UnetLayer &O = n->layers.back();
-    GB_TRY(stage_input(n, x, s));
-    GB_TRY(net_forward(n, s));
+    GB_TRY(reserve(n, 1, true));
+    GB_TRY(stage_input(n, 1, x, s));
+    GB_TRY(net_forward(n, 1, s));
     // dy [cout][P0] -> bf16 rows of the padded output gradient
     const long long cnt = (long long)n->d.cout * P0;
     const float *dys = dy;
@@ -1089,7 +1436,7 @@ extern "C" int gbfwi_unet_gradient(gbfwi_unet *n, const float *x, const float *d
     to_bf16_kernel<<<grid_for(cnt), 256, 0, s>>>(dys, cnt, n->gyb.as<bf16>());
     GB_LAUNCHED();
     GB_CUDA(cudaMemsetAsync(n->g32.p, 0, n->nparam * sizeof(float), s));
-    GB_TRY(net_backward(n, s));
+    GB_TRY(net_backward(n, 1, s));
     GB_CUDA(cudaMemcpyAsync(grad, n->g32.p, n->nparam * sizeof(float),
                             gb_is_device_ptr(grad) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
@@ -1108,27 +1455,32 @@ extern "C" int gbfwi_unet_train_step(gbfwi_unet *n, const float *x, const float 
     const bool dx = gb_is_device_ptr(x), dt = gb_is_device_ptr(target);
     GB_CUDA(cudaMemsetAsync(n->g32.p, 0, n->nparam * sizeof(float), s));
     GB_CUDA(cudaMemsetAsync(n->flag.p, 0, sizeof(int), s));
-    const int nb = 512;
-    double *partial = n->red.as<double>();
-    double *lsum = partial + nb;          // per-sample losses [batch] (<= 1024)
     if (batch > 1024) return GBFWI_EINVAL;
-    for (int b = 0; b < batch; ++b) {
-        const float *xb = x + b * xin;
-        GB_TRY(stage_input(n, xb, s));
-        GB_TRY(net_forward(n, s));
+    const int nblk = 512;
+    int group = std::min(batch_group(n, batch), 64);
+    double *lsum = n->red.as<double>();   // per-sample losses [batch] (<= 1024)
+    double *partial = lsum + 1024;        // [group][nblk]
+    int rc = reserve(n, group, true);
+    for (; rc == GBFWI_ENOMEM && group > 1; rc = reserve(n, group, true)) group = (group + 1) / 2;
+    GB_TRY(rc);
+    for (int b = 0; b < batch; b += group) {
+        const int nb = std::min(group, batch - b);
+        GB_TRY(stage_input(n, nb, x + b * xin, s));
+        GB_TRY(net_forward(n, nb, s));
         const float *tb = target + b * tin;
         if (!dt) {
-            GB_CUDA(cudaMemcpyAsync(n->tgt32.p, tb, tin * sizeof(float), cudaMemcpyHostToDevice, s));
+            GB_CUDA(cudaMemcpyAsync(n->tgt32.p, tb, nb * tin * sizeof(float), cudaMemcpyHostToDevice, s));
             tb = n->tgt32.as<float>();
         }
-        mse_kernel<<<nb, 256, 0, s>>>(n->yout.as<float>(), tb, n->d.cout, O.coutp, P0, 1.f / (float)batch, partial,
-                                      n->gyb.as<bf16>());
+        mse_kernel<<<dim3((unsigned)nblk, (unsigned)nb), 256, 0, s>>>(n->yout.as<float>(), tb, n->d.cout, O.coutp, P0,
+                                                                     1.f / (float)batch, partial, n->gyb.as<bf16>());
         GB_LAUNCHED();
-        mse_finish_kernel<<<1, 32, 0, s>>>(partial, nb, tin, lsum + b, n->flag.as<int>());
+        mse_finish_kernel<<<nb, 128, 0, s>>>(partial, nblk, tin, lsum + b, n->flag.as<int>());
         GB_LAUNCHED();
-        GB_TRY(net_backward(n, s));
+        GB_TRY(net_backward(n, nb, s));
     }
     (void)dx;
+    n->wt_fresh = false;                  // the Adam step below changes the weights
     n->step += 1;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const float c1 = 1.f - powf(b1, (float)n->step), c2 = 1.f - powf(b2, (float)n->step);
