@@ -149,7 +149,7 @@ struct gbfwi_mesh {
     double dx_min = 0;                   // smallest GLL node spacing
 
     // device tables
-    DevBuf d_lm;        // float2 [nz][pitch]  (lambda, mu) times the node's quadrature weight w_i w_j
+    DevBuf d_lm;        // float2 [nz][pitch]  (lambda, mu)
     DevBuf d_minv;      // float  [nz][pitch]  1 / M
     DevBuf d_bnd;       // float4 [nz][pitch]  (Cx, Cz, 1/(M + dt/2 Cx), 1/(M + dt/2 Cz)); edges only
     DevBuf d_bw;        // float4 [nz][pitch]  (Wn_x, Wn_z, Wt_x, Wt_z) Stacey edge weights
@@ -212,7 +212,7 @@ int gb_take_status(gbfwi_mesh *m);
 // shot of a batch)
 // ---------------------------------------------------------------------------
 
-// (resident loops only: MODE_FWD_PC is the forward field with its velocities stored, MODE_RCV the
+// (resident loops only: MODE_FWD_PC is the forward field with its accelerations stored, MODE_RCV the
 // receiver field likewise, driven by the records backwards in time)
 enum StepMode { MODE_FWD = 0, MODE_FWD_PC = 1, MODE_ADJ_G = 2, MODE_ADJ_PC = 3, MODE_RCV = 4 };
 
@@ -261,10 +261,10 @@ struct ResidentArgs {
     float2 *vh;                   // half-step velocity, in place
     float2 *out;                  // level k at slot k - out_k0 (out_ring: k % 3), written for k >= out_from
     int out_from, out_ring, out_k0;
-    float2 *vout;                 // MODE_FWD_PC, MODE_RCV: the velocity that made level k, at the same slot
+    float2 *aout;                 // MODE_FWD_PC, MODE_RCV: the acceleration that made level k, at the same slot
     int reverse;                  // MODE_RCV: the signals run backwards
     const float2 *hist; int hist_k0;   // adjoint: forward level k at slot k - hist_k0
-    const float2 *lm;             // (lambda, mu) times the quadrature weight
+    const float2 *lm;             // (lambda, mu)
     const float *minv;
     const float4 *bnd;
     const float *wxs, *wzs;       // 1-D quadrature weights
@@ -288,12 +288,12 @@ int gb_assemble_strain(const gbfwi_mesh *m, const float *eacc, int B, float *acc
 size_t gb_resident_exchange(const ResidentPlan &p, int nshots, long long NP);   // bytes of the exchange buffer
 int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf &xch, cudaStream_t s);
 
-// Time integrals of the preconditioners from stored levels, B shots (sem_integrals.cu): w, v
-// the field (levels 0 .. nt + 1) and the velocity that made each level (slots 2 .. nt + 1);
+// Time integrals of the preconditioners from stored levels, B shots (sem_integrals.cu): w, a
+// the field (levels 0 .. nt + 1) and the acceleration that made each level (slots 2 .. nt + 1);
 // u null: integrals of w alone (P1, P3), else with the field u backwards in time (P2, P4).
 // acc [B][4][NP]: map 0, and maps 1..3 when strains are asked for; esum: gb_integral_bytes
 size_t gb_integral_bytes(const gbfwi_mesh *m, int B);
-int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *v, const float2 *u, bool strains, float *esum,
+int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *a, const float2 *u, bool strains, float *esum,
                       float *acc, cudaStream_t s);
 
 int gb_launch_step(int mode, int tile, const StepArgs &a, int nbatch, cudaStream_t s);

@@ -604,11 +604,7 @@ __global__ void __launch_bounds__(256) material_kernel(const float *__restrict__
         float4 w = bw[g];
         float cx = rho * vp * w.x + rho * vs * w.z;
         float cz = rho * vp * w.y + rho * vs * w.w;
-        // (lambda, mu) times the quadrature weight w_i w_j of the node, which is
-        // the same in every element that shares it
-        const double w1[4] = {0.1, 49.0 / 90.0, 32.0 / 45.0, 49.0 / 90.0};
-        const float ww = (float)(w1[ix & 3] * w1[iz & 3]);
-        lm[g] = make_float2(ww * lam, ww * mu);
+        lm[g] = make_float2(lam, mu);
         minv[g] = 1.f / M;
         bnd[g] = make_float4(cx, cz, 1.f / (M + 0.5f * dt * cx), 1.f / (M + 0.5f * dt * cz));
     }

@@ -113,7 +113,7 @@ constexpr int kNoLevel = INT_MAX;
 
 // forward launches n in [n0, n1); `need`: first level that is read later
 int fwd_range(const Ctx &c, int mode, int n0, int n1, const Levels &f, int need, float2 *vh, float *seis, float *acc,
-              long long acc_shot_stride, long long acc_comp_stride, float2 *vout = nullptr)
+              long long acc_shot_stride, long long acc_comp_stride, float2 *aout = nullptr)
 {
     StepArgs a;
     base_args(a, c);
@@ -134,7 +134,7 @@ int fwd_range(const Ctx &c, int mode, int n0, int n1, const Levels &f, int need,
     if (c.resident) {
         ResidentArgs r;
         resident_args(r, a, c, n0, n1, f, need);
-        r.vout = vout;
+        r.aout = aout;
         return run_resident(c, mode, r);
     }
     for (int n = n0; n < n1; ++n) {
@@ -149,9 +149,9 @@ int fwd_range(const Ctx &c, int mode, int n0, int n1, const Levels &f, int need,
 }
 
 // adjoint launches j in [j0, j1); the adjoint field cycles through the ring w.
-// MODE_RCV (resident): the field alone, all levels to w and their velocities to vout
+// MODE_RCV (resident): the field alone, all levels to w and their accelerations to aout
 int adj_range(const Ctx &c, int mode, int j0, int j1, const Levels &w, float2 *wh, const Levels &hist,
-              const float *sig, float *acc, long long acc_shot_stride, long long acc_comp_stride, float2 *vout = nullptr)
+              const float *sig, float *acc, long long acc_shot_stride, long long acc_comp_stride, float2 *aout = nullptr)
 {
     const int nt = c.m->d.nt;
     StepArgs a;
@@ -173,7 +173,7 @@ int adj_range(const Ctx &c, int mode, int j0, int j1, const Levels &w, float2 *w
         ResidentArgs r;
         resident_args(r, a, c, j0, j1, w, 0);
         r.reverse = 1;
-        r.vout = vout;
+        r.aout = aout;
         return run_resident(c, mode, r);
     }
     if (c.resident && mode == MODE_ADJ_G) {
@@ -1125,7 +1125,8 @@ static int resident_maps(gbfwi_mesh *m, int nshot, int Bmax, int kind, int tile,
         const int B = std::min(Bmax, nshot - i0);
         const long long lev = B * NP;
         const Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, true};
-        const Levels u{m->w_hist.as<float2>(), lev, 0, false}, v{m->w_snap.as<float2>(), lev, 0, false};
+        const Levels u{m->w_hist.as<float2>(), lev, 0, false};
+        float2 *acc_levels = m->w_snap.as<float2>();
         const Levels w{m->w_adj.as<float2>(), lev, 0, false};
         auto at_rest = [&](const Levels &f) -> int {
             GB_CUDA(cudaMemsetAsync(f.base, 0, 2 * lev * sizeof(float2), s));
@@ -1135,12 +1136,12 @@ static int resident_maps(gbfwi_mesh *m, int nshot, int Bmax, int kind, int tile,
         GB_TRY(at_rest(u));
         GB_CUDA(cudaMemsetAsync(acc, 0, (size_t)B * 4 * NP * sizeof(float), s));
         float *seis = m->w_seis.as<float>();
-        GB_TRY(fwd_range(c, fwd, 0, nt, u, 0, vh, receiver ? seis : nullptr, nullptr, 0, 0, receiver ? nullptr : v.base));
+        GB_TRY(fwd_range(c, fwd, 0, nt, u, 0, vh, receiver ? seis : nullptr, nullptr, 0, 0, receiver ? nullptr : acc_levels));
         if (receiver) {
             GB_TRY(at_rest(w));
-            GB_TRY(adj_range(c, MODE_RCV, 0, nt, w, vh, u, seis, nullptr, 0, 0, v.base));
+            GB_TRY(adj_range(c, MODE_RCV, 0, nt, w, vh, u, seis, nullptr, 0, 0, acc_levels));
         }
-        GB_TRY(gb_time_integrals(m, B, receiver ? w.base : u.base, v.base, receiver ? u.base : nullptr, strains,
+        GB_TRY(gb_time_integrals(m, B, receiver ? w.base : u.base, acc_levels, receiver ? u.base : nullptr, strains,
                                  m->w_eacc.as<float>(), acc, s));
         acc_reduce<<<grid_for(4 * NP), 256, 0, s>>>(acc, B, 4, NP, tot);
         GB_LAUNCHED();

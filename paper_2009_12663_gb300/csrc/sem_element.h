@@ -24,6 +24,13 @@ __device__ __forceinline__ constexpr float D(int q)
 // the factor D[i][k] is zero and its product is left out
 __device__ __forceinline__ constexpr bool dzero(int i, int k) { return i == k && i > 0 && i < 4; }
 
+// GLL quadrature weight w_i w_j of local point (i, j)
+__device__ __forceinline__ constexpr float weight(int i, int j)
+{
+    constexpr double w[5] = {1.0 / 10.0, 49.0 / 90.0, 32.0 / 45.0, 49.0 / 90.0, 1.0 / 10.0};
+    return (float)(w[i] * w[j]);
+}
+
 // derivatives at local point (i, j) of the patch p (index j * 5 + i):
 // gx = d/dxi, ge = d/deta of (ux, uz)
 __device__ __forceinline__ void grad_at(const float2 (&p)[25], int i, int j, float2 &gx, float2 &ge)
@@ -45,7 +52,10 @@ __device__ __forceinline__ void grad_at(const float2 (&p)[25], int i, int j, flo
 // Element nodal forces K u accumulated row by row of local points: the
 // stresses of row j give the xi-part of the nodes of row j and the eta-part
 // of every node, so one row of stresses is live at a time.  lmrow(j, lm)
-// gives row j of (lambda, mu) times the quadrature weight w_i w_j.
+// gives row j of (lambda, mu).  The quadrature weight multiplies the stresses:
+// folded into the moduli it saves 75 products, but the second time differences
+// of P2 and P4 magnify the roundings of the field (the map of a 100 x 25 mesh at
+// 5 Hz moved by 3e-5 when only those roundings changed).
 template <class LmRow>
 __device__ __forceinline__ void element_force(const float2 (&p)[25], LmRow lmrow, float2 (&f)[25])
 {
@@ -59,9 +69,9 @@ __device__ __forceinline__ void element_force(const float2 (&p)[25], LmRow lmrow
             float2 gx, ge;
             grad_at(p, i, j, gx, ge);
             const float l2m = fmaf(2.f, lm[i].y, lm[i].x);
-            txx[i] = fmaf(l2m, gx.x, __fmul_rn(lm[i].x, ge.y));
-            tzz[i] = fmaf(lm[i].x, gx.x, __fmul_rn(l2m, ge.y));
-            txz[i] = __fmul_rn(lm[i].y, __fadd_rn(ge.x, gx.y));
+            txx[i] = __fmul_rn(weight(i, j), fmaf(l2m, gx.x, __fmul_rn(lm[i].x, ge.y)));
+            tzz[i] = __fmul_rn(weight(i, j), fmaf(lm[i].x, gx.x, __fmul_rn(l2m, ge.y)));
+            txz[i] = __fmul_rn(weight(i, j), __fmul_rn(lm[i].y, __fadd_rn(ge.x, gx.y)));
         }
 #pragma unroll
         for (int n = 0; n < 5; ++n)

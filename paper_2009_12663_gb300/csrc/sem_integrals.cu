@@ -6,19 +6,21 @@
 // step: every step a CTA loads its windows twice, sums twice over the elements
 // through shared memory in four colour passes, and reads, adds to and writes
 // four node maps; one step took 38 us at 81 x 21 elements and 5 shots, where
-// the resident loop needs 4.5 us.  Here the passes only store their levels
-// (displacement, and the half-step velocity, whose differences are dt times
-// the acceleration), and the integrals are sums over time at fixed nodes and
-// elements: a thread keeps its sums in registers and streams through the
-// levels (800 steps of those 5 shots: 0.82 ms for the strains, 0.29 ms at the
-// nodes, beside 7.0 ms for the two passes).  Bound by those reads (16 B a node,
-// level and field) and, for the strains, by the few warps their registers allow.
+// the resident loop needs 4.5 us.  Here the passes only store their levels (the
+// displacement, and one field's acceleration), and the integrals are sums over
+// time at fixed nodes and elements: a thread keeps its sums in registers and
+// streams through the levels (800 steps of those 5 shots: 0.85 ms for the
+// strains, 0.36 ms at the nodes, beside 7.1 ms for the two passes).  Bound by
+// those reads (16 B a node, level and field) and, for the strains, by the few
+// warps their registers allow.
 //
 // S0 = sum a . a (one field) or sum (second difference of u) . a, at nodes;
 // S1..S3 = sums of [div div', exx exx' + ezz ezz', gam gam'] of the
 // undivided time differences, at the elements' points, assembled to nodes
-// once at the end.  The differences are those of the stored levels, as in the
-// preconditioner steps, so both round them alike.
+// once at the end.  A step's terms are rounded as in the preconditioner steps
+// (differences of the stored levels, product, then the quadrature weight): where
+// a field has only just arrived the terms are denormal numbers, whose sums are
+// exact in any order, so both forms agree there too about what is zero.
 
 #include <algorithm>
 
@@ -49,7 +51,7 @@ __device__ __forceinline__ void load_difference(const float2 *__restrict__ hi, c
 }
 
 // One thread an element, steps [chunk * steps, + steps) of blockIdx.y, shot
-// blockIdx.z; esum [chunk][shot][75][elements], without the quadrature weight.
+// blockIdx.z; esum [chunk][shot][75][elements].
 // TWO: products of the differences of a and b (step j pairs a's levels j, j + 1
 // with b's nt - j, nt - j + 1); otherwise squares of a's.  Chunks of time give
 // a small mesh enough warps to cover the loads.
@@ -82,9 +84,12 @@ __global__ void __launch_bounds__(128) strain_integral_kernel(const float2 *__re
                 bx = ax;
                 be = ae;
             }
-            s[3 * q] = fmaf(ax.x + ae.y, bx.x + be.y, s[3 * q]);
-            s[3 * q + 1] = fmaf(ax.x, bx.x, fmaf(ae.y, be.y, s[3 * q + 1]));
-            s[3 * q + 2] = fmaf(ae.x + ax.y, be.x + bx.y, s[3 * q + 2]);
+            const float ww = weight(q % 5, q / 5);
+            const float da = __fadd_rn(ax.x, ae.y), db = __fadd_rn(bx.x, be.y);
+            const float ga = __fadd_rn(ae.x, ax.y), gb = __fadd_rn(be.x, bx.y);
+            s[3 * q] = __fadd_rn(s[3 * q], __fmul_rn(ww, __fmul_rn(da, db)));
+            s[3 * q + 1] = __fadd_rn(s[3 * q + 1], __fmul_rn(ww, fmaf(ax.x, bx.x, __fmul_rn(ae.y, be.y))));
+            s[3 * q + 2] = __fadd_rn(s[3 * q + 2], __fmul_rn(ww, __fmul_rn(ga, gb)));
         }
     }
     float *o = esum + ((long long)blockIdx.y * gridDim.z + blockIdx.z) * 75 * ne + e;
@@ -92,12 +97,11 @@ __global__ void __launch_bounds__(128) strain_integral_kernel(const float2 *__re
     for (int q = 0; q < 75; ++q) o[(long long)q * ne] = s[q];
 }
 
-// node maps 1..3 of shot blockIdx.y from the element sums: weight times the
-// sum over time chunks and over the elements around the node
+// node maps 1..3 of shot blockIdx.y: the element sums over time chunks and over
+// the elements around the node
 __global__ void strain_assemble_kernel(const float *__restrict__ esum, int chunks, int nshot, int nex, int nez, int nx, int nz,
                                        int pitch, long long NP, float *__restrict__ acc)
 {
-    constexpr double w[5] = {0.1, 49.0 / 90.0, 32.0 / 45.0, 49.0 / 90.0, 0.1};
     const long long N = (long long)nx * nz;
     const int ne = nex * nez;
     acc += (long long)blockIdx.y * 4 * NP;
@@ -115,64 +119,55 @@ __global__ void strain_assemble_kernel(const float *__restrict__ esum, int chunk
 #pragma unroll
             for (int k = 0; k < 3; ++k) s[k] += t[k];
         }
-        double wi = w[0], wj = w[0];
 #pragma unroll
-        for (int k = 1; k < 4; ++k) {
-            if ((ix & 3) == k) wi = w[k];
-            if ((iz & 3) == k) wj = w[k];
-        }
-        const float ww = (float)(wi * wj);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) acc[(k + 1) * NP + (long long)iz * pitch + ix] = ww * s[k];
+        for (int k = 0; k < 3; ++k) acc[(k + 1) * NP + (long long)iz * pitch + ix] = s[k];
     }
 }
 
-// node map 0 of shot blockIdx.y: v holds the half-step velocity that made the
+// node map 0 of shot blockIdx.y: a holds the acceleration that made the
 // displacement level of its slot.  TWO: u's second difference at levels
 // nt - j + 1, nt - j, nt - j - 1 times the acceleration of step j.
 template <bool TWO>
-__global__ void __launch_bounds__(128) mass_integral_kernel(const float2 *__restrict__ v, const float2 *__restrict__ u,
+__global__ void __launch_bounds__(128) mass_integral_kernel(const float2 *__restrict__ a, const float2 *__restrict__ u,
                                                             long long lev, long long NP, int nx, int nz, int pitch, int nt,
-                                                            float rdt, float *__restrict__ acc)
+                                                            float *__restrict__ acc)
 {
     const long long N = (long long)nx * nz;
     const long long q = blockIdx.x * 128LL + threadIdx.x;
     if (q >= N) return;
     const int iz = (int)(q / nx), ix = (int)(q - (long long)iz * nx);
     const long long g = blockIdx.y * NP + (long long)iz * pitch + ix;
-    v += g + 2 * lev;                                    // step j: slot j + 2
+    a += g + 2 * lev;                                    // step j: slot j + 2
     u += g;
-    float2 vp = make_float2(0.f, 0.f), p0, p1;           // at rest before the first step
+    float2 p0, p1;
     if (TWO) {
         p0 = u[(nt + 1) * lev];
         p1 = u[nt * lev];
     }
     float s = 0.f;
     int j = 0;
-    auto step = [&](float2 vn, float2 p2) {
-        const float ax = __fmul_rn(__fsub_rn(vn.x, vp.x), rdt), az = __fmul_rn(__fsub_rn(vn.y, vp.y), rdt);
+    auto step = [&](float2 an, float2 p2) {
         if (TWO) {
             const float2 f = sub2(sub2(p0, p1), sub2(p1, p2));
-            s += fmaf(f.x, ax, f.y * az);
+            s = __fadd_rn(s, fmaf(f.x, an.x, __fmul_rn(f.y, an.y)));
             p0 = p1;
             p1 = p2;
         } else {
-            s += fmaf(ax, ax, az * az);
+            s = __fadd_rn(s, fmaf(an.x, an.x, __fmul_rn(an.y, an.y)));
         }
-        vp = vn;
     };
     constexpr int U = 8;                                 // steps whose loads are in flight together
     for (; j + U <= nt; j += U) {
-        float2 vn[U], un[U];
+        float2 an[U], un[U];
 #pragma unroll
         for (int i = 0; i < U; ++i) {
-            vn[i] = __ldg(v + (j + i) * lev);
+            an[i] = __ldg(a + (j + i) * lev);
             un[i] = TWO ? __ldg(u + (nt - 1 - j - i) * lev) : make_float2(0.f, 0.f);
         }
 #pragma unroll
-        for (int i = 0; i < U; ++i) step(vn[i], un[i]);
+        for (int i = 0; i < U; ++i) step(an[i], un[i]);
     }
-    for (; j < nt; ++j) step(v[j * lev], TWO ? u[(nt - 1 - j) * lev] : make_float2(0.f, 0.f));
+    for (; j < nt; ++j) step(a[j * lev], TWO ? u[(nt - 1 - j) * lev] : make_float2(0.f, 0.f));
     acc[blockIdx.y * 4 * NP + (long long)iz * pitch + ix] = s;
 }
 
@@ -191,17 +186,16 @@ size_t gb_integral_bytes(const gbfwi_mesh *m, int B)
     return (size_t)strain_chunks(m, B) * B * 75 * m->d.nex * m->d.nez * sizeof(float);
 }
 
-int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *v, const float2 *u, bool strains, float *esum,
+int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *a, const float2 *u, bool strains, float *esum,
                       float *acc, cudaStream_t s)
 {
     const int nt = m->d.nt, ne = m->d.nex * m->d.nez;
     const long long NP = (long long)m->nz * m->pitch, N = (long long)m->nx * m->nz, lev = B * NP;
     const dim3 gm((unsigned)((N + 127) / 128), (unsigned)B);
-    const float rdt = (float)(1.0 / m->d.dt);
     if (u)
-        mass_integral_kernel<true><<<gm, 128, 0, s>>>(v, u, lev, NP, m->nx, m->nz, m->pitch, nt, rdt, acc);
+        mass_integral_kernel<true><<<gm, 128, 0, s>>>(a, u, lev, NP, m->nx, m->nz, m->pitch, nt, acc);
     else
-        mass_integral_kernel<false><<<gm, 128, 0, s>>>(v, v, lev, NP, m->nx, m->nz, m->pitch, nt, rdt, acc);
+        mass_integral_kernel<false><<<gm, 128, 0, s>>>(a, a, lev, NP, m->nx, m->nz, m->pitch, nt, acc);
     GB_LAUNCHED();
     if (!strains) return GBFWI_OK;
     const int nc = strain_chunks(m, B), steps = (nt + nc - 1) / nc;

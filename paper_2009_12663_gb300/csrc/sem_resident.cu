@@ -6,7 +6,7 @@
 // (44 B a node forward, 76 B adjoint, from L2) and start cold each step; a
 // mesh of a few tiles leaves the GPU to launch latency (8 us forward, 23 us
 // adjoint a step measured on 12 x 6 elements).  Here a CTA keeps its tile for
-// all steps: the displacement window, the weighted moduli, the velocity and
+// all steps: the displacement window, the moduli, the velocity and
 // the accumulators stay in shared memory or registers, and between steps a
 // CTA only trades the node lines its neighbours need.  Measured a step: 3.9 us
 // forward (40 x 20 elements, one CTA an SM), 5.3 us with two shots an SM,
@@ -199,10 +199,10 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
 {
     using S = Shape<NT_, MODE>;
     constexpr int NT = S::NT, PS = S::PS, NO = S::NO, NA = S::THREADS, kMaxHalo = S::L.halo;
-    constexpr bool ADJ = S::ADJ, VEL = MODE == MODE_RCV;
+    constexpr bool ADJ = S::ADJ, ACC = MODE == MODE_RCV;
     extern __shared__ float4 rsm[];
     float4 *win0 = rsm;                                          // field window [8][PS], two in the adjoint
-    float4 *lmw = win0 + (ADJ ? 2 : 1) * S::WIN;                 // weighted moduli window [8][PS]
+    float4 *lmw = win0 + (ADJ ? 2 : 1) * S::WIN;                 // moduli window [8][PS]
     float4 *smi = lmw + S::WIN;                                  // 1/M [4][NT]
     float4 *sac = smi + 4 * NT;                                  // adjoint: accelerations [8][NO]
     float4 *sst = sac + 8 * NO;                                  // strain sums [13][NO] (25 points, 2 each)
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
 
     // signals of step n into their half of ssig (asynchronous)
     auto fetch_signals = [&](int n) {
-        const int ts = ADJ || (VEL && a.reverse) ? a.nt - 1 - n : n + 1;
+        const int ts = ADJ || (ACC && a.reverse) ? a.nt - 1 - n : n + 1;
 #pragma unroll 1
         for (int e = t; e < ne; e += NT) {
             const int4 I = sent[e];
@@ -522,15 +522,6 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
         for (int q = t; q < nextra; q += NT) {
             const int rx = q < ncol ? 4 * nex : q - ncol, rz = q < ncol ? q : 4 * nez;
             ob[(4 * ez0 + rz) * pitch + 4 * ex0 + rx] = reinterpret_cast<const float2 *>(w)[sxi[q].z];
-        }
-        if (VEL) {                                                // the velocity that made this level
-            float2 *vb = a.vout + (long long)(k - a.out_k0) * a.lev + fo;
-            if (owns)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) store_row(vb + g00 + j * pitch, vr[2 * j], vr[2 * j + 1]);
-#pragma unroll 1
-            for (int q = t; q < nextra; q += NT)
-                vb[q < ncol ? (4 * ez0 + q) * pitch + a.nx - 1 : (a.nz - 1) * pitch + 4 * ex0 + q - ncol] = svx[q];
         }
         // the next level lies in new pages: have their translation ready
         if (!a.out_ring && t < 2 && k <= a.n1) prefetch_l2(ob + a.lev + (t ? ize - 1 : 4 * ez0) * pitch + 4 * ex0);
@@ -626,6 +617,8 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
             for (int q = 0; q < 9; ++q) zc[q * NT + t] = make_float2(0.f, 0.f);
         }
         bar_sync(1, NA);                                          // shares published, window read
+        // the accelerations of this step, in the slot of the level they make
+        float2 *ab = ACC ? a.aout + (long long)(n + 2 - a.out_k0) * a.lev + fo : nullptr;
         // ---- Newmark update of the owned nodes
         if (owns) {
             // the shares of the elements to the left, above and diagonal
@@ -644,6 +637,7 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
             for (int j = 0; j < 4; ++j) {
                 const float4 m4 = smi[j * NT + t];
                 const float mi[4] = {m4.x, m4.y, m4.z, m4.w};
+                float4 ar[2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const float4 v = vr[2 * j + h], u = win[(2 * j + h) * PS + c0];
@@ -675,7 +669,9 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
                     vr[2 * j + h] = vn;
                     nxt[(2 * j + h) * PS + c0] = un;
                     if (ADJ) sac[(2 * j + h) * NO + oi] = ac;
+                    ar[h] = ac;
                 }
+                if (ACC) store_row(ab + g00 + j * pitch, ar[0], ar[1]);
             }
         }
         // ---- and of the extra lines, one node a thread
@@ -691,6 +687,7 @@ __global__ void __launch_bounds__((Shape<NT_, MODE>::THREADS), (Shape<NT_, MODE>
             if (ADJ) sev[sl] = make_float4(0.5f * (v.x + n2.x), 0.5f * (v.y + n2.y), a2.x, a2.y);
             svx[q] = n2;
             reinterpret_cast<float2 *>(nxt)[X.z] = un;
+            if (ACC) ab[q < ncol ? (4 * ez0 + q) * pitch + a.nx - 1 : (a.nz - 1) * pitch + 4 * ex0 + q - ncol] = a2;
         }
         if (a.ntiles > 1) {
             // ---- the node lines the neighbours need
@@ -777,7 +774,7 @@ const Variant *find_variant(int NT, int mode)
     return nullptr;
 }
 
-// the kernel that runs a mode (MODE_RCV's also stores the velocities)
+// the kernel that runs a mode (MODE_RCV's also stores the accelerations)
 int kernel_mode(int mode) { return mode == MODE_FWD_PC ? MODE_RCV : mode; }
 
 bool fits(int NT, int TX, int TZ)
@@ -895,7 +892,7 @@ int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf
 {
     const Variant *v = find_variant(p.NT, kernel_mode(p.mode));
     if (!v || a.pitch % 4 != 0 || a.fstride % 4 != 0 || a.lev % 4 != 0 || a.acc_comp_stride % 4 != 0 ||
-        a.acc_shot_stride % 4 != 0 || ((uintptr_t)a.vout & 31) || ((uintptr_t)a.u0 & 15) || ((uintptr_t)a.out & 31) || ((uintptr_t)a.vh & 15) ||
+        a.acc_shot_stride % 4 != 0 || ((uintptr_t)a.aout & 31) || ((uintptr_t)a.u0 & 15) || ((uintptr_t)a.out & 31) || ((uintptr_t)a.vh & 15) ||
         ((uintptr_t)a.minv & 15) || ((uintptr_t)a.acc & 15) || ((uintptr_t)a.hist & 31) || ((uintptr_t)a.eacc & 15) || !a.status)
         return GBFWI_EINVAL;
     a.TX = p.TX; a.TZ = p.TZ; a.ntx = p.ntx; a.ntz = p.ntz;
@@ -911,7 +908,7 @@ int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf
         a.u0 += s0 * a.fstride;
         a.vh += s0 * a.fstride;
         a.out += s0 * a.fstride;
-        if (a.vout) a.vout += s0 * a.fstride;
+        if (a.aout) a.aout += s0 * a.fstride;
         if (a.hist) a.hist += s0 * a.fstride;
         if (a.acc) a.acc += s0 * a.acc_shot_stride;
         if (a.eacc) a.eacc += (long long)s0 * a.nex * a.nez * 52;

@@ -110,7 +110,7 @@ __device__ __forceinline__ void element_squares(const float2 *__restrict__ wa, i
 }
 
 // forces of the element whose patch starts at `base` of the field window sw
-// and of the weighted-moduli window slm
+// and of the moduli window slm
 template <int NWXP>
 __device__ __forceinline__ void element_force_window(const float2 *__restrict__ sw, const float2 *__restrict__ slm,
                                                      int base, float2 (&f)[25])

@@ -2,11 +2,9 @@
 resident, sem_integrals.cu) equal those of the preconditioner steps
 (sem_step.cu) on a mesh too large for it that shares the top left corner.
 
-The levels are bitwise the same.  S1..S3 are sums of nt products in another
-order: nt 2^-24 of the largest entry.  S0 takes the acceleration from the
-difference of two velocities, 2^-24 |v| / (dt |a|) <= 2^-24 / (w dt) off a
-step (w dt = 0.12 at 40 Hz), once or twice in a product.  With nt <= 15 both
-are below 2e-6 of the largest entry (asserted 8e-6)."""
+The levels and a step's terms are bitwise the same; the sums of nt terms run
+by element or node instead of by step: nt 2^-24 of the largest entry, below
+2e-6 with nt <= 15 and the elements around a node (asserted 8e-6)."""
 import numpy as np
 import pytest
 
