@@ -295,8 +295,9 @@ def choose_schedule(args, wl, srcs, model):
 
 
 def adjoint_kernel_roofline(ph, sch, nshot, N, peak_gbs):
-    """Average adjoint-step launch duration from the per-phase CUDA events of
-    the last timed gradient, and the algorithmic bandwidth it sustains:
+    """Average duration of an adjoint step (a launch of the step kernels, a
+    step of a resident launch) from the per-phase CUDA events of the last timed
+    gradient, and the algorithmic bandwidth it sustains:
     lanes x algorithmic bytes per launch / launch duration (`lanes` batches
     run their identical phases side by side).  A batched launch of S shots
     reads the material once: (64 S + 12) bytes per point."""
@@ -495,12 +496,14 @@ def run_ours(args):
     tr = traffic_record(f"adjoint_step_{tx}x{tz}_spl{r['spl']}")
     roof = {"bound": "hbm", "achieved": r["achieved"], "peak": pk["hbm_gbs"], "unit": "GB/s",
             "frac": r["frac"], "traffic": (tr or {}).get("bytes_per_launch"),
-            "kernel": f"sem_step_kernel<{tx},{tz},ADJ_G> (adjoint step + gradient correlation)",
+            "kernel": "adjoint step + gradient correlation: a step of sem_resident_kernel<ADJ_G> where the mesh fits "
+                      f"the SMs' shared memory, a launch of sem_step_kernel<{tx},{tz},ADJ_G> otherwise",
             "algorithmic_bytes_per_launch": r["adj_unit"], "avg_launch_us": r["adj_us"],
             "concurrent_lanes": r["lanes"], "peak_kind": pk_kind,
             "meaning": "algorithmic bytes (76 B per point and shot: fields, material, history, accumulators) "
                        "over the CUDA-event launch duration, i.e. effective bandwidth; a lane's per-step "
-                       "working set (~17 MB) stays in L2, so DRAM moves less (traffic)",
+                       "working set stays in shared memory (resident loop) or L2 (~17 MB, step kernels), so DRAM "
+                       "moves less",
             "timing": "CUDA events on each launching stream around every adjoint pass",
             "whole_gradient": {"algorithmic_bytes": step_bytes,
                                "achieved": step_bytes / (grad_ms / 1e3) / 1e9,

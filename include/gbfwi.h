@@ -90,7 +90,11 @@ typedef struct {
     double f0, t0, amp;     /* peak frequency (Hz), delay (s), amplitude */
 } gbfwi_source;
 
-/* Launch schedule (chosen by the autotuner or the caller). */
+/* Launch schedule (chosen by the autotuner or the caller).  On meshes whose
+ * fields fit the SMs' shared memory a launch runs a whole range of time steps
+ * instead of one; it chooses its own tile, and shots beyond shots_per_launch
+ * times streams go together where that costs little memory.  Results do not
+ * depend on the schedule. */
 typedef struct {
     int shots_per_launch;   /* shots advanced together in one launch (>= 1) */
     int tile;               /* element-tile variant, 0..gbfwi_num_tiles()-1 */
@@ -133,7 +137,8 @@ int gbfwi_set_schedule(gbfwi_mesh *mesh, const gbfwi_schedule *sch);
  * alpha = vp, beta = vs, rho): lambda = rho (vp^2 - 2 vs^2), mu = rho vs^2.
  * Checks rho > 0, vp > vs > 0, finite values, and the stability bound
  * dt vp_max / dx_min <= 0.5 (dx_min = smallest GLL node spacing) -> ECFL.
- * Synchronises the stream (the check reads the model on the host). */
+ * The first faulty node decides the error; a rejected model leaves the old one
+ * in place.  Synchronises the stream (the outcome is read on the host). */
 int gbfwi_set_model(gbfwi_mesh *mesh, const float *rho, const float *vp, const float *vs,
                     void *stream);
 
@@ -177,6 +182,8 @@ int gbfwi_adjoint_gradient(gbfwi_mesh *mesh, const int *shot_ids, int nshot,
  * B0: [3][nz][nx] = 1 / (S(H) + damp_factor * median(S(H))) per parameter,
  *     S = Gaussian smoothing of standard deviation smooth_sigma_m metres
  *     (quadrature-weighted average in physical space, truncated at 5 sigma).
+ * Meshes whose time loop is resident keep the levels of a batch of shots (at
+ * most 6 GiB) to form the integrals from.
  * Synchronises the stream.  -> EINVAL, ENOMODEL, ECUDA, ENOMEM. */
 int gbfwi_precond_diag(gbfwi_mesh *mesh, const int *shot_ids, int nshot, int kind,
                        double smooth_sigma_m, double damp_factor, float *H, float *B0,
@@ -395,8 +402,8 @@ int gbfwi_enable_timing(gbfwi_mesh *mesh, int on);
 
 /* Device time (ms) of the forward passes and of the adjoint passes of the
  * most recent timed gbfwi_adjoint_gradient on this mesh, and the number of
- * time-step kernel launches in each (the adjoint passes include the segment
- * recomputation when checkpointing).  -> EINVAL when nothing was timed. */
+ * time steps of shot batches in each, one launch each with the step kernels (the
+ * adjoint passes include the segment recomputation when checkpointing).  -> EINVAL when nothing was timed. */
 int gbfwi_last_phase_times(const gbfwi_mesh *mesh, double *fwd_ms, double *adj_ms,
                            long long *fwd_launches, long long *adj_launches);
 

@@ -1078,7 +1078,7 @@ static int b0_from_map(gbfwi_mesh *m, const float *Hd, float *S1, float *S2, dou
 
 // Shots a resident map run takes at once (0: the preconditioner steps run). Both
 // passes keep their levels, so the batches are smaller than the steps' of Bold
-// shots; a step costs 2 x 5.3 us resident, and 8 us forward (receiver maps) and
+// shots; a step costs about 2 x 5.3 us resident, and 8 us forward (receiver maps) and
 // 38 us a wave of 304 CTAs otherwise (measured at 81 x 21 elements, 5 shots).
 static int map_batch(gbfwi_mesh *m, int nshot, bool receiver, int tile, int Bold, long long NP)
 {

@@ -8,9 +8,9 @@
 // adjoint a step measured on 12 x 6 elements).  Here a CTA keeps its tile for
 // all steps: the displacement window, the moduli, the velocity and
 // the accumulators stay in shared memory or registers, and between steps a
-// CTA only trades the node lines its neighbours need.  Measured a step: 3.9 us
-// forward (40 x 20 elements, one CTA an SM), 5.3 us with two shots an SM,
-// 5.3 to 5.7 us adjoint; the chain of a step is the exchange (1.5 us), the
+// CTA only trades the node lines its neighbours need.  Measured a step: 3.9 to 4.4 us
+// forward (40 x 20 elements, one CTA an SM), 5.7 us with two shots an SM,
+// 5.6 us adjoint; the chain of a step is the exchange (1.5 us), the
 // forces (1.6 us), the update (0.8 us) and the sends (0.4 us).
 //
 // Tile and threads.  A CTA owns TX x TZ elements (chosen at run time) of one
