@@ -274,7 +274,7 @@ def time_unet(dev, peak_tflops: float, iters: int = 5, warmup: int = 3):
     return {"shape": "U-Net 4 levels x 32 base channels, 5 -> 3 channels, 256 x 1024, bf16 / fp32 accumulate",
             "params": net.num_params, "conv_flop_per_inference": flop, **res,
             "inference_tflops": tf, "bf16_peak_tflops": peak_tflops, "inference_frac_of_bf16_peak": tf / peak_tflops,
-            "note": "whole forward (im2col + GEMM + epilogues) over the convolution FLOPs; not part of `value`"}
+            "note": "whole forward (gathered GEMMs + epilogues) over the convolution FLOPs; not part of `value`"}
 
 
 def choose_schedule(args, wl, srcs, model):
