@@ -299,16 +299,23 @@ __global__ void gram_kernel(const double *__restrict__ SS, const double *__restr
 // outputs: a thread takes four columns i, the rows streamed as float4, the sums
 // compensated like the products above (the reads bound it, not the arithmetic).
 // Takes the place of the tensor-core combination there, which fills 64 outputs
-// (n = 1,147,323, 100 rows, one output: 276 us there, 82 us here).
-template <int KB>
+// (n = 1,147,323, 100 rows, one output: 276 us there, 82 us here).  R groups of
+// 256 / R threads share the rows of the same columns where one group would leave
+// SMs idle (whole apply, n = 24,113, 78 rows: 61 us with R = 1, 39 us with 8; n =
+// 170,000, 90 rows: 88 us and 64 us).
+template <int KB, int R>
 __global__ void __launch_bounds__(256) combine_thin_kernel(const float *__restrict__ A1, const float *__restrict__ A2, int k1,
                                                            int ktot, long long lda, const float *__restrict__ coef,
                                                            long long n, float *__restrict__ out, long long ldo,
                                                            const float *__restrict__ dw, const float *__restrict__ Xc,
                                                            long long ldx, float beta)
 {
-    const long long i0 = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
-    if (i0 >= n) return;
+    constexpr int C = 256 / R;                           // threads along the columns
+    const int tx = R == 1 ? threadIdx.x : threadIdx.x % C, ty = R == 1 ? 0 : threadIdx.x / C;
+    const long long i0 = 4 * (blockIdx.x * (long long)C + tx);
+    const bool on = i0 < n;
+    if (R == 1 && !on) return;
+    const int per = (ktot + R - 1) / R, a0 = R == 1 ? 0 : ty * per, a1 = R == 1 ? ktot : on ? min(ktot, (ty + 1) * per) : 0;
     float hi[KB][4], lo[KB][4];
 #pragma unroll
     for (int b = 0; b < KB; ++b)
@@ -325,15 +332,33 @@ __global__ void __launch_bounds__(256) combine_thin_kernel(const float *__restri
             dot2_term(c, v.w, hi[b][3], lo[b][3]);
         }
     };
-    int a = 0;
-    for (; a + 8 <= ktot; a += 8) {
+    int a = a0;
+    for (; a + 8 <= a1; a += 8) {
         float4 v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) v[u] = __ldcs(reinterpret_cast<const float4 *>(row(a + u)));
 #pragma unroll
         for (int u = 0; u < 8; ++u) add(a + u, v[u]);
     }
-    for (; a < ktot; ++a) add(a, __ldcs(reinterpret_cast<const float4 *>(row(a))));
+    for (; a < a1; ++a) add(a, __ldcs(reinterpret_cast<const float4 *>(row(a))));
+    if constexpr (R > 1) {
+        __shared__ float2 sums[KB * 4][256];
+#pragma unroll
+        for (int b = 0; b < KB; ++b)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sums[b * 4 + e][threadIdx.x] = make_float2(hi[b][e], lo[b][e]);
+        __syncthreads();
+        if (ty > 0) return;
+        for (int g = 1; g < R; ++g)
+#pragma unroll
+            for (int b = 0; b < KB; ++b)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 o = sums[b * 4 + e][g * C + tx];
+                    merge_pair(hi[b][e], lo[b][e], o.x, o.y);
+                }
+    }
+    if (!on) return;
 #pragma unroll
     for (int b = 0; b < KB; ++b)
 #pragma unroll
@@ -1281,9 +1306,10 @@ int thin_product(gbfwi_bfgs *h, const float *A1, const float *A2, int k1, int ro
 {
     const long long nc = thin_chunks(h->n);
     if ((size_t)nc * rows * p > h->part.bytes / sizeof(double)) return GBFWI_EINVAL;
-    // about four CTAs an SM: a group takes all rows when the chunks alone give that
+    // about four CTAs an SM: a group takes all rows when the chunks alone give that,
+    // and at least the eight that are reduced together (fewer would be computed with zeros)
     const long long want = std::max<long long>(1, 4 * 152 / nc);
-    const int group = std::min(128, (int)std::max<long long>(1, (rows + want - 1) / want));
+    const int group = std::min(128, (int)std::max<long long>(8, (rows + want - 1) / want));
     const dim3 grid((unsigned)nc, (unsigned)((rows + group - 1) / group));
     const size_t smem = (size_t)group * p * 8 * sizeof(double);
     if (p == 1)
@@ -1327,11 +1353,11 @@ int combine(gbfwi_bfgs *h, const float *A1, const float *A2, int k1, int ktot, c
 {
     const long long n = h->n, ld = h->ld;
     if (ktot >= 1 && nc <= 2) {
-        const unsigned g = (unsigned)((n + 1023) / 1024);
-        if (nc == 1)
-            combine_thin_kernel<1><<<g, 256, 0, s>>>(A1, A2, k1, ktot, ld, coef, n, out, ldo, dw, Xc, ldx, beta);
-        else
-            combine_thin_kernel<2><<<g, 256, 0, s>>>(A1, A2, k1, ktot, ld, coef, n, out, ldo, dw, Xc, ldx, beta);
+        const bool wide = (n + 1023) / 1024 >= 4 * 152;      // the columns alone give an SM four CTAs
+        const unsigned g = (unsigned)(wide ? (n + 1023) / 1024 : (n + 127) / 128);
+        auto kern = nc == 1 ? (wide ? combine_thin_kernel<1, 1> : combine_thin_kernel<1, 8>)
+                            : (wide ? combine_thin_kernel<2, 1> : combine_thin_kernel<2, 8>);
+        kern<<<g, 256, 0, s>>>(A1, A2, k1, ktot, ld, coef, n, out, ldo, dw, Xc, ldx, beta);
         GB_LAUNCHED();
         return GBFWI_OK;
     }
