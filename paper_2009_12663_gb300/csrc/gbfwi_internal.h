@@ -291,10 +291,11 @@ int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf
 // Time integrals of the preconditioners from stored levels, B shots (sem_integrals.cu): w, a
 // the field (levels 0 .. nt + 1) and the acceleration that made each level (slots 2 .. nt + 1);
 // u null: integrals of w alone (P1, P3), else with the field u backwards in time (P2, P4).
-// acc [B][4][NP]: map 0, and maps 1..3 when strains are asked for; esum: gb_integral_bytes
+// acc [B][4][NP]: map 0, and maps 1..3 when strains are asked for; esums: gb_integral_bytes
+// (EINVAL when it holds less)
 size_t gb_integral_bytes(const gbfwi_mesh *m, int B);
-int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *a, const float2 *u, bool strains, float *esum,
-                      float *acc, cudaStream_t s);
+int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *a, const float2 *u, bool strains,
+                      const DevBuf &esums, float *acc, cudaStream_t s);
 
 int gb_launch_step(int mode, int tile, const StepArgs &a, int nbatch, cudaStream_t s);
 int gb_prepare_step(int mode, int tile);   // set kernel attributes outside any stream capture

@@ -1142,7 +1142,7 @@ static int resident_maps(gbfwi_mesh *m, int nshot, int Bmax, int kind, int tile,
             GB_TRY(adj_range(c, MODE_RCV, 0, nt, w, vh, u, seis, nullptr, 0, 0, acc_levels));
         }
         GB_TRY(gb_time_integrals(m, B, receiver ? w.base : u.base, acc_levels, receiver ? u.base : nullptr, strains,
-                                 m->w_eacc.as<float>(), acc, s));
+                                 m->w_eacc, acc, s));
         acc_reduce<<<grid_for(4 * NP), 256, 0, s>>>(acc, B, 4, NP, tot);
         GB_LAUNCHED();
     }

@@ -26,6 +26,7 @@
 
 #include "gbfwi_internal.h"
 #include "sem_element.h"
+#include "size_rules.h"
 
 using namespace sem;
 
@@ -171,25 +172,19 @@ __global__ void __launch_bounds__(128) mass_integral_kernel(const float2 *__rest
     acc[blockIdx.y * 4 * NP + (long long)iz * pitch + ix] = s;
 }
 
-// time chunks of the strain sums: about ten warps an SM, at least 16 steps each
-int strain_chunks(const gbfwi_mesh *m, int B)
-{
-    const long long warps = ((long long)m->d.nex * m->d.nez + 31) / 32 * B;
-    const long long want = std::max<long long>(1, 152 * 10 / warps);
-    return (int)std::min<long long>({want, std::max(1, m->d.nt / 16), 64});
-}
-
 }  // namespace
 
 size_t gb_integral_bytes(const gbfwi_mesh *m, int B)
 {
-    return (size_t)strain_chunks(m, B) * B * 75 * m->d.nex * m->d.nez * sizeof(float);
+    return sizes::integral_bytes((long long)m->d.nex * m->d.nez, m->d.nt, B);
 }
 
-int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *a, const float2 *u, bool strains, float *esum,
-                      float *acc, cudaStream_t s)
+int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 *a, const float2 *u, bool strains,
+                      const DevBuf &esums, float *acc, cudaStream_t s)
 {
     const int nt = m->d.nt, ne = m->d.nex * m->d.nez;
+    if (strains && esums.bytes < gb_integral_bytes(m, B)) return GBFWI_EINVAL;
+    float *esum = esums.as<float>();
     const long long NP = (long long)m->nz * m->pitch, N = (long long)m->nx * m->nz, lev = B * NP;
     const dim3 gm((unsigned)((N + 127) / 128), (unsigned)B);
     if (u)
@@ -198,7 +193,7 @@ int gb_time_integrals(const gbfwi_mesh *m, int B, const float2 *w, const float2 
         mass_integral_kernel<false><<<gm, 128, 0, s>>>(a, a, lev, NP, m->nx, m->nz, m->pitch, nt, acc);
     GB_LAUNCHED();
     if (!strains) return GBFWI_OK;
-    const int nc = strain_chunks(m, B), steps = (nt + nc - 1) / nc;
+    const int nc = sizes::strain_chunks(ne, nt), steps = (nt + nc - 1) / nc;
     const dim3 gs((unsigned)((ne + 127) / 128), (unsigned)nc, (unsigned)B);
     if (u)
         strain_integral_kernel<true><<<gs, 128, 0, s>>>(w, u, lev, NP, m->pitch, m->d.nex, ne, nt, steps, esum);

@@ -1,0 +1,47 @@
+"""Calls that take their shots in several batches, the last of them smaller,
+against the same shots in other batches."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+import paper_2009_12663_gb300 as gb  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+H, DT = 50.0, 5e-4
+
+
+def mesh(nex, nez, nt, nshot, nrec=29, same=False, **sched):
+    """Shots along the surface, or all at one place."""
+    L = nex * H
+    src = [dict(x=L * (0.5 if same else (i + 0.5) / nshot), z=20.0, type=0, f0=8.0, t0=0.05, amp=1e12) for i in range(nshot)]
+    rec = np.stack([np.linspace(0.0, L, nrec), np.zeros(nrec)], axis=1)
+    m = gb.Mesh(nex, nez, H, DT, nt, src, rec)
+    m.set_schedule(**sched)
+    x, z = (torch.tensor(a, device=DEV) for a in m.node_coords())
+    vp = 2600.0 + 300.0 * torch.sin(x / 900.0) + 0.2 * z
+    m.set_model(*(a.float().contiguous() for a in (2000.0 + 0.01 * x, vp, vp / 1.8)))
+    return m
+
+
+def raw_map(m, ids, kind):
+    raw, B0 = (torch.zeros(3, m.nz, m.nx, device=DEV) for _ in range(2))
+    m.precond_diag(ids, kind, 100.0, 1.0, raw, B0)
+    return raw
+
+
+# Levels of 6 GiB hold three of these shots: batches of 3, .., 1 and 3, 2.  A
+# forward map sums squares, so it is the sum of the shots' own maps (different
+# shots).  A receiver map is the modulus of a sum: of equal shots it is nshot times
+# one shot's.  The chunks of time are those of any batch, so both sides differ by the
+# FP32 additions of the shots (nshot 2^-24) and the products of the maps' finish (8
+# 2^-24 on each side); where a field has only just arrived, by roundings of denormals.
+@pytest.mark.parametrize("nex,nez,nshot,nt,kind", [(126, 46, 13, 1333, 3), (160, 60, 5, 500, 4)])
+def test_map_in_ragged_batches_is_the_sum_of_its_shots(nex, nez, nshot, nt, kind):
+    m = mesh(nex, nez, nt, nshot, same=kind == 4)
+    total = torch.zeros(3, m.nz, m.nx, device=DEV, dtype=torch.float64)
+    whole = raw_map(m, list(range(nshot)), kind).double()   # first: no other call has grown the buffers
+    for i in range(nshot):
+        total += raw_map(m, [i], kind).double()
+    assert whole.abs().max() > 0
+    assert bool(((whole - total).abs() <= (nshot + 16) * 2.0 ** -24 * total + 1e-30 * total.max()).all())
