@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "gbfwi_internal.h"
+#include "size_rules.h"
 
 namespace {
 
@@ -513,11 +514,17 @@ int check_shots(const gbfwi_mesh *m, const int *shot_ids, int nshot)
     return GBFWI_OK;
 }
 
-// the exchange buffer of the resident loop (before any work is queued)
-int reserve_exchange(gbfwi_mesh *m, int mode, int B, long long NP)
+// The exchange buffer of the resident loop for `nshot` shots taken `most` at a
+// time (before any work is queued).  The last batch has a plan of its own, which may take
+// more shots in one launch than that of the others.
+int reserve_exchange(gbfwi_mesh *m, int mode, int nshot, int most, long long NP)
 {
-    ResidentPlan *p = gb_resident_plan(m, mode, B);
-    return p ? m->w_xch.ensure(gb_resident_exchange(*p, B, NP)) : GBFWI_EINVAL;
+    for (int B : {most, sizes::last_batch(nshot, most)}) {
+        const ResidentPlan *p = gb_resident_plan(m, mode, B);
+        if (!p) return GBFWI_EINVAL;
+        GB_TRY(m->w_xch.ensure(gb_resident_exchange(*p, B, NP)));
+    }
+    return GBFWI_OK;
 }
 
 // Shots advanced together by forward runs that keep no history, and whether
@@ -551,7 +558,7 @@ extern "C" int gbfwi_forward(gbfwi_mesh *m, const int *shot_ids, int nshot, floa
     const int Bmax = forward_batch(m, nshot, resident);
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
     const bool dev_out = gb_is_device_ptr(seis);
-    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, Bmax, NP));
+    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, nshot, Bmax, NP));
     GB_TRY(m->w_hist.ensure((size_t)3 * Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
@@ -595,7 +602,7 @@ extern "C" int gbfwi_misfit(gbfwi_mesh *m, const int *shot_ids, int nshot, const
     bool resident = false;
     const int Bmax = forward_batch(m, nshot, resident);
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
-    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, Bmax, NP));
+    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, nshot, Bmax, NP));
     GB_TRY(m->w_hist.ensure((size_t)3 * Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
@@ -851,11 +858,10 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
     const int L = resident ? 1 : std::max(1, std::min(m->sch.streams, nbatch));
     const size_t eacc_shot = (size_t)m->d.nex * m->d.nez * 52 * sizeof(float);
     if (resident) GB_TRY(m->w_eacc.ensure(eacc_shot * Bmax));
-    if (resident)
-        for (int B : {Bmax, nshot - (nbatch - 1) * Bmax}) {
-            GB_TRY(reserve_exchange(m, MODE_FWD, B, NP));
-            GB_TRY(reserve_exchange(m, MODE_ADJ_G, B, NP));
-        }
+    if (resident) {
+        GB_TRY(reserve_exchange(m, MODE_FWD, nshot, Bmax, NP));
+        GB_TRY(reserve_exchange(m, MODE_ADJ_G, nshot, Bmax, NP));
+    }
 
     // lanes: 0 = the mesh's own buffers on the caller's stream, 1.. = extra streams
     while ((int)m->lanes.size() < L - 1) m->lanes.push_back(new gbfwi_mesh::Lane());
@@ -1111,10 +1117,8 @@ static int resident_maps(gbfwi_mesh *m, int nshot, int Bmax, int kind, int tile,
     if (!rc && strains) rc = m->w_eacc.ensure(gb_integral_bytes(m, Bmax));
     if (!rc && receiver) rc = m->w_seis.ensure(seis_shot * Bmax * sizeof(float));
     if (!rc) rc = m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2));
-    for (int B : {Bmax, nshot - (nshot - 1) / Bmax * Bmax}) {
-        if (!rc) rc = reserve_exchange(m, fwd, B, NP);
-        if (!rc && receiver) rc = reserve_exchange(m, MODE_RCV, B, NP);
-    }
+    if (!rc) rc = reserve_exchange(m, fwd, nshot, Bmax, NP);
+    if (!rc && receiver) rc = reserve_exchange(m, MODE_RCV, nshot, Bmax, NP);
     if (rc) {
         for (DevBuf *b : big) b->release();
         return rc;
@@ -1170,8 +1174,7 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     const long long small = kSmallHistory / ((levels + 2) * NP * (long long)sizeof(float2));
     const int Bmax = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
     const bool resident = receiver && gb_resident_plan(m, MODE_FWD, Bmax);
-    if (resident)
-        for (int B : {Bmax, nshot - (nshot - 1) / Bmax * Bmax}) GB_TRY(reserve_exchange(m, MODE_FWD, B, NP));
+    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, nshot, Bmax, NP));
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
     const long long lev = (long long)Bmax * NP;
     const double dt = m->d.dt;

@@ -44,20 +44,14 @@
 #include <climits>
 
 #include "gbfwi_internal.h"
+#include "resident_plan.h"
 #include "sem_element.h"
 #include "sm100.h"
 
+using namespace resident;
 using namespace sem;
 
 namespace {
-
-// What a tile of NT element threads can hold: window cells ((TX+2) (TZ+2)),
-// owned elements and exchanged nodes a thread (limits checked by fits()).
-struct Limits { int cells, owned, halo; };
-constexpr Limits limits_of(int NT)
-{
-    return NT == 64 ? Limits{90, 49, 5} : NT == 128 ? Limits{153, 105, 4} : Limits{220, 162, 4};
-}
 
 template <int NT_, int MODE>
 struct Shape {
@@ -65,15 +59,11 @@ struct Shape {
     static constexpr Limits L = limits_of(NT_);
     static constexpr int NT = NT_;                              // element threads
     static constexpr int PS = L.cells, NO = L.owned;
-    static constexpr int NP = ADJ ? (NO + 31) / 32 * 32 : 0;    // correlation threads (adjoint)
+    static constexpr int NP = corr_threads(NT_, ADJ);           // correlation threads (adjoint)
     static constexpr int THREADS = NT + NP;
-    static constexpr int WIN = 8 * PS;                          // float4 of one window
-    // resident CTAs: as many as shared memory holds
-    static constexpr int MINB = ADJ ? (NT == 64 ? 3 : 1) : (NT == 64 ? 6 : NT == 128 ? 3 : 2);
-    // float4: field window (two in the adjoint), moduli window, 1/M; adjoint:
-    // accelerations [8], strain sums [13] and mass sums [4] of every owned element
-    static constexpr int F4 = (ADJ ? 3 : 2) * WIN + 4 * NT + (ADJ ? 25 * NO : 0);
-    static constexpr size_t bytes = (size_t)F4 * 16 + (size_t)(9 * NT) * sizeof(float2);   // before the Tail
+    static constexpr int WIN = window_f4(NT_);                  // float4 of one window
+    static constexpr int MINB = blocks_per_sm(NT_, ADJ);
+    static constexpr int F4 = head_f4(NT_, ADJ);                // float4 before the exchange inside the tile
 };
 
 struct Word2 { unsigned long long x, z; };
@@ -140,33 +130,6 @@ __device__ __forceinline__ float2 load2(const void *p)
     float2 v;
     asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
     return v;
-}
-
-// Shared memory behind the windows and per-element arrays, in floats (every
-// piece a multiple of 4 floats)
-struct Tail {
-    int edge, ev, vx, xi, ent, sig, inj, grp, rec, recw, recv, send, total;
-};
-__host__ __device__ inline int up4(int v) { return (v + 3) & ~3; }
-__host__ __device__ inline Tail tail_of(bool adj, bool one_tile, int TX, int TZ, int edge_cap, int grp_cap, int ent_cap, int rec_cap)
-{
-    Tail q;
-    int o = 0;
-    auto take = [&](int n) { const int at = o; o += up4(n); return at; };
-    q.edge = take(4 * edge_cap);                  // Stacey factors of the tile's absorbing edges (float4)
-    q.ev = take(adj ? 4 * edge_cap : 0);          // mean velocity and acceleration there (two float2)
-    q.vx = take(2 * (4 * (TX + TZ) + 1));         // velocity of the extra node lines (float2)
-    q.xi = take(4 * (4 * (TX + TZ) + 1));         // their places (int4, see the element threads)
-    q.ent = take(4 * ent_cap);                    // injection entries: (offset x, offset z, weight x, weight z)
-    q.sig = take(4 * ent_cap);                    // their signals, two steps
-    q.inj = take(2 * grp_cap);                    // injected forces (float2)
-    q.grp = take(grp_cap + 1);                    // first entry of every group
-    q.rec = take(4 * rec_cap);                    // recorded receivers: id and the cells of their patch (int, 4 shorts)
-    q.recw = take(25 * rec_cap);                  // their weights
-    q.recv = take(one_tile ? 0 : 2 * (20 * (TX + TZ) + 25));   // nodes to receive and to send (int2: node, window slot)
-    q.send = take(one_tile ? 0 : 2 * (20 * (TX + TZ) + 25));
-    q.total = o;
-    return q;
 }
 
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
@@ -756,12 +719,13 @@ namespace {
 
 using Kernel = void (*)(const ResidentArgs);
 
-struct Variant { int NT, MODE, threads; Kernel fn; size_t bytes; };
+struct Variant { int NT, MODE, threads; Kernel fn; };
 
 template <int NT, int MODE>
-constexpr Variant variant() { 
-    return {NT, MODE, Shape<NT, MODE>::THREADS, sem_resident_kernel<NT, MODE>, Shape<NT, MODE>::bytes};
- }
+constexpr Variant variant()
+{
+    return {NT, MODE, Shape<NT, MODE>::THREADS, sem_resident_kernel<NT, MODE>};
+}
 
 const Variant kVariants[] = {variant<64, MODE_FWD>(),   variant<128, MODE_FWD>(),   variant<192, MODE_FWD>(),
                              variant<64, MODE_RCV>(),   variant<128, MODE_RCV>(),   variant<192, MODE_RCV>(),
@@ -776,13 +740,6 @@ const Variant *find_variant(int NT, int mode)
 
 // the kernel that runs a mode (MODE_RCV's also stores the accelerations)
 int kernel_mode(int mode) { return mode == MODE_FWD_PC ? MODE_RCV : mode; }
-
-bool fits(int NT, int TX, int TZ)
-{
-    const Limits L = limits_of(NT);
-    return (TX + 1) * (TZ + 1) <= NT && (TX + 2) * (TZ + 2) <= L.cells && TX * TZ <= L.owned &&
-           20 * (TX + TZ) + 25 <= L.halo * NT;
-}
 
 // resident CTAs of a variant on the current device (0: none)
 int slots_of(const Variant &v, size_t smem, int *nsm)
@@ -800,66 +757,20 @@ int slots_of(const Variant &v, size_t smem, int *nsm)
     return occ * *nsm;
 }
 
-// edge slots of a tile: the sides it can touch
-int edge_cap(int TX, int TZ, int ntx, int ntz, bool free_top)
-{
-    return (4 * TZ + 1) * (ntx == 1 ? 2 : 1) + (4 * TX + 1) * (ntz == 1 && !free_top ? 2 : 1);
-}
-
-size_t smem_of(const Variant &v, int TX, int TZ, int ntx, int ntz, bool free_top, int grp_cap, int ent_cap, int rec_cap)
-{
-    return v.bytes + sizeof(float) * (size_t)tail_of(v.MODE == MODE_ADJ_G, ntx * ntz == 1, TX, TZ, edge_cap(TX, TZ, ntx, ntz, free_top),
-                                                     grp_cap, ent_cap, rec_cap).total;
-}
-
 }  // namespace
 
-// Plan of the resident loop for `shots` shots in `mode`: the tile whose model
-// time per shot and step is smallest among those of which at least one whole
-// shot is resident at once.  null: the mesh does not fit (the step kernels of
-// sem_step.cu run).
+// Plan of the resident loop for `shots` shots in `mode` (best_tile).  null: the
+// mesh does not fit (the step kernels of sem_step.cu run).
 ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
 {
     if (mode == MODE_ADJ_PC) return nullptr;
     for (ResidentPlan *p : m->plans)
         if (p->mode == mode && p->wanted == shots) return p->NT ? p : nullptr;
-    ResidentPlan best;
-    best.mode = mode;
-    best.wanted = shots;
-    double best_cost = 1e300;
-    const int nex = m->d.nex, nez = m->d.nez;
-    for (const Variant &v : kVariants) {
-        if (v.MODE != kernel_mode(mode)) continue;
-        int nsm = 0, slots = 0;
-        size_t known = 0;                        // shared bytes `slots` was looked up for
-        for (int tx = 1; tx < v.NT; ++tx) {
-            // shapes with equal tile counts differ only in their padding: balance them
-            int tz = std::min(v.NT / (tx + 1) - 1, nez);
-            if (tz < 1 || tx > nex) continue;
-            const int ntx = (nex + tx - 1) / tx, ntz = (nez + tz - 1) / tz;
-            const int TX = (nex + ntx - 1) / ntx, TZ = (nez + ntz - 1) / ntz;
-            if (!fits(v.NT, TX, TZ)) continue;
-            const long long T = (long long)ntx * ntz;
-            const size_t smem = smem_of(v, TX, TZ, ntx, ntz, m->d.free_surface_top, 8, 8, 0);
-            if (smem != known) slots = slots_of(v, smem, &nsm);
-            known = smem;
-            const int cap = (int)std::min<long long>(shots, slots / T);
-            for (int c = 1; c <= cap; ++c) {
-                // a step takes the larger of a warp's latency (with the exchange
-                // between tiles) and the busiest SM's issue time
-                const double warps = ((TX + 1) * (TZ + 1) + 31) / 32 * (double)((c * T + nsm - 1) / nsm);
-                // (us; measured: 4.2 us forward and 5.7 us adjoint a step with one CTA an SM,
-                // 5.3 us forward with two)
-                const double issue = (v.MODE != MODE_ADJ_G ? 0.43 : 0.90) * warps;
-                const double lat = (v.MODE != MODE_ADJ_G ? 2.6 : 3.6) + (T > 1 ? 1.2 : 0.0) + 0.05 * warps;
-                const double cost = ((shots + c - 1) / c) * std::max(issue, lat);
-                if (cost < best_cost * (1 - 1e-9)) {
-                    best_cost = cost;
-                    best.NT = v.NT; best.TX = TX; best.TZ = TZ; best.ntx = ntx; best.ntz = ntz;
-                }
-            }
-        }
-    }
+    const bool adj = kernel_mode(mode) == MODE_ADJ_G;
+    const Tile best = best_tile(m->d.nex, m->d.nez, m->d.free_surface_top, adj, shots, [&](int NT, size_t smem, int &nsm) {
+        const Variant *v = find_variant(NT, kernel_mode(mode));
+        return v ? slots_of(*v, smem, &nsm) : 0;
+    });
     ResidentPlan *p = new ResidentPlan();
     p->mode = mode;
     p->wanted = shots;
@@ -879,7 +790,7 @@ ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
     p->ent_cap = fwd ? p->lists.src_entries_most : p->lists.rec_entries_most;
     p->rec_cap = fwd ? p->lists.recorded_most : 0;
     int nsm = 0;
-    p->smem = smem_of(*v, p->TX, p->TZ, p->ntx, p->ntz, m->d.free_surface_top, p->grp_cap, p->ent_cap, p->rec_cap);
+    p->smem = smem_bytes(best.NT, adj, p->TX, p->TZ, p->ntx, p->ntz, m->d.free_surface_top, p->grp_cap, p->ent_cap, p->rec_cap);
     const int slots = slots_of(*v, p->smem, &nsm);
     p->per_launch = p->grp_cap < 32767 ? slots / (p->ntx * p->ntz) : 0;
     if (p->per_launch < 1) return nullptr;
@@ -895,6 +806,7 @@ int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf
         a.acc_shot_stride % 4 != 0 || ((uintptr_t)a.aout & 31) || ((uintptr_t)a.u0 & 15) || ((uintptr_t)a.out & 31) || ((uintptr_t)a.vh & 15) ||
         ((uintptr_t)a.minv & 15) || ((uintptr_t)a.acc & 15) || ((uintptr_t)a.hist & 31) || ((uintptr_t)a.eacc & 15) || !a.status)
         return GBFWI_EINVAL;
+    if (xch.bytes < gb_resident_exchange(p, nshots, a.fstride)) return GBFWI_EINVAL;
     a.TX = p.TX; a.TZ = p.TZ; a.ntx = p.ntx; a.ntz = p.ntz;
     a.ntiles = p.ntx * p.ntz;
     a.edge_cap = edge_cap(p.TX, p.TZ, p.ntx, p.ntz, a.free_top);
@@ -938,5 +850,5 @@ int gb_assemble_strain(const gbfwi_mesh *m, const float *eacc, int B, float *acc
 
 size_t gb_resident_exchange(const ResidentPlan &p, int nshots, long long NP)
 {
-    return p.ntx * p.ntz > 1 ? (size_t)32 * std::min(nshots, p.per_launch) * NP : 16;
+    return exchange_bytes(p.ntx * p.ntz, nshots, p.per_launch, NP);
 }

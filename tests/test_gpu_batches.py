@@ -45,3 +45,21 @@ def test_map_in_ragged_batches_is_the_sum_of_its_shots(nex, nez, nshot, nt, kind
         total += raw_map(m, [i], kind).double()
     assert whole.abs().max() > 0
     assert bool(((whole - total).abs() <= (nshot + 16) * 2.0 ** -24 * total + 1e-30 * total.max()).all())
+
+
+# the last batch (19, 13 and 20 shots of 43, 37 and 44) takes more of them in one launch
+# than the first of 24; 50 shots of a mesh of one tile
+@pytest.mark.parametrize("nex,nez,nshot,spl", [(280, 10, 43, 24), (253, 24, 37, 24), (110, 37, 44, 24), (14, 8, 50, 3)])
+def test_records_of_ragged_batches_are_those_of_single_shots(nex, nez, nshot, spl):
+    nt, ids = 40, list(range(nshot))
+    m = mesh(nex, nez, nt, nshot, shots_per_launch=spl)
+    seis = torch.zeros(nshot, 29, 2, nt, device=DEV)
+    obs = torch.zeros_like(seis)
+    f = m.misfit(ids, obs)                               # first: no other call has grown the buffers
+    m.forward(ids, seis)
+    one, each = torch.zeros(1, 29, 2, nt, device=DEV), 0.0
+    for i in ids:
+        m.forward([i], one)
+        assert torch.equal(one[0], seis[i]), i           # the fields do not depend on the batch
+        each += m.misfit([i], obs[:1])
+    assert f > 0 and abs(f - each) <= 1e-13 * nshot * f   # FP64 sums of the shots' misfits

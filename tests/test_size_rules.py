@@ -7,10 +7,10 @@ import subprocess
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2009_12663_gb300", "csrc")
 
 
-def run(tmp_path, body):
+def run(tmp_path, body, head=""):
     src = tmp_path / "rules.cpp"
-    src.write_text("#include <cstdio>\n#include <initializer_list>\n#include \"size_rules.h\"\nusing namespace sizes;\n"
-                   "int main() {\n  int bad = 0;\n" + body + "  return bad != 0;\n}\n")
+    src.write_text("#include <cstdio>\n#include <initializer_list>\n#include \"resident_plan.h\"\n#include \"size_rules.h\"\n"
+                   "using namespace resident;\nusing namespace sizes;\n" + head + "int main() {\n  int bad = 0;\n" + body + "  return bad != 0;\n}\n")
     exe = str(tmp_path / "rules")
     subprocess.check_call(["g++", "-std=c++17", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", exe])
     r = subprocess.run([exe], capture_output=True, text=True)
@@ -32,3 +32,53 @@ def test_strain_sums_of_every_batch_fit_the_buffer_of_the_first(tmp_path):
             }
           }
 """)
+
+
+# an SM of 228 KB shared memory (1 KB a CTA taken by the system), 152 of them; registers let
+# at least the CTAs of the launch bounds in, and shared memory decides here
+PLAN = r"""
+struct Plan { Tile t; int per_launch; };
+static int slots(int NT, bool adj, size_t smem) {
+  if (smem > 227 * 1024 - 64) return 0;
+  return 152 * (int)std::min<size_t>(228 * 1024 / (smem + 1024), 2048 / (NT + corr_threads(NT, adj)));
+}
+static Plan plan(int nex, int nez, bool adj, int shots, int injected = 4) {
+  const Tile t = best_tile(nex, nez, true, adj, shots, [&](int NT, size_t smem, int &nsm) { nsm = 152; return slots(NT, adj, smem); });
+  if (!t.NT) return {t, 0};
+  const size_t smem = smem_bytes(t.NT, adj, t.TX, t.TZ, t.ntx, t.ntz, true, injected, injected, adj ? 0 : 8);
+  return {t, slots(t.NT, adj, smem) / (t.ntx * t.ntz)};
+}
+"""
+
+
+def test_exchange_of_every_batch_fits_what_both_batch_sizes_reserve(tmp_path):
+    """Forward runs: the last batch has a plan of its own, which may take more
+    shots a launch than the first batch's (the grid holds such calls), so both
+    count in what is reserved."""
+    run(tmp_path, r"""
+  int wider = 0;
+  for (auto [nex, nez] : {std::pair{5, 3}, {40, 20}, {57, 46}, {106, 40}, {110, 37}, {253, 24}, {280, 10}, {340, 70}})
+    for (int spl : {1, 8, 24})
+      for (int nshot : {1, 5, 13, 24, 37, 43, 44, 61}) {
+        const Plan all = plan(nex, nez, false, nshot);
+        if (all.per_launch < 1) continue;
+        const int most = std::min(nshot, std::max(all.per_launch, spl)), last = last_batch(nshot, most);
+        const long long nodes = (4LL * nez + 1) * (4 * nex + 4);
+        size_t reserved = 0, first = 0;
+        for (int B : {most, last}) {
+          const Plan p = plan(nex, nez, false, B);
+          reserved = std::max(reserved, exchange_bytes(p.t.ntx * p.t.ntz, B, p.per_launch, nodes));
+          if (B == most) first = reserved;
+        }
+        for (int i0 = 0; i0 < nshot; i0 += most) {
+          const int B = std::min(most, nshot - i0);
+          const Plan p = plan(nex, nez, false, B);
+          for (int s0 = 0; s0 < B; s0 += p.per_launch) {      // the launches of a batch, 32 bytes a node and shot
+            const size_t used = p.t.ntx * p.t.ntz > 1 ? 32 * (size_t)std::min(p.per_launch, B - s0) * nodes : 0;
+            if (used > reserved) { std::printf("%d x %d, %d shots by %d\n", nex, nez, nshot, most); ++bad; }
+            if (used > first) ++wider;
+          }
+        }
+      }
+  if (!wider) { std::printf("no last batch needs more than the first\n"); ++bad; }
+""", "#include <utility>\n" + PLAN)
