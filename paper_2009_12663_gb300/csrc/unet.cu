@@ -38,6 +38,9 @@
 #include <vector>
 
 #include "gbfwi_internal.h"
+#include "size_rules.h"
+
+using namespace sizes;
 
 typedef __nv_bfloat16 bf16;
 
@@ -47,7 +50,7 @@ namespace {
 // BF16 GEMM on the tensor cores
 // ---------------------------------------------------------------------------
 
-constexpr int GBK = 32;        // k extent of a staged tile
+constexpr int GBK = sizes::kGemmBK;   // k extent of a staged tile
 constexpr int GPAD = 8;        // bf16 padding per shared row (ldmatrix rows on distinct banks)
 constexpr int GTHREADS = 256;  // 8 warps, each owning a 32 x 32 block of C
 constexpr int GSTAGES = 3;     // cp.async pipeline depth (tiles in flight + 1)
@@ -949,10 +952,6 @@ namespace {
 
 long long npix(const gbfwi_unet *n, int l) { return (long long)(n->d.height >> l) * (n->d.width >> l); }
 
-// tile extents by output rows
-constexpr int bm_of(int M) { return M <= 32 ? 32 : (M <= 64 ? 64 : 128); }
-constexpr int bn_of(int BM) { return 256 * 32 / BM; }
-
 template <class K>
 int allow_smem(K kern, size_t smem, bool (&done)[64])
 {
@@ -968,7 +967,7 @@ int allow_smem(K kern, size_t smem, bool (&done)[64])
 template <int BM, bool AK, bool BK, bool GA>
 int launch_gemm(const GemmArgs &g, int samples, cudaStream_t s)
 {
-    constexpr int BN = bn_of(BM);
+    constexpr int BN = gemm_bn(BM);
     dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), (unsigned)(g.splits * samples));
     using T = GemmTile<BM, BN, AK, BK>;
     constexpr size_t smem = (size_t)kStages<GA> * (T::AE + T::BE) * sizeof(bf16);
@@ -986,25 +985,6 @@ int launch_gemm_bm(const GemmArgs &g, int samples, bool a_km, bool b_nk, cudaStr
         return b_nk ? launch_gemm<BM, false, true, true>(g, samples, s) : launch_gemm<BM, false, false, true>(g, samples, s);
     if (a_km) return b_nk ? GBFWI_EINVAL : launch_gemm<BM, true, false, false>(g, samples, s);
     return b_nk ? launch_gemm<BM, false, true, false>(g, samples, s) : launch_gemm<BM, false, false, false>(g, samples, s);
-}
-
-// k range of a split of an (M x N) output over K: enough splits to fill the
-// SMs, each at least four tiles long.  The rule fixes where the sums are cut, so
-// it depends on one sample's shape only.
-int split_chunk(int M, int N, int K, long long part_cap, int *splits_out)
-{
-    const int BM = bm_of(M), BN = bn_of(BM);
-    const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
-    int splits = 1;
-    if (tiles < 2 * 152 && K >= 8 * GBK) {
-        long long want = (2 * 152 + tiles - 1) / tiles;
-        want = std::min<long long>(want, K / (4 * GBK));
-        want = std::min<long long>(want, std::max<long long>(1, part_cap / ((long long)M * N)));
-        splits = (int)std::max<long long>(1, want);
-    }
-    const int kchunk = (int)(((K + splits - 1) / splits + GBK - 1) / GBK * GBK);
-    *splits_out = (K + kchunk - 1) / kchunk;
-    return kchunk;
 }
 
 // Sum of the split partials [sample][split][M][N] in the scratch with the GEMM's
@@ -1036,14 +1016,15 @@ int gemm(gbfwi_unet *net, int samples, Operand A, bool a_km, Operand B, const Co
         return GBFWI_EINVAL;
     if (!src && (B.ld % 8 || ((uintptr_t)B.p & 15))) return GBFWI_EINVAL;
     if (src && (src->W % 8 || ((uintptr_t)src->s1 & 15) || ((uintptr_t)src->s2 & 15))) return GBFWI_EINVAL;
-    const int BM = bm_of(M);
+    const int BM = gemm_bm(M);
     int splits = 1;
     const int kchunk = split_chunk(M, N, K, net->part_cap, &splits);
-    const bool partial = splits > 1 || (accumulate && samples > 1);
-    // samples whose partials fit the scratch together
-    const int fit = partial ? (int)std::max<long long>(1, net->part_cap / ((long long)M * N * splits)) : samples;
+    // samples whose partials fit the scratch together (a wide layer's gradient alone is
+    // larger than it: one sample after another then, each added to the output)
+    const int fit = gemm_samples((long long)M * N, splits, samples, accumulate, net->part_cap);
     for (int b0 = 0; b0 < samples; b0 += fit) {
         const int nb = std::min(fit, samples - b0);
+        const bool partial = gemm_partial(splits, nb, accumulate);
         GemmArgs g{};
         g.A = A.p + b0 * A.bs; g.lda = A.ld; g.abs_ = A.bs;
         if (src) {
@@ -1085,7 +1066,7 @@ int gemm(gbfwi_unet *net, int samples, Operand A, bool a_km, Operand B, const Co
 template <int BM>
 int launch_dx(const GemmArgs &g, int samples, cudaStream_t s)
 {
-    constexpr int BN = bn_of(BM);
+    constexpr int BN = gemm_bn(BM);
     using T = GemmTile<BM, BN, true, false>;
     constexpr size_t smem = (size_t)GSTAGES * (T::AE + T::BE) * sizeof(bf16);
     static bool attr_done[64] = {};
@@ -1133,10 +1114,10 @@ int conv_bwd(gbfwi_unet *n, int nb, const UnetLayer &L, const ConvSrc &src, cons
     g.kchunk = split_chunk(L.kcp, (int)P, L.coutp, n->part_cap, &splits);
     g.Cf = dX; g.ldc = P; g.cbs = L.cin * P;
     g.src = ConvSrc{G, G, L.cout, 0, 0, src.H, src.W, L.cout * P, 0};
-    const int BM = bm_of(L.cin);
+    const int BM = gemm_bm(L.cin);
     // a CTA per tap while the tiles alone leave most SMs idle (48 tiles: 38 us, 27 us
     // with the sum; 128 tiles: 21 us, 36 us with it)
-    const long long tiles = (P + bn_of(BM) - 1) / bn_of(BM) * ((L.cin + BM - 1) / BM) * nb, taps = 9LL * nb * L.cin * P;
+    const long long tiles = (P + gemm_bn(BM) - 1) / gemm_bn(BM) * ((L.cin + BM - 1) / BM) * nb, taps = 9LL * nb * L.cin * P;
     if (tiles < 64 && taps <= n->part_cap) {
         g.partial = 1;
         g.Cf = n->part.as<float>();

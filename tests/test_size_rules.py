@@ -82,3 +82,42 @@ def test_exchange_of_every_batch_fits_what_both_batch_sizes_reserve(tmp_path):
       }
   if (!wider) { std::printf("no last batch needs more than the first\n"); ++bad; }
 """, "#include <utility>\n" + PLAN)
+
+
+def test_partials_of_unet_products_fit_the_scratch(tmp_path):
+    """Every 3x3 layer's forward product and weight gradient over the networks
+    the library accepts, alone and in batches: partials within the scratch, which
+    some layers' weight gradients do not fit even alone."""
+    run(tmp_path, r"""
+  const long long cap = 32LL << 20;
+  int wide = 0;
+  for (int levels = 1; levels <= 6; ++levels)
+    for (int base : {8, 32, 64, 96})
+      for (int unit : {1, 2, 8})                               // coarsest level of unit x 8 unit pixels
+        for (int samples : {1, 2, 5, 64}) {
+          auto check = [&](int M, int N, int K, bool accumulate) {
+            int splits = 0;
+            const int kchunk = split_chunk(M, N, K, cap, &splits);
+            const long long outputs = (long long)M * N;
+            const int fit = gemm_samples(outputs, splits, samples, accumulate, cap);
+            if (accumulate && outputs > cap) ++wide;
+            if (fit < 1 || fit > samples || kchunk % kGemmBK || (long long)kchunk * splits < K) ++bad;
+            for (int b0 = 0; b0 < samples; b0 += fit) {
+              const int nb = std::min(fit, samples - b0);
+              if (gemm_partial(splits, nb, accumulate) ? nb * splits * outputs > cap : accumulate && nb > 1) {
+                std::printf("levels %d base %d: %d x %d over %d, %d samples\n", levels, base, M, N, K, nb);
+                ++bad;
+              }
+            }
+          };
+          for (int l = 0; l < levels; ++l) {
+            const int ch = base << l, below = l ? ch / 2 : 5, px = (unit << (levels - 1 - l)) * ((8 * unit) << (levels - 1 - l));
+            for (int cin : {below, ch, 3 * ch}) {              // encoder, second convolutions, decoder
+              const int kcp = (9 * cin + 7) / 8 * 8;
+              check(ch, px, kcp, false);
+              check(ch, kcp, px, true);
+            }
+          }
+        }
+  if (!wide) { std::printf("no layer is wider than the scratch\n"); ++bad; }
+""")
