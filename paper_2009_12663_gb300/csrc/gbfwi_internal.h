@@ -3,7 +3,9 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <map>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "gbfwi.h"
@@ -114,15 +116,14 @@ struct TileLists {
 };
 
 // Tile of the resident time loop (sem_resident.cu) for one kind of pass and
-// number of shots; its injection groups pack the node as thread * 32 + q, q =
-// j * 5 + i the node of the thread's element that owns it.
+// number of shots; the injection groups of its lists pack the node as thread * 32 +
+// q, q = j * 5 + i the node of the thread's element that owns it.
 struct ResidentPlan {
-    int mode = 0, wanted = 0;
     int NT = 0, TX = 0, TZ = 0, ntx = 0, ntz = 0;   // NT 0: the mesh does not fit
     int per_launch = 0;                              // shots of which every tile is resident at once
     int grp_cap = 0, ent_cap = 0, rec_cap = 0;       // most injected nodes, their entries and receivers of a tile
     size_t smem = 0;
-    TileLists lists;
+    const TileLists *lists = nullptr;
 };
 
 // ---------------------------------------------------------------------------
@@ -175,7 +176,11 @@ struct gbfwi_mesh {
         ~Lane() { if (st) cudaStreamDestroy(st); }
     };
     std::vector<Lane *> lanes;
-    std::vector<ResidentPlan *> plans;  // of the resident time loop
+    // plans of the resident time loop by mode and number of shots, and the lists of
+    // their tile shapes (TX, TZ): kept with the mesh, so that a plan or a list in use is
+    // never freed.  A plan is a few numbers; the shapes are at most a few hundred.
+    std::map<std::pair<int, int>, ResidentPlan> plans;
+    std::map<std::pair<int, int>, TileLists> plan_lists;
     DevBuf w_eacc;                      // its strain sums by element
     DevBuf w_xch;                       // its exchange of node lines between tiles
     DevBuf w_chk;                       // model checks (and a model given on the host)
@@ -281,12 +286,12 @@ struct ResidentArgs {
     int *status;
 };
 
-ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots);
+const ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots);
 // acc components 0 and 1 of B shots from the elements' strain sums
 int gb_assemble_strain(const gbfwi_mesh *m, const float *eacc, int B, float *acc, long long acc_shot_stride, long long cs,
                        cudaStream_t s);
 size_t gb_resident_exchange(const ResidentPlan &p, int nshots, long long NP);   // bytes of the exchange buffer
-int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf &xch, cudaStream_t s);
+int gb_launch_resident(const ResidentPlan &p, int mode, ResidentArgs a, int nshots, DevBuf &xch, cudaStream_t s);
 
 // Time integrals of the preconditioners from stored levels, B shots (sem_integrals.cu): w, a
 // the field (levels 0 .. nt + 1) and the acceleration that made each level (slots 2 .. nt + 1);

@@ -36,7 +36,6 @@ gbfwi_mesh::~gbfwi_mesh()
     for (auto &g : graphs) cudaGraphExecDestroy(g.exec);
     if (cap_stream) cudaStreamDestroy(cap_stream);
     for (Lane *l : lanes) delete l;
-    for (ResidentPlan *p : plans) delete p;
 }
 
 extern "C" int gbfwi_enable_timing(gbfwi_mesh *m, int on)

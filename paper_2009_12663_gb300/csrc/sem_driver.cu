@@ -99,15 +99,15 @@ void resident_args(ResidentArgs &r, const StepArgs &a, const Ctx &c, int n0, int
 
 int run_resident(const Ctx &c, int mode, ResidentArgs &r)
 {
-    ResidentPlan *p = gb_resident_plan(c.m, mode, c.B);
+    const ResidentPlan *p = gb_resident_plan(c.m, mode, c.B);
     if (!p) return GBFWI_EINVAL;
     const bool fwd = mode == MODE_FWD || mode == MODE_FWD_PC;
-    r.gptr = (fwd ? p->lists.src_gptr : p->lists.rec_gptr).as<int>();
-    r.groups = (fwd ? p->lists.src_groups : p->lists.rec_groups).as<InjGroup>();
-    r.entries = (fwd ? p->lists.src_entries : p->lists.rec_entries).as<InjEntry>();
-    r.rec_tptr = p->lists.rec_tptr.as<int>();
-    r.rec_list = p->lists.rec_list.as<int>();
-    return gb_launch_resident(*p, r, c.B, c.m->w_xch, c.s);
+    r.gptr = (fwd ? p->lists->src_gptr : p->lists->rec_gptr).as<int>();
+    r.groups = (fwd ? p->lists->src_groups : p->lists->rec_groups).as<InjGroup>();
+    r.entries = (fwd ? p->lists->src_entries : p->lists->rec_entries).as<InjEntry>();
+    r.rec_tptr = p->lists->rec_tptr.as<int>();
+    r.rec_list = p->lists->rec_list.as<int>();
+    return gb_launch_resident(*p, mode, r, c.B, c.m->w_xch, c.s);
 }
 
 constexpr int kNoLevel = INT_MAX;
@@ -532,7 +532,7 @@ int reserve_exchange(gbfwi_mesh *m, int mode, int nshot, int most, long long NP)
 // at once (three levels and a velocity each), the step kernels the schedule's.
 int forward_batch(gbfwi_mesh *m, int nshot, bool &resident)
 {
-    ResidentPlan *p = gb_resident_plan(m, MODE_FWD, nshot);
+    const ResidentPlan *p = gb_resident_plan(m, MODE_FWD, nshot);
     resident = p != nullptr;
     return std::min(nshot, p ? std::max(p->per_launch, m->sch.shots_per_launch) : m->sch.shots_per_launch);
 }

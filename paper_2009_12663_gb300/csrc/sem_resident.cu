@@ -760,48 +760,42 @@ int slots_of(const Variant &v, size_t smem, int *nsm)
 }  // namespace
 
 // Plan of the resident loop for `shots` shots in `mode` (best_tile).  null: the
-// mesh does not fit (the step kernels of sem_step.cu run).
-ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
+// mesh does not fit (the step kernels of sem_step.cu run), or the lists of the tile
+// could not be allocated this time (asked again by the next call).
+const ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
 {
     if (mode == MODE_ADJ_PC) return nullptr;
-    for (ResidentPlan *p : m->plans)
-        if (p->mode == mode && p->wanted == shots) return p->NT ? p : nullptr;
+    const auto known = m->plans.find({mode, shots});
+    if (known != m->plans.end()) return known->second.NT ? &known->second : nullptr;
     const bool adj = kernel_mode(mode) == MODE_ADJ_G;
     const Tile best = best_tile(m->d.nex, m->d.nez, m->d.free_surface_top, adj, shots, [&](int NT, size_t smem, int &nsm) {
         const Variant *v = find_variant(NT, kernel_mode(mode));
         return v ? slots_of(*v, smem, &nsm) : 0;
     });
-    ResidentPlan *p = new ResidentPlan();
-    p->mode = mode;
-    p->wanted = shots;
-    if (m->plans.size() >= 64) {                 // bounded cache
-        cudaDeviceSynchronize();                 // its lists may be in use
-        delete m->plans.front();
-        m->plans.erase(m->plans.begin());
+    ResidentPlan p;
+    if (best.NT) {
+        TileLists &lists = m->plan_lists[{best.TX, best.TZ}];
+        if (!lists.built && gb_build_lists(m, best.TX, best.TZ, true, lists) != GBFWI_OK) return nullptr;
+        // with the real injection lists: how many shots fit one launch
+        const bool fwd = mode == MODE_FWD || mode == MODE_FWD_PC;
+        p.TX = best.TX; p.TZ = best.TZ; p.ntx = best.ntx; p.ntz = best.ntz;
+        p.lists = &lists;
+        p.grp_cap = fwd ? lists.src_most : lists.rec_most;
+        p.ent_cap = fwd ? lists.src_entries_most : lists.rec_entries_most;
+        p.rec_cap = fwd ? lists.recorded_most : 0;
+        p.smem = smem_bytes(best.NT, adj, p.TX, p.TZ, p.ntx, p.ntz, m->d.free_surface_top, p.grp_cap, p.ent_cap, p.rec_cap);
+        int nsm = 0;
+        const int slots = slots_of(*find_variant(best.NT, kernel_mode(mode)), p.smem, &nsm);
+        p.per_launch = p.grp_cap < 32767 ? std::min(slots / (p.ntx * p.ntz), 60000) : 0;
+        if (p.per_launch >= 1) p.NT = best.NT;
     }
-    m->plans.push_back(p);
-    if (!best.NT) return nullptr;
-    p->TX = best.TX; p->TZ = best.TZ; p->ntx = best.ntx; p->ntz = best.ntz;
-    if (gb_build_lists(m, p->TX, p->TZ, true, p->lists) != GBFWI_OK) return nullptr;
-    // with the real injection lists: how many shots fit one launch
-    const Variant *v = find_variant(best.NT, kernel_mode(mode));
-    const bool fwd = mode == MODE_FWD || mode == MODE_FWD_PC;
-    p->grp_cap = fwd ? p->lists.src_most : p->lists.rec_most;
-    p->ent_cap = fwd ? p->lists.src_entries_most : p->lists.rec_entries_most;
-    p->rec_cap = fwd ? p->lists.recorded_most : 0;
-    int nsm = 0;
-    p->smem = smem_bytes(best.NT, adj, p->TX, p->TZ, p->ntx, p->ntz, m->d.free_surface_top, p->grp_cap, p->ent_cap, p->rec_cap);
-    const int slots = slots_of(*v, p->smem, &nsm);
-    p->per_launch = p->grp_cap < 32767 ? slots / (p->ntx * p->ntz) : 0;
-    if (p->per_launch < 1) return nullptr;
-    p->per_launch = std::min(p->per_launch, 60000);
-    p->NT = best.NT;
-    return p;
+    const ResidentPlan &kept = m->plans[{mode, shots}] = p;
+    return kept.NT ? &kept : nullptr;
 }
 
-int gb_launch_resident(const ResidentPlan &p, ResidentArgs a, int nshots, DevBuf &xch, cudaStream_t s)
+int gb_launch_resident(const ResidentPlan &p, int mode, ResidentArgs a, int nshots, DevBuf &xch, cudaStream_t s)
 {
-    const Variant *v = find_variant(p.NT, kernel_mode(p.mode));
+    const Variant *v = find_variant(p.NT, kernel_mode(mode));
     if (!v || a.pitch % 4 != 0 || a.fstride % 4 != 0 || a.lev % 4 != 0 || a.acc_comp_stride % 4 != 0 ||
         a.acc_shot_stride % 4 != 0 || ((uintptr_t)a.aout & 31) || ((uintptr_t)a.u0 & 15) || ((uintptr_t)a.out & 31) || ((uintptr_t)a.vh & 15) ||
         ((uintptr_t)a.minv & 15) || ((uintptr_t)a.acc & 15) || ((uintptr_t)a.hist & 31) || ((uintptr_t)a.eacc & 15) || !a.status)

@@ -63,3 +63,18 @@ def test_records_of_ragged_batches_are_those_of_single_shots(nex, nez, nshot, sp
         assert torch.equal(one[0], seis[i]), i           # the fields do not depend on the batch
         each += m.misfit([i], obs[:1])
     assert f > 0 and abs(f - each) <= 1e-13 * nshot * f   # FP64 sums of the shots' misfits
+
+
+def test_many_shot_counts_on_one_mesh():
+    """A study with changing minibatches: every number of shots and kind of pass
+    keeps its plan, and none loses it to the others."""
+    nshot, nt = 40, 30
+    m = mesh(23, 19, nt, nshot, shots_per_launch=2)
+    seis, again = (torch.zeros(nshot, 29, 2, nt, device=DEV) for _ in range(2))
+    m.forward(list(range(nshot)), seis)
+    first = raw_map(m, [0, 1], 2)
+    for k in range(1, nshot + 1):
+        m.forward(list(range(k)), again[:k])
+        assert torch.equal(again[:k], seis[:k]), k
+        raw_map(m, list(range(k)), 1 + k % 2)
+    assert torch.equal(raw_map(m, [0, 1], 2), first)
