@@ -179,6 +179,7 @@ int adj_range(const Ctx &c, int mode, int j0, int j1, const Levels &w, float2 *w
     }
     if (c.resident && mode == MODE_ADJ_G) {
         ResidentArgs r;
+        if (hist.lev != w.lev) return GBFWI_EINVAL;            // the kernel has one stride for both
         resident_args(r, a, c, j0, j1, w, j1 < nt ? j1 : kNoLevel);
         r.hist = hist.base;
         r.hist_k0 = hist.k0;
@@ -649,8 +650,9 @@ extern "C" int gbfwi_misfit(gbfwi_mesh *m, const int *shot_ids, int nshot, const
 
 namespace {
 
+// buffers for the largest batch; a batch of B shots lays its levels out B * NP apart
 struct BatchHist {
-    Levels full;               // ckpt == 0
+    float2 *full = nullptr;    // ckpt == 0: nt + 2 levels
     float2 *ring = nullptr;    // ckpt > 0: 3-slot ring for the forward pass
     float2 *seg = nullptr;     // ckpt > 0: C + 2 slots
     float2 *snap = nullptr;    // ckpt > 0: [nseg][3][B][NP]: u_{sC}, u_{sC+1}, vh_{sC}
@@ -686,7 +688,7 @@ int alloc_hist(gbfwi_mesh *m, const LaneRef &L, int B, int ckpt, long long NP, B
     long long lev = (long long)B * NP;
     if (ckpt <= 0 || ckpt >= nt) {
         GB_TRY(L.hist->ensure((size_t)(nt + 2) * lev * sizeof(float2)));
-        h.full = Levels{L.hist->as<float2>(), lev, 0, false};
+        h.full = L.hist->as<float2>();
         h.C = 0;
     } else {
         h.C = ckpt;
@@ -719,8 +721,8 @@ int forward_pass(const Ctx &c, BatchHist &h, float *seis)
     float2 *vh = h.vh;
     GB_CUDA(cudaMemsetAsync(vh, 0, lev * sizeof(float2), c.s));
     if (h.C == 0) {
-        GB_CUDA(cudaMemsetAsync(h.full.base, 0, 2 * lev * sizeof(float2), c.s));
-        return fwd_range(c, MODE_FWD, 0, nt, h.full, 0, vh, seis, nullptr, 0, 0);
+        GB_CUDA(cudaMemsetAsync(h.full, 0, 2 * lev * sizeof(float2), c.s));
+        return fwd_range(c, MODE_FWD, 0, nt, Levels{h.full, lev, 0, false}, 0, vh, seis, nullptr, 0, 0);
     }
     GB_CUDA(cudaMemsetAsync(h.ring, 0, 3 * lev * sizeof(float2), c.s));
     const Levels ring{h.ring, lev, 0, true};
@@ -747,7 +749,7 @@ int adjoint_pass(const Ctx &c, BatchHist &h, int mode, const float *sig, float *
     GB_CUDA(cudaMemsetAsync(h.wring, 0, 3 * lev * sizeof(float2), c.s));
     GB_CUDA(cudaMemsetAsync(wh, 0, lev * sizeof(float2), c.s));
     if (h.C == 0) {
-        return adj_range(c, mode, 0, nt, wring, wh, h.full, sig, acc, acc_shot_stride, acc_comp_stride);
+        return adj_range(c, mode, 0, nt, wring, wh, Levels{h.full, lev, 0, false}, sig, acc, acc_shot_stride, acc_comp_stride);
     }
     for (int sg = h.nseg - 1; sg >= 0; --sg) {
         int n0 = sg * h.C, n1 = std::min(nt, n0 + h.C);

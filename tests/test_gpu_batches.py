@@ -78,3 +78,22 @@ def test_many_shot_counts_on_one_mesh():
         assert torch.equal(again[:k], seis[:k]), k
         raw_map(m, list(range(k)), 1 + k % 2)
     assert torch.equal(raw_map(m, [0, 1], 2), first)
+
+
+# Batches of 10 and 8 (10 and 3), the whole history or checkpoints.  FP32 sums over the shots
+# and in the chain rule: nshot 2^-24 of the shots' moduli, and of each shot's largest
+# entry times nt where its terms cancel; asserted twice that.
+@pytest.mark.parametrize("nshot,spl,ckpt", [(18, 10, 0), (13, 10, 0), (18, 10, 100)])
+def test_gradient_in_ragged_batches_is_the_sum_of_its_shots(nshot, spl, ckpt):
+    nt, ids = 500, list(range(nshot))
+    m = mesh(46, 42, nt, nshot, shots_per_launch=spl, ckpt_every=ckpt)
+    obs = torch.zeros(nshot, 29, 2, nt, device=DEV)
+    grad, one = (torch.zeros(3, m.nz, m.nx, device=DEV) for _ in range(2))
+    f = m.adjoint_gradient(ids, obs, grad)
+    total, size, each = torch.zeros_like(grad).double(), torch.zeros_like(grad).double(), 0.0
+    for i in ids:
+        each += m.adjoint_gradient([i], obs[:1], one)
+        total += one
+        size += one.abs() + nt * one.abs().amax(dim=(1, 2), keepdim=True)
+    assert f > 0 and abs(f - each) <= 1e-13 * nshot * f
+    assert bool(((grad - total).abs() <= 2 * nshot * 2.0 ** -24 * size).all())
