@@ -515,27 +515,40 @@ int check_shots(const gbfwi_mesh *m, const int *shot_ids, int nshot)
     return GBFWI_OK;
 }
 
-// The exchange buffer of the resident loop for `nshot` shots taken `most` at a
-// time (before any work is queued).  The last batch has a plan of its own, which may take
-// more shots in one launch than that of the others.
-int reserve_exchange(gbfwi_mesh *m, int mode, int nshot, int most, long long NP)
+// Shots taken `most` at a time, and whether batches of that size and the last one
+// run as resident loops.  The last batch has plans of its own: it may take more shots in one
+// launch than the others (the exchange buffer is sized for both), or none at all
+// where its tile does not hold the receivers' lists (the step kernels serve it).
+struct Batches {
+    int most = 0, last = 0;
+    bool resident_most = false, resident_last = false;
+    bool resident(int B) const { return B == most ? resident_most : resident_last; }
+};
+
+// ... for passes in all of `modes`; reserves the exchange (before any work is queued)
+int plan_batches(gbfwi_mesh *m, std::initializer_list<int> modes, int nshot, int most, long long NP, Batches &b)
 {
-    for (int B : {most, sizes::last_batch(nshot, most)}) {
-        const ResidentPlan *p = gb_resident_plan(m, mode, B);
-        if (!p) return GBFWI_EINVAL;
-        GB_TRY(m->w_xch.ensure(gb_resident_exchange(*p, B, NP)));
-    }
+    b = Batches{most, sizes::last_batch(nshot, most)};
+    auto resident = [&](int B) {
+        return std::all_of(modes.begin(), modes.end(), [&](int mode) { return gb_resident_plan(m, mode, B) != nullptr; });
+    };
+    b.resident_most = resident(most);
+    b.resident_last = b.resident_most && resident(b.last);
+    for (int B : {most, b.last})
+        if (b.resident(B))
+            for (int mode : modes) GB_TRY(m->w_xch.ensure(gb_resident_exchange(*gb_resident_plan(m, mode, B), B, NP)));
     return GBFWI_OK;
 }
 
-// Shots advanced together by forward runs that keep no history, and whether
-// as resident launches: the resident loop takes as many shots as fit the SMs
-// at once (three levels and a velocity each), the step kernels the schedule's.
-int forward_batch(gbfwi_mesh *m, int nshot, bool &resident)
+// Batches of forward runs that keep no history: the resident loop takes as many
+// shots as fit the SMs at once (three levels and a velocity each), the step kernels
+// the schedule's.
+int forward_batches(gbfwi_mesh *m, int nshot, long long NP, Batches &b)
 {
     const ResidentPlan *p = gb_resident_plan(m, MODE_FWD, nshot);
-    resident = p != nullptr;
-    return std::min(nshot, p ? std::max(p->per_launch, m->sch.shots_per_launch) : m->sch.shots_per_launch);
+    const int scheduled = std::min(nshot, m->sch.shots_per_launch);
+    GB_TRY(plan_batches(m, {MODE_FWD}, nshot, p ? std::min(nshot, std::max(p->per_launch, scheduled)) : scheduled, NP, b));
+    return b.resident_most || b.most == scheduled ? GBFWI_OK : plan_batches(m, {MODE_FWD}, nshot, scheduled, NP, b);
 }
 
 }  // namespace
@@ -555,11 +568,11 @@ extern "C" int gbfwi_forward(gbfwi_mesh *m, const int *shot_ids, int nshot, floa
     GB_TRY(gb_build_tile_lists(m, tile));
     const int nt = m->d.nt;
     const long long NP = (long long)m->nz * m->pitch;
-    bool resident = false;
-    const int Bmax = forward_batch(m, nshot, resident);
+    Batches batches;
+    GB_TRY(forward_batches(m, nshot, NP, batches));
+    const int Bmax = batches.most;
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
     const bool dev_out = gb_is_device_ptr(seis);
-    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, nshot, Bmax, NP));
     GB_TRY(m->w_hist.ensure((size_t)3 * Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
@@ -567,7 +580,7 @@ extern "C" int gbfwi_forward(gbfwi_mesh *m, const int *shot_ids, int nshot, floa
     GB_CUDA(cudaMemcpyAsync(m->w_shots.p, shot_ids, nshot * sizeof(int), cudaMemcpyHostToDevice, s));
     for (int i0 = 0; i0 < nshot; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
-        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, resident};
+        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, batches.resident(B)};
         const Levels ring{m->w_hist.as<float2>(), (long long)B * NP, 0, true};
         GB_CUDA(cudaMemsetAsync(ring.base, 0, 3 * ring.lev * sizeof(float2), s));
         GB_CUDA(cudaMemsetAsync(m->w_vh.p, 0, ring.lev * sizeof(float2), s));
@@ -600,10 +613,10 @@ extern "C" int gbfwi_misfit(gbfwi_mesh *m, const int *shot_ids, int nshot, const
     GB_TRY(gb_build_tile_lists(m, tile));
     const int nt = m->d.nt;
     const long long NP = (long long)m->nz * m->pitch;
-    bool resident = false;
-    const int Bmax = forward_batch(m, nshot, resident);
+    Batches batches;
+    GB_TRY(forward_batches(m, nshot, NP, batches));
+    const int Bmax = batches.most;
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
-    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, nshot, Bmax, NP));
     GB_TRY(m->w_hist.ensure((size_t)3 * Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2)));
     GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
@@ -621,7 +634,7 @@ extern "C" int gbfwi_misfit(gbfwi_mesh *m, const int *shot_ids, int nshot, const
     GB_CUDA(cudaMemsetAsync(flag, 0, 16, s));
     for (int i0 = 0; i0 < nshot; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
-        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, resident};
+        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, batches.resident(B)};
         const Levels ring{m->w_hist.as<float2>(), (long long)B * NP, 0, true};
         GB_CUDA(cudaMemsetAsync(ring.base, 0, 3 * ring.lev * sizeof(float2), s));
         GB_CUDA(cudaMemsetAsync(m->w_vh.p, 0, ring.lev * sizeof(float2), s));
@@ -854,16 +867,13 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
     const long long levels = full ? nt + 2 : 3LL * ((nt + ckpt - 1) / ckpt) + ckpt + 6;
     const long long small = kSmallHistory / (levels * NP * (long long)sizeof(float2));
     int Bmax = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
-    const bool resident = gb_resident_plan(m, MODE_FWD, Bmax) && gb_resident_plan(m, MODE_ADJ_G, Bmax);
-    if (!resident) Bmax = std::min(m->sch.shots_per_launch, nshot);
+    Batches batches;
+    GB_TRY(plan_batches(m, {MODE_FWD, MODE_ADJ_G}, nshot, Bmax, NP, batches));
+    if (!batches.resident_most) Bmax = std::min(m->sch.shots_per_launch, nshot);
     const int nbatch = (nshot + Bmax - 1) / Bmax;
-    const int L = resident ? 1 : std::max(1, std::min(m->sch.streams, nbatch));
+    const int L = batches.resident_most ? 1 : std::max(1, std::min(m->sch.streams, nbatch));
     const size_t eacc_shot = (size_t)m->d.nex * m->d.nez * 52 * sizeof(float);
-    if (resident) GB_TRY(m->w_eacc.ensure(eacc_shot * Bmax));
-    if (resident) {
-        GB_TRY(reserve_exchange(m, MODE_FWD, nshot, Bmax, NP));
-        GB_TRY(reserve_exchange(m, MODE_ADJ_G, nshot, Bmax, NP));
-    }
+    if (batches.resident_most) GB_TRY(m->w_eacc.ensure(eacc_shot * Bmax));
 
     // lanes: 0 = the mesh's own buffers on the caller's stream, 1.. = extra streams
     while ((int)m->lanes.size() < L - 1) m->lanes.push_back(new gbfwi_mesh::Lane());
@@ -930,6 +940,7 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
         BatchHist &h = hs[l];
         cudaStream_t ls = lr.st;
         const int B = std::min(Bmax, nshot - i0);
+        const bool resident = batches.resident_most && batches.resident(B);
         auto step = [&]() -> int {
             auto mark = [&](int i) -> int {
                 if (m->timing) GB_CUDA(cudaEventRecord(m->ev[i], ls));
@@ -1094,8 +1105,9 @@ static int map_batch(gbfwi_mesh *m, int nshot, bool receiver, int tile, int Bold
     int B = (int)std::min<long long>(nshot, kMapHistory / shot);
     if (B < 1 || !gb_resident_plan(m, MODE_FWD, B)) return 0;
     B = (nshot + (nshot + B - 1) / B - 1) / ((nshot + B - 1) / B);      // equal batches
-    const ResidentPlan *f = gb_resident_plan(m, receiver ? MODE_FWD : MODE_FWD_PC, B), *r = receiver ? gb_resident_plan(m, MODE_RCV, B) : f;
-    if (!f || !r) return 0;
+    const int fwd = receiver ? MODE_FWD : MODE_FWD_PC, rcv = receiver ? MODE_RCV : fwd, last = sizes::last_batch(nshot, B);
+    const ResidentPlan *f = gb_resident_plan(m, fwd, B), *r = gb_resident_plan(m, rcv, B);
+    if (!f || !r || !gb_resident_plan(m, fwd, last) || !gb_resident_plan(m, rcv, last)) return 0;
     const TileShape &t = kTiles[tile];
     const long long ctas = (long long)((m->d.nex + t.tx - 1) / t.tx) * ((m->d.nez + t.tz - 1) / t.tz) * Bold;
     const double launches = (B + f->per_launch - 1) / f->per_launch + (receiver ? (B + r->per_launch - 1) / r->per_launch : 0);
@@ -1119,8 +1131,8 @@ static int resident_maps(gbfwi_mesh *m, int nshot, int Bmax, int kind, int tile,
     if (!rc && strains) rc = m->w_eacc.ensure(gb_integral_bytes(m, Bmax));
     if (!rc && receiver) rc = m->w_seis.ensure(seis_shot * Bmax * sizeof(float));
     if (!rc) rc = m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2));
-    if (!rc) rc = reserve_exchange(m, fwd, nshot, Bmax, NP);
-    if (!rc && receiver) rc = reserve_exchange(m, MODE_RCV, nshot, Bmax, NP);
+    Batches batches;
+    if (!rc) rc = receiver ? plan_batches(m, {fwd, MODE_RCV}, nshot, Bmax, NP, batches) : plan_batches(m, {fwd}, nshot, Bmax, NP, batches);
     if (rc) {
         for (DevBuf *b : big) b->release();
         return rc;
@@ -1175,8 +1187,8 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     const long long levels = !receiver ? 4 : ck <= 0 || ck >= nt ? nt + 6 : 3LL * ((nt + ck - 1) / ck) + ck + 10;
     const long long small = kSmallHistory / ((levels + 2) * NP * (long long)sizeof(float2));
     const int Bmax = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
-    const bool resident = receiver && gb_resident_plan(m, MODE_FWD, Bmax);
-    if (resident) GB_TRY(reserve_exchange(m, MODE_FWD, nshot, Bmax, NP));
+    Batches batches;
+    if (receiver) GB_TRY(plan_batches(m, {MODE_FWD}, nshot, Bmax, NP, batches));
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
     const long long lev = (long long)Bmax * NP;
     const double dt = m->d.dt;
@@ -1204,7 +1216,7 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     }
     for (int i0 = 0; i0 < nshot && !done; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
-        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, resident};
+        Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, batches.resident(B)};
         float *acc = m->w_pc.as<float>();
         GB_CUDA(cudaMemsetAsync(acc, 0, (size_t)B * 4 * NP * sizeof(float), s));
         long long blev = (long long)B * NP;

@@ -84,10 +84,10 @@ def test_many_shot_counts_on_one_mesh():
 # and in the chain rule: nshot 2^-24 of the shots' moduli, and of each shot's largest
 # entry times nt where its terms cancel; asserted twice that.
 @pytest.mark.parametrize("nshot,spl,ckpt", [(18, 10, 0), (13, 10, 0), (18, 10, 100)])
-def test_gradient_in_ragged_batches_is_the_sum_of_its_shots(nshot, spl, ckpt):
+def test_gradient_in_ragged_batches_is_the_sum_of_its_shots(nshot, spl, ckpt, nrec=29):
     nt, ids = 500, list(range(nshot))
-    m = mesh(46, 42, nt, nshot, shots_per_launch=spl, ckpt_every=ckpt)
-    obs = torch.zeros(nshot, 29, 2, nt, device=DEV)
+    m = mesh(46, 42, nt, nshot, nrec=nrec, shots_per_launch=spl, ckpt_every=ckpt)
+    obs = torch.zeros(nshot, nrec, 2, nt, device=DEV)
     grad, one = (torch.zeros(3, m.nz, m.nx, device=DEV) for _ in range(2))
     f = m.adjoint_gradient(ids, obs, grad)
     total, size, each = torch.zeros_like(grad).double(), torch.zeros_like(grad).double(), 0.0
@@ -97,3 +97,27 @@ def test_gradient_in_ragged_batches_is_the_sum_of_its_shots(nshot, spl, ckpt):
         size += one.abs() + nt * one.abs().amax(dim=(1, 2), keepdim=True)
     assert f > 0 and abs(f - each) <= 1e-13 * nshot * f
     assert bool(((grad - total).abs() <= 2 * nshot * 2.0 ** -24 * size).all())
+
+
+# Many receivers: a tile's lists take its shared memory, and the tile chosen for some numbers
+# of shots no longer fits while that of others does (18 shots by 10 and 2000
+# receivers: the adjoint loop is resident for 10 shots and not for 8).  Such calls mix
+# both forms; within a shot they sum the strains by element or by node (nt 2^-24 of
+# the shot's largest entry, within the bound above).
+@pytest.mark.parametrize("nrec", [1000, 2000, 3000])
+@pytest.mark.parametrize("nshot", [13, 18])
+def test_gradient_where_a_batch_does_not_fit(nrec, nshot):
+    test_gradient_in_ragged_batches_is_the_sum_of_its_shots(nshot, 10, 0, nrec)
+
+
+@pytest.mark.parametrize("nrec", [2000, 6000, 12000])
+def test_records_where_a_batch_does_not_fit(nrec):
+    nt, nshot = 20, 23
+    m = mesh(46, 42, nt, nshot, nrec=nrec, shots_per_launch=9)
+    seis, one = torch.zeros(nshot, nrec, 2, nt, device=DEV), torch.zeros(1, nrec, 2, nt, device=DEV)
+    m.forward(list(range(nshot)), seis)
+    for i in range(nshot):
+        m.forward([i], one)
+        assert torch.equal(one[0], seis[i]), i
+    for kind in (1, 2):
+        assert bool(torch.isfinite(raw_map(m, list(range(nshot)), kind)).all())
