@@ -1368,7 +1368,7 @@ int combine(gbfwi_bfgs *h, const float *A1, const float *A2, int k1, int ktot, c
         int cn = std::min(64, nc - c0);
         size_t smem = (size_t)std::max(ktot, 1) * 64 * sizeof(float);
         if (smem > 48 * 1024)
-            GB_CUDA(cudaFuncSetAttribute(combine_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            GB_TRY(gb_allow_smem((const void *)combine_kernel<64>));
         combine_kernel<64><<<grid_n(n) / 2 + 1, 128, smem, s>>>(A1, A2, k1, ktot, ld, coef, c0, cn, n, out, ldo, dw,
                                                               Xc, ldx, beta);
         GB_LAUNCHED();
@@ -1406,7 +1406,7 @@ int launch_middle(gbfwi_bfgs *h, const double *T, int q, double gamma, float *co
     auto kern = k <= 32 ? middle_col_kernel<1> : k <= 64 ? middle_col_kernel<2> : k <= 128 ? middle_col_kernel<4>
                                                                                        : middle_kernel;
     if (bytes > 48 * 1024)
-        GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        GB_TRY(gb_allow_smem((const void *)kern));
     kern<<<q, 256, bytes, s>>>(T, h->dSY, h->dYBY, k, h->kmax, q, gamma, mats, coef, coefd);
     GB_LAUNCHED();
     return GBFWI_OK;
@@ -1651,7 +1651,7 @@ int launch_pivchol(const double *G, int p, double tol, double *work, double *coe
     const size_t ws = (3 * (size_t)p * p + 2 * (size_t)p) * sizeof(double);
     const int use_smem = ws <= 200 * 1024;
     if (use_smem)
-        GB_CUDA(cudaFuncSetAttribute(gram_pivchol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ws));
+        GB_TRY(gb_allow_smem((const void *)gram_pivchol_kernel));
     gram_pivchol_kernel<<<1, 512, use_smem ? ws : 0, s>>>(G, p, tol, work, coef, r_out, flag, use_smem);
     GB_LAUNCHED();
     return GBFWI_OK;
@@ -1663,7 +1663,7 @@ int launch_eig(const double *T, int r, int rank, double *work, double *lam, floa
     const int use_smem = we <= 200 * 1024;
     const int npair = (r + 1) / 2;
     auto kern = npair <= 32 ? eig_select_kernel<1> : npair <= 64 ? eig_select_kernel<2> : eig_select_kernel<4>;
-    if (use_smem) GB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)we));
+    if (use_smem) GB_TRY(gb_allow_smem((const void *)kern));
     kern<<<1, 1024, use_smem ? we : 0, s>>>(T, r, rank, work, lam, coef, flag, use_smem);
     GB_LAUNCHED();
     return GBFWI_OK;
@@ -1826,10 +1826,10 @@ int lowrank_randomized(gbfwi_bfgs *h, const float *X, int p, int rank, unsigned 
         GB_LAUNCHED();
         const size_t wl = (size_t)2 * r * r * sizeof(double);
         const int lu_smem = wl <= 200 * 1024;
-        if (lu_smem) GB_CUDA(cudaFuncSetAttribute(lu_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wl));
+        if (lu_smem) GB_TRY(gb_allow_smem((const void *)lu_kernel));
         lu_kernel<<<1, 512, lu_smem ? wl : 0, s>>>(A, R2, perm, r, flag, lu_smem);
         GB_LAUNCHED();
-        if (lu_smem) GB_CUDA(cudaFuncSetAttribute(lu_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wl));
+        if (lu_smem) GB_TRY(gb_allow_smem((const void *)lu_solve_kernel));
         lu_solve_kernel<<<r, 32, lu_smem ? wl : 0, s>>>(A, R2, perm, Bm, r, Om, lu_smem);
         GB_LAUNCHED();
         sym_kernel<<<1, 512, 0, s>>>(Om, r);

@@ -50,6 +50,11 @@ long long gb_launches_so_far();
 // device buffers
 // ---------------------------------------------------------------------------
 
+// Lets `kernel` use all the dynamic shared memory of a block, once per device: the attribute
+// belongs to the process, and one that followed each launch's size would be lowered by
+// another host thread between a launch's setting of it and the launch.
+int gb_allow_smem(const void *kernel);
+
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;

@@ -11,6 +11,7 @@
 #include <cstring>
 #include <atomic>
 #include <mutex>
+#include <set>
 
 #include "gbfwi_internal.h"
 
@@ -65,6 +66,22 @@ int gb_nonfinite(const char *what)
 {
     snprintf(g_nonfinite, sizeof(g_nonfinite), "non-finite value: %s", what);
     return GBFWI_ENONFINITE;
+}
+
+int gb_allow_smem(const void *kernel)
+{
+    static std::mutex mutex;
+    static std::set<std::pair<int, const void *>> done;
+    int dev = 0, most = 0;
+    GB_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mutex);
+    if (done.count({dev, kernel})) return GBFWI_OK;
+    cudaFuncAttributes at;
+    GB_CUDA(cudaFuncGetAttributes(&at, kernel));
+    GB_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    GB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes));
+    done.insert({dev, kernel});
+    return GBFWI_OK;
 }
 
 int DevBuf::ensure(size_t nbytes)

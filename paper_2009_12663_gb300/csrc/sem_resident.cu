@@ -748,8 +748,7 @@ int slots_of(const Variant &v, size_t smem, int *nsm)
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || !coop ||
-        smem > (size_t)most - 64 ||
-        cudaFuncSetAttribute(v.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        smem > (size_t)most - 64 || gb_allow_smem((const void *)v.fn) != GBFWI_OK ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, v.fn, v.threads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -806,7 +805,7 @@ int gb_launch_resident(const ResidentPlan &p, int mode, ResidentArgs a, int nsho
     a.edge_cap = edge_cap(p.TX, p.TZ, p.ntx, p.ntz, a.free_top);
     a.grp_cap = p.grp_cap; a.ent_cap = p.ent_cap; a.rec_cap = p.rec_cap;
     const size_t smem = p.smem;
-    GB_CUDA(cudaFuncSetAttribute(v->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    GB_TRY(gb_allow_smem((const void *)v->fn));
     const ResidentArgs all = a;
     for (int s0 = 0; s0 < nshots; s0 += p.per_launch) {
         const int B = std::min(p.per_launch, nshots - s0);
