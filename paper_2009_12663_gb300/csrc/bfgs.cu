@@ -1507,7 +1507,8 @@ extern "C" int gbfwi_bfgs_create(long long n, int kmax, const float *B0, gbfwi_b
         (pad && cudaMemset2D(h->Y + n, h->ld * 4, 0, pad, (size_t)kmax) != cudaSuccess) ||
         (pad && cudaMemset2D(h->BY + n, h->ld * 4, 0, pad, (size_t)kmax) != cudaSuccess) ||
         cudaMemset(base + oM, 0, oF + 32 - oM) != cudaSuccess ||
-        cudaMemcpy(h->B0, B0, (size_t)n * sizeof(float), cudaMemcpyDefault) != cudaSuccess) {
+        cudaMemcpy(h->B0, B0, (size_t)n * sizeof(float), cudaMemcpyDefault) != cudaSuccess ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess) {     // work on other streams may follow at once
         gb_set_last_cuda_error(cudaGetLastError(), "initialise the BFGS store", __FILE__, __LINE__);
         delete h;
         return GBFWI_ECUDA;

@@ -65,3 +65,22 @@ def test_threads_do_not_disturb_each_other():
     for t in threads:
         t.join()
     assert not wrong, wrong
+
+
+def test_a_store_is_complete_when_it_is_created():
+    """Creation takes no stream: work queued on another one must not overtake it,
+    however busy the default stream is."""
+    n, k = 5000, 6
+    want = bfgs_work(n, k)
+    torch.cuda.synchronize()
+    busy = torch.zeros(4096, 4096, device=DEV)
+    torch.matmul(busy, busy)
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    for _ in range(40):
+        torch.matmul(busy, busy)                         # some 50 ms on the default stream
+    with torch.cuda.stream(st):
+        got = bfgs_work(n, k)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
