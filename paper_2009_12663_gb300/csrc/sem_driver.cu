@@ -540,15 +540,54 @@ int plan_batches(gbfwi_mesh *m, std::initializer_list<int> modes, int nshot, int
     return GBFWI_OK;
 }
 
-// Batches of forward runs that keep no history: the resident loop takes as many
-// shots as fit the SMs at once (three levels and a velocity each), the step kernels
-// the schedule's.
-int forward_batches(gbfwi_mesh *m, int nshot, long long NP, Batches &b)
+// Shots of a batch where the resident loop takes it, and where it does not (`resident`
+// false: it is not asked).  A call prefers more shots at once than its schedule asks for;
+// where their buffers do not fit the memory that is left, it goes back to the schedule's
+// number, and to the step kernels.
+struct Choice { int most, stepped; bool resident; };
+
+// gives back the buffers that grow with a batch (a cudaFree waits for work that uses them)
+void release_batch_buffers(gbfwi_mesh *m)
+{
+    for (DevBuf *b : {&m->w_hist, &m->w_snap, &m->w_vh, &m->w_adj, &m->w_wh, &m->w_seis, &m->w_lacc, &m->w_pc, &m->w_eacc, &m->w_xch})
+        b->release();
+    for (gbfwi_mesh::Lane *l : m->lanes)
+        for (DevBuf *b : {&l->hist, &l->snap, &l->vh, &l->adj, &l->wh, &l->seis, &l->acc}) b->release();
+}
+
+// reserve(batches) for the first of the choices whose buffers fit; passes in `modes` are those
+// the resident loop would run
+template <class Reserve>
+int reserve_batches(gbfwi_mesh *m, std::initializer_list<int> modes, int nshot, const std::vector<Choice> &choices, Batches &b,
+                    Reserve reserve)
+{
+    const long long NP = (long long)m->nz * m->pitch;
+    return sizes::first_that_fits(choices, GBFWI_ENOMEM, [&](const Choice &c) -> int {
+        b = Batches();
+        if (c.resident && modes.size()) GB_TRY(plan_batches(m, modes, nshot, c.most, NP, b));
+        if (!b.resident_most) b = Batches{c.stepped, sizes::last_batch(nshot, c.stepped)};
+        return reserve(b);
+    }, [&] { release_batch_buffers(m); });
+}
+
+// Forward runs that keep no history: the resident loop takes as many shots as fit
+// the SMs at once (three levels and a velocity each), the step kernels the
+// schedule's.  seis_shot: values of a shot's records that the mesh keeps (0: the caller
+// does); fixed(): the buffers that do not grow with the batch
+template <class Fixed>
+int reserve_forward(gbfwi_mesh *m, int nshot, size_t seis_shot, Batches &b, Fixed fixed)
 {
     const ResidentPlan *p = gb_resident_plan(m, MODE_FWD, nshot);
+    const long long NP = (long long)m->nz * m->pitch;
     const int scheduled = std::min(nshot, m->sch.shots_per_launch);
-    GB_TRY(plan_batches(m, {MODE_FWD}, nshot, p ? std::min(nshot, std::max(p->per_launch, scheduled)) : scheduled, NP, b));
-    return b.resident_most || b.most == scheduled ? GBFWI_OK : plan_batches(m, {MODE_FWD}, nshot, scheduled, NP, b);
+    const int preferred = p ? std::min(nshot, std::max(p->per_launch, scheduled)) : scheduled;
+    const std::vector<Choice> choices = {{preferred, scheduled, p != nullptr}, {scheduled, scheduled, true}, {scheduled, scheduled, false}};
+    return reserve_batches(m, {MODE_FWD}, nshot, choices, b, [&](const Batches &c) -> int {
+        GB_TRY(fixed());
+        GB_TRY(m->w_hist.ensure((size_t)3 * c.most * NP * sizeof(float2)));
+        GB_TRY(m->w_vh.ensure((size_t)c.most * NP * sizeof(float2)));
+        return seis_shot ? m->w_seis.ensure(seis_shot * c.most * sizeof(float)) : GBFWI_OK;
+    });
 }
 
 }  // namespace
@@ -568,15 +607,12 @@ extern "C" int gbfwi_forward(gbfwi_mesh *m, const int *shot_ids, int nshot, floa
     GB_TRY(gb_build_tile_lists(m, tile));
     const int nt = m->d.nt;
     const long long NP = (long long)m->nz * m->pitch;
-    Batches batches;
-    GB_TRY(forward_batches(m, nshot, NP, batches));
-    const int Bmax = batches.most;
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
     const bool dev_out = gb_is_device_ptr(seis);
-    GB_TRY(m->w_hist.ensure((size_t)3 * Bmax * NP * sizeof(float2)));
-    GB_TRY(m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2)));
-    GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
-    if (!dev_out) GB_TRY(m->w_seis.ensure(seis_shot * Bmax * sizeof(float)));
+    Batches batches;
+    GB_TRY(reserve_forward(m, nshot, dev_out ? 0 : seis_shot, batches,
+                           [&] { return m->w_shots.ensure((size_t)nshot * sizeof(int)); }));
+    const int Bmax = batches.most;
     GB_CUDA(cudaMemcpyAsync(m->w_shots.p, shot_ids, nshot * sizeof(int), cudaMemcpyHostToDevice, s));
     for (int i0 = 0; i0 < nshot; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
@@ -613,17 +649,16 @@ extern "C" int gbfwi_misfit(gbfwi_mesh *m, const int *shot_ids, int nshot, const
     GB_TRY(gb_build_tile_lists(m, tile));
     const int nt = m->d.nt;
     const long long NP = (long long)m->nz * m->pitch;
-    Batches batches;
-    GB_TRY(forward_batches(m, nshot, NP, batches));
-    const int Bmax = batches.most;
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
-    GB_TRY(m->w_hist.ensure((size_t)3 * Bmax * NP * sizeof(float2)));
-    GB_TRY(m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2)));
-    GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
-    GB_TRY(m->w_seis.ensure(seis_shot * Bmax * sizeof(float)));
-    const int npart = kMisfitBlocks * Bmax;
-    GB_TRY(m->w_red.ensure((size_t)(npart + 8) * sizeof(double) + 4096));
-    GB_TRY(m->w_flag.ensure(16));
+    const int npart = kMisfitBlocks * nshot;
+    Batches batches;
+    GB_TRY(reserve_forward(m, nshot, seis_shot, batches, [&]() -> int {
+        GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
+        GB_TRY(m->w_red.ensure((size_t)(npart + 8) * sizeof(double) + 4096));
+        GB_TRY(m->w_flag.ensure(16));
+        return gb_is_device_ptr(d_obs) ? GBFWI_OK : m->w_obs.ensure(seis_shot * nshot * sizeof(float));
+    }));
+    const int Bmax = batches.most;
     const void *obs_d = nullptr;
     GB_TRY(stage_in(m->w_obs, d_obs, seis_shot * nshot * sizeof(float), s, &obs_d));
     double *partial = m->w_red.as<double>();
@@ -866,47 +901,55 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
     const bool full = ckpt <= 0 || ckpt >= nt;
     const long long levels = full ? nt + 2 : 3LL * ((nt + ckpt - 1) / ckpt) + ckpt + 6;
     const long long small = kSmallHistory / (levels * NP * (long long)sizeof(float2));
-    int Bmax = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
-    Batches batches;
-    GB_TRY(plan_batches(m, {MODE_FWD, MODE_ADJ_G}, nshot, Bmax, NP, batches));
-    if (!batches.resident_most) Bmax = std::min(m->sch.shots_per_launch, nshot);
-    const int nbatch = (nshot + Bmax - 1) / Bmax;
-    const int L = batches.resident_most ? 1 : std::max(1, std::min(m->sch.streams, nbatch));
+    const int stepped = std::min(m->sch.shots_per_launch, nshot);
+    const int scheduled = (int)std::min<long long>(nshot, (long long)m->sch.shots_per_launch * m->sch.streams);
+    const int preferred = (int)std::min<long long>(nshot, std::max<long long>(scheduled, small));
     const size_t eacc_shot = (size_t)m->d.nex * m->d.nez * 52 * sizeof(float);
-    if (batches.resident_most) GB_TRY(m->w_eacc.ensure(eacc_shot * Bmax));
-
-    // lanes: 0 = the mesh's own buffers on the caller's stream, 1.. = extra streams
-    while ((int)m->lanes.size() < L - 1) m->lanes.push_back(new gbfwi_mesh::Lane());
-    std::vector<LaneRef> lanes{lane0(m, s)};
-    for (int l = 1; l < L; ++l) {
-        gbfwi_mesh::Lane *ln = m->lanes[l - 1];
-        if (!ln->st) GB_CUDA(cudaStreamCreateWithFlags(&ln->st, cudaStreamNonBlocking));
-        lanes.push_back(
-            LaneRef{&ln->hist, &ln->snap, &ln->vh, &ln->adj, &ln->wh, &ln->seis, &ln->batch, &ln->acc, ln->st});
-    }
-    std::vector<BatchHist> hs(L);
-    for (int l = 0; l < L; ++l) {
-        GB_TRY(alloc_hist(m, lanes[l], Bmax, ckpt, NP, hs[l], true));
-        GB_TRY(lanes[l].seis->ensure(seis_shot * Bmax * sizeof(float)));
-        GB_TRY(lanes[l].batch->ensure((size_t)Bmax * sizeof(int)));
-        GB_TRY(lanes[l].acc->ensure((size_t)Bmax * 5 * NP * sizeof(float)));
-    }
     // per-shot accumulators and misfit partials, reduced once in shot order at
     // the end: the result does not depend on batching or lanes
-    GB_TRY(m->w_acc.ensure((size_t)nshot * 5 * NP * sizeof(float)));
-    GB_TRY(m->w_grad.ensure((size_t)5 * NP * sizeof(float)));
-    GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
     const int npart = kMisfitBlocks * nshot;
-    GB_TRY(m->w_red.ensure((size_t)(npart + 8) * sizeof(double) + 4096));
-    GB_TRY(m->w_flag.ensure(16));
+    const bool dev_grad = gb_is_device_ptr(grad);
+    auto fixed_buffers = [&]() -> int {
+        GB_TRY(m->w_acc.ensure((size_t)nshot * 5 * NP * sizeof(float)));
+        GB_TRY(m->w_grad.ensure((size_t)5 * NP * sizeof(float)));
+        GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
+        GB_TRY(m->w_red.ensure((size_t)(npart + 8) * sizeof(double) + 4096));
+        GB_TRY(m->w_flag.ensure(16));
+        if (!dev_grad) GB_TRY(m->w_tmp.ensure((size_t)3 * N * sizeof(float)));
+        return gb_is_device_ptr(d_obs) ? GBFWI_OK : m->w_obs.ensure(seis_shot * nshot * sizeof(float));
+    };
+    // lanes: 0 = the mesh's own buffers on the caller's stream, 1.. = extra streams
+    int nbatch = 0, L = 0;
+    std::vector<LaneRef> lanes;
+    std::vector<BatchHist> hs;
+    Batches batches;
+    const std::vector<Choice> choices = {{preferred, stepped, true}, {scheduled, stepped, true}, {stepped, stepped, false}};
+    GB_TRY(reserve_batches(m, {MODE_FWD, MODE_ADJ_G}, nshot, choices, batches, [&](const Batches &b) -> int {
+        GB_TRY(fixed_buffers());
+        nbatch = (nshot + b.most - 1) / b.most;
+        L = b.resident_most ? 1 : std::max(1, std::min(m->sch.streams, nbatch));
+        if (b.resident_most) GB_TRY(m->w_eacc.ensure(eacc_shot * b.most));
+        while ((int)m->lanes.size() < L - 1) m->lanes.push_back(new gbfwi_mesh::Lane());
+        lanes.assign(1, lane0(m, s));
+        for (int l = 1; l < L; ++l) {
+            gbfwi_mesh::Lane *ln = m->lanes[l - 1];
+            if (!ln->st) GB_CUDA(cudaStreamCreateWithFlags(&ln->st, cudaStreamNonBlocking));
+            lanes.push_back(
+                LaneRef{&ln->hist, &ln->snap, &ln->vh, &ln->adj, &ln->wh, &ln->seis, &ln->batch, &ln->acc, ln->st});
+        }
+        hs.assign(L, BatchHist());
+        for (int l = 0; l < L; ++l) {
+            GB_TRY(alloc_hist(m, lanes[l], b.most, ckpt, NP, hs[l], true));
+            GB_TRY(lanes[l].seis->ensure(seis_shot * b.most * sizeof(float)));
+            GB_TRY(lanes[l].batch->ensure((size_t)b.most * sizeof(int)));
+            GB_TRY(lanes[l].acc->ensure((size_t)b.most * 5 * NP * sizeof(float)));
+        }
+        return GBFWI_OK;
+    }));
+    const int Bmax = batches.most;
     const void *obs_d = nullptr;
     GB_TRY(stage_in(m->w_obs, d_obs, seis_shot * nshot * sizeof(float), s, &obs_d));
-    const bool dev_grad = gb_is_device_ptr(grad);
-    float *grad_d = grad;
-    if (!dev_grad) {
-        GB_TRY(m->w_tmp.ensure((size_t)3 * N * sizeof(float)));
-        grad_d = m->w_tmp.as<float>();
-    }
+    float *grad_d = dev_grad ? grad : m->w_tmp.as<float>();
     double *partial = m->w_red.as<double>();
     double *mis_d = partial + npart;
     int *flag = m->w_flag.as<int>();
@@ -940,7 +983,7 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
         BatchHist &h = hs[l];
         cudaStream_t ls = lr.st;
         const int B = std::min(Bmax, nshot - i0);
-        const bool resident = batches.resident_most && batches.resident(B);
+        const bool resident = batches.resident(B);
         auto step = [&]() -> int {
             auto mark = [&](int i) -> int {
                 if (m->timing) GB_CUDA(cudaEventRecord(m->ev[i], ls));
@@ -1116,27 +1159,28 @@ static int map_batch(gbfwi_mesh *m, int nshot, bool receiver, int tile, int Bold
     return here < steps ? B : 0;
 }
 
-// The integrals of every shot (summed into tot) from stored levels.  GBFWI_ENOMEM
-// before anything is queued when the levels do not fit: nothing is kept then.
+// buffers of resident_maps
+static int reserve_maps(gbfwi_mesh *m, int nshot, int Bmax, bool receiver, bool strains)
+{
+    const long long NP = (long long)m->nz * m->pitch;
+    const size_t levels = (size_t)(m->d.nt + 2) * Bmax * NP * sizeof(float2);
+    Batches b;
+    GB_TRY(receiver ? plan_batches(m, {MODE_FWD, MODE_RCV}, nshot, Bmax, NP, b) : plan_batches(m, {MODE_FWD_PC}, nshot, Bmax, NP, b));
+    GB_TRY(m->w_hist.ensure(levels));
+    GB_TRY(m->w_snap.ensure(levels));
+    if (receiver) GB_TRY(m->w_adj.ensure(levels));
+    if (receiver) GB_TRY(m->w_seis.ensure((size_t)m->nrec * 2 * m->d.nt * Bmax * sizeof(float)));
+    if (strains) GB_TRY(m->w_eacc.ensure(gb_integral_bytes(m, Bmax)));
+    GB_TRY(m->w_pc.ensure((size_t)Bmax * 4 * NP * sizeof(float)));
+    return m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2));
+}
+
+// the integrals of every shot (summed into tot) from stored levels
 static int resident_maps(gbfwi_mesh *m, int nshot, int Bmax, int kind, int tile, float *tot, long long NP, cudaStream_t s)
 {
     const int nt = m->d.nt;
     const bool receiver = kind == 2 || kind == 4, strains = kind >= 3;
     const int fwd = receiver ? MODE_FWD : MODE_FWD_PC;
-    const size_t levels = (size_t)(nt + 2) * Bmax * NP * sizeof(float2), seis_shot = (size_t)m->nrec * 2 * nt;
-    DevBuf *big[] = {&m->w_hist, &m->w_snap, &m->w_adj, &m->w_eacc};
-    int rc = m->w_hist.ensure(levels);
-    if (!rc) rc = m->w_snap.ensure(levels);
-    if (!rc && receiver) rc = m->w_adj.ensure(levels);
-    if (!rc && strains) rc = m->w_eacc.ensure(gb_integral_bytes(m, Bmax));
-    if (!rc && receiver) rc = m->w_seis.ensure(seis_shot * Bmax * sizeof(float));
-    if (!rc) rc = m->w_vh.ensure((size_t)Bmax * NP * sizeof(float2));
-    Batches batches;
-    if (!rc) rc = receiver ? plan_batches(m, {fwd, MODE_RCV}, nshot, Bmax, NP, batches) : plan_batches(m, {fwd}, nshot, Bmax, NP, batches);
-    if (rc) {
-        for (DevBuf *b : big) b->release();
-        return rc;
-    }
     float *acc = m->w_pc.as<float>();
     float2 *vh = m->w_vh.as<float2>();
     for (int i0 = 0; i0 < nshot; i0 += Bmax) {
@@ -1186,35 +1230,43 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     const int ck = m->sch.ckpt_every;
     const long long levels = !receiver ? 4 : ck <= 0 || ck >= nt ? nt + 6 : 3LL * ((nt + ck - 1) / ck) + ck + 10;
     const long long small = kSmallHistory / ((levels + 2) * NP * (long long)sizeof(float2));
-    const int Bmax = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
-    Batches batches;
-    if (receiver) GB_TRY(plan_batches(m, {MODE_FWD}, nshot, Bmax, NP, batches));
+    const int scheduled = std::min(m->sch.shots_per_launch, nshot);
+    const int preferred = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
-    const long long lev = (long long)Bmax * NP;
     const double dt = m->d.dt;
 
-    const int Bmap = map_batch(m, nshot, receiver, tile, Bmax, NP);
-    GB_TRY(m->w_vh.ensure(lev * sizeof(float2)));
-    GB_TRY(m->w_pc.ensure((size_t)std::max(Bmax, Bmap) * 4 * NP * sizeof(float)));
-    GB_TRY(m->w_grad.ensure((size_t)5 * NP * sizeof(float)));
-    GB_TRY(m->w_shots.ensure((size_t)nshot * sizeof(int)));
+    const int Bmap = map_batch(m, nshot, receiver, tile, preferred, NP);
+    auto fixed_buffers = [&]() -> int {
+        GB_TRY(m->w_grad.ensure((size_t)5 * NP * sizeof(float)));
+        GB_TRY(m->w_tmp.ensure((size_t)9 * N * sizeof(float) + 4096));
+        return m->w_shots.ensure((size_t)nshot * sizeof(int));
+    };
+    // the maps from stored levels where their buffers fit, else the preconditioner steps
+    BatchHist h;
+    Batches batches;
+    int rc = fixed_buffers();
+    if (!rc && Bmap) rc = reserve_maps(m, nshot, Bmap, receiver, kind >= 3);
+    const bool from_levels = Bmap && rc == GBFWI_OK;
+    if (!from_levels) {
+        if (rc && rc != GBFWI_ENOMEM) return rc;
+        if (rc) release_batch_buffers(m);
+        const auto steps = [&](const Batches &b) -> int {
+            GB_TRY(fixed_buffers());
+            GB_TRY(m->w_vh.ensure((size_t)b.most * NP * sizeof(float2)));
+            GB_TRY(m->w_pc.ensure((size_t)b.most * 4 * NP * sizeof(float)));
+            if (!receiver) return m->w_hist.ensure((size_t)3 * b.most * NP * sizeof(float2));
+            GB_TRY(alloc_hist(m, lane0(m, s), b.most, ck, NP, h, true));
+            return m->w_seis.ensure(seis_shot * b.most * sizeof(float));
+        };
+        const std::vector<Choice> choices = {{preferred, preferred, receiver}, {scheduled, scheduled, receiver}, {scheduled, scheduled, false}};
+        GB_TRY(reserve_batches(m, {MODE_FWD}, nshot, choices, batches, steps));
+    }
     GB_CUDA(cudaMemcpyAsync(m->w_shots.p, shot_ids, nshot * sizeof(int), cudaMemcpyHostToDevice, s));
     float *tot = m->w_grad.as<float>();
     GB_CUDA(cudaMemsetAsync(tot, 0, 4 * NP * sizeof(float), s));
-    bool done = false;
-    if (Bmap) {
-        const int rc = resident_maps(m, nshot, Bmap, kind, tile, tot, NP, s);
-        if (rc && rc != GBFWI_ENOMEM) return rc;
-        done = rc == GBFWI_OK;
-    }
-    BatchHist h;
-    if (!done && receiver) {
-        GB_TRY(alloc_hist(m, lane0(m, s), Bmax, m->sch.ckpt_every, NP, h, true));
-        GB_TRY(m->w_seis.ensure(seis_shot * Bmax * sizeof(float)));
-    } else if (!done) {
-        GB_TRY(m->w_hist.ensure((size_t)3 * lev * sizeof(float2)));
-    }
-    for (int i0 = 0; i0 < nshot && !done; i0 += Bmax) {
+    if (from_levels) GB_TRY(resident_maps(m, nshot, Bmap, kind, tile, tot, NP, s));
+    const int Bmax = batches.most;
+    for (int i0 = 0; i0 < nshot && !from_levels; i0 += Bmax) {
         int B = std::min(Bmax, nshot - i0);
         Ctx c{m, &m->lists[tile], tile, B, s, m->w_shots.as<int>() + i0, NP, batches.resident(B)};
         float *acc = m->w_pc.as<float>();
@@ -1239,7 +1291,6 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     // (second difference) . a (x 1/dt)
     float f0 = (kind == 1 || kind == 3) ? (float)dt : (float)(1.0 / dt);
     float f1 = (float)(1.0 / dt);
-    GB_TRY(m->w_tmp.ensure((size_t)9 * N * sizeof(float) + 4096));
     float *Hd = m->w_tmp.as<float>();
     float *S1 = Hd + 3 * N, *S2 = Hd + 6 * N;
     precond_finish<<<grid_for(N), 256, 0, s>>>(tot, m->d_model.as<float>(), m->d_wx.as<float>(),

@@ -11,6 +11,22 @@ namespace sizes {
 // shots of the last of the batches that take `nshot` shots `most` at a time
 inline int last_batch(int nshot, int most) { return nshot - (nshot - 1) / most * most; }
 
+// Tries reserve(choice) for the choices in order, the preferred one first, until one
+// does not fail with `no_memory`; what a failed one holds is given back before the next.
+template <class Choices, class Reserve, class Release>
+int first_that_fits(const Choices &choices, int no_memory, Reserve reserve, Release release)
+{
+    int rc = no_memory;
+    bool first = true;
+    for (const auto &c : choices) {
+        if (!first) release();
+        first = false;
+        rc = reserve(c);
+        if (rc != no_memory) break;
+    }
+    return rc;
+}
+
 // Time chunks of the strain sums of the preconditioner maps (sem_integrals.cu):
 // about five warps an SM from one shot, at least 16 steps each.  By the mesh and
 // the time axis only: a rule on the warps of a whole batch let a smaller batch

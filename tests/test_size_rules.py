@@ -121,3 +121,23 @@ def test_partials_of_unet_products_fit_the_scratch(tmp_path):
         }
   if (!wide) { std::printf("no layer is wider than the scratch\n"); ++bad; }
 """)
+
+
+def test_less_is_reserved_when_memory_is_short(tmp_path):
+    """Choices in order until one fits; what a failed one took is given back first;
+    other errors end the search."""
+    run(tmp_path, r"""
+  for (int room = 0; room <= 40; ++room) {
+    int held = 0, released = 0;
+    auto reserve = [&](int want) {                   // in pieces of three, like a call's buffers
+      for (int got = 0; got < want; got += 3, held += 3)
+        if (held + 3 > room) return -2;
+      return 0;
+    };
+    const int rc = first_that_fits(std::initializer_list<int>{36, 12, 3}, -2, reserve, [&] { held = 0; ++released; });
+    const int want = room >= 36 ? 36 : room >= 12 ? 12 : 3;
+    if (rc != (room >= 3 ? 0 : -2) || (rc == 0 && held != want) || released != (want == 36 ? 0 : want == 12 ? 1 : 2)) ++bad;
+  }
+  int asked = 0;
+  if (first_that_fits(std::initializer_list<int>{2, 1}, -2, [&](int) { ++asked; return -1; }, [] {}) != -1 || asked != 1) ++bad;
+""")
