@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "gbfwi_internal.h"
@@ -945,7 +946,6 @@ struct gbfwi_unet {
     DevBuf red, flag;                   // loss partials / result, non-finite flag
     long long part_cap = 0;
     int nb = 0;                         // samples the activation buffers hold
-    bool grads = false;                 // the gradient buffers are there too
 };
 
 namespace {
@@ -1284,25 +1284,23 @@ int stage_input(gbfwi_unet *n, int nb, const float *x, cudaStream_t s)
     return GBFWI_OK;
 }
 
-// Activation buffers for nb samples, and the gradients' when grads.  Grown on
-// demand: inference needs neither the gradients nor more than one sample.
-int reserve(gbfwi_unet *n, int nb, bool grads)
+// Activation and gradient buffers for nb samples.  The larger ones are allocated
+// beside those that are there and take their place together, so a failure leaves
+// the network with what it had (one sample's from its creation on).
+int reserve(gbfwi_unet *n, int nb)
 {
-    if (nb <= n->nb && (n->grads || !grads)) return GBFWI_OK;
-    nb = std::max(nb, n->nb);
+    if (nb <= n->nb) return GBFWI_OK;
     const int Lv = n->d.levels;
     const long long P0 = npix(n, 0);
     const UnetLayer &O = n->layers.back();
-    int rc = GBFWI_OK;
-    auto need = [&](DevBuf &b, long long bytes) {
-        if (!rc) rc = b.ensure((size_t)std::max<long long>(bytes * nb, 16));
-    };
+    std::vector<std::pair<DevBuf *, size_t>> list;
+    auto need = [&](DevBuf &b, long long bytes) { list.push_back({&b, (size_t)std::max<long long>(bytes * nb, 16)}); };
     const size_t F = sizeof(float), B2 = sizeof(bf16);
-    n->nb = 0;                          // until all of it is there
     need(n->xin32, (long long)n->d.cin * P0 * F);
     need(n->xb, (long long)n->d.cin * P0 * B2);
     need(n->tgt32, (long long)n->d.cout * P0 * F);
     need(n->yout, (long long)O.coutp * P0 * F);
+    need(n->gyb, (long long)O.coutp * P0 * B2);
     long long cmax = (long long)O.coutp * P0;
     for (int l = 0; l < Lv; ++l) {
         const long long P = npix(n, l);
@@ -1313,20 +1311,20 @@ int reserve(gbfwi_unet *n, int nb, bool grads)
         if (l <= Lv - 2) {
             need(n->da[l], n->ch[l] * P * B2);
             need(n->dd[l], n->ch[l] * P * B2);
+            need(n->dcat[l], (long long)(n->ch[l + 1] + n->ch[l]) * P * F);
         }
     }
-    if (grads || n->grads) {
-        need(n->gyb, (long long)O.coutp * P0 * B2);
-        for (int l = 0; l <= Lv - 2; ++l) need(n->dcat[l], (long long)(n->ch[l + 1] + n->ch[l]) * npix(n, l) * F);
-        need(n->fA, cmax * F);
-        need(n->fP, cmax * F);
-        need(n->gb, cmax * B2);
-        need(n->rsum, (long long)std::max(n->ch[Lv - 1], O.coutp) * F);
-        if (!rc) rc = n->wt.ensure((size_t)n->nparam * B2);
+    need(n->fA, cmax * F);
+    need(n->fP, cmax * F);
+    need(n->gb, cmax * B2);
+    need(n->rsum, (long long)std::max(n->ch[Lv - 1], O.coutp) * F);
+    std::vector<DevBuf> fresh(list.size());
+    for (size_t i = 0; i < list.size(); ++i) GB_TRY(fresh[i].ensure(list[i].second));
+    for (size_t i = 0; i < list.size(); ++i) {
+        std::swap(list[i].first->p, fresh[i].p);
+        std::swap(list[i].first->bytes, fresh[i].bytes);
     }
-    if (rc) return rc;
     n->nb = nb;
-    n->grads = n->grads || grads;
     return GBFWI_OK;
 }
 
@@ -1394,7 +1392,8 @@ extern "C" int gbfwi_unet_create(const gbfwi_unet_desc *d, gbfwi_unet **out)
     need(n->part, n->part_cap * F);
     need(n->red, (1024 + 512 * 64) * sizeof(double));
     need(n->flag, 16);
-    if (!rc) rc = reserve(n, 1, true);
+    need(n->wt, n->nparam * B2);
+    if (!rc) rc = reserve(n, 1);
     if (rc) {
         delete n;
         return rc;
@@ -1470,7 +1469,6 @@ extern "C" int gbfwi_unet_forward(gbfwi_unet *n, const float *x, float *y, void 
     GB_TRY(gb_check_local(x, y));
     cudaStream_t s = (cudaStream_t)stream;
     const long long P0 = npix(n, 0);
-    GB_TRY(reserve(n, 1, true));
     GB_TRY(stage_input(n, 1, x, s));
     GB_TRY(net_forward(n, 1, s));
     const long long cnt = (long long)n->d.cout * P0;
@@ -1491,7 +1489,6 @@ extern "C" int gbfwi_unet_gradient(gbfwi_unet *n, const float *x, const float *d
     cudaStream_t s = (cudaStream_t)stream;
     const long long P0 = npix(n, 0);
     const UnetLayer &O = n->layers.back();
-    GB_TRY(reserve(n, 1, true));
     GB_TRY(stage_input(n, 1, x, s));
     GB_TRY(net_forward(n, 1, s));
     // dy [cout][P0] -> bf16 rows of the padded output gradient
@@ -1530,8 +1527,8 @@ extern "C" int gbfwi_unet_train_step(gbfwi_unet *n, const float *x, const float 
     int group = std::min(batch_group(n, batch), 64);
     double *lsum = n->red.as<double>();   // per-sample losses [batch] (<= 1024)
     double *partial = lsum + 1024;        // [group][nblk]
-    int rc = reserve(n, group, true);
-    for (; rc == GBFWI_ENOMEM && group > 1; rc = reserve(n, group, true)) group = (group + 1) / 2;
+    int rc = reserve(n, group);
+    for (; rc == GBFWI_ENOMEM && group > 1; rc = reserve(n, group)) group = (group + 1) / 2;
     GB_TRY(rc);
     for (int b = 0; b < batch; b += group) {
         const int nb = std::min(group, batch - b);

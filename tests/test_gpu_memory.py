@@ -5,6 +5,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 import paper_2009_12663_gb300 as gb  # noqa: E402
+from paper_2009_12663_gb300 import learned  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -22,15 +23,15 @@ def mesh():
     return m
 
 
-def fill():
-    """Device memory taken until LEFT bytes are free."""
+def fill(left=LEFT):
+    """Device memory taken until `left` bytes are free."""
     held = []
     torch.cuda.empty_cache()
     while True:
         free = torch.cuda.mem_get_info()[0]
-        if free <= LEFT + (4 << 20):
+        if free <= left + (4 << 20):
             return held
-        held.append(torch.empty(min(free - LEFT, 8 << 30), dtype=torch.uint8, device=DEV))
+        held.append(torch.empty(min(free - left, 8 << 30), dtype=torch.uint8, device=DEV))
 
 
 def test_a_schedule_that_fits_runs_when_memory_is_short():
@@ -56,3 +57,34 @@ def test_a_schedule_that_fits_runs_when_memory_is_short():
     # the map by steps instead of from levels: sums of NT non-negative terms in another order
     for c in range(3):
         assert (a[1][c] - b[1][c]).abs().max() <= 2 * NT * 2.0 ** -24 * a[1][c].max()
+
+
+def test_training_takes_fewer_samples_at_once_when_memory_is_short():
+    """Samples add to the gradients in order, however many are taken at once; a
+    failed step leaves the network able to go on."""
+    batch, Hn, Wn = 64, 32, 128
+    gen = torch.Generator(device=DEV).manual_seed(4)
+    x = torch.randn(batch, 5, Hn, Wn, generator=gen, device=DEV)
+    t = torch.randn(batch, 3, Hn, Wn, generator=gen, device=DEV)
+
+    def network():
+        net = gb.Unet(levels=4, base=32, cin=5, cout=3, height=Hn, width=Wn)
+        net.set_params(torch.tensor(learned.he_init(net, 1), device=DEV))
+        return net
+    net = network()
+    p, q = torch.zeros(net.num_params, device=DEV), torch.zeros(net.num_params, device=DEV)
+    y, y2 = torch.zeros(3, Hn, Wn, device=DEV), torch.zeros(3, Hn, Wn, device=DEV)
+    losses = [net.train_step(x, t, 1e-3) for _ in range(2)]
+    net.get_params(p)
+    net.forward(x[0].contiguous(), y)
+    del net
+    net, x0 = network(), x[0].contiguous()
+    held = fill(96 << 20)                                # all 64 samples' buffers take some 400 MB
+    try:
+        again = [net.train_step(x, t, 1e-3) for _ in range(2)]
+        net.forward(x0, y2)
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    net.get_params(q)
+    assert again == losses and torch.equal(p, q) and torch.equal(y, y2)
