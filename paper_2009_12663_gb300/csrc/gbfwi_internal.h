@@ -116,8 +116,11 @@ struct TileLists {
     DevBuf rec_entries;
     DevBuf rec_tptr;     // int [ntiles + 1]   receivers recorded by each tile
     DevBuf rec_list;     // int receiver ids, grouped by tile
-    // largest numbers of a tile: groups and entries of one source / of the receivers, receivers recorded
-    int src_most = 0, rec_most = 0, src_entries_most = 0, rec_entries_most = 0, recorded_most = 0;
+};
+
+// largest numbers of a tile: groups and entries of one source / of the receivers, receivers recorded
+struct ListSizes {
+    int src_groups = 0, src_entries = 0, rec_groups = 0, rec_entries = 0, recorded = 0;
 };
 
 // Tile of the resident time loop (sem_resident.cu) for one kind of pass and
@@ -186,6 +189,9 @@ struct gbfwi_mesh {
     // never freed.  A plan is a few numbers; the shapes are at most a few hundred.
     std::map<std::pair<int, int>, ResidentPlan> plans;
     std::map<std::pair<int, int>, TileLists> plan_lists;
+    std::map<std::pair<int, int>, ListSizes> plan_sizes;
+    struct InjectedNode { int ix, iz, entries; };
+    std::vector<InjectedNode> rec_nodes;   // nodes the receivers' signals act on, for gb_list_sizes
     DevBuf w_eacc;                      // its strain sums by element
     DevBuf w_xch;                       // its exchange of node lines between tiles
     DevBuf w_chk;                       // model checks (and a model given on the host)
@@ -213,6 +219,8 @@ struct gbfwi_mesh {
 int gb_build_tile_lists(gbfwi_mesh *m, int tile);
 // lists of the TX x TZ element tiling; per_thread: nodes packed for ResidentPlan
 int gb_build_lists(gbfwi_mesh *m, int TX, int TZ, bool per_thread, TileLists &L);
+// sizes of the per-thread lists of a tile shape, without building them
+const ListSizes &gb_list_sizes(gbfwi_mesh *m, int TX, int TZ);
 // after the work on the mesh has completed: GBFWI_ETIMEOUT (and the flag
 // cleared) when a step kernel's bounded wait gave up since the last check
 int gb_take_status(gbfwi_mesh *m);

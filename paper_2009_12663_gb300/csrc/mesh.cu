@@ -539,17 +539,6 @@ int gb_build_lists(gbfwi_mesh *m, int TX, int TZ, bool per_thread, TileLists &L)
         return GBFWI_OK;
     };
     if (sgptr.empty()) sgptr.assign(ntiles + 1, 0);
-    auto most = [](const std::vector<int> &gp, const std::vector<InjGroup> &gr, size_t q, int &groups, int &entries) {
-        if (gp[q + 1] <= gp[q]) return;
-        groups = std::max(groups, gp[q + 1] - gp[q]);
-        entries = std::max(entries, gr[gp[q + 1] - 1].end - gr[gp[q]].begin);
-    };
-    for (size_t q = 0; q + 1 < sgptr.size(); ++q)
-        if ((q + 1) % (ntiles + 1)) most(sgptr, sgroups, q, L.src_most, L.src_entries_most);
-    for (int t = 0; t < ntiles; ++t) {
-        most(rgptr, rgroups, t, L.rec_most, L.rec_entries_most);
-        L.recorded_most = std::max(L.recorded_most, tcount[t + 1] - tcount[t]);
-    }
     GB_TRY(up(L.src_gptr, sgptr.data(), sgptr.size() * sizeof(int)));
     GB_TRY(up(L.src_groups, sgroups.data(), sgroups.size() * sizeof(InjGroup)));
     GB_TRY(up(L.src_entries, sentries.data(), sentries.size() * sizeof(InjEntry)));
@@ -560,6 +549,38 @@ int gb_build_lists(gbfwi_mesh *m, int TX, int TZ, bool per_thread, TileLists &L)
     GB_TRY(up(L.rec_list, rlist.data(), rlist.size() * sizeof(int)));
     L.built = true;
     return GBFWI_OK;
+}
+
+const ListSizes &gb_list_sizes(gbfwi_mesh *m, int TX, int TZ)
+{
+    const auto known = m->plan_sizes.find({TX, TZ});
+    if (known != m->plan_sizes.end()) return known->second;
+    if (m->rec_nodes.empty()) {
+        std::map<std::pair<int, int>, int> at;
+        for (int r = 0; r < m->nrec; ++r)
+            for (int q = 0; q < 25; ++q)
+                if (m->rec_w[(size_t)r * 25 + q] != 0.0f) at[{4 * m->rec_ez[r] + q / 5, 4 * m->rec_ex[r] + q % 5}]++;
+        for (const auto &n : at) m->rec_nodes.push_back({n.first.second, n.first.first, n.second});
+    }
+    const int ntx = (m->d.nex + TX - 1) / TX, ntz = (m->d.nez + TZ - 1) / TZ;
+    auto tile_of = [&](int ix, int iz) {
+        return std::min(iz / 4, m->d.nez - 1) / TZ * ntx + std::min(ix / 4, m->d.nex - 1) / TX;
+    };
+    ListSizes S;
+    std::vector<int> count((size_t)ntx * ntz, 0), entries(count);
+    for (const auto &nodes : m->src_nodes) {
+        for (const auto &n : nodes) S.src_groups = std::max(S.src_groups, ++count[tile_of(n.ix, n.iz)]);
+        for (const auto &n : nodes) count[tile_of(n.ix, n.iz)] = 0;
+    }
+    S.src_entries = S.src_groups;                // a source acts on a node once
+    for (const auto &n : m->rec_nodes) {
+        const int t = tile_of(n.ix, n.iz);
+        S.rec_groups = std::max(S.rec_groups, ++count[t]);
+        S.rec_entries = std::max(S.rec_entries, entries[t] += n.entries);
+    }
+    std::fill(count.begin(), count.end(), 0);
+    for (int r = 0; r < m->nrec; ++r) S.recorded = std::max(S.recorded, ++count[m->rec_ez[r] / TZ * ntx + m->rec_ex[r] / TX]);
+    return m->plan_sizes[{TX, TZ}] = S;
 }
 
 // ---------------------------------------------------------------------------

@@ -78,15 +78,19 @@ inline size_t smem_bytes(int NT, bool adj, int TX, int TZ, int ntx, int ntz, boo
                                                                  grp_cap, ent_cap, rec_cap).total;
 }
 
-struct Tile { int NT = 0, TX = 0, TZ = 0, ntx = 0, ntz = 0; };   // NT 0: none
+struct Tile { int NT, TX, TZ, ntx, ntz; };   // NT 0: none
 
 // The tile whose model time per step of all `shots` is smallest among those of
-// which at least one whole shot is resident at once.  slots(NT, smem, nsm) gives the resident
-// CTAs of a variant on the device and its SMs.
-template <class Slots>
-Tile best_tile(int nex, int nez, bool free_top, bool adj, int shots, Slots slots)
+// which at least one whole shot is resident at once, also with the lists of the
+// acquisition.  slots(NT, smem, nsm) gives the resident CTAs of a variant on the device and its
+// SMs; usable(tile) whether a shot is resident with its lists.  Whether any tile is found
+// depends on the mesh and the acquisition only, not on `shots`: gradients of the
+// resident loop and of the step kernels round alike but for the order of the strain
+// sums, so a mesh keeps to one of them whatever its batches.
+template <class Slots, class Usable>
+Tile best_tile(int nex, int nez, bool free_top, bool adj, int shots, Slots slots, Usable usable)
 {
-    Tile best;
+    Tile best{};
     double best_cost = 1e300;
     for (int NT : kTileThreads) {
         int nsm = 0, have = 0;
@@ -103,6 +107,7 @@ Tile best_tile(int nex, int nez, bool free_top, bool adj, int shots, Slots slots
             if (smem != known) have = slots(NT, smem, nsm);
             known = smem;
             const int cap = (int)std::min<long long>(shots, have / T);
+            int asked = -1;                      // usable(): not asked yet
             for (int c = 1; c <= cap; ++c) {
                 // a step takes the larger of a warp's latency (with the exchange
                 // between tiles) and the busiest SM's issue time
@@ -113,8 +118,11 @@ Tile best_tile(int nex, int nez, bool free_top, bool adj, int shots, Slots slots
                 const double lat = (adj ? 3.6 : 2.6) + (T > 1 ? 1.2 : 0.0) + 0.05 * warps;
                 const double cost = ((shots + c - 1) / c) * std::max(issue, lat);
                 if (cost < best_cost * (1 - 1e-9)) {
+                    const Tile t{NT, TX, TZ, ntx, ntz};
+                    if (asked < 0) asked = usable(t);
+                    if (!asked) break;
                     best_cost = cost;
-                    best.NT = NT; best.TX = TX; best.TZ = TZ; best.ntx = ntx; best.ntz = ntz;
+                    best = t;
                 }
             }
         }

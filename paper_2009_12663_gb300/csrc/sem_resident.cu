@@ -766,27 +766,32 @@ const ResidentPlan *gb_resident_plan(gbfwi_mesh *m, int mode, int shots)
     if (mode == MODE_ADJ_PC) return nullptr;
     const auto known = m->plans.find({mode, shots});
     if (known != m->plans.end()) return known->second.NT ? &known->second : nullptr;
-    const bool adj = kernel_mode(mode) == MODE_ADJ_G;
-    const Tile best = best_tile(m->d.nex, m->d.nez, m->d.free_surface_top, adj, shots, [&](int NT, size_t smem, int &nsm) {
+    const bool adj = kernel_mode(mode) == MODE_ADJ_G, fwd = mode == MODE_FWD || mode == MODE_FWD_PC;
+    auto slots = [&](int NT, size_t smem, int &nsm) {
         const Variant *v = find_variant(NT, kernel_mode(mode));
         return v ? slots_of(*v, smem, &nsm) : 0;
-    });
+    };
+    // with the injection and record lists of the tile shape: shots that fit one launch
+    auto with_lists = [&](const Tile &t) {
+        const ListSizes &n = gb_list_sizes(m, t.TX, t.TZ);
+        ResidentPlan p;
+        p.NT = t.NT; p.TX = t.TX; p.TZ = t.TZ; p.ntx = t.ntx; p.ntz = t.ntz;
+        p.grp_cap = fwd ? n.src_groups : n.rec_groups;
+        p.ent_cap = fwd ? n.src_entries : n.rec_entries;
+        p.rec_cap = fwd ? n.recorded : 0;
+        p.smem = smem_bytes(t.NT, adj, t.TX, t.TZ, t.ntx, t.ntz, m->d.free_surface_top, p.grp_cap, p.ent_cap, p.rec_cap);
+        int nsm = 0;
+        p.per_launch = p.grp_cap < 32767 ? std::min(slots(t.NT, p.smem, nsm) / (t.ntx * t.ntz), 60000) : 0;
+        return p;
+    };
+    const Tile best = best_tile(m->d.nex, m->d.nez, m->d.free_surface_top, adj, shots, slots,
+                                [&](const Tile &t) { return with_lists(t).per_launch >= 1; });
     ResidentPlan p;
     if (best.NT) {
         TileLists &lists = m->plan_lists[{best.TX, best.TZ}];
         if (!lists.built && gb_build_lists(m, best.TX, best.TZ, true, lists) != GBFWI_OK) return nullptr;
-        // with the real injection lists: how many shots fit one launch
-        const bool fwd = mode == MODE_FWD || mode == MODE_FWD_PC;
-        p.TX = best.TX; p.TZ = best.TZ; p.ntx = best.ntx; p.ntz = best.ntz;
+        p = with_lists(best);
         p.lists = &lists;
-        p.grp_cap = fwd ? lists.src_most : lists.rec_most;
-        p.ent_cap = fwd ? lists.src_entries_most : lists.rec_entries_most;
-        p.rec_cap = fwd ? lists.recorded_most : 0;
-        p.smem = smem_bytes(best.NT, adj, p.TX, p.TZ, p.ntx, p.ntz, m->d.free_surface_top, p.grp_cap, p.ent_cap, p.rec_cap);
-        int nsm = 0;
-        const int slots = slots_of(*find_variant(best.NT, kernel_mode(mode)), p.smem, &nsm);
-        p.per_launch = p.grp_cap < 32767 ? std::min(slots / (p.ntx * p.ntz), 60000) : 0;
-        if (p.per_launch >= 1) p.NT = best.NT;
     }
     const ResidentPlan &kept = m->plans[{mode, shots}] = p;
     return kept.NT ? &kept : nullptr;

@@ -42,11 +42,16 @@ static int slots(int NT, bool adj, size_t smem) {
   if (smem > 227 * 1024 - 64) return 0;
   return 152 * (int)std::min<size_t>(228 * 1024 / (smem + 1024), 2048 / (NT + corr_threads(NT, adj)));
 }
-static Plan plan(int nex, int nez, bool adj, int shots, int injected = 4) {
-  const Tile t = best_tile(nex, nez, true, adj, shots, [&](int NT, size_t smem, int &nsm) { nsm = 152; return slots(NT, adj, smem); });
-  if (!t.NT) return {t, 0};
-  const size_t smem = smem_bytes(t.NT, adj, t.TX, t.TZ, t.ntx, t.ntz, true, injected, injected, adj ? 0 : 8);
-  return {t, slots(t.NT, adj, smem) / (t.ntx * t.ntz)};
+// receivers along the surface: those of a tile, on five nodes each
+static Plan plan(int nex, int nez, bool adj, int shots, int nrec = 8) {
+  auto all = [&](int NT, size_t smem, int &nsm) { nsm = 152; return slots(NT, adj, smem); };
+  auto launch = [&](const Tile &t) {
+    const int rec = (nrec * t.TX + nex - 1) / nex;
+    const size_t smem = smem_bytes(t.NT, adj, t.TX, t.TZ, t.ntx, t.ntz, true, adj ? 4 * t.TX + 1 : 8, adj ? 5 * rec : 8, adj ? 0 : rec);
+    return slots(t.NT, adj, smem) / (t.ntx * t.ntz);
+  };
+  const Tile t = best_tile(nex, nez, true, adj, shots, all, [&](const Tile &c) { return launch(c) >= 1; });
+  return {t, t.NT ? launch(t) : 0};
 }
 """
 
@@ -141,3 +146,23 @@ def test_less_is_reserved_when_memory_is_short(tmp_path):
   int asked = 0;
   if (first_that_fits(std::initializer_list<int>{2, 1}, -2, [&](int) { ++asked; return -1; }, [] {}) != -1 || asked != 1) ++bad;
 """)
+
+
+def test_whether_a_mesh_is_resident_does_not_depend_on_the_shots(tmp_path):
+    """Some shots choose a tile that many receivers' lists do not fit: another one
+    takes its place."""
+    run(tmp_path, r"""
+  int fit = 0, not_fit = 0;
+  for (auto [nex, nez] : {std::pair{12, 6}, {46, 42}, {60, 30}, {110, 37}, {340, 70}, {700, 80}})
+    for (bool adj : {false, true})
+      for (int nrec : {10, 1000, 2000, 3000, 12000, 100000}) {
+        const bool one = plan(nex, nez, adj, 1, nrec).per_launch >= 1;
+        (one ? fit : not_fit)++;
+        for (int shots = 2; shots <= 40; ++shots)
+          if ((plan(nex, nez, adj, shots, nrec).per_launch >= 1) != one) {
+            std::printf("%d x %d, %d receivers, %d shots\n", nex, nez, nrec, shots);
+            ++bad;
+          }
+      }
+  if (!fit || !not_fit) ++bad;
+""", "#include <utility>\n" + PLAN)
