@@ -93,8 +93,10 @@ typedef struct {
 /* Launch schedule (chosen by the autotuner or the caller).  On meshes whose
  * fields fit the SMs' shared memory a launch runs a whole range of time steps
  * instead of one; it chooses its own tile, and shots beyond shots_per_launch
- * times streams go together where that costs little memory.  Results do not
- * depend on the schedule. */
+ * times streams go together where that costs little memory.  Records, misfits
+ * and gradients do not depend on the schedule; preconditioner maps do in their
+ * rounding only (whether their time integrals are summed from stored levels or
+ * step by step), and so do gradients where memory is too short for such a launch. */
 typedef struct {
     int shots_per_launch;   /* shots advanced together in one launch (>= 1) */
     int tile;               /* element-tile variant, 0..gbfwi_num_tiles()-1 */

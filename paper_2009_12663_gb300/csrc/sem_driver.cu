@@ -1140,8 +1140,13 @@ static int b0_from_map(gbfwi_mesh *m, const float *Hd, float *S1, float *S2, dou
 
 // Shots a resident map run takes at once (0: the preconditioner steps run). Both
 // passes keep their levels, so the batches are smaller than the steps' of Bold
-// shots; a step costs about 2 x 5.3 us resident, and 8 us forward (receiver maps) and
-// 38 us a wave of 304 CTAs otherwise (measured at 81 x 21 elements, 5 shots).
+// shots; a step costs about 5.3 us a launch resident, and 8 us forward (receiver maps) and
+// 36 to 51 us a wave of 304 CTAs otherwise.  P4 measured from levels and by steps, 24 shots in one
+// batch of steps: 40 x 20 elements, 300 steps: 3.8 and 13 ms; 81 x 21: 5.1 and 24 ms; 160 x 60, 200 steps
+// (batches of 8 from levels): 19 and 82 ms; 340 x 70, 600 steps (one by one): 183 and 577 ms.  The steps
+// win where few shots of a long run on a small mesh fit the memory for levels and
+// the schedule lets many run together (40 x 20, 16000 steps, 24 shots a launch: 3.27 and 0.69 s; one a launch:
+// 3.27 and 14.9 s).  Where both are close the rule loses 12% at most (81 x 21, 6000 steps, four streams).
 static int map_batch(gbfwi_mesh *m, int nshot, bool receiver, int tile, int Bold, long long NP)
 {
     const long long shot = (receiver ? 3 : 2) * (m->d.nt + 2LL) * NP * (long long)sizeof(float2);
