@@ -540,6 +540,10 @@ int plan_batches(gbfwi_mesh *m, std::initializer_list<int> modes, int nshot, int
     return GBFWI_OK;
 }
 
+// Most shots a call takes together beyond what its schedule asks for in one launch
+// (blockIdx.y counts the shots of a batch)
+constexpr long long kMostShots = 65535;
+
 // Shots of a batch where the resident loop takes it, and where it does not (`resident`
 // false: it is not asked).  A call prefers more shots at once than its schedule asks for;
 // where their buffers do not fit the memory that is left, it goes back to the schedule's
@@ -902,8 +906,8 @@ extern "C" int gbfwi_adjoint_gradient(gbfwi_mesh *m, const int *shot_ids, int ns
     const long long levels = full ? nt + 2 : 3LL * ((nt + ckpt - 1) / ckpt) + ckpt + 6;
     const long long small = kSmallHistory / (levels * NP * (long long)sizeof(float2));
     const int stepped = std::min(m->sch.shots_per_launch, nshot);
-    const int scheduled = (int)std::min<long long>(nshot, (long long)m->sch.shots_per_launch * m->sch.streams);
-    const int preferred = (int)std::min<long long>(nshot, std::max<long long>(scheduled, small));
+    const int scheduled = (int)std::min<long long>({nshot, (long long)m->sch.shots_per_launch * m->sch.streams, kMostShots});
+    const int preferred = (int)std::min<long long>({nshot, std::max<long long>(scheduled, small), kMostShots});
     const size_t eacc_shot = (size_t)m->d.nex * m->d.nez * 52 * sizeof(float);
     // per-shot accumulators and misfit partials, reduced once in shot order at
     // the end: the result does not depend on batching or lanes
@@ -1150,7 +1154,7 @@ static int b0_from_map(gbfwi_mesh *m, const float *Hd, float *S1, float *S2, dou
 static int map_batch(gbfwi_mesh *m, int nshot, bool receiver, int tile, int Bold, long long NP)
 {
     const long long shot = (receiver ? 3 : 2) * (m->d.nt + 2LL) * NP * (long long)sizeof(float2);
-    int B = (int)std::min<long long>(nshot, kMapHistory / shot);
+    int B = (int)std::min<long long>({nshot, kMapHistory / shot, kMostShots});
     if (B < 1 || !gb_resident_plan(m, MODE_FWD, B)) return 0;
     B = (nshot + (nshot + B - 1) / B - 1) / ((nshot + B - 1) / B);      // equal batches
     const int fwd = receiver ? MODE_FWD : MODE_FWD_PC, rcv = receiver ? MODE_RCV : fwd, last = sizes::last_batch(nshot, B);
@@ -1236,7 +1240,8 @@ extern "C" int gbfwi_precond_diag(gbfwi_mesh *m, const int *shot_ids, int nshot,
     const long long levels = !receiver ? 4 : ck <= 0 || ck >= nt ? nt + 6 : 3LL * ((nt + ck - 1) / ck) + ck + 10;
     const long long small = kSmallHistory / ((levels + 2) * NP * (long long)sizeof(float2));
     const int scheduled = std::min(m->sch.shots_per_launch, nshot);
-    const int preferred = (int)std::min<long long>(nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small));
+    const int preferred =
+        (int)std::min<long long>({nshot, std::max<long long>((long long)m->sch.shots_per_launch * m->sch.streams, small), kMostShots});
     const size_t seis_shot = (size_t)m->nrec * 2 * nt;
     const double dt = m->d.dt;
 

@@ -122,3 +122,22 @@ def test_records_where_a_batch_does_not_fit(nrec):
         assert torch.equal(one[0], seis[i]), i
     for kind in (1, 2):
         assert bool(torch.isfinite(raw_map(m, list(range(nshot)), kind)).all())
+
+
+def test_more_shots_than_a_grid_has_rows():
+    """70000 shots of the smallest kind fit the memory a call takes beyond its
+    schedule, but not one launch.  All equal: each gives the first one's part."""
+    nshot, nt = 70000, 2
+    m = mesh(5, 3, nt, nshot, nrec=2, same=True, shots_per_launch=2, streams=2)
+    ids = list(range(nshot))
+    obs = torch.ones(nshot, 2, 2, nt, device=DEV)
+    grad, one = (torch.zeros(3, m.nz, m.nx, device=DEV) for _ in range(2))
+    f1 = m.adjoint_gradient([0], obs[:1], one)
+    f = m.adjoint_gradient(ids, obs, grad)
+    assert f1 > 0 and abs(f - nshot * f1) <= 1e-15 * nshot * f    # one FP64 addition a shot
+    assert abs(m.misfit(ids, obs) - f) <= 1e-15 * nshot * f
+    # one FP32 addition a shot (their error grows like the number of equal terms: nshot 2^-24)
+    assert (grad - nshot * one).abs().max() <= nshot * 2.0 ** -24 * nshot * one.abs().max()
+    for kind in (1, 2):
+        raw, first = raw_map(m, ids, kind), raw_map(m, [0], kind)
+        assert (raw - nshot * first).abs().max() <= nshot * 2.0 ** -24 * nshot * first.max()
