@@ -37,19 +37,29 @@ def _signature(nex, nez, nshot, nrec, nt, gpu_name, space):
 
 def schedule_bytes(nx, nz, nshot, nrec, nt, spl, streams, ckpt):
     """Device bytes of gbfwi_adjoint_gradient's work buffers for a schedule
-    on the full time axis (the layout of sem_driver.cu)."""
+    on the full time axis (the layout of sem_driver.cu), the larger of its two
+    forms: the resident loop, whose one batch holds the shots of all lanes, with the
+    elements' strain sums and the exchange between tiles; and the step kernels
+    with a batch per lane.  (What the resident loop takes beyond its schedule it gives
+    back when memory is short.)"""
     pitch = (nx + 3) // 4 * 4
     NP = nz * pitch
+
+    def lane(B):
+        lev = B * NP * 8                               # one float2 time level of a batch
+        if ckpt <= 0 or ckpt >= nt:
+            hist = (nt + 2) * lev
+        else:
+            nseg = -(-nt // ckpt)
+            hist = (3 + ckpt + 2 + 1) * lev + nseg * 3 * lev
+        return hist + lev * (1 + 3 + 1) + B * nrec * 2 * nt * 4 + B * 5 * NP * 4
+
     B = min(spl, nshot)
     lanes = max(1, min(streams, -(-nshot // B)))
-    lev = B * NP * 8                                   # one float2 time level of a batch
-    if ckpt <= 0 or ckpt >= nt:
-        hist = (nt + 2) * lev
-    else:
-        nseg = -(-nt // ckpt)
-        hist = (3 + ckpt + 2 + 1) * lev + nseg * 3 * lev
-    per_lane = hist + lev * (1 + 3 + 1) + B * nrec * 2 * nt * 4 + B * 5 * NP * 4
-    return lanes * per_lane + nshot * 5 * NP * 4 + 5 * NP * 4 + nshot * nrec * 2 * nt * 4
+    together = min(spl * streams, nshot)
+    elements = (nx - 1) // 4 * ((nz - 1) // 4)
+    resident = lane(together) + together * (52 * 4 * elements + 32 * NP)
+    return max(lanes * lane(B), resident) + nshot * 5 * NP * 4 + 5 * NP * 4 + nshot * nrec * 2 * nt * 4
 
 
 def tune(nex, nez, h, dt, nt, sources, rec_xz, model, probe_nt=200, repeats=3, tiles=None,
