@@ -1518,7 +1518,7 @@ extern "C" int gbfwi_unet_train_step(gbfwi_unet *n, const float *x, const float 
     const long long P0 = npix(n, 0);
     const UnetLayer &O = n->layers.back();
     const long long xin = (long long)n->d.cin * P0, tin = (long long)n->d.cout * P0;
-    const bool dx = gb_is_device_ptr(x), dt = gb_is_device_ptr(target);
+    const bool dt = gb_is_device_ptr(target);
     GB_CUDA(cudaMemsetAsync(n->g32.p, 0, n->nparam * sizeof(float), s));
     GB_CUDA(cudaMemsetAsync(n->flag.p, 0, sizeof(int), s));
     if (batch > 1024) return GBFWI_EINVAL;
@@ -1546,7 +1546,6 @@ extern "C" int gbfwi_unet_train_step(gbfwi_unet *n, const float *x, const float 
         GB_LAUNCHED();
         GB_TRY(net_backward(n, nb, s));
     }
-    (void)dx;
     n->wt_fresh = false;                  // the Adam step below changes the weights
     n->step += 1;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -1584,9 +1583,7 @@ extern "C" int gbfwi_resample(const float *src, int channels, int sh, int sw, fl
         !gb_is_device_ptr(src) || !gb_is_device_ptr(dst))
         return GBFWI_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    GB_TRY(launch_resample(src, channels, sh, sw, dst, dh, dw, op, nullptr, 0, s));
-    GB_LAUNCHED();
-    return GBFWI_OK;
+    return launch_resample(src, channels, sh, sw, dst, dh, dw, op, nullptr, 0, s);
 }
 
 extern "C" int gbfwi_unet_features(gbfwi_mesh *m, const float *rho, const float *vp, const float *vs, double sigma_m,
