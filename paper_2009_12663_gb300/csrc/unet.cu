@@ -934,6 +934,7 @@ struct gbfwi_unet {
     long long nparam = 0;
     long long step = 0;                 // Adam steps taken
     DevBuf p32, g32, m32, v32, pb;      // master params, grads, Adam moments, bf16 copy
+    DevBuf arena;                       // holds the buffers of the samples, from xin32 to gb but for wt
     DevBuf xin32, xb, tgt32;            // input (FP32 staging, bf16), target staging
     DevBuf ea[kMaxLevels], e[kMaxLevels], pl[kMaxLevels], da[kMaxLevels], dd[kMaxLevels];
     DevBuf yout, gyb;                   // output [coutp][P0] FP32, its gradient (bf16)
@@ -1284,9 +1285,9 @@ int stage_input(gbfwi_unet *n, int nb, const float *x, cudaStream_t s)
     return GBFWI_OK;
 }
 
-// Activation and gradient buffers for nb samples.  The larger ones are allocated
-// beside those that are there and take their place together, so a failure leaves
-// the network with what it had (one sample's from its creation on).
+// Activation and gradient buffers for nb samples, pieces of one allocation.  The larger
+// one is made beside the one that is there and takes its place, so a failure
+// leaves the network with what it had (one sample's from its creation on).
 int reserve(gbfwi_unet *n, int nb)
 {
     if (nb <= n->nb) return GBFWI_OK;
@@ -1294,7 +1295,11 @@ int reserve(gbfwi_unet *n, int nb)
     const long long P0 = npix(n, 0);
     const UnetLayer &O = n->layers.back();
     std::vector<std::pair<DevBuf *, size_t>> list;
-    auto need = [&](DevBuf &b, long long bytes) { list.push_back({&b, (size_t)std::max<long long>(bytes * nb, 16)}); };
+    size_t total = 0;
+    auto need = [&](DevBuf &b, long long bytes) {
+        list.push_back({&b, (size_t)(bytes * nb + 255) / 256 * 256});
+        total += list.back().second;
+    };
     const size_t F = sizeof(float), B2 = sizeof(bf16);
     need(n->xin32, (long long)n->d.cin * P0 * F);
     need(n->xb, (long long)n->d.cin * P0 * B2);
@@ -1318,11 +1323,14 @@ int reserve(gbfwi_unet *n, int nb)
     need(n->fP, cmax * F);
     need(n->gb, cmax * B2);
     need(n->rsum, (long long)std::max(n->ch[Lv - 1], O.coutp) * F);
-    std::vector<DevBuf> fresh(list.size());
-    for (size_t i = 0; i < list.size(); ++i) GB_TRY(fresh[i].ensure(list[i].second));
-    for (size_t i = 0; i < list.size(); ++i) {
-        std::swap(list[i].first->p, fresh[i].p);
-        std::swap(list[i].first->bytes, fresh[i].bytes);
+    DevBuf fresh;
+    GB_TRY(fresh.ensure(total));
+    std::swap(n->arena.p, fresh.p);
+    std::swap(n->arena.bytes, fresh.bytes);
+    size_t at = 0;
+    for (const auto &piece : list) {
+        piece.first->lend(n->arena.as<char>() + at, piece.second);
+        at += piece.second;
     }
     n->nb = nb;
     return GBFWI_OK;
