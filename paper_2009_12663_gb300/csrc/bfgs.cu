@@ -84,9 +84,12 @@ __device__ __forceinline__ void dot2_term(float a, float b, float &hi, float &lo
 // The sums of eight rows are then reduced together over the warp in
 // compensated pairs, each exchange halving the values a lane holds: 9 merges
 // instead of 40, and FP32 ones (the FP64 pipe takes 16 cycles a warp
-// instruction); FP64 only over the warps.  Bound by the row reads (459 MB for
-// 100 rows of n = 1,147,323): 108 us, 317 us with each row reduced in FP64,
-// 160 us with a CTA per row and chunk, which reads the column again for each row.
+// instruction); FP64 only over the warps.  Against exact sums the error is 0.1e-16
+// to 7e-16 of the sum of moduli, 0.1e-16 to 3e-16 with an FP64 tree over the threads.
+// 100 rows of n = 1,147,323 (459 MB) take 108 us, 63% of the measured HBM rate (317 us
+// with each row reduced in FP64, 160 us with a CTA per row and chunk, which
+// reads the column again for each row): the 16 warps an SM that its registers allow
+// wait for their loads half of the time, at 43% of the issue slots.
 // part[chunk][a][b] is summed over the chunks by thin_reduce.
 constexpr int kThinChunk = 4096;           // elements of a chunk: 256 threads x 16
 

@@ -9,10 +9,11 @@
 // the resident loop needs 4.5 us.  Here the passes only store their levels (the
 // displacement, and one field's acceleration), and the integrals are sums over
 // time at fixed nodes and elements: a thread keeps its sums in registers and
-// streams through the levels (800 steps of those 5 shots: 0.85 ms for the
-// strains, 0.36 ms at the nodes, beside 7.1 ms for the two passes).  Bound by
-// those reads (16 B a node, level and field) and, for the strains, by the few
-// warps their registers allow.
+// streams through the levels (800 steps of those 5 shots: 0.61 ms for the strains
+// and 0.02 ms for their assembly, 0.36 ms at the nodes, beside 7.0 ms for the
+// two passes).  Bound by those reads (16 B a node, level and field) and, for the
+// strains, by the few warps their registers allow: 14 chunks of time there; five took
+// 0.85 ms.
 //
 // S0 = sum a . a (one field) or sum (second difference of u) . a, at nodes;
 // S1..S3 = sums of [div div', exx exx' + ezz ezz', gam gam'] of the
